@@ -7,6 +7,7 @@
 
 #include "kmv.cuh"
 #include "kmv_dispatch.cuh"
+#include "kmvfix_kernels.cuh"
 #include "kmvtc_kernels.cuh"
 
 namespace krr {
@@ -223,17 +224,40 @@ static ExpFFConsts make_exp_consts() {
 }
 
 // ---------------------------------------------------------- reduction
-template <typename T, int MAXM>
-__global__ void kmv_reduce_kernel(const T *__restrict__ part, int splits, int M,
-                                  int64_t N, int m, T lambda, const T *__restrict__ V,
-                                  int64_t ldv, T *__restrict__ Y, int64_t ldy) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= N) return;
-  for (int c = 0; c < m; ++c) {
-    T acc = 0;
-    for (int sp = 0; sp < splits; ++sp) acc += part[((int64_t)sp * M + c) * N + i];
-    Y[(int64_t)c * ldy + i] = V ? acc + lambda * V[(int64_t)c * ldv + i] : acc;
+// Y = the sum of the splits' partial sums (+ lambda V).  A block takes 32
+// rows; its 8 warps take every eighth split each and the warps' sums are
+// added in warp order, so a small N with many splits neither leaves the GPU
+// to a few threads nor chains all the loads in one thread (N = 4096, 64
+// splits: 7.4 us with one thread a row and column, 3.6 us this way).
+constexpr int KRED_WARPS = 8;
+template <typename T>
+__global__ void __launch_bounds__(32 * KRED_WARPS)
+kmv_reduce_kernel(const T *__restrict__ part, int splits, int M, int64_t N, T lambda,
+                  const T *__restrict__ V, int64_t ldv, T *__restrict__ Y, int64_t ldy) {
+  __shared__ T red[KRED_WARPS][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t i = (int64_t)blockIdx.x * 32 + lane;
+  const int c = blockIdx.y;
+  T acc = 0;
+  if (i < N) {
+#pragma unroll 4
+    for (int sp = warp; sp < splits; sp += KRED_WARPS) acc += part[((int64_t)sp * M + c) * N + i];
   }
+  red[warp][lane] = acc;
+  __syncthreads();
+  if (warp != 0 || i >= N) return;
+#pragma unroll
+  for (int w = 1; w < KRED_WARPS; ++w) acc += red[w][lane];
+  Y[(int64_t)c * ldy + i] = V ? acc + lambda * V[(int64_t)c * ldv + i] : acc;
+}
+
+template <typename T>
+static krr_status kmv_reduce(const T *part, int splits, int M, int64_t N, int m, T lambda,
+                             const T *V, int64_t ldv, T *Y, int64_t ldy, cudaStream_t s) {
+  kmv_reduce_kernel<T><<<dim3(ceil_div(N, 32), m), 32 * KRED_WARPS, 0, s>>>(
+      part, splits, M, N, lambda, V, ldv, Y, ldy);
+  KRR_LAUNCH_CHECK();
+  return KRR_OK;
 }
 
 static int pad_m(int m) {
@@ -380,9 +404,7 @@ static krr_status kmv_tc(const PointsF32 &P, float lambda, const float *V, int64
       set_error("tensor-core product launch failed: %s", cudaGetErrorString(e));
       return KRR_ECUDA;
     }
-    kmv_reduce_kernel<float, 16><<<ceil_div(N, 256), 256, 0, s>>>(
-        part.p, nsplit, M, N, mg, lambda, Vg, ldv, Y + (int64_t)c0 * ldy, ldy);
-    KRR_LAUNCH_CHECK();
+    KRR_TRY(kmv_reduce<float>(part.p, nsplit, M, N, mg, lambda, Vg, ldv, Y + (int64_t)c0 * ldy, ldy, s));
   }
   return KRR_OK;
 }
@@ -421,45 +443,68 @@ krr_status kmv_f32(const PointsF32 &P, float lambda, const float *V, int64_t ldv
       set_error("fused product launch failed: %s", cudaGetErrorString(e));
       return KRR_ECUDA;
     }
-    kmv_reduce_kernel<float, 16><<<ceil_div(N, 256), 256, 0, s>>>(
-        part.p, nsplit, M, N, mg, lambda, Vg, ldv, Y + (int64_t)c0 * ldy, ldy);
-    KRR_LAUNCH_CHECK();
+    KRR_TRY(kmv_reduce<float>(part.p, nsplit, M, N, mg, lambda, Vg, ldv, Y + (int64_t)c0 * ldy, ldy, s));
   }
   return KRR_OK;
 }
 
-krr_status kmv_f64(const double *Xd, int64_t N, int d, int kern, double sigma,
-                   double lambda, const double *V, int64_t ldv, int m, double *Y,
-                   int64_t ldy, cudaStream_t s, DevBuf<double> &part) {
-  if (N == 0 || m == 0) return KRR_OK;
+cudaError_t launch_kmvfix_any(int kern, int DP, int M, dim3 grid, cudaStream_t s,
+                              const KmvFixArgs &a);
+
+// Float64 product between row points (Xr, ur) and column points (Xc, uc) of
+// one scale; known as in PointsF64.
+static krr_status f64_products(const double *Xr, const int2 *ur, int64_t Nr, const double *Xc,
+                               const int2 *uc, int64_t N, int d, int kern, double sigma,
+                               const FixScale *scale, int known, double lambda, bool shift,
+                               const double *V, int64_t ldv, int m, double *Y, int64_t ldy, cudaStream_t s,
+                               DevBuf<double> &part) {
   const int dp = (d + 3) / 4 * 4;
-  double inv_scale = (kern == KGAUSS) ? 1.0 / (2.0 * sigma * sigma) : 1.0 / sigma;
+  const double inv_scale = (kern == KGAUSS) ? 1.0 / (2.0 * sigma * sigma) : 1.0 / sigma;
   for (int c0 = 0; c0 < m; c0 += 16) {
     const int mg = (m - c0 < 16) ? (m - c0) : 16;
     const int M = pad_m(mg);
-    const int64_t row_tiles = (N + KMV64_THREADS - 1) / KMV64_THREADS;
-    const int splits = choose_splits(row_tiles, N, KMV64_TJ, 4, 4);
-    int64_t chunk = (N + splits - 1) / splits;
-    chunk = (chunk + KMV64_TJ - 1) / KMV64_TJ * KMV64_TJ;
-    const int nsplit = (int)((N + chunk - 1) / chunk);
-    const size_t need = (size_t)nsplit * M * N;
+    const double *Vg = V + (int64_t)c0 * ldv;
+    // one grid for both kernels, so that their partial sums have one layout:
+    // about two waves of eight fixed-point CTAs a SM
+    const int rows = KFIX_THREADS * kmvfix_rows_per_thread(dp);
+    const int64_t fix_tiles = (Nr + rows - 1) / rows;
+    const int splits = choose_splits(fix_tiles, N, KFIX_TJ, 8, 2);
+    int64_t chunk;
+    int nsplit;
+    split_shape(N, splits, KFIX_TJ, &chunk, &nsplit);
+    const size_t need = (size_t)nsplit * M * Nr;
     if (part.n < need) KRR_TRY(part.alloc(need, s));
-    Kmv64Args a{Xd, N, Xd, d, V + (int64_t)c0 * ldv, ldv, N, mg, chunk, inv_scale, part.p};
     KmvTimer tm(1);
     tm.begin(s);
-    cudaError_t e = launch_kmv64_any(kern, dp, M, dim3((unsigned)row_tiles, nsplit), s, a);
+    cudaError_t e = cudaSuccess;
+    if (known != 0) {
+      const KmvFixArgs a{ur, Nr, uc, scale, Vg, ldv, N, mg, chunk, part.p};
+      e = launch_kmvfix_any(kern, dp, M, dim3((unsigned)fix_tiles, nsplit), s, a);
+      count_launch();
+    }
+    if (known != 1 && e == cudaSuccess) {
+      const int64_t row_tiles = (Nr + KMV64_THREADS - 1) / KMV64_THREADS;
+      const Kmv64Args a{Xr, Nr, Xc, d, Vg, ldv, N, mg, chunk, inv_scale, part.p,
+                        known < 0 ? scale : nullptr};
+      e = launch_kmv64_any(kern, dp, M, dim3((unsigned)row_tiles, nsplit), s, a);
+      count_launch();
+    }
     tm.end(s);
-    count_launch();
     if (e != cudaSuccess) {
       set_error("float64 product launch failed: %s", cudaGetErrorString(e));
       return KRR_ECUDA;
     }
-    kmv_reduce_kernel<double, 16><<<ceil_div(N, 256), 256, 0, s>>>(
-        part.p, nsplit, M, N, mg, lambda, V + (int64_t)c0 * ldv, ldv,
-        Y + (int64_t)c0 * ldy, ldy);
-    KRR_LAUNCH_CHECK();
+    KRR_TRY(kmv_reduce<double>(part.p, nsplit, M, Nr, mg, lambda, shift ? Vg : nullptr, ldv,
+                               Y + (int64_t)c0 * ldy, ldy, s));
   }
   return KRR_OK;
+}
+
+krr_status kmv_f64(const PointsF64 &P, double lambda, const double *V, int64_t ldv, int m,
+                   double *Y, int64_t ldy, cudaStream_t s, DevBuf<double> &part) {
+  if (P.N == 0 || m == 0) return KRR_OK;
+  return f64_products(P.X, P.u.p, P.N, P.X, P.u.p, P.N, P.d, P.kern, P.sigma, P.scale.p, P.known,
+                      lambda, true, V, ldv, m, Y, ldy, s, part);
 }
 
 __global__ void kmvffsym_reduce_kernel(const double *__restrict__ rowpart,
@@ -576,10 +621,7 @@ krr_status kff_cross(const PointsFF &R, const PointsFF &P, double lambda, const 
       set_error("float-float product launch failed: %s", cudaGetErrorString(e));
       return KRR_ECUDA;
     }
-    kmv_reduce_kernel<double, 16><<<ceil_div(Nr, 256), 256, 0, s>>>(
-        part.p, nsplit, M, Nr, mg, square ? lambda : 0.0,
-        square ? V + (int64_t)c0 * ldv : nullptr, ldv, Y + (int64_t)c0 * ldy, ldy);
-    KRR_LAUNCH_CHECK();
+    KRR_TRY(kmv_reduce<double>(part.p, nsplit, M, Nr, mg, square ? lambda : 0.0, square ? V + (int64_t)c0 * ldv : nullptr, ldv, Y + (int64_t)c0 * ldy, ldy, s));
   }
   return KRR_OK;
 }
@@ -614,9 +656,7 @@ krr_status kcross_f32(const PointsF32 &R, const PointsF32 &P, const float *V, in
       set_error("prediction product launch failed: %s", cudaGetErrorString(e));
       return KRR_ECUDA;
     }
-    kmv_reduce_kernel<float, 16><<<ceil_div(Nr, 256), 256, 0, s>>>(
-        part.p, nsplit, M, Nr, mg, 0.0f, nullptr, 0, Y + (int64_t)c0 * ldy, ldy);
-    KRR_LAUNCH_CHECK();
+    KRR_TRY(kmv_reduce<float>(part.p, nsplit, M, Nr, mg, 0.0f, nullptr, 0, Y + (int64_t)c0 * ldy, ldy, s));
   }
   return KRR_OK;
 }
@@ -625,30 +665,13 @@ krr_status kcross_f64(const double *Xr, int64_t Nr, const double *Xd, int64_t N,
                       int kern, double sigma, const double *V, int64_t ldv, int m, double *Y,
                       int64_t ldy, cudaStream_t s, DevBuf<double> &part) {
   if (N == 0 || Nr == 0 || m == 0) return KRR_OK;
-  const int dp = (d + 3) / 4 * 4;
-  double inv_scale = (kern == KGAUSS) ? 1.0 / (2.0 * sigma * sigma) : 1.0 / sigma;
-  for (int c0 = 0; c0 < m; c0 += 16) {
-    const int mg = (m - c0 < 16) ? (m - c0) : 16;
-    const int M = pad_m(mg);
-    const int64_t row_tiles = (Nr + KMV64_THREADS - 1) / KMV64_THREADS;
-    const int splits = choose_splits(row_tiles, N, KMV64_TJ, 4, 4);
-    int64_t chunk = (N + splits - 1) / splits;
-    chunk = (chunk + KMV64_TJ - 1) / KMV64_TJ * KMV64_TJ;
-    const int nsplit = (int)((N + chunk - 1) / chunk);
-    const size_t need = (size_t)nsplit * M * Nr;
-    if (part.n < need) KRR_TRY(part.alloc(need, s));
-    Kmv64Args a{Xr, Nr, Xd, d, V + (int64_t)c0 * ldv, ldv, N, mg, chunk, inv_scale, part.p};
-    cudaError_t e = launch_kmv64_any(kern, dp, M, dim3((unsigned)row_tiles, nsplit), s, a);
-    count_launch();
-    if (e != cudaSuccess) {
-      set_error("prediction product launch failed: %s", cudaGetErrorString(e));
-      return KRR_ECUDA;
-    }
-    kmv_reduce_kernel<double, 16><<<ceil_div(Nr, 256), 256, 0, s>>>(
-        part.p, nsplit, M, Nr, mg, 0.0, nullptr, 0, Y + (int64_t)c0 * ldy, ldy);
-    KRR_LAUNCH_CHECK();
-  }
-  return KRR_OK;
+  DevBuf<FixScale> scale;
+  DevBuf<int2> ur, uc;
+  KRR_TRY(fix_scale(Xr, Nr, Xd, N, d, kern, sigma, s, scale));
+  KRR_TRY(fix_points(Xr, Nr, d, kern, scale.p, s, ur));
+  KRR_TRY(fix_points(Xd, N, d, kern, scale.p, s, uc));
+  return f64_products(Xr, ur.p, Nr, Xd, uc.p, N, d, kern, sigma, scale.p, -1, 0.0, false, V, ldv,
+                      m, Y, ldy, s, part);
 }
 
 // Same product with caller-provided split scratch of `scratch_elems` doubles:
@@ -676,17 +699,15 @@ krr_status kmv_f64_with_scratch(const double *Xd, int64_t N, int d, int kern, do
     int64_t chunk = (N + splits - 1) / splits;
     chunk = (chunk + KMV64_TJ - 1) / KMV64_TJ * KMV64_TJ;
     const int nsplit = (int)((N + chunk - 1) / chunk);
-    Kmv64Args a{Xd, N, Xd, d, V + (int64_t)c0 * ldv, ldv, N, mg, chunk, inv_scale, scratch};
+    Kmv64Args a{Xd, N, Xd, d, V + (int64_t)c0 * ldv, ldv, N, mg, chunk, inv_scale, scratch,
+                nullptr};
     cudaError_t e = launch_kmv64_any(kern, dp, M, dim3((unsigned)row_tiles, nsplit), s, a);
     count_launch();
     if (e != cudaSuccess) {
       set_error("float64 product launch failed: %s", cudaGetErrorString(e));
       return KRR_ECUDA;
     }
-    kmv_reduce_kernel<double, 16><<<ceil_div(N, 256), 256, 0, s>>>(
-        scratch, nsplit, M, N, mg, lambda, V + (int64_t)c0 * ldv, ldv,
-        Y + (int64_t)c0 * ldy, ldy);
-    KRR_LAUNCH_CHECK();
+    KRR_TRY(kmv_reduce<double>(scratch, nsplit, M, N, mg, lambda, V + (int64_t)c0 * ldv, ldv, Y + (int64_t)c0 * ldy, ldy, s));
   }
   return KRR_OK;
 }
@@ -728,34 +749,34 @@ krr_status convert_f32_to_f64(const float *src, double *dst, int64_t n, cudaStre
 }
 
 // ---------------------------------------------------- kernel columns
-// One thread per (row, column) pair; the selected points are staged in
-// shared memory (nc <= 128 points of <= 32 coordinates).
+// One thread per row and 32 columns a CTA; the float64 form, for point sets
+// whose range does not allow the fixed-point one.
 __global__ void kernel_columns_kernel(const double *__restrict__ X, int64_t N, int d,
                                       int kern, double sigma,
                                       const int64_t *__restrict__ cols, int nc,
-                                      double *__restrict__ G, int64_t ldg) {
-  extern __shared__ double sp[];
-  for (int idx = threadIdx.x; idx < nc * d; idx += blockDim.x)
-    sp[idx] = X[cols[idx / d] * d + idx % d];
+                                      double *__restrict__ G, int64_t ldg,
+                                      const FixScale *__restrict__ scale) {
+  __shared__ double sp[32 * 32];
+  if (scale->ok) return;
+  const int c0 = blockIdx.y * 32, cn = min(32, nc - c0);
+  for (int idx = threadIdx.x; idx < cn * d; idx += blockDim.x)
+    sp[idx] = X[cols[c0 + idx / d] * d + idx % d];
   __syncthreads();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= N) return;
   double xi[32];
   for (int k = 0; k < d; ++k) xi[k] = X[i * d + k];
-  for (int c = 0; c < nc; ++c)
-    G[(int64_t)c * ldg + i] = kappa_point_f64(xi, sp + c * d, d, kern, sigma);
+  for (int c = 0; c < cn; ++c)
+    G[(int64_t)(c0 + c) * ldg + i] = kappa_point_f64(xi, sp + c * d, d, kern, sigma);
 }
 
-krr_status kernel_columns_f64(const double *Xd, int64_t N, int d, int kern, double sigma,
-                              const int64_t *cols, int nc, double *G, int64_t ldg,
-                              cudaStream_t s) {
-  if (nc == 0 || N == 0) return KRR_OK;
-  for (int c0 = 0; c0 < nc; c0 += 128) {
-    const int ncg = (nc - c0 < 128) ? nc - c0 : 128;
-    const size_t smem = (size_t)ncg * d * sizeof(double);
-    KRR_TRY(raise_smem_limit(kernel_columns_kernel, smem));
-    kernel_columns_kernel<<<ceil_div(N, 128), 128, smem, s>>>(
-        Xd, N, d, kern, sigma, cols + c0, ncg, G + (int64_t)c0 * ldg, ldg);
+krr_status kernel_columns_f64(const PointsF64 &P, const int64_t *cols, int nc, double *G,
+                              int64_t ldg, cudaStream_t s) {
+  if (nc == 0 || P.N == 0) return KRR_OK;
+  if (P.known != 0) KRR_TRY(kfix_columns(P, cols, nc, G, ldg, s));
+  if (P.known != 1) {
+    kernel_columns_kernel<<<dim3(ceil_div(P.N, 128), ceil_div(nc, 32)), 128, 0, s>>>(
+        P.X, P.N, P.d, P.kern, P.sigma, cols, nc, G, ldg, P.scale.p);
     KRR_LAUNCH_CHECK();
   }
   return KRR_OK;

@@ -4,6 +4,7 @@
 #include <cuda.h>
 
 #include "common.cuh"
+#include "kfix.cuh"
 
 namespace krr {
 
@@ -92,6 +93,39 @@ int kmvtc_rows_per_cta(int KC, int M);
 void set_product_path(int path);
 int product_path();
 
+// Points of the float64 products: the caller's array and its fixed-point
+// coordinates (kfix.cuh).  Whether the range of the points allows the
+// fixed-point kernels is known on the device only (scale->ok) until a caller
+// waits for it: known is 1 or 0 then, -1 before, when a product launches both
+// kernels and the one that does not apply returns at once.
+struct PointsF64 {
+  const double *X = nullptr;
+  int64_t N = 0;
+  int d = 0;
+  int kern = 0;
+  double sigma = 0.0;
+  DevBuf<FixScale> scale;
+  DevBuf<int2> u;       // N x dp, dp = d rounded up to a multiple of 4
+  int known = -1;
+};
+
+// wait: read scale->ok back (synchronises s), for points that serve many
+// launches.
+krr_status prepare_points_f64(const double *Xd, int64_t N, int d, int kern, double sigma,
+                              cudaStream_t s, PointsF64 &P, bool wait);
+
+// Common scale of one or two point sets (B may be NULL) and the integer
+// coordinates of one set under it.
+krr_status fix_scale(const double *A, int64_t na, const double *B, int64_t nb, int d, int kern,
+                     double sigma, cudaStream_t s, DevBuf<FixScale> &out);
+krr_status fix_points(const double *Xd, int64_t N, int d, int kern, const FixScale *scale,
+                      cudaStream_t s, DevBuf<int2> &u);
+
+// G (nc columns, ld ldg) = A(:, cols) from fixed-point coordinates; writes
+// nothing when the range does not allow them.
+krr_status kfix_columns(const PointsF64 &P, const int64_t *cols, int nc, double *G, int64_t ldg,
+                        cudaStream_t s);
+
 // Prediction products (no shift): Y (Nr x m) = K(rows, columns) V.
 krr_status kcross_f32(const PointsF32 &R, const PointsF32 &P, const float *V, int64_t ldv,
                       int m, float *Y, int64_t ldy, cudaStream_t s, DevBuf<float> &part);
@@ -135,10 +169,9 @@ int tuned_splits(int kern, int dp, int M, int64_t N);
 krr_status kmv_f32(const PointsF32 &P, float lambda, const float *V, int64_t ldv,
                    int m, float *Y, int64_t ldy, cudaStream_t s, DevBuf<float> &part);
 
-// Y (m x ldy, float64) = (A + lambda I) V (m x ldv, float64); Xd N x d float64.
-krr_status kmv_f64(const double *Xd, int64_t N, int d, int kern, double sigma,
-                   double lambda, const double *V, int64_t ldv, int m, double *Y,
-                   int64_t ldy, cudaStream_t s, DevBuf<double> &part);
+// Y (m x ldy, float64) = (A + lambda I) V (m x ldv, float64).
+krr_status kmv_f64(const PointsF64 &P, double lambda, const double *V, int64_t ldv, int m,
+                   double *Y, int64_t ldy, cudaStream_t s, DevBuf<double> &part);
 
 // kmv_f64 with caller-provided scratch for the split partial sums (no
 // allocation); KRR_EINVAL if N x padded(m) exceeds scratch_elems.
@@ -183,8 +216,7 @@ __device__ __forceinline__ double kappa_point_f64(const double *a, const double 
 }
 
 // G (nc x ldg column-major, rows 0..N-1) = A(:, cols), float64.
-krr_status kernel_columns_f64(const double *Xd, int64_t N, int d, int kern,
-                              double sigma, const int64_t *cols, int nc, double *G,
+krr_status kernel_columns_f64(const PointsF64 &P, const int64_t *cols, int nc, double *G,
                               int64_t ldg, cudaStream_t s);
 
 // out[i] = kappa(x_i, x_i) for all i (float64).

@@ -33,6 +33,7 @@ struct Kmv64Args {
   int64_t chunk;
   double inv_scale;
   double *part;
+  const FixScale *scale;   // may be NULL, see kmv64_kernel
 };
 
 template <int KERN, int DP>
@@ -75,7 +76,7 @@ cudaError_t launch_kmv64_m(int M, dim3 grid, cudaStream_t s, const Kmv64Args &a)
     kmv64_kernel<KERN, DP, MM><<<grid, KMV64_THREADS, 0, s>>>(a.Xr, a.Nr, a.X, a.d,  \
                                                              a.V, a.ldv, a.N, a.m,  \
                                                              a.chunk, a.inv_scale,  \
-                                                             a.part);               \
+                                                             a.part, a.scale);      \
     break;
     KRR_CASE(1) KRR_CASE(2) KRR_CASE(4) KRR_CASE(8) KRR_CASE(16)
 #undef KRR_CASE

@@ -23,6 +23,7 @@
 #pragma once
 
 #include "common.cuh"
+#include "kfix.cuh"
 
 namespace krr {
 
@@ -268,13 +269,16 @@ __device__ __forceinline__ double kappa_f64(double s, double inv_scale) {
 }
 
 // Xr (Nr x d) row points; X (N x d) column points; part: splits x M x Nr.
+// scale (optional): returns at once when the fixed-point kernel has done the
+// product (kmvfix_kernels.cuh).
 template <int KERN, int DP, int M>
 __global__ void __launch_bounds__(KMV64_THREADS)
 kmv64_kernel(const double *__restrict__ Xr, int64_t Nr, const double *__restrict__ X, int d,
              const double *__restrict__ V, int64_t ldv, int64_t N, int m, int64_t chunk,
-             double inv_scale, double *__restrict__ part) {
+             double inv_scale, double *__restrict__ part, const FixScale *__restrict__ scale) {
   __shared__ double sx[KMV64_TJ][DP];
   __shared__ double sv[KMV64_TJ][M];
+  if (scale && scale->ok) return;
   const int tid = threadIdx.x;
   const int64_t i = (int64_t)blockIdx.x * KMV64_THREADS + tid;
   const int64_t j_begin = (int64_t)blockIdx.y * chunk;

@@ -389,7 +389,8 @@ krr_status rpcholesky_device(const double *Xd, int64_t N, int d, int kern, doubl
   KRR_LAUNCH_CHECK();
   double maxdiag = 0.0;
   KRR_CUDA_TRY(cudaMemcpyAsync(&maxdiag, maxd.p, sizeof(double), cudaMemcpyDeviceToHost, s));
-  KRR_CUDA_TRY(cudaStreamSynchronize(s));
+  PointsF64 P64;   // waits for s
+  KRR_TRY(prepare_points_f64(Xd, N, d, kern, sigma, s, P64, true));
   const double thr = (double)N * 2.220446049250313e-16 * maxdiag;
 
   DevBuf<int64_t> draws, cand;
@@ -452,7 +453,7 @@ krr_status rpcholesky_device(const double *Xd, int64_t N, int d, int kern, doubl
       nc = hcounts[1];
     }
     // G = A(:, S') - F(:, 0:rank) F(S', 0:rank)^T
-    KRR_TRY(kernel_columns_f64(Xd, N, d, kern, sigma, cand.p, nc, G.p, N, s));
+    KRR_TRY(kernel_columns_f64(P64, cand.p, nc, G.p, N, s));
     if (rank > 0) {
       gather_rows_kernel<<<ceil_div((int64_t)nc * rank, 256), 256, 0, s>>>(f->F, N, rank,
                                                                          cand.p, nc, Fs.p);

@@ -80,11 +80,13 @@ krr_status pcg_solve_device(const double *Xd, int64_t N, int d, int kern, double
     DevBuf<double> part;
     DevBuf<float> vsplit;
     PointsFF Pff;
+    PointsF64 P64;
     const bool ff = (prec == KRR_PREC_FLOAT_FLOAT);
     if (ff) KRR_TRY(prepare_points_ff(Xd, N, d, kern, sigma, s, Pff));
+    else KRR_TRY(prepare_points_f64(Xd, N, d, kern, sigma, s, P64, true));
     auto product = [&](const double *in, double *out, cudaStream_t st) {
       if (ff) return kmv_ff(Pff, lambda, in, N, m, out, N, st, part, vsplit);
-      return kmv_f64(Xd, N, d, kern, sigma, lambda, in, N, m, out, N, st, part);
+      return kmv_f64(P64, lambda, in, N, m, out, N, st, part);
     };
     PcgOps<double> ops;
     PrecondWs pws;
@@ -524,10 +526,10 @@ krr_status escalate_refine(Escalation &e, cudaStream_t s) {
   // from the float64 product
   bool res64 = false;
   const double *Xdev = nullptr;
+  PointsF64 P64;
   auto residual = [&]() -> krr_status {
     if (res64)
-      KRR_TRY(kmv_f64(Xdev, N, e.d, e.kern, e.sigma, e.lambda, e.alpha, N, m, e.mx, N, s,
-                      part64));
+      KRR_TRY(kmv_f64(P64, e.lambda, e.alpha, N, m, e.mx, N, s, part64));
     else
       KRR_TRY(kmv_ff(*e.Pff, e.lambda, e.alpha, N, m, e.mx, N, s, *e.ffpart, *e.ffvsplit));
     e.entries += kmv_entries(N);
@@ -545,6 +547,7 @@ krr_status escalate_refine(Escalation &e, cudaStream_t s) {
       if (res64) break;
       res64 = true;
       KRR_TRY(device_view(e.X, (size_t)N * e.d, s, X64, &Xdev));
+      KRR_TRY(prepare_points_f64(Xdev, N, e.d, e.kern, e.sigma, s, P64, true));
       KRR_TRY(residual());
       worst = escalation_worst(e);
       e.relres = worst;
