@@ -53,6 +53,45 @@ static thread_local cudaStream_t g_alloc_stream = nullptr;
 void set_alloc_stream(cudaStream_t s) { g_alloc_stream = s; }
 cudaStream_t alloc_stream() { return g_alloc_stream; }
 
+cudaError_t pool_malloc(void **p, size_t bytes, cudaStream_t s) {
+  constexpr int kMaxDevices = 64;
+  static std::mutex mtx;
+  static cudaMemPool_t pools[kMaxDevices] = {};
+  static bool tried[kMaxDevices] = {};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  cudaMemPool_t pool = nullptr;
+  if (dev >= 0 && dev < kMaxDevices) {
+    std::lock_guard<std::mutex> lk(mtx);
+    if (!tried[dev]) {
+      tried[dev] = true;
+      cudaMemPoolProps props = {};
+      props.allocType = cudaMemAllocationTypePinned;
+      props.location.type = cudaMemLocationTypeDevice;
+      props.location.id = dev;
+      unsigned long long keep = kPoolKeepBytes;
+      cudaMemPool_t np = nullptr;
+      if (cudaMemPoolCreate(&np, &props) == cudaSuccess) {
+        if (cudaMemPoolSetAttribute(np, cudaMemPoolAttrReleaseThreshold, &keep) == cudaSuccess)
+          pools[dev] = np;
+        else
+          cudaMemPoolDestroy(np);
+      }
+      cudaGetLastError();
+    }
+    pool = pools[dev];
+  }
+  if (pool) {
+    e = cudaMallocFromPoolAsync(p, bytes, pool, s);
+    if (e == cudaSuccess) return e;
+    cudaGetLastError();
+    cudaMemPoolTrimTo(pool, 0);
+    cudaGetLastError();
+  }
+  return cudaMallocAsync(p, bytes, s);
+}
+
 bool is_device_ptr(const void *p) {
   if (!p) return false;
   cudaPointerAttributes a;
@@ -362,16 +401,19 @@ krr_status krr_kmatvec(const double *X, int64_t N, int d, krr_kernel kern, doubl
     DevBuf<float> vsplit;
     KRR_TRY(kmv_ff(P, lambda, Vd, N, m, out.dev, N, s, part, vsplit));
   } else {
-    PointsF32 P;
-    KRR_TRY(prepare_points_f32(Xd, N, d, kern, sigma, s, P));
-    KRR_TRY(prepare_points_tc(Xd, s, P));
-    DevBuf<float> v32, y32, part;
-    KRR_TRY(v32.alloc((size_t)N * m, s));
-    KRR_TRY(y32.alloc((size_t)N * m, s));
-    KRR_TRY(convert_f64_to_f32(Vd, v32.p, N * m, s));
-    KRR_TRY(kmv_f32(P, (float)lambda, v32.p, N, m, y32.p, N, s, part));
-    KRR_TRY(tc5_check_fault(s));
-    KRR_TRY(convert_f32_to_f64(y32.p, out.dev, N * m, s));
+    bool done = false;
+    KRR_TRY(kmv_tc5_call(nullptr, 0, Xd, N, d, kern, sigma, lambda, Vd, m, out.dev, s, &done));
+    if (!done) {
+      PointsF32 P;
+      KRR_TRY(prepare_points_product(Xd, N, d, kern, sigma, s, P));
+      DevBuf<float> v32, y32, part;
+      KRR_TRY(v32.alloc((size_t)N * m, s));
+      KRR_TRY(y32.alloc((size_t)N * m, s));
+      KRR_TRY(convert_f64_to_f32(Vd, v32.p, N * m, s));
+      KRR_TRY(kmv_f32(P, (float)lambda, v32.p, N, m, y32.p, N, s, part));
+      KRR_TRY(convert_f32_to_f64(y32.p, out.dev, N * m, s));
+      if (P.nh5 > 0) KRR_TRY(tc5_check_fault(s));
+    }
   }
   return out.finish(s);
 }
@@ -435,28 +477,20 @@ krr_status krr_predict(const double *Xtrain, int64_t N, int d, krr_kernel kern, 
     DevBuf<double> part;
     KRR_TRY(kcross_f64(Td, Nt, Xd, N, d, kern, sigma, Ad, N, m, o.dev, Nt, s, part));
   } else {
-    PointsF32 P, R;
-    KRR_TRY(prepare_points_f32(Xd, N, d, kern, sigma, s, P));
-    KRR_TRY(prepare_points_f32(Td, Nt, d, kern, sigma, s, R, P.mean.p));
-    // the tcgen05 rectangular product when both point sets have split operands
-    bool tc5 = false;
-    if (product_path() == 0) {
-      int bad_p = 0, bad_r = 0;
-      KRR_TRY(prepare_points_tc5(Xd, s, P, &bad_p));
-      if (P.nh5 > 0) KRR_TRY(prepare_points_tc5(Td, s, R, &bad_r));
-      tc5 = P.nh5 > 0 && R.nh5 > 0;
-    }
-    DevBuf<float> a32, y32, part;
-    KRR_TRY(a32.alloc((size_t)N * m, s));
-    KRR_TRY(y32.alloc((size_t)Nt * m, s));
-    KRR_TRY(convert_f64_to_f32(Ad, a32.p, N * m, s));
-    if (tc5) {
-      KRR_TRY(kmv_tc5(R, P, 0.0f, false, a32.p, N, m, y32.p, Nt, s, part));
-      KRR_TRY(tc5_check_fault(s));
-    } else {
+    // the tcgen05 rectangular product when both point sets fit its split
+    bool done = false;
+    KRR_TRY(kmv_tc5_call(Td, Nt, Xd, N, d, kern, sigma, 0.0, Ad, m, o.dev, s, &done));
+    if (!done) {
+      PointsF32 P, R;
+      KRR_TRY(prepare_points_f32(Xd, N, d, kern, sigma, s, P));
+      KRR_TRY(prepare_points_f32(Td, Nt, d, kern, sigma, s, R, P.mean.p));
+      DevBuf<float> a32, y32, part;
+      KRR_TRY(a32.alloc((size_t)N * m, s));
+      KRR_TRY(y32.alloc((size_t)Nt * m, s));
+      KRR_TRY(convert_f64_to_f32(Ad, a32.p, N * m, s));
       KRR_TRY(kcross_f32(R, P, a32.p, N, m, y32.p, Nt, s, part));
+      KRR_TRY(convert_f32_to_f64(y32.p, o.dev, Nt * m, s));
     }
-    KRR_TRY(convert_f32_to_f64(y32.p, o.dev, Nt * m, s));
   }
   return o.finish(s);
 }

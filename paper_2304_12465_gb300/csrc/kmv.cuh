@@ -13,7 +13,7 @@ namespace krr {
 struct PointsF32 {
   DevBuf<float> xt;   // N x dp
   DevBuf<float> cn;   // N
-  DevBuf<double> mean;  // d, the centre subtracted from every point
+  DevBuf<double> mean;  // d, the centre subtracted (empty when it was given)
   int dp = 0;
   int d = 0;
   int64_t N = 0;
@@ -32,6 +32,11 @@ struct PointsF32 {
   int nh5 = 0, csep5 = 0;
 };
 
+// mean[k] = the mean of coordinate k (d doubles, allocated here); zero
+// (optional) is a device flag cleared on the way.
+krr_status points_mean(const double *Xd, int64_t N, int d, cudaStream_t s, DevBuf<double> &mean,
+                       int *zero = nullptr);
+
 // mean_dev (optional, d doubles on the device): centre to use instead of the
 // points' own mean (prediction prepares test points with the training mean).
 // dp (optional): padded dimension (a multiple of 4 in [d, 32]) instead of the
@@ -49,9 +54,17 @@ krr_status prepare_points_f32(const double *Xd, int64_t N, int d, int kern,
 krr_status prepare_points_tc(const double *Xd, cudaStream_t s, PointsF32 &P,
                              bool with_tc5 = true);
 
+// Points of a square float32 product (kmv_f32) by the process's path: the
+// tcgen05 operands alone when they apply, else the float32 points and, where
+// it applies, the mma.sync layout.  Synchronises s.
+krr_status prepare_points_product(const double *Xd, int64_t N, int d, int kern, double sigma,
+                                  cudaStream_t s, PointsF32 &P);
+
 // Builds only the tcgen05 operands of P (P.nh5 > 0); *bad = 1 (and nh5 = 0)
-// when a point is outside the split's range.  Synchronises s.
-krr_status prepare_points_tc5(const double *Xd, cudaStream_t s, PointsF32 &P, int *bad);
+// when a point is outside the split's range.  P's kern, sigma, N and d are
+// set, and its mean unless mean_dev gives the centre.  Synchronises s.
+krr_status prepare_points_tc5(const double *Xd, cudaStream_t s, PointsF32 &P, int *bad,
+                              const double *mean_dev = nullptr);
 
 // tcgen05 product Y (R.N x m) = K(R, P) V, + lambda V when square (R is P);
 // both point sets carry tcgen05 operands prepared with the same centre and
@@ -61,6 +74,15 @@ krr_status prepare_points_tc5(const double *Xd, cudaStream_t s, PointsF32 &P, in
 krr_status kmv_tc5(const PointsF32 &R, const PointsF32 &P, float lambda, bool square,
                    const float *V, int64_t ldv, int m, float *Y, int64_t ldy, cudaStream_t s,
                    DevBuf<float> &part, bool quiet = false);
+
+// One whole tcgen05 product from and to float64 arrays: Y = K(Xr, X) V, or (A
+// + lambda I) V when Xr is NULL.  Every launch is issued before the host
+// learns whether the points fit the split: *done = false when the path does
+// not apply or they did not fit (Y is then to be computed another way).
+// Synchronises s.
+krr_status kmv_tc5_call(const double *Xr, int64_t Nr, const double *Xd, int64_t N, int d,
+                        int kern, double sigma, double lambda, const double *V, int m, double *Y,
+                        cudaStream_t s, bool *done);
 
 // Epilogue variant of the tcgen05 product (see krr_set_product_variant), and
 // the autotuner's choice and per-variant times for a square shape.

@@ -20,30 +20,56 @@ namespace krr {
 // as c1 + c2 + c3; writes the row operand xa and the column operand xb
 // (kb = 2 nh + csep blocks of 16 halves each, stored K-block-major: block q
 // of point i at (q N + i) 16).  A coordinate or c outside the split's range
-// sets *bad.
+// sets *bad.  xa or xb may be NULL (a rectangular product needs one of them).
 // cshift is added to c on both sides (7 for the Gaussian: D = log2 kappa + 14).
-__global__ void prepare_tc5_kernel(const double *__restrict__ X, int64_t N, int d, int nh,
-                                   int csep, const double *__restrict__ mean, double scale,
-                                   double cshift, __half *__restrict__ xa,
-                                   __half *__restrict__ xb, int *__restrict__ bad) {
+// A block of 16 halves is assembled in registers and stored as two 16-byte
+// words; half by half the stores took 66 us at N = 1e5, d = 16 (both
+// operands), like this 24 us.
+template <int NH, int CSEP>
+__global__ void __launch_bounds__(128)
+prepare_tc5_kernel(const double *__restrict__ X, int64_t N, int d,
+                   const double *__restrict__ mean, double scale, double cshift,
+                   uint4 *__restrict__ xa, uint4 *__restrict__ xb, int *__restrict__ bad) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= N) return;
-  // element t of block q of this point
-  auto at = [&](__half *base, int q, int t) -> __half & { return base[((int64_t)q * N + i) * 16 + t]; };
+  auto store = [&](uint4 *base, int q, const uint32_t (&w)[8]) {
+    if (!base) return;
+    uint4 *dst = base + ((int64_t)q * N + i) * 2;
+    dst[0] = make_uint4(w[0], w[1], w[2], w[3]);
+    dst[1] = make_uint4(w[4], w[5], w[6], w[7]);
+  };
+  auto pack = [](__half lo, __half hi) {
+    return (uint32_t)__half_as_ushort(lo) | ((uint32_t)__half_as_ushort(hi) << 16);
+  };
   double nrm = 0.0;
   bool out_of_range = false;
-  for (int k = 0; k < nh * 16; ++k) {
-    const double v = (k < d) ? (X[i * d + k] - mean[k]) * scale : 0.0;
-    if (!(fabs(v) <= (double)T5_MAX_COORD)) out_of_range = true;
-    const __half h = __double2half(v);
-    const double hv = (double)__half2float(h);
-    const __half l = __double2half(v - hv);
-    const double e = hv + (double)__half2float(l);
-    nrm = fma(e, e, nrm);
-    at(xa, k / 16, k % 16) = h;
-    at(xb, k / 16, k % 16) = h;
-    at(xa, nh + k / 16, k % 16) = l;
-    at(xb, nh + k / 16, k % 16) = l;
+  uint32_t hw[8];
+#pragma unroll
+  for (int b = 0; b < NH; ++b) {
+    uint32_t lw[8];
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+      __half h[2], l[2];
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int k = b * 16 + 2 * t + u;
+        const double v = (k < d) ? (X[i * d + k] - mean[k]) * scale : 0.0;
+        if (!(fabs(v) <= (double)T5_MAX_COORD)) out_of_range = true;
+        h[u] = __double2half(v);
+        const double hv = (double)__half2float(h[u]);
+        l[u] = __double2half(v - hv);
+        const double e = hv + (double)__half2float(l[u]);
+        nrm = fma(e, e, nrm);
+      }
+      hw[t] = pack(h[0], h[1]);
+      lw[t] = pack(l[0], l[1]);
+    }
+    store(xa, NH + b, lw);
+    store(xb, NH + b, lw);
+    if (b + 1 < NH || CSEP) {
+      store(xa, b, hw);
+      store(xb, b, hw);
+    }
   }
   const double c = -0.5 * nrm + cshift;
   if (!(fabs(c) <= (double)T5_MAX_C)) out_of_range = true;
@@ -53,18 +79,21 @@ __global__ void prepare_tc5_kernel(const double *__restrict__ X, int64_t N, int 
   const __half c3 = __double2half(r1 - (double)__half2float(c2));
   const __half one = __double2half(1.0), zero = __double2half(0.0);
   // c-part: its own block, or positions 10..15 of the last H block (those
-  // coordinates are beyond d, so their H and L entries are zero)
-  const int qc = csep ? 2 * nh : nh - 1, off = csep ? 0 : 10;
-  if (csep)
-    for (int t = 6; t < 16; ++t) {
-      at(xa, qc, t) = zero;
-      at(xb, qc, t) = zero;
-    }
-  const __half pa_c[6] = {c1, c2, c3, one, one, one};
-  const __half pb_c[6] = {one, one, one, c1, c2, c3};
-  for (int t = 0; t < 6; ++t) {
-    at(xa, qc, off + t) = pa_c[t];
-    at(xb, qc, off + t) = pb_c[t];
+  // coordinates are beyond d, so their H and L entries are zero); the row
+  // operand holds (c1, c2, c3, 1, 1, 1), the column operand (1, 1, 1, c1, c2, c3)
+  const uint32_t pa[3] = {pack(c1, c2), pack(c3, one), pack(one, one)};
+  const uint32_t pb[3] = {pack(one, one), pack(one, c1), pack(c2, c3)};
+  if (CSEP) {
+    const uint32_t z = pack(zero, zero);
+    const uint32_t wa[8] = {pa[0], pa[1], pa[2], z, z, z, z, z};
+    const uint32_t wb[8] = {pb[0], pb[1], pb[2], z, z, z, z, z};
+    store(xa, 2 * NH, wa);
+    store(xb, 2 * NH, wb);
+  } else {
+    const uint32_t wa[8] = {hw[0], hw[1], hw[2], hw[3], hw[4], pa[0], pa[1], pa[2]};
+    const uint32_t wb[8] = {hw[0], hw[1], hw[2], hw[3], hw[4], pb[0], pb[1], pb[2]};
+    store(xa, NH - 1, wa);
+    store(xb, NH - 1, wb);
   }
   if (out_of_range) *bad = 1;
 }
@@ -108,38 +137,57 @@ static krr_status encode_operand_map(CUtensorMap *map, const uint16_t *ptr, int6
   return KRR_OK;
 }
 
-// Builds P's tcgen05 operands (P.nh5 > 0 on success; left at 0 when a point is
-// outside the split's range).  P was prepared by prepare_points_f32.
-krr_status prepare_points_tc5(const double *Xd, cudaStream_t s, PointsF32 &P, int *h_bad_out) {
-  P.nh5 = 0;
-  *h_bad_out = 0;
-  if (P.kern == KLAPLACE || P.d > 32 || P.N == 0) return KRR_OK;
+// Allocates and fills P's tcgen05 operands and encodes their maps (P.nh5 >
+// 0); a point outside the split's range sets *bad_dev (cleared by the
+// caller).  rows, cols: which operands are wanted.
+static krr_status tc5_operands(const double *Xd, cudaStream_t s, PointsF32 &P, const double *mean,
+                               bool rows, bool cols, int *bad_dev) {
   const int nh = t5_nh(P.d), csep = t5_csep(P.d), kb = t5_kb(nh, csep);
   const double log2e = 1.4426950408889634;
   const double scale = (P.kern == KGAUSS) ? std::sqrt(log2e) / P.sigma : std::sqrt(5.0) / P.sigma;
-  KRR_TRY(P.xa5.alloc((size_t)P.N * kb * 16, s));
-  KRR_TRY(P.xb5.alloc((size_t)P.N * kb * 16, s));
+  if (rows) KRR_TRY(P.xa5.alloc((size_t)P.N * kb * 16, s));
+  if (cols) KRR_TRY(P.xb5.alloc((size_t)P.N * kb * 16, s));
+  uint4 *xa = reinterpret_cast<uint4 *>(rows ? P.xa5.p : nullptr);
+  uint4 *xb = reinterpret_cast<uint4 *>(cols ? P.xb5.p : nullptr);
+  const double cshift = P.kern == KGAUSS ? 7.0 : 0.0;
+  const unsigned grid = ceil_div(P.N, 128);
+#define KRR_PREP(NH, CS)                                                                     \
+  if (nh == NH && csep == CS)                                                                \
+  prepare_tc5_kernel<NH, CS><<<grid, 128, 0, s>>>(Xd, P.N, P.d, mean, scale, cshift, xa, xb, \
+                                                  bad_dev)
+  KRR_PREP(1, 0);
+  KRR_PREP(1, 1);
+  KRR_PREP(2, 0);
+  KRR_PREP(2, 1);
+#undef KRR_PREP
+  KRR_LAUNCH_CHECK();
+  if (rows) KRR_TRY(encode_operand_map(&P.ma5, P.xa5.p, P.N, kb));
+  if (cols) KRR_TRY(encode_operand_map(&P.mb5, P.xb5.p, P.N, kb));
+  P.nh5 = nh;
+  P.csep5 = csep;
+  return KRR_OK;
+}
+
+// Builds P's tcgen05 operands (P.nh5 > 0 on success; left at 0 when a point is
+// outside the split's range) with the centre mean_dev, or P.mean.
+krr_status prepare_points_tc5(const double *Xd, cudaStream_t s, PointsF32 &P, int *h_bad_out,
+                              const double *mean_dev) {
+  P.nh5 = 0;
+  *h_bad_out = 0;
+  if (P.kern == KLAPLACE || P.d > 32 || P.N == 0) return KRR_OK;
   DevBuf<int> bad;
   KRR_TRY(bad.alloc(1, s));
   KRR_CUDA_TRY(cudaMemsetAsync(bad.p, 0, sizeof(int), s));
-  prepare_tc5_kernel<<<ceil_div(P.N, 256), 256, 0, s>>>(
-      Xd, P.N, P.d, nh, csep, P.mean.p, scale, P.kern == KGAUSS ? 7.0 : 0.0,
-      reinterpret_cast<__half *>(P.xa5.p),
-      reinterpret_cast<__half *>(P.xb5.p), bad.p);
-  KRR_LAUNCH_CHECK();
+  KRR_TRY(tc5_operands(Xd, s, P, mean_dev ? mean_dev : P.mean.p, true, true, bad.p));
   int h_bad = 0;
   KRR_CUDA_TRY(cudaMemcpyAsync(&h_bad, bad.p, sizeof(int), cudaMemcpyDeviceToHost, s));
   KRR_CUDA_TRY(cudaStreamSynchronize(s));
   if (h_bad) {
+    P.nh5 = 0;
     P.xa5.release();
     P.xb5.release();
     *h_bad_out = 1;
-    return KRR_OK;
   }
-  KRR_TRY(encode_operand_map(&P.ma5, P.xa5.p, P.N, kb));
-  KRR_TRY(encode_operand_map(&P.mb5, P.xb5.p, P.N, kb));
-  P.nh5 = nh;
-  P.csep5 = csep;
   return KRR_OK;
 }
 
@@ -203,11 +251,16 @@ krr_status tc5_wait_selftest(long long budget, cudaStream_t s) {
 }
 
 // ------------------------------------------------------------ reduction
+// TV5: the type of V and Y.  flags (optional): {a point outside the split's
+// range, a bounded wait gave up}, for one read-back after the product.
+template <typename TV5>
 __global__ void t5_reduce_kernel(const float *__restrict__ part, int64_t Nr, int m, int M, int C,
                                  int64_t T, int G, int J, int CG, const int *__restrict__ vexp,
-                                 float lambda, const float *__restrict__ V, int64_t ldv,
-                                 float *__restrict__ Y, int64_t ldy) {
+                                 double lambda, const TV5 *__restrict__ V, int64_t ldv,
+                                 TV5 *__restrict__ Y, int64_t ldy, const int *__restrict__ fault,
+                                 int *__restrict__ flags) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (flags && i == 0) flags[1] = *fault;
   if (i >= Nr) return;
   const int64_t rb = i / T5_RB;
   const int r = (int)(i % T5_RB);
@@ -222,7 +275,7 @@ __global__ void t5_reduce_kernel(const float *__restrict__ part, int64_t Nr, int
     }
     if (vexp) acc = ldexp(acc, -14 - vexp[c]);
     Y[(int64_t)c * ldy + i] =
-        V ? (float)(acc + (double)lambda * (double)V[(int64_t)c * ldv + i]) : (float)acc;
+        V ? (TV5)(acc + lambda * (double)V[(int64_t)c * ldv + i]) : (TV5)acc;
   }
 }
 
@@ -231,7 +284,8 @@ __global__ void t5_reduce_kernel(const float *__restrict__ part, int64_t Nr, int
 // v_2cp, v_2cp+1, v_2cp+1} of point t TN + jl times vscale (zero beyond Nc
 // or m); vscale = 2^-14 for the Gaussian, whose kernel values come scaled by
 // 2^14.
-__global__ void t5_vdup_kernel(const float *__restrict__ V, int64_t ldv, int64_t Nc, int m,
+template <typename TV5>
+__global__ void t5_vdup_kernel(const TV5 *__restrict__ V, int64_t ldv, int64_t Nc, int m,
                                int MP, int C, int TN, float vscale, float4 *__restrict__ vdup) {
   const int64_t total = (int64_t)C * MP * TN;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
@@ -242,8 +296,8 @@ __global__ void t5_vdup_kernel(const float *__restrict__ V, int64_t ldv, int64_t
     const int64_t j = t * TN + jl;
     float va = 0.0f, vb = 0.0f;
     if (j < Nc) {
-      if (2 * cp < m) va = V[(int64_t)(2 * cp) * ldv + j] * vscale;
-      if (2 * cp + 1 < m) vb = V[(int64_t)(2 * cp + 1) * ldv + j] * vscale;
+      if (2 * cp < m) va = (float)V[(int64_t)(2 * cp) * ldv + j] * vscale;
+      if (2 * cp + 1 < m) vb = (float)V[(int64_t)(2 * cp + 1) * ldv + j] * vscale;
     }
     vdup[e] = make_float4(va, va, vb, vb);
   }
@@ -252,7 +306,8 @@ __global__ void t5_vdup_kernel(const float *__restrict__ V, int64_t ldv, int64_t
 // Largest |v| of each right-hand side (m <= 8) over this block's grid-stride
 // share of the Nc points: bmax[block][c].
 constexpr int T5_VMAX_BLOCKS = 256;
-__global__ void t5_vmax_kernel(const float *__restrict__ V, int64_t ldv, int64_t Nc, int m,
+template <typename TV5>
+__global__ void t5_vmax_kernel(const TV5 *__restrict__ V, int64_t ldv, int64_t Nc, int m,
                                float *__restrict__ bmax) {
   __shared__ float red[8][8];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -261,7 +316,7 @@ __global__ void t5_vmax_kernel(const float *__restrict__ V, int64_t ldv, int64_t
     if (c < m)
       for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < Nc;
            j += (int64_t)gridDim.x * blockDim.x)
-        mx = fmaxf(mx, fabsf(V[(int64_t)c * ldv + j]));
+        mx = fmaxf(mx, fabsf((float)V[(int64_t)c * ldv + j]));
     for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
     if (lane == 0) red[warp][c] = mx;
   }
@@ -286,7 +341,8 @@ __device__ __forceinline__ uint32_t t5_pack_halves(__half lo, __half hi) {
 // holds {B(2q, g), B(2q + 1, g)}, {B(2q + 8, g), B(2q + 9, g)} over the
 // batch's columns (zero beyond Nc, m or 2M).  Every block derives the scales
 // from bmax (gmax blocks); block 0 also stores vexp for the reduction.
-__global__ void t5_vfrag_kernel(const float *__restrict__ V, int64_t ldv, int64_t Nc, int m,
+template <typename TV5>
+__global__ void t5_vfrag_kernel(const TV5 *__restrict__ V, int64_t ldv, int64_t Nc, int m,
                                 int M, int C, int TN, const float *__restrict__ bmax, int gmax,
                                 uint2 *__restrict__ frag, int *__restrict__ vexp) {
   __shared__ float sc[8];
@@ -324,7 +380,7 @@ __global__ void t5_vfrag_kernel(const float *__restrict__ V, int64_t ldv, int64_
     auto slot = [&](int k) -> __half {
       const int64_t j = j0 + k;
       if (!live || c >= m || j >= Nc) return __float2half_rn(0.0f);
-      const float vs = V[(int64_t)c * ldv + j] * sc[c];
+      const float vs = (float)V[(int64_t)c * ldv + j] * sc[c];
       const __half h = __float2half_rn(vs);
       return lo ? __float2half_rn(vs - __half2float(h)) : h;
     };
@@ -407,8 +463,9 @@ static int *t5_vexp(float *part, const T5Geometry &g, int M) {
 
 // Stages V for this geometry and launches the product; returns the launch's
 // error.  part must hold t5_scratch_floats(g, M) floats.
+template <typename TV5>
 static cudaError_t t5_launch(const PointsF32 &R, const PointsF32 &P, int M, int variant,
-                             const T5Geometry &g, const float *Vg, int64_t ldv, int mg,
+                             const T5Geometry &g, const TV5 *Vg, int64_t ldv, int mg,
                              float *part, int *fault, cudaStream_t s, bool timed) {
   float *vbuf = part + t5_npart(g, M);
   cudaError_t e = cudaSuccess;
@@ -456,8 +513,9 @@ static cudaError_t t5_launch(const PointsF32 &R, const PointsF32 &P, int M, int 
 }
 
 // Variant for this product: forced, cached, tuned now, or the default.
+template <typename TV5>
 static int choose_variant(const PointsF32 &R, const PointsF32 &P, bool square, int M,
-                          const float *Vg,
+                          const TV5 *Vg,
                           int64_t ldv, int mg, DevBuf<float> &part, int *fault, cudaStream_t s,
                           bool quiet) {
   const int forced = g_t5_variant.load();
@@ -513,9 +571,10 @@ static int choose_variant(const PointsF32 &R, const PointsF32 &P, bool square, i
   return tune.best;
 }
 
-krr_status kmv_tc5(const PointsF32 &R, const PointsF32 &P, float lambda, bool square,
-                   const float *V, int64_t ldv, int m, float *Y, int64_t ldy, cudaStream_t s,
-                   DevBuf<float> &part, bool quiet) {
+template <typename TV5>
+static krr_status tc5_products(const PointsF32 &R, const PointsF32 &P, double lambda, bool square,
+                               const TV5 *V, int64_t ldv, int m, TV5 *Y, int64_t ldy,
+                               cudaStream_t s, DevBuf<float> &part, bool quiet, int *flags) {
   const int64_t Nr = R.N, Nc = P.N;
   if (Nr == 0 || Nc == 0 || m == 0) return KRR_OK;
   KRR_REQUIRE(R.nh5 > 0 && P.nh5 == R.nh5 && P.csep5 == R.csep5 && R.kern == P.kern,
@@ -525,7 +584,7 @@ krr_status kmv_tc5(const PointsF32 &R, const PointsF32 &P, float lambda, bool sq
   for (int c0 = 0; c0 < m; c0 += 8) {
     const int mg = std::min(8, m - c0);
     const int M = mg <= 2 ? 2 : mg <= 4 ? 4 : 8;
-    const float *Vg = V + (int64_t)c0 * ldv;
+    const TV5 *Vg = V + (int64_t)c0 * ldv;
     const int variant = choose_variant(R, P, square, M, Vg, ldv, mg, part, fault, s, quiet);
     const T5Geometry g = t5_geometry(Nr, Nc, t5_variant_tn(variant));
     const size_t need = t5_scratch_floats(g, M);
@@ -536,12 +595,53 @@ krr_status kmv_tc5(const PointsF32 &R, const PointsF32 &P, float lambda, bool sq
       return KRR_ECUDA;
     }
     const int CG = t5_variant_ew(variant) / 4;
-    t5_reduce_kernel<<<ceil_div(Nr, 256), 256, 0, s>>>(
+    t5_reduce_kernel<TV5><<<ceil_div(Nr, 256), 256, 0, s>>>(
         part.p, Nr, mg, M, g.C, g.T, g.G, g.J, CG,
         t5_variant_tv(variant) ? t5_vexp(part.p, g, M) : nullptr, lambda, square ? Vg : nullptr,
-        ldv, Y + (int64_t)c0 * ldy, ldy);
+        ldv, Y + (int64_t)c0 * ldy, ldy, fault, flags);
     KRR_LAUNCH_CHECK();
   }
+  return KRR_OK;
+}
+
+krr_status kmv_tc5(const PointsF32 &R, const PointsF32 &P, float lambda, bool square,
+                   const float *V, int64_t ldv, int m, float *Y, int64_t ldy, cudaStream_t s,
+                   DevBuf<float> &part, bool quiet) {
+  return tc5_products<float>(R, P, (double)lambda, square, V, ldv, m, Y, ldy, s, part, quiet,
+                             nullptr);
+}
+
+krr_status kmv_tc5_call(const double *Xr, int64_t Nr, const double *Xd, int64_t N, int d,
+                        int kern, double sigma, double lambda, const double *V, int m, double *Y,
+                        cudaStream_t s, bool *done) {
+  *done = false;
+  if (product_path() != 0 || kern == KLAPLACE || d > 32) return KRR_OK;
+  PointsF32 P, R;
+  auto set = [&](PointsF32 &Q, int64_t n) {
+    Q.dp = (d + 3) / 4 * 4;
+    Q.d = d;
+    Q.N = n;
+    Q.kern = kern;
+    Q.sigma = sigma;
+  };
+  set(P, N);
+  DevBuf<int> flags;
+  KRR_TRY(flags.alloc(2, s));
+  KRR_TRY(points_mean(Xd, N, d, s, P.mean, flags.p));
+  KRR_TRY(tc5_operands(Xd, s, P, P.mean.p, Xr == nullptr, true, flags.p));
+  if (Xr) {
+    set(R, Nr);
+    KRR_TRY(tc5_operands(Xr, s, R, P.mean.p, true, false, flags.p));
+  }
+  DevBuf<float> part;
+  // the shift as the float32 products apply it
+  KRR_TRY(tc5_products<double>(Xr ? R : P, P, (double)(float)lambda, Xr == nullptr, V, N, m, Y,
+                               Xr ? Nr : N, s, part, false, flags.p));
+  int h[2] = {0, 0};
+  KRR_CUDA_TRY(cudaMemcpyAsync(h, flags.p, sizeof(h), cudaMemcpyDeviceToHost, s));
+  KRR_CUDA_TRY(cudaStreamSynchronize(s));
+  if (h[1]) return tc5_check_fault(s);
+  *done = h[0] == 0;
   return KRR_OK;
 }
 

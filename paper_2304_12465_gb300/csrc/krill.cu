@@ -580,16 +580,24 @@ krr_status krill_product64(const krill_precond *P, KrillFF &Q, const double *bet
 krr_status krill_points_tc5(const krill_precond *P, cudaStream_t s, KrillTC5 &T) {
   T.ok = false;
   if (P->kern == KLAPLACE || product_path() == 1 || P->d > 32) return KRR_OK;
-  KRR_TRY(prepare_points_f32(P->X, P->N, P->d, P->kern, P->sigma, s, T.all));
+  auto set = [&](PointsF32 &Q, int64_t n) {
+    Q.dp = (P->d + 3) / 4 * 4;
+    Q.d = P->d;
+    Q.N = n;
+    Q.kern = P->kern;
+    Q.sigma = P->sigma;
+  };
+  set(T.all, P->N);
+  set(T.centers, P->k);
+  KRR_TRY(points_mean(P->X, P->N, P->d, s, T.all.mean));
   DevBuf<double> xc;
   KRR_TRY(xc.alloc((size_t)P->k * P->d, s));
   gather_points_kernel<<<ceil_div((int64_t)P->k * P->d, 256), 256, 0, s>>>(P->X, P->d, P->S,
                                                                           P->k, xc.p);
   KRR_LAUNCH_CHECK();
-  KRR_TRY(prepare_points_f32(xc.p, P->k, P->d, P->kern, P->sigma, s, T.centers, T.all.mean.p));
   int bad_all = 0, bad_c = 0;
   KRR_TRY(prepare_points_tc5(P->X, s, T.all, &bad_all));
-  KRR_TRY(prepare_points_tc5(xc.p, s, T.centers, &bad_c));
+  KRR_TRY(prepare_points_tc5(xc.p, s, T.centers, &bad_c, T.all.mean.p));
   T.ok = !bad_all && !bad_c && T.all.nh5 > 0 && T.centers.nh5 > 0;
   return KRR_OK;
 }
