@@ -140,138 +140,6 @@ krr_status gemm(const Gemm<T> &g, cudaStream_t s, int split_k) {
   return KRR_OK;
 }
 
-// ------------------------------------------- float-float Schur update
-// C(M x N) -= A(M x K) B(K x N) for float64 data, with the products and sums
-// in float-float arithmetic on the float32 pipes (float64 runs at a small
-// fraction of the float32 rate on this GPU).  Each float64 input is split
-// into hi = fl32(a) and lo = fl32(a - hi) (48 bits) when its tile is staged;
-// a product is hi_a hi_b, split exactly into p + e with an FMA (Dekker's
-// TwoProduct), plus the cross terms hi_a lo_b + lo_a hi_b (lo_a lo_b, below
-// 2^-48 |a b|, is dropped); p enters the running sum through Knuth's
-// error-free TwoSum, the rounding error and e through a float32 correction.
-// The pair (sum, correction) is renormalised once per K tile.  Intrinsics
-// keep the compiler from contracting or reassociating the error-free steps.
-// Error: about 2^-48 sqrt(K) max_k |sum_{l<=k} a_il b_lj| per entry.
-__global__ void __launch_bounds__(G_THREADS)
-gemm_sub_ff_kernel(int M, int N, int K, const double *__restrict__ A, int64_t sai,
-                   int64_t sak, const double *__restrict__ B, int64_t sbk, int64_t sbj,
-                   double *__restrict__ C, int64_t ldc) {
-  __shared__ float Ah[GB_K][GB_M + 1], Al[GB_K][GB_M + 1];
-  __shared__ float Bh[GB_K][GB_N + 1], Bl[GB_K][GB_N + 1];
-  const int tid = threadIdx.x;
-  const int tx = tid % 16, ty = tid / 16;
-  const int i0 = blockIdx.x * GB_M, j0 = blockIdx.y * GB_N;
-  // outputs (row ty + 16 r, columns tx + 16 (2 h) and tx + 16 (2 h + 1)) as
-  // packed pairs: every step below is one FMUL2 / FFMA2 / FADD2 for two
-  // outputs, x - y written as fma(y, -1, x) (the same single rounding)
-  float2 sh[4][2], sl[4][2];
-#pragma unroll
-  for (int r = 0; r < 4; ++r)
-#pragma unroll
-    for (int h = 0; h < 2; ++h) sh[r][h] = sl[r][h] = make_float2(0.0f, 0.0f);
-  const float2 m1 = make_float2(-1.0f, -1.0f);
-  const bool a_kfast = (sak == 1 && sai != 1);
-  const bool b_kfast = (sbk == 1 && sbj != 1);
-  for (int k0 = 0; k0 < K; k0 += GB_K) {
-#pragma unroll
-    for (int e = 0; e < (GB_M * GB_K) / G_THREADS; ++e) {
-      const int idx = tid + e * G_THREADS;
-      int ii, kk;
-      if (a_kfast) { kk = idx % GB_K; ii = idx / GB_K; }
-      else { ii = idx % GB_M; kk = idx / GB_M; }
-      const int gi = i0 + ii, gk = k0 + kk;
-      const double v = (gi < M && gk < K) ? A[(int64_t)gi * sai + (int64_t)gk * sak] : 0.0;
-      const float h = __double2float_rn(v);
-      Ah[kk][ii] = h;
-      Al[kk][ii] = __double2float_rn(v - (double)h);
-    }
-#pragma unroll
-    for (int e = 0; e < (GB_N * GB_K) / G_THREADS; ++e) {
-      const int idx = tid + e * G_THREADS;
-      int jj, kk;
-      if (b_kfast) { kk = idx % GB_K; jj = idx / GB_K; }
-      else { jj = idx % GB_N; kk = idx / GB_N; }
-      const int gj = j0 + jj, gk = k0 + kk;
-      const double v = (gj < N && gk < K) ? B[(int64_t)gk * sbk + (int64_t)gj * sbj] : 0.0;
-      const float h = __double2float_rn(v);
-      Bh[kk][jj] = h;
-      Bl[kk][jj] = __double2float_rn(v - (double)h);
-    }
-    __syncthreads();
-#pragma unroll 4
-    for (int kk = 0; kk < GB_K; ++kk) {
-      float2 ah[4], nah[4], nal[4], bh[2], bl[2];
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const float a = Ah[kk][ty + 16 * r], al = Al[kk][ty + 16 * r];
-        ah[r] = make_float2(a, a);
-        nah[r] = make_float2(-a, -a);
-        nal[r] = make_float2(-al, -al);
-      }
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        bh[h] = make_float2(Bh[kk][tx + 32 * h], Bh[kk][tx + 32 * h + 16]);
-        bl[h] = make_float2(Bl[kk][tx + 32 * h], Bl[kk][tx + 32 * h + 16]);
-      }
-#pragma unroll
-      for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          // p = hi_a hi_b; en = -(hi_a hi_b - p) - hi_a lo_b - lo_a hi_b (the
-          // negated product error and cross terms, each step exact or
-          // rounded once as in the scalar form)
-          const float2 p = __fmul2_rn(ah[r], bh[h]);
-          float2 en = __ffma2_rn(nah[r], bh[h], p);
-          en = __ffma2_rn(nah[r], bl[h], en);
-          en = __ffma2_rn(nal[r], bh[h], en);
-          // TwoSum(sh, p)
-          const float2 t = __fadd2_rn(sh[r][h], p);
-          const float2 z = __ffma2_rn(sh[r][h], m1, t);
-          const float2 tz = __ffma2_rn(z, m1, t);
-          const float2 err = __fadd2_rn(__ffma2_rn(tz, m1, sh[r][h]), __ffma2_rn(z, m1, p));
-          sh[r][h] = t;
-          sl[r][h] = __fadd2_rn(sl[r][h], __ffma2_rn(en, m1, err));
-        }
-    }
-    __syncthreads();
-    // renormalise once per tile (TwoSum): the correction stays below an ulp
-    // of the sum, so its own roundings stay at the float-float level
-#pragma unroll
-    for (int r = 0; r < 4; ++r)
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const float2 t = __fadd2_rn(sh[r][h], sl[r][h]);
-        const float2 z = __ffma2_rn(sh[r][h], m1, t);
-        sl[r][h] = __fadd2_rn(__ffma2_rn(__ffma2_rn(z, m1, t), m1, sh[r][h]),
-                              __ffma2_rn(z, m1, sl[r][h]));
-        sh[r][h] = t;
-      }
-  }
-#pragma unroll
-  for (int r = 0; r < 4; ++r)
-#pragma unroll
-    for (int h = 0; h < 2; ++h)
-#pragma unroll
-      for (int e = 0; e < 2; ++e) {
-        const int gi = i0 + ty + 16 * r, gj = j0 + tx + 32 * h + 16 * e;
-        if (gi < M && gj < N) {
-          double *dst = C + (int64_t)gi + (int64_t)gj * ldc;
-          const float hi = e ? sh[r][h].y : sh[r][h].x, lo = e ? sl[r][h].y : sl[r][h].x;
-          *dst = *dst - ((double)hi + (double)lo);
-        }
-      }
-}
-
-krr_status gemm_sub_ff(const Gemm<double> &g, cudaStream_t s) {
-  if (g.M <= 0 || g.N <= 0 || g.K <= 0) return KRR_OK;
-  KRR_REQUIRE(g.alpha == -1.0 && g.beta == 1.0, "gemm_sub_ff: C -= A B only");
-  dim3 grid((g.M + GB_M - 1) / GB_M, (g.N + GB_N - 1) / GB_N, 1);
-  gemm_sub_ff_kernel<<<grid, G_THREADS, 0, s>>>(g.M, g.N, g.K, g.A, g.sai, g.sak, g.B, g.sbk,
-                                                g.sbj, g.C, g.ldc);
-  KRR_LAUNCH_CHECK();
-  return KRR_OK;
-}
-
 // ------------------------------------------------------------ Gram (F^T F)
 // Lower-triangular output tiles only.  float input: each K tile of GB_K
 // products is summed in float32, then added to a float-float accumulator

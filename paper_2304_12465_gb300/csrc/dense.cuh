@@ -25,10 +25,15 @@ struct Gemm {
 template <typename T>
 krr_status gemm(const Gemm<T> &g, cudaStream_t s, int split_k = 1);
 
-// C -= A B (alpha = -1, beta = 1) for float64 data with float-float products
-// and sums on the float32 pipes: about 2^-48 sqrt(K) times the largest
-// partial sum per entry.
-krr_status gemm_sub_ff(const Gemm<double> &g, cudaStream_t s);
+// C (N x nc, ldc) -= A (N x K, lda) B^T for float64 matrices with entries in
+// [-1, 1] whose products' sums stay below 4 in magnitude, on the tensor cores
+// by digits (digits.cuh): row c of B starts at B + rows[c] (rows NULL: B + c)
+// with a step of ldb between its K entries and updates column cmap[c] of C
+// (cmap NULL: c).  frag: dig_frag_elems(nc, K) elements of scratch.
+size_t dig_frag_elems(int nc, int K);
+krr_status dig_gemm_sub(const double *A, int64_t lda, int64_t N, int K, const double *B,
+                        int64_t ldb, const int64_t *rows, int nc, double *C, int64_t ldc,
+                        const int *cmap, uint2 *frag, cudaStream_t s);
 
 // Lower triangle of C (r x r, column-major) = F^T F for F N x r column-major.
 // float F: float32 products summed in float32 over 16-term chunks, the chunk

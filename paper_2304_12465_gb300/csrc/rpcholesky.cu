@@ -3,9 +3,12 @@
 // Per block: (1) fixed-point pivot sampling from the residual diagonal
 // (residuals at or below the drop threshold carry no weight) and
 // Unique in first-occurrence order; (2) G = A(:,S') from the kernel function
-// minus the Schur term F(:,1:i) F(S',1:i)^T (GEMM); (3) Cholesky of G(S',S')
-// pivot by pivot with the drop rule; (4) the new columns G R^{-1} by forward
-// substitution, fused with the residual-diagonal downdate.
+// minus the Schur term F(:,1:i) F(S',1:i)^T (by digits on the tensor cores);
+// (3) Cholesky of G(S',S') pivot by pivot with the drop rule; (4) the new
+// columns G R^{-1}, by groups of columns: the groups before them on the tensor
+// cores, then forward substitution, fused with the residual-diagonal downdate.
+#include <algorithm>
+
 #include "dense.cuh"
 #include "handles.cuh"
 #include "kmv.cuh"
@@ -53,80 +56,113 @@ sample_chunk_sums_kernel(const double *__restrict__ dres, int64_t N, double dflo
   }
 }
 
-// One CTA: prefix of chunk sums, ndraw draws (one warp per draw), then Unique
-// (first-occurrence order) by one thread.
+// Exclusive prefix of v over the block's threads, and the block's total.
+__device__ __forceinline__ uint64_t block_scan_u64(uint64_t v, uint64_t *total,
+                                                   uint64_t (&warp_sums)[SMP_THREADS / 32]) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint64_t incl = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint64_t u = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += u;
+  }
+  __syncthreads();   // a previous scan's sums have been read
+  if (lane == 31) warp_sums[warp] = incl;
+  __syncthreads();
+  uint64_t before = 0, all = 0;
+#pragma unroll
+  for (int w = 0; w < SMP_THREADS / 32; ++w) {
+    if (w < warp) before += warp_sums[w];
+    all += warp_sums[w];
+  }
+  *total = all;
+  return before + incl - v;
+}
+
+// One CTA a draw: the chunk that holds the target (from the chunk sums), then
+// the entry inside it, each by a block-wide prefix over consecutive shares.
+// One CTA for all draws took 490 us for 100 draws at N = 1e5 (a chunk's scan
+// by one warp, thirteen draws a warp, the chunk sums by one thread).
+// counts[0] = ndraw, or 0 when every weight is zero.
 __global__ void __launch_bounds__(SMP_THREADS)
 sample_draw_kernel(const double *__restrict__ dres, int64_t N, double dfloor, int fbits,
-                   int64_t chunk,
-                   const uint64_t *__restrict__ csum, int nchunks, uint64_t seed,
-                   uint64_t t, int ndraw, int64_t *__restrict__ draws,
-                   int64_t *__restrict__ cand, int *__restrict__ counts) {
-  __shared__ uint64_t cpre[SMP_MAX_CHUNKS];
-  __shared__ uint64_t total;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (threadIdx.x == 0) {
-    uint64_t run = 0;
-    for (int c = 0; c < nchunks; ++c) {
-      run += csum[c];
-      cpre[c] = run;
-    }
-    total = run;
+                   int64_t chunk, const uint64_t *__restrict__ csum, int nchunks, uint64_t seed,
+                   uint64_t t, int ndraw, int64_t *__restrict__ draws, int *__restrict__ counts) {
+  __shared__ uint64_t ws[SMP_THREADS / 32];
+  __shared__ uint64_t s_local;
+  __shared__ int s_chunk;
+  const int tid = threadIdx.x, j = blockIdx.x;
+  const int per = (nchunks + SMP_THREADS - 1) / SMP_THREADS;
+  const int c0 = min(nchunks, tid * per), c1 = min(nchunks, c0 + per);
+  uint64_t mine = 0, total;
+  for (int c = c0; c < c1; ++c) mine += csum[c];
+  uint64_t run = block_scan_u64(mine, &total, ws);
+  if (j == 0 && tid == 0) counts[0] = total ? ndraw : 0;
+  if (total == 0) return;
+  uint64_t ctr[4] = {t, (uint64_t)j, 0ull, 0ull}, out[4];
+  philox4x64_10(ctr, seed, kTagPivots, out);
+  const uint64_t target = scale_u64(out[0], total);
+  // smallest chunk whose inclusive prefix exceeds the target
+  if (target >= run && target < run + mine) {
+    int c = c0;
+    while (target >= run + csum[c]) run += csum[c++];
+    s_chunk = c;
+    s_local = target - run;
   }
   __syncthreads();
-  if (total == 0) {
-    if (threadIdx.x == 0) {
-      counts[0] = 0;
-      counts[1] = 0;
+  uint64_t tl = s_local;
+  const int64_t b1 = min(N, (int64_t)(s_chunk + 1) * chunk);
+  constexpr int PER = 8;
+  for (int64_t b0 = (int64_t)s_chunk * chunk; b0 < b1; b0 += SMP_THREADS * PER) {
+    const int64_t i0 = b0 + (int64_t)tid * PER;
+    uint64_t w[PER];
+    mine = 0;
+#pragma unroll
+    for (int e = 0; e < PER; ++e) {
+      w[e] = (i0 + e < b1) ? fixed_weight(dres[i0 + e], dfloor, fbits) : 0ull;
+      mine += w[e];
     }
+    uint64_t part;
+    run = block_scan_u64(mine, &part, ws);
+    if (tl < part) {
+      if (tl >= run && tl < run + mine) {
+        int e = 0;
+        while (tl >= run + w[e]) run += w[e++];
+        draws[j] = i0 + e;
+      }
+      return;
+    }
+    tl -= part;
+  }
+}
+
+// Unique: the distinct draws in first-occurrence order; one thread a draw.
+constexpr int UNIQUE_THREADS = 1024;
+__global__ void __launch_bounds__(UNIQUE_THREADS)
+sample_unique_kernel(const int64_t *__restrict__ draws, int64_t *__restrict__ cand,
+                     int *__restrict__ counts) {
+  __shared__ int64_t sd[UNIQUE_THREADS];
+  __shared__ int wsum[UNIQUE_THREADS / 32];
+  const int j = threadIdx.x, lane = j & 31, warp = j >> 5, n = counts[0];
+  if (n == 0) {
+    if (j == 0) counts[1] = 0;
     return;
   }
-  for (int j = warp; j < ndraw; j += SMP_THREADS / 32) {
-    uint64_t ctr[4] = {t, (uint64_t)j, 0ull, 0ull}, out[4];
-    philox4x64_10(ctr, seed, kTagPivots, out);
-    const uint64_t target = scale_u64(out[0], total);
-    // smallest chunk whose inclusive prefix exceeds the target
-    int lo = 0, hi = nchunks - 1;
-    while (lo < hi) {
-      const int mid = (lo + hi) >> 1;
-      if (cpre[mid] > target) hi = mid; else lo = mid + 1;
-    }
-    const uint64_t base = cpre[lo] - csum[lo];
-    const uint64_t tl = target - base;
-    const int64_t b0 = (int64_t)lo * chunk, b1 = min(N, b0 + chunk);
-    uint64_t run = 0;
-    int64_t pick = b1 - 1;
-    for (int64_t off = b0; off < b1; off += 32) {
-      const int64_t i = off + lane;
-      const uint64_t w = (i < b1) ? fixed_weight(dres[i], dfloor, fbits) : 0ull;
-      uint64_t incl = w;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint64_t v = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += v;
-      }
-      const uint64_t tot = __shfl_sync(0xffffffffu, incl, 31);
-      if (run + tot > tl) {
-        const unsigned hit = __ballot_sync(0xffffffffu, run + incl > tl);
-        pick = off + (__ffs(hit) - 1);
-        break;
-      }
-      run += tot;
-    }
-    if (lane == 0) draws[j] = pick;
-  }
+  const int64_t v = j < n ? draws[j] : -1;
+  sd[j] = v;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    int nc = 0;
-    for (int j = 0; j < ndraw; ++j) {
-      const int64_t v = draws[j];
-      bool seen = false;
-      for (int c = 0; c < nc; ++c)
-        if (cand[c] == v) { seen = true; break; }
-      if (!seen) cand[nc++] = v;
-    }
-    counts[0] = ndraw;
-    counts[1] = nc;
+  bool first = j < n;
+  for (int i = 0; i < j && first; ++i) first = sd[i] != v;
+  const unsigned b = __ballot_sync(0xffffffffu, first);
+  if (lane == 0) wsum[warp] = __popc(b);
+  __syncthreads();
+  int pos = __popc(b & ((1u << lane) - 1u)), all = 0;
+  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
+    if (w < warp) pos += wsum[w];
+    all += wsum[w];
   }
+  if (first) cand[pos] = v;
+  if (j == 0) counts[1] = all;
 }
 
 krr_status rpc_sample_device(const double *dres, int64_t N, double dfloor, uint64_t seed,
@@ -140,8 +176,10 @@ krr_status rpc_sample_device(const double *dres, int64_t N, double dfloor, uint6
   sample_chunk_sums_kernel<<<nchunks, SMP_THREADS, 0, s>>>(dres, N, dfloor, fbits, chunk,
                                                            csum.p);
   KRR_LAUNCH_CHECK();
-  sample_draw_kernel<<<1, SMP_THREADS, 0, s>>>(dres, N, dfloor, fbits, chunk, csum.p, nchunks,
-                                               seed, t, ndraw, draws, cand, counts);
+  sample_draw_kernel<<<ndraw, SMP_THREADS, 0, s>>>(dres, N, dfloor, fbits, chunk, csum.p, nchunks,
+                                                   seed, t, ndraw, draws, counts);
+  KRR_LAUNCH_CHECK();
+  sample_unique_kernel<<<1, (ndraw + 31) / 32 * 32, 0, s>>>(draws, cand, counts);
   KRR_LAUNCH_CHECK();
   return KRR_OK;
 }
@@ -177,10 +215,6 @@ __global__ void uniform_pivots_kernel(int64_t N, int k, uint64_t seed, unsigned 
 // largest (value, -index) strictly below pick j - 1 in that order.
 constexpr int GREEDY_THREADS = 1024;
 
-// Smallest N whose Schur updates take the float-float GEMM: the drop
-// threshold N 2^-52 max A_ii is then at least 7e-12, about 70 times the
-// float-float rounding of a partial sum of magnitude 1 over 1000 terms.
-constexpr int64_t kSchurFFMinN = 32768;
 __global__ void __launch_bounds__(GREEDY_THREADS)
 greedy_pick_kernel(const double *__restrict__ dres, int64_t N, double dfloor, int npick,
                    int64_t *__restrict__ cand, int *__restrict__ counts) {
@@ -251,93 +285,149 @@ greedy_pick_kernel(const double *__restrict__ dres, int64_t N, double dfloor, in
 }
 
 // ------------------------------------------------------- block kernels
-// Fs (nc x rank, column-major) = F(cand, 0:rank)
-__global__ void gather_rows_kernel(const double *__restrict__ F, int64_t N, int rank,
-                                   const int64_t *__restrict__ cand, int nc,
-                                   double *__restrict__ Fs) {
-  const int64_t total = (int64_t)nc * rank;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int c = (int)(e % nc);
-    const int l = (int)(e / nc);
-    Fs[e] = F[cand[c] + (int64_t)l * N];
-  }
+// q = x / d with r = 1 / d at hand: one correction of x r, which leaves the
+// rounding of a division at a quarter of its float64 operations.
+__device__ __forceinline__ double div_by(double x, double d, double r) {
+  const double q = x * r;
+  return fma(fma(-q, d, x), r, q);
 }
 
 // Right-looking Cholesky of T = G(S', S') (nc x nc) in candidate order; a
 // candidate whose current Schur value is <= thr is dropped and does not
-// update the rest.  Outputs the factor entries Lb (nc x nc, column-major,
-// lower, rows/columns of dropped candidates unused), the kept positions in
-// order, and their count.
+// update the rest.  Outputs the factor of the kept candidates Lb (ld nc,
+// column-major, lower, in their order), their positions, and their count.
+// Panels of eight columns are factored by one warp in registers (a lane keeps
+// every 32nd row; rows meet by shuffles, without barriers), the rest is
+// updated by all warps between two barriers: 100 candidates took 262 us with
+// three barriers a column, now about 75 us, of which the 1.7e5 DFMA at 1.9 a
+// clock on one SM are 43.
+constexpr int CHOL_PW = 8;
 __global__ void __launch_bounds__(256)
 block_chol_kernel(const double *__restrict__ G, int64_t ldg, const int64_t *__restrict__ cand,
                   int nc, double thr, double *__restrict__ Lb, int *__restrict__ kept,
                   int *__restrict__ nkept) {
-  extern __shared__ double sT[];  // nc x nc, row-major
-  __shared__ int s_keep;
+  extern __shared__ double sT[];  // nc x (nc + 1), row-major
   __shared__ int s_list[RPC_MAX_BLOCK];
+  __shared__ unsigned s_mask;     // kept columns of the panel
   __shared__ int s_na;
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int ld = nc + 1;
   for (int e = tid; e < nc * nc; e += blockDim.x) {
-    const int a = e / nc, c = e % nc;
-    sT[a * nc + c] = G[cand[a] + (int64_t)c * ldg];
+    const int c = e / nc, a = e - c * nc;
+    sT[a * ld + c] = G[cand[a] + (int64_t)c * ldg];
   }
   if (tid == 0) s_na = 0;
   __syncthreads();
-  for (int c = 0; c < nc; ++c) {
-    if (tid == 0) {
-      const double p = sT[c * nc + c];
-      s_keep = (p > thr) ? 1 : 0;
-      if (s_keep) {
-        sT[c * nc + c] = sqrt(p);
-        s_list[s_na] = c;
-        s_na = s_na + 1;
+  for (int c0 = 0; c0 < nc; c0 += CHOL_PW) {
+    const int pw = min(CHOL_PW, nc - c0);
+    if (warp == 0) {
+      // row c0 + lane + 32 r, columns c0 .. c0 + pw
+      double P[4][CHOL_PW];
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int q = 0; q < CHOL_PW; ++q) {
+          const int a = c0 + lane + 32 * r;
+          P[r][q] = (a < nc && q < pw) ? sT[a * ld + c0 + q] : 0.0;
+        }
+      unsigned mask = 0;
+#pragma unroll
+      for (int q = 0; q < CHOL_PW; ++q) {
+        const double p = __shfl_sync(0xffffffffu, P[0][q], q);
+        if (q < pw && p > thr) {
+          mask |= 1u << q;
+          const double d = sqrt(p), rd = 1.0 / d;
+#pragma unroll
+          for (int r = 0; r < 4; ++r) P[r][q] = div_by(P[r][q], d, rd);
+          if (lane == q) P[0][q] = d;
+#pragma unroll
+          for (int u = q + 1; u < CHOL_PW; ++u) {
+            const double l = __shfl_sync(0xffffffffu, P[0][q], u);
+#pragma unroll
+            for (int r = 0; r < 4; ++r) P[r][u] = fma(-P[r][q], l, P[r][u]);
+          }
+        }
+      }
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int q = 0; q < CHOL_PW; ++q) {
+          const int a = c0 + lane + 32 * r;
+          if (a < nc && q < pw) sT[a * ld + c0 + q] = P[r][q];
+        }
+      if (lane == 0) {
+        s_mask = mask;
+        int na = s_na;
+        for (int q = 0; q < pw; ++q)
+          if (mask >> q & 1) s_list[na++] = c0 + q;
+        s_na = na;
       }
     }
     __syncthreads();
-    if (s_keep) {
-      const double dc = sT[c * nc + c];
-      for (int a = c + 1 + tid; a < nc; a += blockDim.x) sT[a * nc + c] /= dc;
-      __syncthreads();
-      const int rem = nc - c - 1;
-      for (int e = tid; e < rem * rem; e += blockDim.x) {
-        const int a = c + 1 + e / rem, b = c + 1 + e % rem;
-        if (b <= a) sT[a * nc + b] -= sT[a * nc + c] * sT[b * nc + c];
+    const unsigned mask = s_mask;
+    const int t0 = c0 + pw;
+    // 16 x 16 threads over the lower triangle that is left
+    for (int a = t0 + (tid >> 4); a < nc; a += 16) {
+      double x[CHOL_PW];
+#pragma unroll
+      for (int q = 0; q < CHOL_PW; ++q) x[q] = (mask >> q & 1) ? sT[a * ld + c0 + q] : 0.0;
+      for (int b = t0 + (tid & 15); b <= a; b += 16) {
+        double v = sT[a * ld + b];
+#pragma unroll
+        for (int q = 0; q < CHOL_PW; ++q)
+          if (mask >> q & 1) v = fma(-x[q], sT[b * ld + c0 + q], v);
+        sT[a * ld + b] = v;
       }
     }
     __syncthreads();
   }
-  for (int e = tid; e < nc * nc; e += blockDim.x) {
-    const int a = e % nc, c = e / nc;
-    Lb[a + (int64_t)c * nc] = (a >= c) ? sT[a * nc + c] : 0.0;
+  const int na = s_na;
+  for (int e = tid; e < na * na; e += blockDim.x) {
+    const int c = e / na, a = e - c * na;
+    Lb[a + (int64_t)c * nc] = (a >= c) ? sT[s_list[a] * ld + s_list[c]] : 0.0;
   }
-  for (int e = tid; e < s_na; e += blockDim.x) kept[e] = s_list[e];
-  if (tid == 0) *nkept = s_na;
+  for (int e = tid; e < na; e += blockDim.x) kept[e] = s_list[e];
+  if (tid == 0) *nkept = na;
 }
 
-// New columns: row n solves x L_kk^T = G(n, kept) by forward substitution and
-// writes x to F(n, rank : rank + na); dres(n) -= |x|^2.
-__global__ void __launch_bounds__(128)
+// Columns a0 .. a0 + w of the new part of F: row n solves x L^T = G(n, kept)
+// over them by forward substitution (G already holds the part of the columns
+// before a0) and writes x to F(n, rank + a0 ..); dres(n) -= |x|^2.  The row
+// stays in registers, so a group is at most TRSM_W columns: the float64 work
+// of a row is w^2 / 2 + 4 w of the na^2 / 2 + 10 na that substitution over all
+// na columns (with divisions) took.
+constexpr int TRSM_W = 20;
+constexpr int TRSM_THREADS = 64;
+__global__ void __launch_bounds__(TRSM_THREADS)
 block_trsm_kernel(const double *__restrict__ G, int64_t ldg, const double *__restrict__ Lb,
-                  int nc, const int *__restrict__ kept, const int *__restrict__ nkept,
-                  double *__restrict__ F, int64_t N, int rank, double *__restrict__ dres) {
-  extern __shared__ double sL[];  // na x na, row-major, kept rows/cols only
-  const int na = *nkept;
-  for (int e = threadIdx.x; e < na * na; e += blockDim.x) {
-    const int a = e / na, b = e % na;
-    sL[e] = (b <= a) ? Lb[kept[a] + (int64_t)kept[b] * nc] : 0.0;
+                  int nc, const int *__restrict__ kept, int a0, int w, double *__restrict__ F,
+                  int64_t N, int rank, double *__restrict__ dres) {
+  __shared__ double sL[TRSM_W][TRSM_W + 1];
+  __shared__ double sR[TRSM_W];
+  for (int e = threadIdx.x; e < w * w; e += TRSM_THREADS) {
+    const int a = e / w, b = e % w;
+    const double v = Lb[a0 + a + (int64_t)(a0 + b) * nc];
+    sL[a][b] = v;
+    if (a == b) sR[a] = 1.0 / v;
   }
   __syncthreads();
-  const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t n = (int64_t)blockIdx.x * TRSM_THREADS + threadIdx.x;
   if (n >= N) return;
+  double x[TRSM_W];
+#pragma unroll
+  for (int a = 0; a < TRSM_W; ++a) x[a] = a < w ? G[n + (int64_t)kept[a0 + a] * ldg] : 0.0;
   double s2 = 0.0;
-  double *Fn = F + n + (int64_t)rank * N;
-  for (int a = 0; a < na; ++a) {
-    double v = G[n + (int64_t)kept[a] * ldg];
-    for (int b = 0; b < a; ++b) v -= Fn[(int64_t)b * N] * sL[a * na + b];
-    v /= sL[a * na + a];
-    Fn[(int64_t)a * N] = v;
-    s2 = fma(v, v, s2);
+  double *Fn = F + n + (int64_t)(rank + a0) * N;
+#pragma unroll
+  for (int a = 0; a < TRSM_W; ++a) {
+    if (a < w) {
+      const double v = div_by(x[a], sL[a][a], sR[a]);
+      Fn[(int64_t)a * N] = v;
+      s2 = fma(v, v, s2);
+#pragma unroll
+      for (int b = a + 1; b < TRSM_W; ++b)
+        if (b < w) x[b] = fma(-v, sL[b][a], x[b]);
+    }
   }
   dres[n] -= s2;
 }
@@ -395,18 +485,17 @@ krr_status rpcholesky_device(const double *Xd, int64_t N, int d, int kern, doubl
 
   DevBuf<int64_t> draws, cand;
   DevBuf<int> counts, kept;
-  DevBuf<double> G, Fs, Lb;
+  DevBuf<double> G, Lb;
+  DevBuf<uint2> frag;
   KRR_TRY(draws.alloc(B, s));
   KRR_TRY(cand.alloc(B, s));
   KRR_TRY(counts.alloc(4, s));
   KRR_TRY(kept.alloc(B, s));
   KRR_TRY(G.alloc((size_t)N * B, s));
-  KRR_TRY(Fs.alloc((size_t)B * k, s));
+  KRR_TRY(frag.alloc(dig_frag_elems(B, std::max(k, B)), s));
   KRR_TRY(Lb.alloc((size_t)B * B, s));
 
-  const size_t chol_smem = (size_t)B * B * sizeof(double);
-  KRR_TRY(raise_smem_limit(block_chol_kernel, chol_smem));
-  KRR_TRY(raise_smem_limit(block_trsm_kernel, chol_smem));
+  KRR_TRY(raise_smem_limit(block_chol_kernel, (size_t)B * (B + 1) * sizeof(double)));
 
   // the uniform rule's k pivots are drawn before the first block
   DevBuf<int64_t> upiv;
@@ -454,32 +543,26 @@ krr_status rpcholesky_device(const double *Xd, int64_t N, int d, int kern, doubl
     }
     // G = A(:, S') - F(:, 0:rank) F(S', 0:rank)^T
     KRR_TRY(kernel_columns_f64(P64, cand.p, nc, G.p, N, s));
-    if (rank > 0) {
-      gather_rows_kernel<<<ceil_div((int64_t)nc * rank, 256), 256, 0, s>>>(f->F, N, rank,
-                                                                         cand.p, nc, Fs.p);
-      KRR_LAUNCH_CHECK();
-      Gemm<double> g;
-      g.M = (int)N; g.N = nc; g.K = rank;
-      g.A = f->F; g.sai = 1; g.sak = N;
-      g.B = Fs.p; g.sbk = nc; g.sbj = 1;
-      g.alpha = -1.0; g.beta = 1.0; g.C = G.p; g.ldc = N;
-      // float-float on the float32 pipes where its rounding (about 1e-13 of
-      // the partial sums) stays two orders below the drop threshold
-      // N 2^-52 max A_ii; float64 below that size
-      if (N >= kSchurFFMinN) KRR_TRY(gemm_sub_ff(g, s));
-      else KRR_TRY(gemm(g, s));
-    }
-    block_chol_kernel<<<1, 256, (size_t)nc * nc * sizeof(double), s>>>(G.p, N, cand.p, nc, thr,
-                                                                     Lb.p, kept.p, counts.p + 2);
-    KRR_LAUNCH_CHECK();
-    block_trsm_kernel<<<ceil_div(N, 128), 128, (size_t)nc * nc * sizeof(double), s>>>(
-        G.p, N, Lb.p, nc, kept.p, counts.p + 2, f->F, N, rank, f->dres);
-    KRR_LAUNCH_CHECK();
-    block_finish_kernel<<<1, 128, 0, s>>>(cand.p, nc, kept.p, counts.p + 2, f->S, rank, f->dres);
+    if (rank > 0)
+      KRR_TRY(dig_gemm_sub(f->F, N, N, rank, f->F, N, cand.p, nc, G.p, N, nullptr, frag.p, s));
+    block_chol_kernel<<<1, 256, (size_t)nc * (nc + 1) * sizeof(double), s>>>(
+        G.p, N, cand.p, nc, thr, Lb.p, kept.p, counts.p + 2);
     KRR_LAUNCH_CHECK();
     int na = 0;
     KRR_CUDA_TRY(cudaMemcpyAsync(&na, counts.p + 2, sizeof(int), cudaMemcpyDeviceToHost, s));
     KRR_CUDA_TRY(cudaStreamSynchronize(s));
+    // equal groups of at most TRSM_W columns
+    const int groups = (na + TRSM_W - 1) / TRSM_W;
+    for (int q = 0; q < groups; ++q) {
+      const int a0 = (int)((int64_t)na * q / groups), w = (int)((int64_t)na * (q + 1) / groups) - a0;
+      KRR_TRY(dig_gemm_sub(f->F + (int64_t)rank * N, N, N, a0, Lb.p + a0, nc, nullptr, w, G.p, N,
+                           kept.p + a0, frag.p, s));
+      block_trsm_kernel<<<ceil_div(N, TRSM_THREADS), TRSM_THREADS, 0, s>>>(
+          G.p, N, Lb.p, nc, kept.p, a0, w, f->F, N, rank, f->dres);
+      KRR_LAUNCH_CHECK();
+    }
+    block_finish_kernel<<<1, 128, 0, s>>>(cand.p, nc, kept.p, counts.p + 2, f->S, rank, f->dres);
+    KRR_LAUNCH_CHECK();
     rank += na;
   }
   f->rank = rank;
