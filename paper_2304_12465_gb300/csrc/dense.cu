@@ -1,144 +1,13 @@
-// Dense building blocks: strided SIMT GEMM (float32 / float64), blocked
-// float64 Cholesky and blocked lower-triangular inverse.  Used for the k x k
-// cores of Alg. 1 (lambda I + F^T F) and Alg. 2 (B^T B + H), the Schur update
-// of Alg. 3 and the triangular solves of both preconditioners.
+// Dense building blocks of the k x k cores of Alg. 1 (lambda I + F^T F) and
+// Alg. 2 (B^T B + H): Gram product, blocked float64 Cholesky and the inverse of
+// its factor.
+#include <algorithm>
+
 #include "dense.cuh"
 
 namespace krr {
 
 constexpr int GB_M = 64, GB_N = 64, GB_K = 16, G_THREADS = 256;
-
-template <typename T>
-__global__ void __launch_bounds__(G_THREADS)
-gemm_kernel(int M, int N, int K, const T *__restrict__ A, int64_t sai, int64_t sak,
-            const T *__restrict__ B, int64_t sbk, int64_t sbj, T *__restrict__ out,
-            int64_t ldo, int64_t slice_stride, int kslice, T alpha, T beta, int direct) {
-  __shared__ T As[GB_K][GB_M + 1];
-  __shared__ T Bs[GB_K][GB_N + 1];
-  const int tid = threadIdx.x;
-  const int tx = tid % 16, ty = tid / 16;
-  const int i0 = blockIdx.x * GB_M, j0 = blockIdx.y * GB_N;
-  const int kb = blockIdx.z * kslice;
-  const int ke = min(K, kb + kslice);
-  T acc[4][4];
-#pragma unroll
-  for (int r = 0; r < 4; ++r)
-#pragma unroll
-    for (int c = 0; c < 4; ++c) acc[r][c] = 0;
-  const bool a_kfast = (sak == 1 && sai != 1);
-  const bool b_kfast = (sbk == 1 && sbj != 1);
-  for (int k0 = kb; k0 < ke; k0 += GB_K) {
-#pragma unroll
-    for (int e = 0; e < (GB_M * GB_K) / G_THREADS; ++e) {
-      const int idx = tid + e * G_THREADS;
-      int ii, kk;
-      if (a_kfast) { kk = idx % GB_K; ii = idx / GB_K; }
-      else { ii = idx % GB_M; kk = idx / GB_M; }
-      const int gi = i0 + ii, gk = k0 + kk;
-      As[kk][ii] = (gi < M && gk < ke) ? A[(int64_t)gi * sai + (int64_t)gk * sak] : T(0);
-    }
-#pragma unroll
-    for (int e = 0; e < (GB_N * GB_K) / G_THREADS; ++e) {
-      const int idx = tid + e * G_THREADS;
-      int jj, kk;
-      if (b_kfast) { kk = idx % GB_K; jj = idx / GB_K; }
-      else { jj = idx % GB_N; kk = idx / GB_N; }
-      const int gj = j0 + jj, gk = k0 + kk;
-      Bs[kk][jj] = (gj < N && gk < ke) ? B[(int64_t)gk * sbk + (int64_t)gj * sbj] : T(0);
-    }
-    __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < GB_K; ++kk) {
-      T a[4], b[4];
-#pragma unroll
-      for (int r = 0; r < 4; ++r) a[r] = As[kk][ty + 16 * r];
-#pragma unroll
-      for (int c = 0; c < 4; ++c) b[c] = Bs[kk][tx + 16 * c];
-#pragma unroll
-      for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) acc[r][c] = fma(a[r], b[c], acc[r][c]);
-    }
-    __syncthreads();
-  }
-  T *o = out + (int64_t)blockIdx.z * slice_stride;
-#pragma unroll
-  for (int r = 0; r < 4; ++r)
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const int gi = i0 + ty + 16 * r, gj = j0 + tx + 16 * c;
-      if (gi < M && gj < N) {
-        T *dst = o + (int64_t)gi + (int64_t)gj * ldo;
-        if (direct) *dst = (beta == T(0)) ? alpha * acc[r][c] : fma(alpha, acc[r][c], beta * *dst);
-        else *dst = acc[r][c];
-      }
-    }
-}
-
-// C = beta C + alpha * sum_z P_z, P_z (M x N, ld M) in slices.
-template <typename T>
-__global__ void gemm_combine_kernel(int M, int N, const T *__restrict__ P, int slices,
-                                    T alpha, T beta, T *__restrict__ C, int64_t ldc) {
-  const int64_t total = (int64_t)M * N;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int i = (int)(e % M), j = (int)(e / M);
-    T acc = 0;
-    for (int z = 0; z < slices; ++z) acc += P[(int64_t)z * total + e];
-    T *c = C + (int64_t)i + (int64_t)j * ldc;
-    *c = (beta == T(0)) ? alpha * acc : beta * (*c) + alpha * acc;
-  }
-}
-
-int gemm_auto_split(int M, int N, int K) {
-  const int64_t tiles = (int64_t)((M + GB_M - 1) / GB_M) * ((N + GB_N - 1) / GB_N);
-  const int64_t want = (int64_t)num_sms() * 4;
-  if (tiles >= want || K < 4 * GB_K) return 1;
-  int64_t sk = (want + tiles - 1) / tiles;
-  const int64_t maxk = K / (8 * GB_K);
-  if (sk > maxk) sk = maxk;
-  if (sk > 64) sk = 64;
-  return (int)(sk < 1 ? 1 : sk);
-}
-
-template <typename T>
-krr_status gemm(const Gemm<T> &g, cudaStream_t s, int split_k) {
-  if (g.M <= 0 || g.N <= 0) return KRR_OK;
-  if (g.K <= 0) {
-    // C = beta C
-    DevBuf<T> z;
-    KRR_TRY(z.alloc((size_t)g.M * g.N, s));
-    KRR_CUDA_TRY(cudaMemsetAsync(z.p, 0, sizeof(T) * (size_t)g.M * g.N, s));
-    gemm_combine_kernel<T><<<ceil_div((int64_t)g.M * g.N, 256), 256, 0, s>>>(
-        g.M, g.N, z.p, 1, g.alpha, g.beta, g.C, g.ldc);
-    KRR_LAUNCH_CHECK();
-    return KRR_OK;
-  }
-  if (split_k < 1) split_k = 1;
-  int kslice = (g.K + split_k - 1) / split_k;
-  kslice = (kslice + GB_K - 1) / GB_K * GB_K;
-  const int slices = (g.K + kslice - 1) / kslice;
-  dim3 grid((g.M + GB_M - 1) / GB_M, (g.N + GB_N - 1) / GB_N, slices);
-  if (slices == 1) {
-    gemm_kernel<T><<<grid, G_THREADS, 0, s>>>(g.M, g.N, g.K, g.A, g.sai, g.sak, g.B, g.sbk,
-                                             g.sbj, g.C, g.ldc, 0, kslice, g.alpha, g.beta, 1);
-    KRR_LAUNCH_CHECK();
-    return KRR_OK;
-  }
-  DevBuf<T> P;
-  KRR_TRY(P.alloc((size_t)slices * g.M * g.N, s));
-  gemm_kernel<T><<<grid, G_THREADS, 0, s>>>(g.M, g.N, g.K, g.A, g.sai, g.sak, g.B, g.sbk,
-                                           g.sbj, P.p, g.M, (int64_t)g.M * g.N, kslice,
-                                           T(1), T(0), 0);
-  KRR_LAUNCH_CHECK();
-  int64_t total = (int64_t)g.M * g.N;
-  int blocks = ceil_div(total, 256);
-  if (blocks > num_sms() * 16) blocks = num_sms() * 16;
-  gemm_combine_kernel<T><<<blocks, 256, 0, s>>>(g.M, g.N, P.p, slices, g.alpha, g.beta,
-                                                g.C, g.ldc);
-  KRR_LAUNCH_CHECK();
-  return KRR_OK;
-}
 
 // ------------------------------------------------------------ Gram (F^T F)
 // Lower-triangular output tiles only.  float input: each K tile of GB_K
@@ -279,87 +148,115 @@ krr_status gram_lower(const T *F, int64_t N, int r, double *C, cudaStream_t s) {
 template krr_status gram_lower<float>(const float *, int64_t, int, double *, cudaStream_t);
 template krr_status gram_lower<double>(const double *, int64_t, int, double *, cudaStream_t);
 
-template krr_status gemm<double>(const Gemm<double> &, cudaStream_t, int);
-template krr_status gemm<float>(const Gemm<float> &, cudaStream_t, int);
-
 // ------------------------------------------------------------ Cholesky
-constexpr int CH_NB = 64;
+// Right-looking blocked Cholesky of the k x k cores.  The float64 pipe does
+// 1.9 DFMA a clock on one SM, so what one block does alone is kept small: the
+// diagonal block is 32 wide (11000 DFMA to factor and as many to invert it; a
+// 64-wide one took 168 us), its inverse turns the panel's triangular solve
+// into a product spread over the SMs by eight rows, and the trailing update
+// touches the lower triangle only.
+constexpr int CH_NB = 32;
+constexpr int CH_PANEL_ROWS = 8;
 
-// Factors the w x w diagonal block at A (lda) in place (lower) and writes the
-// inverse of its factor to Dinv (CH_NB x CH_NB, column-major, zero padded).
-// factor == 0: the block already holds a lower factor; only invert it.
-__global__ void __launch_bounds__(256)
-potrf_diag_kernel(double *__restrict__ A, int w, int64_t lda, double *__restrict__ Dinv,
+// Factors the w x w diagonal block at A (lda) in place (lower; factor == 0:
+// it already holds the factor) and writes the inverse of its factor to Dinv
+// (CH_NB x CH_NB, column-major, zero padded).  blockIdx.x: block of a batch of
+// diagonal blocks, CH_NB apart (n: size of the whole matrix).
+__global__ void __launch_bounds__(128)
+potrf_diag_kernel(double *__restrict__ A, int n, int64_t lda, double *__restrict__ Dinv,
                   int *__restrict__ status, int factor) {
-  extern __shared__ double smem[];
-  double *sA = smem;                        // CH_NB x (CH_NB+1)
-  double *sW = smem + CH_NB * (CH_NB + 1);  // CH_NB x (CH_NB+1)
-  const int tid = threadIdx.x;
-  constexpr int LD = CH_NB + 1;
-  for (int e = tid; e < w * w; e += blockDim.x) {
-    const int i = e % w, j = e / w;
-    sA[i * LD + j] = (i >= j) ? A[i + (int64_t)j * lda] : 0.0;
-  }
+  __shared__ double sA[CH_NB][CH_NB + 1], sW[CH_NB][CH_NB + 1];
+  const int o = blockIdx.x * CH_NB, w = min(CH_NB, n - o);
+  A += o + (int64_t)o * lda;
+  Dinv += (int64_t)blockIdx.x * CH_NB * CH_NB;
+  const int tid = threadIdx.x, i = tid & 31, q = tid >> 5;
+  for (int j = q; j < CH_NB; j += 4)
+    sA[i][j] = (i < w && j < w && i >= j) ? A[i + (int64_t)j * lda] : (i == j ? 1.0 : 0.0);
   __syncthreads();
   if (factor) {
     for (int j = 0; j < w; ++j) {
-      if (tid == 0) {
-        const double p = sA[j * LD + j];
-        if (!(p > 0.0)) atomicExch(status, 1);
-        sA[j * LD + j] = sqrt(p);
+      const double p = sA[j][j];
+      const double d = sqrt(p), rd = 1.0 / d;
+      __syncthreads();
+      if (q == 0) {
+        if (i == j) {
+          if (!(p > 0.0)) atomicExch(status, 1);
+          sA[j][j] = d;
+        } else if (i > j) {
+          const double x = sA[i][j], t = x * rd;
+          sA[i][j] = fma(fma(-t, d, x), rd, t);
+        }
       }
       __syncthreads();
-      const double dj = sA[j * LD + j];
-      for (int i = j + 1 + tid; i < w; i += blockDim.x) sA[i * LD + j] /= dj;
-      __syncthreads();
-      const int rem = w - j - 1;
-      for (int e = tid; e < rem * rem; e += blockDim.x) {
-        const int i = j + 1 + e % rem, l = j + 1 + e / rem;
-        if (l <= i) sA[i * LD + l] -= sA[i * LD + j] * sA[l * LD + j];
-      }
+      const double l = sA[i][j];
+      for (int c = j + 1 + q; c <= i; c += 4) sA[i][c] = fma(-l, sA[c][j], sA[i][c]);
       __syncthreads();
     }
-    for (int e = tid; e < w * w; e += blockDim.x) {
-      const int i = e % w, j = e / w;
-      if (i >= j) A[i + (int64_t)j * lda] = sA[i * LD + j];
-    }
+    for (int j = q; j < w; j += 4)
+      if (i >= j && i < w) A[i + (int64_t)j * lda] = sA[i][j];
   }
-  // inverse of the lower factor, one column per thread (forward substitution)
-  if (tid < CH_NB) {
-    const int c = tid;
-    for (int i = 0; i < CH_NB; ++i) {
-      double v = 0.0;
-      if (c < w && i < w && i >= c) {
-        v = (i == c) ? 1.0 : 0.0;
-        for (int l = c; l < i; ++l) v -= sA[i * LD + l] * sW[l * LD + c];
-        v /= sA[i * LD + i];
-      }
-      sW[i * LD + c] = v;
-    }
+  // inverse by forward substitution: four threads a column (partial sums of
+  // every fourth term, added by shuffles)
+  const int c = tid >> 2, t = tid & 3;
+  for (int r = 0; r < CH_NB; ++r) {
+    double v = 0.0;
+    for (int l = c + t; l < r; l += 4) v = fma(-sA[r][l], sW[l][c], v);
+    v += __shfl_xor_sync(0xffffffffu, v, 1);
+    v += __shfl_xor_sync(0xffffffffu, v, 2);
+    if (t == 0) sW[r][c] = r < c ? 0.0 : ((r == c ? 1.0 : 0.0) + v) / sA[r][r];
+    __syncwarp();
   }
   __syncthreads();
-  for (int e = tid; e < CH_NB * CH_NB; e += blockDim.x) {
-    const int i = e % CH_NB, j = e / CH_NB;
-    Dinv[i + j * CH_NB] = sW[i * LD + j];
+  for (int j = q; j < CH_NB; j += 4) Dinv[i + j * CH_NB] = (i < w && j < w) ? sW[i][j] : 0.0;
+}
+
+// A21 (r x w) <- A21 Dinv^T, eight rows a block.
+__global__ void __launch_bounds__(256)
+potrf_panel_kernel(double *__restrict__ A21, int r, int w, int64_t lda,
+                   const double *__restrict__ Dinv) {
+  __shared__ double sD[CH_NB][CH_NB + 1], sX[CH_PANEL_ROWS][CH_NB + 1];
+  const int tid = threadIdx.x;
+  for (int e = tid; e < CH_NB * CH_NB; e += 256) sD[e % CH_NB][e / CH_NB] = Dinv[e];
+  const int row = tid & 7, j = tid >> 3;   // 8 rows x 32 columns
+  const int i = blockIdx.x * CH_PANEL_ROWS + row;
+  sX[row][j] = (i < r && j < w) ? A21[i + (int64_t)j * lda] : 0.0;
+  __syncthreads();
+  double v = 0.0;
+#pragma unroll 8
+  for (int l = 0; l < CH_NB; ++l) v = fma(sX[row][l], sD[j][l], v);   // Dinv is lower
+  if (i < r && j < w) A21[i + (int64_t)j * lda] = v;
+}
+
+// A22 -= A21 A21^T on the lower triangle, 32 x 32 tiles (one a block).
+__global__ void __launch_bounds__(256)
+potrf_update_kernel(double *__restrict__ A21, int r, int w, int64_t lda) {
+  __shared__ double sI[CH_NB][33], sJ[CH_NB][33];   // [column of A21][row]
+  int t = blockIdx.x, ti = (int)((sqrtf(8.0f * t + 1.0f) - 1.0f) * 0.5f);
+  while (ti * (ti + 1) / 2 > t) --ti;
+  while ((ti + 1) * (ti + 2) / 2 <= t) ++ti;
+  const int tj = t - ti * (ti + 1) / 2;
+  const int tid = threadIdx.x;
+  for (int e = tid; e < CH_NB * 32; e += 256) {
+    const int l = e >> 5, x = e & 31;
+    const int i = ti * 32 + x, j = tj * 32 + x;
+    sI[l][x] = (i < r && l < w) ? A21[i + (int64_t)l * lda] : 0.0;
+    sJ[l][x] = (j < r && l < w) ? A21[j + (int64_t)l * lda] : 0.0;
   }
-}
-
-static krr_status diag_block(double *A, int w, int64_t lda, double *Dinv, int *status,
-                             int factor, cudaStream_t s) {
-  const size_t smem = 2 * CH_NB * (CH_NB + 1) * sizeof(double);
-  KRR_TRY(raise_smem_limit(potrf_diag_kernel, smem));
-  potrf_diag_kernel<<<1, 256, smem, s>>>(A, w, lda, Dinv, status, factor);
-  KRR_LAUNCH_CHECK();
-  return KRR_OK;
-}
-
-__global__ void copy_block_kernel(const double *__restrict__ src, int64_t lds, int rows,
-                                  int cols, double *__restrict__ dst, int64_t ldd) {
-  const int64_t total = (int64_t)rows * cols;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int i = (int)(e % rows), j = (int)(e / rows);
-    dst[i + j * ldd] = src[i + j * lds];
+  __syncthreads();
+  double *A22 = A21 + (int64_t)w * lda;
+  const int x = tid & 31, y = tid >> 5;   // row x, columns y + 8 u
+  double acc[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 8
+  for (int l = 0; l < CH_NB; ++l) {
+    const double a = sI[l][x];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) acc[u] = fma(a, sJ[l][y + 8 * u], acc[u]);
+  }
+  const int i = ti * 32 + x;
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int j = tj * 32 + y + 8 * u;
+    if (i < r && j <= i) A22[i + (int64_t)j * lda] -= acc[u];
   }
 }
 
@@ -368,32 +265,20 @@ krr_status potrf_lower(double *A, int n, int64_t lda, cudaStream_t s) {
   DevBuf<int> status;
   KRR_TRY(status.alloc(1, s));
   KRR_CUDA_TRY(cudaMemsetAsync(status.p, 0, sizeof(int), s));
-  DevBuf<double> dinv, T;
+  DevBuf<double> dinv;
   KRR_TRY(dinv.alloc(CH_NB * CH_NB, s));
-  KRR_TRY(T.alloc((size_t)n * CH_NB, s));
   for (int o = 0; o < n; o += CH_NB) {
-    const int w = (n - o < CH_NB) ? n - o : CH_NB;
+    const int w = std::min(CH_NB, n - o);
     double *Abb = A + o + (int64_t)o * lda;
-    KRR_TRY(diag_block(Abb, w, lda, dinv.p, status.p, 1, s));
+    potrf_diag_kernel<<<1, 128, 0, s>>>(Abb, w, lda, dinv.p, status.p, 1);
+    KRR_LAUNCH_CHECK();
     const int r = n - o - w;
     if (r <= 0) break;
-    double *A21 = Abb + w;
-    // T (r x w) = A21 Dinv^T
-    Gemm<double> g;
-    g.M = r; g.N = w; g.K = w;
-    g.A = A21; g.sai = 1; g.sak = lda;
-    g.B = dinv.p; g.sbk = CH_NB; g.sbj = 1;
-    g.alpha = 1.0; g.beta = 0.0; g.C = T.p; g.ldc = r;
-    KRR_TRY(gemm(g, s));
-    copy_block_kernel<<<ceil_div((int64_t)r * w, 256), 256, 0, s>>>(T.p, r, r, w, A21, lda);
+    potrf_panel_kernel<<<ceil_div(r, CH_PANEL_ROWS), 256, 0, s>>>(Abb + w, r, w, lda, dinv.p);
     KRR_LAUNCH_CHECK();
-    // A22 -= T T^T
-    Gemm<double> u;
-    u.M = r; u.N = r; u.K = w;
-    u.A = T.p; u.sai = 1; u.sak = r;
-    u.B = T.p; u.sbk = r; u.sbj = 1;
-    u.alpha = -1.0; u.beta = 1.0; u.C = A21 + (int64_t)w * lda; u.ldc = lda;
-    KRR_TRY(gemm(u, s, gemm_auto_split(r, r, w)));
+    const int tiles = (r + 31) / 32;
+    potrf_update_kernel<<<tiles * (tiles + 1) / 2, 256, 0, s>>>(Abb + w, r, w, lda);
+    KRR_LAUNCH_CHECK();
   }
   int h = 0;
   KRR_CUDA_TRY(cudaMemcpyAsync(&h, status.p, sizeof(int), cudaMemcpyDeviceToHost, s));
@@ -406,42 +291,91 @@ krr_status potrf_lower(double *A, int n, int64_t lda, cudaStream_t s) {
   return KRR_OK;
 }
 
+// W <- the inverses of the diagonal blocks, zero elsewhere.
+__global__ void trinv_init_kernel(const double *__restrict__ Dinv, int n, double *__restrict__ W) {
+  const int64_t total = (int64_t)n * n;
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
+       e += (int64_t)gridDim.x * blockDim.x) {
+    const int j = (int)(e / n), i = (int)(e - (int64_t)j * n);
+    const int b = i / CH_NB;
+    W[e] = (b == j / CH_NB)
+               ? Dinv[(int64_t)b * CH_NB * CH_NB + (i - b * CH_NB) + (j - b * CH_NB) * CH_NB]
+               : 0.0;
+  }
+}
+
+// One half of a doubling step of the inverse: the pairs of size-h diagonal
+// blocks (rows p 2h .. of the first, + h of the second) whose inverses W holds.
+//   first  half: T21 = L21 W11          (columns of W11 are lower: k >= column)
+//   second half: W21 = -W22 T21         (rows of W22 are lower: k <= row)
+// T (n x n, only the blocks below the pairs' diagonals) is scratch.  A block
+// does a 32 x 32 tile over the k that are not zero.
+template <bool FIRST>
+__global__ void __launch_bounds__(256)
+trinv_level_kernel(const double *__restrict__ L, int64_t lda, int n, int h, double *__restrict__ W,
+                   double *__restrict__ T) {
+  __shared__ double sX[32][33], sY[32][33];   // [k][row], [k][column]
+  const int o = blockIdx.z * 2 * h;            // first row of the pair
+  const int r0 = o + h + blockIdx.x * 32, c0 = o + blockIdx.y * 32;
+  if (r0 >= n) return;
+  const int rows = min(o + 2 * h, n);
+  const int tid = threadIdx.x, x = tid & 31, y = tid >> 5;
+  double acc[4] = {0.0, 0.0, 0.0, 0.0};
+  const int kb = FIRST ? c0 : o + h, ke = FIRST ? o + h : min(r0 + 32, rows);
+  for (int k0 = kb; k0 < ke; k0 += 32) {
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int kk = y + 8 * u, k = k0 + kk;
+      // X(row, k): contiguous in rows; Y(k, column): contiguous in k
+      double a = 0.0, b = 0.0;
+      if (r0 + x < rows && k < ke)
+        a = FIRST ? L[r0 + x + (int64_t)k * lda] : W[r0 + x + (int64_t)k * n];
+      const int kx = k0 + x;
+      if (kx < ke) b = FIRST ? W[kx + (int64_t)(c0 + kk) * n] : T[kx + (int64_t)(c0 + kk) * n];
+      sX[kk][x] = a;
+      sY[x][kk] = b;
+    }
+    __syncthreads();
+#pragma unroll 8
+    for (int l = 0; l < 32; ++l) {
+      const double a = sX[l][x];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) acc[u] = fma(a, sY[l][y + 8 * u], acc[u]);
+    }
+  }
+  if (r0 + x < rows)
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int64_t e = r0 + x + (int64_t)(c0 + y + 8 * u) * n;
+      if (FIRST) T[e] = acc[u];
+      else W[e] = -acc[u];
+    }
+}
+
+// Inverse by doubling: the diagonal blocks' inverses (one launch), then pairs
+// of inverted blocks of 32, 64, ... joined by two products a level, all pairs
+// of a level in one launch.  Row by row of blocks (each row a product with
+// everything before it) it was a chain of small grids: 30 launches and 9 ms at
+// n = 1000.
 krr_status trinv_lower(const double *L, int n, int64_t lda, double *W, cudaStream_t s) {
   if (n <= 0) return KRR_OK;
-  KRR_CUDA_TRY(cudaMemsetAsync(W, 0, sizeof(double) * (size_t)n * n, s));
-  DevBuf<int> status;
-  KRR_TRY(status.alloc(1, s));
-  KRR_CUDA_TRY(cudaMemsetAsync(status.p, 0, sizeof(int), s));
   const int nb = (n + CH_NB - 1) / CH_NB;
   DevBuf<double> dinv, T;
   KRR_TRY(dinv.alloc((size_t)nb * CH_NB * CH_NB, s));
-  KRR_TRY(T.alloc((size_t)CH_NB * n, s));
-  for (int b = 0; b < nb; ++b) {
-    const int o = b * CH_NB;
-    const int w = (n - o < CH_NB) ? n - o : CH_NB;
-    KRR_TRY(diag_block(const_cast<double *>(L) + o + (int64_t)o * lda, w, lda,
-                       dinv.p + (size_t)b * CH_NB * CH_NB, status.p, 0, s));
-    copy_block_kernel<<<ceil_div((int64_t)w * w, 256), 256, 0, s>>>(
-        dinv.p + (size_t)b * CH_NB * CH_NB, CH_NB, w, w, W + o + (int64_t)o * n, n);
+  KRR_TRY(T.alloc((size_t)n * n, s));
+  potrf_diag_kernel<<<nb, 128, 0, s>>>(const_cast<double *>(L), n, lda, dinv.p, nullptr, 0);
+  KRR_LAUNCH_CHECK();
+  const int64_t g = std::min<int64_t>(((int64_t)n * n + 255) / 256, (int64_t)num_sms() * 16);
+  trinv_init_kernel<<<(unsigned)g, 256, 0, s>>>(dinv.p, n, W);
+  KRR_LAUNCH_CHECK();
+  for (int h = CH_NB; h < n; h *= 2) {
+    const int pairs = (n - h + 2 * h - 1) / (2 * h);   // pairs with a second block
+    const dim3 grid(h / 32, h / 32, pairs);
+    trinv_level_kernel<true><<<grid, 256, 0, s>>>(L, lda, n, h, W, T.p);
     KRR_LAUNCH_CHECK();
-  }
-  for (int b = 1; b < nb; ++b) {
-    const int o = b * CH_NB;
-    const int w = (n - o < CH_NB) ? n - o : CH_NB;
-    // T (w x o) = L(o:o+w, 0:o) W(0:o, 0:o)
-    Gemm<double> g;
-    g.M = w; g.N = o; g.K = o;
-    g.A = L + o; g.sai = 1; g.sak = lda;
-    g.B = W; g.sbk = 1; g.sbj = n;
-    g.alpha = 1.0; g.beta = 0.0; g.C = T.p; g.ldc = w;
-    KRR_TRY(gemm(g, s));
-    // W(o:o+w, 0:o) = -Dinv_b T
-    Gemm<double> h;
-    h.M = w; h.N = o; h.K = w;
-    h.A = dinv.p + (size_t)b * CH_NB * CH_NB; h.sai = 1; h.sak = CH_NB;
-    h.B = T.p; h.sbk = 1; h.sbj = w;
-    h.alpha = -1.0; h.beta = 0.0; h.C = W + o; h.ldc = n;
-    KRR_TRY(gemm(h, s));
+    trinv_level_kernel<false><<<grid, 256, 0, s>>>(L, lda, n, h, W, T.p);
+    KRR_LAUNCH_CHECK();
   }
   return KRR_OK;
 }
@@ -476,24 +410,6 @@ krr_status transpose_square(const double *A, int n, double *B, cudaStream_t s) {
   if (n <= 0) return KRR_OK;
   dim3 grid((n + 31) / 32, (n + 31) / 32), block(32, 8);
   transpose_kernel<<<grid, block, 0, s>>>(A, n, B);
-  KRR_LAUNCH_CHECK();
-  return KRR_OK;
-}
-
-__global__ void symmetrize_kernel(double *A, int n, int64_t lda) {
-  const int64_t total = (int64_t)n * n;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int i = (int)(e % n), j = (int)(e / n);
-    if (j > i) A[i + (int64_t)j * lda] = A[j + (int64_t)i * lda];
-  }
-}
-
-krr_status symmetrize_lower(double *A, int n, int64_t lda, cudaStream_t s) {
-  if (n <= 0) return KRR_OK;
-  int blocks = ceil_div((int64_t)n * n, 256);
-  if (blocks > num_sms() * 16) blocks = num_sms() * 16;
-  symmetrize_kernel<<<blocks, 256, 0, s>>>(A, n, lda);
   KRR_LAUNCH_CHECK();
   return KRR_OK;
 }

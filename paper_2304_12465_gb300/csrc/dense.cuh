@@ -1,29 +1,11 @@
-// Dense building blocks (dense.cu): a strided SIMT GEMM, the blocked float64
-// Cholesky factorisation and the blocked inverse of a lower-triangular factor.
+// Dense building blocks (dense.cu, digits.cu): products by digits, the Gram
+// product, the blocked float64 Cholesky factorisation and the inverse of a
+// lower-triangular factor.
 #pragma once
 
 #include "common.cuh"
 
 namespace krr {
-
-// C(MxN, column-major, ldc) = alpha * A(MxK) B(KxN) + beta * C, where element
-// (i, k) of A is A[i*sai + k*sak] and element (k, j) of B is B[k*sbk + j*sbj].
-// split_k > 1 sums K in slices through a workspace, in a fixed order.
-template <typename T>
-struct Gemm {
-  int M = 0, N = 0, K = 0;
-  T alpha = 1;
-  const T *A = nullptr;
-  int64_t sai = 0, sak = 0;
-  const T *B = nullptr;
-  int64_t sbk = 0, sbj = 0;
-  T beta = 0;
-  T *C = nullptr;
-  int64_t ldc = 0;
-};
-
-template <typename T>
-krr_status gemm(const Gemm<T> &g, cudaStream_t s, int split_k = 1);
 
 // C (N x nc, ldc) -= A (N x K, lda) B^T for float64 matrices with entries in
 // [-1, 1] whose products' sums stay below 4 in magnitude, on the tensor cores
@@ -42,9 +24,6 @@ krr_status dig_gemm_sub(const double *A, int64_t lda, int64_t N, int K, const do
 template <typename T>
 krr_status gram_lower(const T *F, int64_t N, int r, double *C, cudaStream_t s);
 
-// Picks a split-K count that fills the machine for a long, thin reduction.
-int gemm_auto_split(int M, int N, int K);
-
 // In-place lower Cholesky of the n x n column-major matrix A (lda): on return
 // the lower triangle holds L with A = L L^T (the upper triangle is scratch).
 // Returns KRR_ECHOL if a pivot is not positive (NaN included).
@@ -59,8 +38,5 @@ krr_status add_diagonal(double *A, int n, int64_t lda, double v, cudaStream_t s)
 
 // B = A^T for n x n column-major matrices (no aliasing).
 krr_status transpose_square(const double *A, int n, double *B, cudaStream_t s);
-
-// Mirror the lower triangle into the upper one.
-krr_status symmetrize_lower(double *A, int n, int64_t lda, cudaStream_t s);
 
 }  // namespace krr

@@ -11,6 +11,7 @@
 // uses a product that regenerates the N x k block A(:,S) twice per
 // application in float32 (u = A(:,S) beta, then A(S,:) u), with the
 // preconditioner W^T W, W = L^{-1}, P = L L^T.
+#include <algorithm>
 #include <chrono>
 
 #include "dense.cuh"
@@ -214,10 +215,10 @@ __global__ void kss_kernel(const double *__restrict__ X, int d, int kern, double
   H[e] = kappa_point_f64(X + S[i] * d, X + S[j] * d, d, kern, sigma);
 }
 
-__global__ void h_finish_kernel(double *__restrict__ H, int k, double lambda, double shift_scale) {
-  // trace by one block, then H = lambda A + shift I
+// shift = shift_scale tr(A(S,S)), one block
+__global__ void h_trace_kernel(const double *__restrict__ H, int k, double shift_scale,
+                               double *__restrict__ shift) {
   __shared__ double red[32];
-  __shared__ double tr;
   double t = 0.0;
   for (int i = threadIdx.x; i < k; i += blockDim.x) t += H[i + (int64_t)i * k];
   t = warp_sum(t);
@@ -226,13 +227,27 @@ __global__ void h_finish_kernel(double *__restrict__ H, int k, double lambda, do
   if (threadIdx.x == 0) {
     double s = 0.0;
     for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[w];
-    tr = s;
+    *shift = shift_scale * s;
   }
-  __syncthreads();
-  const double shift = shift_scale * tr;
-  for (int64_t e = threadIdx.x; e < (int64_t)k * k; e += blockDim.x) {
-    const int i = (int)(e % k), j = (int)(e / k);
-    H[e] = lambda * H[e] + ((i == j) ? shift : 0.0);
+}
+
+// H = lambda A + shift I
+__global__ void h_finish_kernel(double *__restrict__ H, int k, double lambda,
+                                const double *__restrict__ shift) {
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < (int64_t)k * k;
+       e += (int64_t)gridDim.x * blockDim.x)
+    H[e] = lambda * H[e] + ((e % (k + 1)) == 0 ? *shift : 0.0);
+}
+
+// P (lower triangle B^T B) += H, mirrored into the upper triangle.
+__global__ void add_symmetric_kernel(const double *__restrict__ H, int k, double *__restrict__ P) {
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < (int64_t)k * k;
+       e += (int64_t)gridDim.x * blockDim.x) {
+    const int j = (int)(e / k), i = (int)(e - (int64_t)j * k);
+    if (i < j) continue;
+    const double v = P[e] + H[e];
+    P[e] = v;
+    P[j + (int64_t)i * k] = v;
   }
 }
 
@@ -452,8 +467,15 @@ krr_status krill_build_device(krill_precond *P, cudaStream_t s) {
   kss_kernel<<<ceil_div((int64_t)k * k, 256), 256, 0, s>>>(P->X, P->d, P->kern, P->sigma, P->S,
                                                           k, P->H);
   KRR_LAUNCH_CHECK();
-  h_finish_kernel<<<1, 1024, 0, s>>>(P->H, k, P->lambda, (double)N * 2.220446049250313e-16);
-  KRR_LAUNCH_CHECK();
+  {
+    DevBuf<double> shift;
+    KRR_TRY(shift.alloc(1, s));
+    h_trace_kernel<<<1, 1024, 0, s>>>(P->H, k, (double)N * 2.220446049250313e-16, shift.p);
+    KRR_LAUNCH_CHECK();
+    const int64_t g = std::min<int64_t>(((int64_t)k * k + 255) / 256, (int64_t)num_sms() * 16);
+    h_finish_kernel<<<(unsigned)g, 256, 0, s>>>(P->H, k, P->lambda, shift.p);
+    KRR_LAUNCH_CHECK();
+  }
   // Phi and its row lists
   DevBuf<int32_t> rows, col_n;
   DevBuf<float> vals, col_v;
@@ -495,14 +517,11 @@ krr_status krill_build_device(krill_precond *P, cudaStream_t s) {
   }
   // P = B^T B + H
   KRR_TRY(dev_alloc(&P->P, (size_t)k * k));
-  KRR_CUDA_TRY(cudaMemcpyAsync(P->P, P->H, sizeof(double) * k * k, cudaMemcpyDeviceToDevice, s));
+  KRR_TRY(gram_lower<double>(P->Bsk, sr, k, P->P, s));
   {
-    Gemm<double> g;
-    g.M = k; g.N = k; g.K = sr;
-    g.A = P->Bsk; g.sai = sr; g.sak = 1;
-    g.B = P->Bsk; g.sbk = 1; g.sbj = sr;
-    g.alpha = 1.0; g.beta = 1.0; g.C = P->P; g.ldc = k;
-    KRR_TRY(gemm(g, s, gemm_auto_split(k, k, sr)));
+    const int64_t g = std::min<int64_t>(((int64_t)k * k + 255) / 256, (int64_t)num_sms() * 16);
+    add_symmetric_kernel<<<(unsigned)g, 256, 0, s>>>(P->H, k, P->P);
+    KRR_LAUNCH_CHECK();
   }
   KRR_TRY(dev_alloc(&P->L, (size_t)k * k));
   KRR_CUDA_TRY(cudaMemcpyAsync(P->L, P->P, sizeof(double) * k * k, cudaMemcpyDeviceToDevice, s));
