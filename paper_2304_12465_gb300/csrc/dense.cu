@@ -165,35 +165,49 @@ constexpr int CH_PANEL_ROWS = 8;
 __global__ void __launch_bounds__(128)
 potrf_diag_kernel(double *__restrict__ A, int n, int64_t lda, double *__restrict__ Dinv,
                   int *__restrict__ status, int factor) {
-  __shared__ double sA[CH_NB][CH_NB + 1], sW[CH_NB][CH_NB + 1];
+  __shared__ double sA[CH_NB][CH_NB + 1], sW[CH_NB][CH_NB + 1], sR[CH_NB];
+  __shared__ unsigned short order[CH_NB * (CH_NB + 1) / 2];
   const int o = blockIdx.x * CH_NB, w = min(CH_NB, n - o);
   A += o + (int64_t)o * lda;
   Dinv += (int64_t)blockIdx.x * CH_NB * CH_NB;
   const int tid = threadIdx.x, i = tid & 31, q = tid >> 5;
   for (int j = q; j < CH_NB; j += 4)
     sA[i][j] = (i < w && j < w && i >= j) ? A[i + (int64_t)j * lda] : (i == j ? 1.0 : 0.0);
+  // the lower triangle's entries, last column first: those that the update of
+  // column j touches are a prefix, which the threads share without idle lanes
+  for (int j = q; j < CH_NB; j += 4) {
+    const int m = CH_NB - 1 - j;   // entries of the columns after j
+    if (i >= j) order[m * (m + 1) / 2 + (i - j)] = (unsigned short)(i << 8 | j);
+  }
   __syncthreads();
   if (factor) {
-    for (int j = 0; j < w; ++j) {
-      const double p = sA[j][j];
-      const double d = sqrt(p), rd = 1.0 / d;
-      __syncthreads();
+    for (int j = 0; j < CH_NB; ++j) {
       if (q == 0) {
+        const double p = sA[j][j];
+        double d, r;
+        sqrt_and_inverse(p, &d, &r);
         if (i == j) {
           if (!(p > 0.0)) atomicExch(status, 1);
           sA[j][j] = d;
+          sR[j] = r;
         } else if (i > j) {
-          const double x = sA[i][j], t = x * rd;
-          sA[i][j] = fma(fma(-t, d, x), rd, t);
+          const double x = sA[i][j], t = x * r;
+          sA[i][j] = fma(fma(-t, d, x), r, t);
         }
       }
       __syncthreads();
-      const double l = sA[i][j];
-      for (int c = j + 1 + q; c <= i; c += 4) sA[i][c] = fma(-l, sA[c][j], sA[i][c]);
+      const int m = CH_NB - 1 - j, cnt = m * (m + 1) / 2;
+      for (int e = tid; e < cnt; e += 128) {
+        const int a = order[e] >> 8, c = order[e] & 255;
+        sA[a][c] = fma(-sA[a][j], sA[c][j], sA[a][c]);
+      }
       __syncthreads();
     }
     for (int j = q; j < w; j += 4)
       if (i >= j && i < w) A[i + (int64_t)j * lda] = sA[i][j];
+  } else {
+    if (tid < CH_NB) sR[tid] = 1.0 / sA[tid][tid];
+    __syncthreads();
   }
   // inverse by forward substitution: four threads a column (partial sums of
   // every fourth term, added by shuffles)
@@ -203,7 +217,7 @@ potrf_diag_kernel(double *__restrict__ A, int n, int64_t lda, double *__restrict
     for (int l = c + t; l < r; l += 4) v = fma(-sA[r][l], sW[l][c], v);
     v += __shfl_xor_sync(0xffffffffu, v, 1);
     v += __shfl_xor_sync(0xffffffffu, v, 2);
-    if (t == 0) sW[r][c] = r < c ? 0.0 : ((r == c ? 1.0 : 0.0) + v) / sA[r][r];
+    if (t == 0) sW[r][c] = r < c ? 0.0 : (r == c ? sR[r] : v * sR[r]);
     __syncwarp();
   }
   __syncthreads();

@@ -23,8 +23,8 @@ namespace krr {
 // sets *bad.  xa or xb may be NULL (a rectangular product needs one of them).
 // cshift is added to c on both sides (7 for the Gaussian: D = log2 kappa + 14).
 // A block of 16 halves is assembled in registers and stored as two 16-byte
-// words; half by half the stores took 66 us at N = 1e5, d = 16 (both
-// operands), like this 24 us.
+// words, and what follows the difference and the scaling, which are float64
+// (at 1.9 operations a clock and SM they bound the kernel), is float32.
 template <int NH, int CSEP>
 __global__ void __launch_bounds__(128)
 prepare_tc5_kernel(const double *__restrict__ X, int64_t N, int d,
@@ -41,7 +41,14 @@ prepare_tc5_kernel(const double *__restrict__ X, int64_t N, int d,
   auto pack = [](__half lo, __half hi) {
     return (uint32_t)__half_as_ushort(lo) | ((uint32_t)__half_as_ushort(hi) << 16);
   };
-  double nrm = 0.0;
+  // |h + l|^2 as an unevaluated float sum: the three products of a square are
+  // exact in float32 (h and l have 11 bits)
+  float sh = 0.0f, sl = 0.0f;
+  auto add = [&](float v) {
+    const float t = __fadd_rn(sh, v), z = __fsub_rn(t, sh);
+    sl = __fadd_rn(sl, __fadd_rn(__fsub_rn(sh, __fsub_rn(t, z)), __fsub_rn(v, z)));
+    sh = t;
+  };
   bool out_of_range = false;
   uint32_t hw[8];
 #pragma unroll
@@ -49,17 +56,22 @@ prepare_tc5_kernel(const double *__restrict__ X, int64_t N, int d,
     uint32_t lw[8];
 #pragma unroll
     for (int t = 0; t < 8; ++t) {
-      __half h[2], l[2];
+      __half h[2] = {__ushort_as_half(0), __ushort_as_half(0)}, l[2] = {h[0], h[0]};
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
         const int k = b * 16 + 2 * t + u;
-        const double v = (k < d) ? (X[i * d + k] - mean[k]) * scale : 0.0;
-        if (!(fabs(v) <= (double)T5_MAX_COORD)) out_of_range = true;
-        h[u] = __double2half(v);
-        const double hv = (double)__half2float(h[u]);
-        l[u] = __double2half(v - hv);
-        const double e = hv + (double)__half2float(l[u]);
-        nrm = fma(e, e, nrm);
+        if (k < d) {
+          const double v = (X[i * d + k] - mean[k]) * scale;
+          const float vh = (float)v, vl = (float)(v - (double)vh);
+          if (!(fabsf(vh) <= T5_MAX_COORD)) out_of_range = true;
+          h[u] = __float2half_rn(vh);
+          const float hf = __half2float(h[u]);
+          l[u] = __float2half_rn(__fadd_rn(__fsub_rn(vh, hf), vl));
+          const float lf = __half2float(l[u]);
+          add(__fmul_rn(hf, hf));
+          add(__fmul_rn(2.0f * hf, lf));
+          sl = __fmaf_rn(lf, lf, sl);
+        }
       }
       hw[t] = pack(h[0], h[1]);
       lw[t] = pack(l[0], l[1]);
@@ -71,7 +83,7 @@ prepare_tc5_kernel(const double *__restrict__ X, int64_t N, int d,
       store(xb, b, hw);
     }
   }
-  const double c = -0.5 * nrm + cshift;
+  const double c = -0.5 * ((double)sh + (double)sl) + cshift;
   if (!(fabs(c) <= (double)T5_MAX_C)) out_of_range = true;
   const __half c1 = __double2half(c);
   const double r1 = c - (double)__half2float(c1);
@@ -277,6 +289,43 @@ __global__ void t5_reduce_kernel(const float *__restrict__ part, int64_t Nr, int
     Y[(int64_t)c * ldy + i] =
         V ? (TV5)(acc + lambda * (double)V[(int64_t)c * ldv + i]) : (TV5)acc;
   }
+}
+
+// The same sums for row blocks that many CTAs share (few rows against many
+// columns, or a small product): 32 rows a block, whose eight warps take every
+// eighth segment each; the warps' sums are added in warp order.  With one
+// thread a row the chain of loads took 13.3 us at N = 2000 (32 segments a row)
+// and 16.2 us at 1000 rows by 2e5 columns (78).
+constexpr int T5_RED_WARPS = 8;
+template <typename TV5>
+__global__ void __launch_bounds__(32 * T5_RED_WARPS)
+t5_reduce_many_kernel(const float *__restrict__ part, int64_t Nr, int m, int M, int C, int64_t T,
+                      int G, int J, int CG, const int *__restrict__ vexp, double lambda,
+                      const TV5 *__restrict__ V, int64_t ldv, TV5 *__restrict__ Y, int64_t ldy,
+                      const int *__restrict__ fault, int *__restrict__ flags) {
+  __shared__ double red[T5_RED_WARPS][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t i0 = (int64_t)blockIdx.x * 32, i = i0 + lane;
+  const int c = blockIdx.y;
+  if (flags && i0 == 0 && c == 0 && threadIdx.x == 0) flags[1] = *fault;
+  const int64_t rb = i0 / T5_RB;
+  const int r = (int)(i0 % T5_RB) + lane;
+  const int b_lo = t5_cta_of(rb * C, T, G);
+  const int b_hi = t5_cta_of(rb * C + C - 1, T, G);
+  double acc = 0.0;
+  for (int b = b_lo + warp; b <= b_hi; b += T5_RED_WARPS) {
+    const int64_t j = rb - ((int64_t)b * T / G) / C;
+    for (int cg = 0; cg < CG; ++cg)
+      acc += (double)part[((((int64_t)b * J + j) * CG + cg) * M + c) * T5_RB + r];
+  }
+  red[warp][lane] = acc;
+  __syncthreads();
+  if (warp != 0 || i >= Nr) return;
+#pragma unroll
+  for (int w = 1; w < T5_RED_WARPS; ++w) acc += red[w][lane];
+  if (vexp) acc = ldexp(acc, -14 - vexp[c]);
+  Y[(int64_t)c * ldy + i] =
+      V ? (TV5)(acc + lambda * (double)V[(int64_t)c * ldv + i]) : (TV5)acc;
 }
 
 // Right-hand sides of the column points as the kernel's shared tiles hold
@@ -595,10 +644,16 @@ static krr_status tc5_products(const PointsF32 &R, const PointsF32 &P, double la
       return KRR_ECUDA;
     }
     const int CG = t5_variant_ew(variant) / 4;
-    t5_reduce_kernel<TV5><<<ceil_div(Nr, 256), 256, 0, s>>>(
-        part.p, Nr, mg, M, g.C, g.T, g.G, g.J, CG,
-        t5_variant_tv(variant) ? t5_vexp(part.p, g, M) : nullptr, lambda, square ? Vg : nullptr,
-        ldv, Y + (int64_t)c0 * ldy, ldy, fault, flags);
+    const int *vexp = t5_variant_tv(variant) ? t5_vexp(part.p, g, M) : nullptr;
+    const TV5 *Vs = square ? Vg : nullptr;
+    TV5 *Yg = Y + (int64_t)c0 * ldy;
+    // more than four CTAs a row block: the grouped sum
+    if ((int64_t)g.C * g.G > 4 * g.T)
+      t5_reduce_many_kernel<TV5><<<dim3(ceil_div(Nr, 32), mg), 32 * T5_RED_WARPS, 0, s>>>(
+          part.p, Nr, mg, M, g.C, g.T, g.G, g.J, CG, vexp, lambda, Vs, ldv, Yg, ldy, fault, flags);
+    else
+      t5_reduce_kernel<TV5><<<ceil_div(Nr, 256), 256, 0, s>>>(
+          part.p, Nr, mg, M, g.C, g.T, g.G, g.J, CG, vexp, lambda, Vs, ldv, Yg, ldy, fault, flags);
     KRR_LAUNCH_CHECK();
   }
   return KRR_OK;

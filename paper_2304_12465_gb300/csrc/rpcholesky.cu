@@ -336,7 +336,8 @@ block_chol_kernel(const double *__restrict__ G, int64_t ldg, const int64_t *__re
         const double p = __shfl_sync(0xffffffffu, P[0][q], q);
         if (q < pw && p > thr) {
           mask |= 1u << q;
-          const double d = sqrt(p), rd = 1.0 / d;
+          double d, rd;
+          sqrt_and_inverse(p, &d, &rd);
 #pragma unroll
           for (int r = 0; r < 4; ++r) P[r][q] = div_by(P[r][q], d, rd);
           if (lane == q) P[0][q] = d;
