@@ -391,7 +391,7 @@ krr_status krr_kmatvec(const double *X, int64_t N, int d, krr_kernel kern, doubl
   KRR_TRY(out.init(Y, (size_t)N * m, s));
   if (prec == KRR_PREC_FP64) {
     PointsF64 P;
-    KRR_TRY(prepare_points_f64(Xd, N, d, kern, sigma, s, P, false));
+    KRR_TRY(prepare_points_f64(Xd, N, d, kern, sigma, s, P, fixsym_applies(N, d, m, false)));
     DevBuf<double> part;
     KRR_TRY(kmv_f64(P, lambda, Vd, N, m, out.dev, N, s, part));
   } else if (prec == KRR_PREC_FLOAT_FLOAT) {

@@ -6,9 +6,15 @@
 
 namespace krr {
 
-cudaError_t launch_kmvfix_gauss(int DP, int M, dim3 g, cudaStream_t s, const KmvFixArgs &a);
-cudaError_t launch_kmvfix_laplace(int DP, int M, dim3 g, cudaStream_t s, const KmvFixArgs &a);
-cudaError_t launch_kmvfix_matern(int DP, int M, dim3 g, cudaStream_t s, const KmvFixArgs &a);
+#define KRR_DECL(K)                                                                       \
+  cudaError_t launch_kmvfix_##K(int, int, dim3, cudaStream_t, const KmvFixArgs &);          \
+  cudaError_t launch_kmvfix_ff_##K(int, int, dim3, cudaStream_t, const KmvFixArgs &);       \
+  cudaError_t launch_kmvfixsym_##K(int, int, cudaStream_t, const KmvFixSymArgs &);          \
+  cudaError_t launch_kmvfixsym_ff_##K(int, int, cudaStream_t, const KmvFixSymArgs &);
+KRR_DECL(gauss)
+KRR_DECL(laplace)
+KRR_DECL(matern)
+#undef KRR_DECL
 cudaError_t launch_kfix_columns_gauss(int, const int2 *, int64_t, const FixScale *,
                                       const int64_t *, int, double *, int64_t, cudaStream_t);
 cudaError_t launch_kfix_columns_laplace(int, const int2 *, int64_t, const FixScale *,
@@ -55,7 +61,7 @@ fix_range_kernel(const double *__restrict__ X, int64_t total, int d, int skip,
 
 // Centre and fraction bits from the blocks' ranges; one warp.
 __global__ void fix_scale_kernel(const double *__restrict__ part, int blocks, int d, int kern,
-                                 double s_hi, double s_lo, FixScale *__restrict__ out) {
+                                 int ff, double s_hi, double s_lo, FixScale *__restrict__ out) {
   const int k = threadIdx.x;
   double lo = INFINITY, hi = -INFINITY;
   if (k < d)
@@ -73,35 +79,38 @@ __global__ void fix_scale_kernel(const double *__restrict__ part, int blocks, in
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) half = fmax(half, __shfl_xor_sync(0xffffffffu, half, o));
   if (k != 0) return;
-  const int e_max = kern == KGAUSS ? kFixMaxExpGauss
-                                   : kern == KMATERN ? kFixMaxExpMatern : kFixMaxExpLaplace;
+  const int lim[2][3] = {{kFixMaxExpGauss, kFixMaxExpLaplace, kFixMaxExpMatern},
+                         {kFixFFMaxExpGauss, kFixFFMaxExpLaplace, kFixFFMaxExpMatern}};
+  const int e_max = lim[ff][kern];
   // 2^e above the half-range with room for the coordinate rounding
   int e = kFixMinExp;
   while (e <= e_max && half * (1.0 + 0x1p-26) >= ldexp(1.0, e)) ++e;
   out->ok = e <= e_max ? 1 : 0;
+  e = min(e, e_max);
   out->s_hi = s_hi;
   out->s_lo = s_lo;
+  out->s1_max = 0;
+  out->r2_scale = 0.0;
   if (kern == KLAPLACE) {
+    out->limb = 0;
     out->q = 58 - e;
     out->r = 4 - e;
-    out->s1_max = 0;
-    out->r2_scale = 0.0;
-  } else {
-    out->q = 57 - e;
-    out->r = 30 - 2 * e;
-    out->r2_scale = ldexp(1.0, 30 - 2 * out->q);
-    // (with e = 1 every sum of squares stays below E = 512)
-    out->s1_max = e == 1 ? INT64_MAX
-                         : e <= kFixMaxExpGauss ? (int64_t)((1022ull << 54) >> (28 - out->r)) : 0;
+    return;
   }
+  out->limb = ff ? kFixFFLimb : kFixLimb;
+  out->q = (ff ? 53 : 57) - e;
+  out->r = (ff ? 26 : 30) - 2 * e;
+  const int left = (ff ? 24 : 28) - out->r;   // left shift of S1 to 54 fraction bits
+  out->r2_scale = ldexp(1.0, 30 - 2 * out->q);
+  // (without a shift every sum of squares stays below E = 512)
+  out->s1_max = left == 0 ? INT64_MAX : (int64_t)((1022ull << 54) >> left);
 }
 
 __global__ void fix_convert_kernel(const double *__restrict__ X, int64_t N, int d, int dp,
-                                   int laplace, const FixScale *__restrict__ scale,
-                                   int2 *__restrict__ u) {
+                                   const FixScale *__restrict__ scale, int2 *__restrict__ u) {
   if (!scale->ok) return;
   const double s_hi = scale->s_hi, s_lo = scale->s_lo;
-  const int q = scale->q;
+  const int q = scale->q, limb = scale->limb;
   const int64_t total = N * dp;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
        e += (int64_t)gridDim.x * blockDim.x) {
@@ -110,10 +119,10 @@ __global__ void fix_convert_kernel(const double *__restrict__ X, int64_t N, int 
     int2 v = make_int2(0, 0);
     if (k < d) {
       const int64_t c = fix_coord(X[i * d + k], scale->ctr[k], s_hi, s_lo, q);
-      if (laplace) {
+      if (limb == 0) {
         v = make_int2((int)(uint32_t)(uint64_t)c, (int)(c >> 32));
       } else {
-        fix_limbs(c, &v.x, &v.y);
+        fix_limbs(c, limb, &v.x, &v.y);
       }
     }
     u[e] = v;
@@ -121,7 +130,7 @@ __global__ void fix_convert_kernel(const double *__restrict__ X, int64_t N, int 
 }
 
 krr_status fix_scale(const double *A, int64_t na, const double *B, int64_t nb, int d, int kern,
-                     double sigma, cudaStream_t s, DevBuf<FixScale> &out) {
+                     double sigma, bool ff, cudaStream_t s, DevBuf<FixScale> &out) {
   KRR_REQUIRE(d >= 1 && d <= 32, "d must be in [1, 32]");
   // sqrt(log2 e / 2), log2 e and sqrt(5) as unevaluated sums, divided by sigma
   static const double num[3][2] = {{0x1.b2da4e9808a53p-1, -0x1.dede1a6b5e413p-56},
@@ -144,17 +153,17 @@ krr_status fix_scale(const double *A, int64_t na, const double *B, int64_t nb, i
     fix_range_kernel<<<gb, FIX_RANGE_THREADS, 0, s>>>(B, nb * d, d, ga, part.p);
     KRR_LAUNCH_CHECK();
   }
-  fix_scale_kernel<<<1, 32, 0, s>>>(part.p, ga + gb, d, kern, s_hi, s_lo, out.p);
+  fix_scale_kernel<<<1, 32, 0, s>>>(part.p, ga + gb, d, kern, ff ? 1 : 0, s_hi, s_lo, out.p);
   KRR_LAUNCH_CHECK();
   return KRR_OK;
 }
 
-krr_status fix_points(const double *Xd, int64_t N, int d, int kern, const FixScale *scale,
-                      cudaStream_t s, DevBuf<int2> &u) {
+krr_status fix_points(const double *Xd, int64_t N, int d, const FixScale *scale, cudaStream_t s,
+                      DevBuf<int2> &u) {
   const int dp = (d + 3) / 4 * 4;
   KRR_TRY(u.alloc((size_t)N * dp, s));
   const int64_t g = std::min<int64_t>((N * dp + 255) / 256, (int64_t)num_sms() * 16);
-  fix_convert_kernel<<<(unsigned)g, 256, 0, s>>>(Xd, N, d, dp, kern == KLAPLACE, scale, u.p);
+  fix_convert_kernel<<<(unsigned)g, 256, 0, s>>>(Xd, N, d, dp, scale, u.p);
   KRR_LAUNCH_CHECK();
   return KRR_OK;
 }
@@ -167,23 +176,37 @@ krr_status prepare_points_f64(const double *Xd, int64_t N, int d, int kern, doub
   P.kern = kern;
   P.sigma = sigma;
   P.known = -1;
-  KRR_TRY(fix_scale(Xd, N, nullptr, 0, d, kern, sigma, s, P.scale));
-  KRR_TRY(fix_points(Xd, N, d, kern, P.scale.p, s, P.u));
+  KRR_TRY(fix_scale(Xd, N, nullptr, 0, d, kern, sigma, false, s, P.scale));
+  KRR_TRY(fix_points(Xd, N, d, P.scale.p, s, P.u));
   if (wait) {
     int ok = 0;
     KRR_CUDA_TRY(cudaMemcpyAsync(&ok, &P.scale.p->ok, sizeof(int), cudaMemcpyDeviceToHost, s));
     KRR_CUDA_TRY(cudaStreamSynchronize(s));
-    P.known = ok ? 1 : 0;
+    P.known = ok;
   }
   return KRR_OK;
 }
 
-cudaError_t launch_kmvfix_any(int kern, int DP, int M, dim3 g, cudaStream_t s,
+cudaError_t launch_kmvfix_any(int kern, bool ff, int DP, int M, dim3 g, cudaStream_t s,
                               const KmvFixArgs &a) {
   switch (kern) {
-    case KGAUSS: return launch_kmvfix_gauss(DP, M, g, s, a);
-    case KLAPLACE: return launch_kmvfix_laplace(DP, M, g, s, a);
-    case KMATERN: return launch_kmvfix_matern(DP, M, g, s, a);
+    case KGAUSS: return ff ? launch_kmvfix_ff_gauss(DP, M, g, s, a) : launch_kmvfix_gauss(DP, M, g, s, a);
+    case KLAPLACE:
+      return ff ? launch_kmvfix_ff_laplace(DP, M, g, s, a) : launch_kmvfix_laplace(DP, M, g, s, a);
+    case KMATERN:
+      return ff ? launch_kmvfix_ff_matern(DP, M, g, s, a) : launch_kmvfix_matern(DP, M, g, s, a);
+  }
+  return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_kmvfixsym_any(int kern, bool ff, int DP, int M, cudaStream_t s,
+                                 const KmvFixSymArgs &a) {
+  switch (kern) {
+    case KGAUSS: return ff ? launch_kmvfixsym_ff_gauss(DP, M, s, a) : launch_kmvfixsym_gauss(DP, M, s, a);
+    case KLAPLACE:
+      return ff ? launch_kmvfixsym_ff_laplace(DP, M, s, a) : launch_kmvfixsym_laplace(DP, M, s, a);
+    case KMATERN:
+      return ff ? launch_kmvfixsym_ff_matern(DP, M, s, a) : launch_kmvfixsym_matern(DP, M, s, a);
   }
   return cudaErrorInvalidValue;
 }

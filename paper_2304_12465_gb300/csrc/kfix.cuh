@@ -41,15 +41,22 @@
 
 namespace krr {
 
-// Scaled half-range limit 2^e of each kernel function (index: kernel code).
+// Scaled half-range limit 2^e of each kernel function for the float64 products
+// and for the float-float ones (about 2^-46 an entry), whose limits are where
+// the coordinate rounding reaches that.
 constexpr int kFixMaxExpGauss = 4, kFixMaxExpMatern = 6, kFixMaxExpLaplace = 5;
+constexpr int kFixFFMaxExpGauss = 4, kFixFFMaxExpMatern = 5, kFixFFMaxExpLaplace = 9;
 constexpr int kFixMinExp = 1;    // a smaller range gains nothing: E is kept at 2^-54
 constexpr int kFixLimb = 29;
+// The float-float products keep |u| < 2^53 with low limbs of 25 bits and leave
+// out S3 but for its mean over low limbs: what is missing stays below d 2^(2 e
+// - 56) of E at the accepted ranges, and two multiply-adds a coordinate remain.
+constexpr int kFixFFLimb = 25;
 constexpr int kFixTab = 256;
 
 // What the conversion and the products of one point set (or two: rows and
 // columns) share.  Lives in device memory, so that no launch waits for the
-// host; ok == 0 leaves the work to the float64 kernels.
+// host; ok == 0 leaves the work to the float64 or float-float kernels.
 struct FixScale {
   double ctr[32];
   double s_hi, s_lo;     // scale factor as an unevaluated sum
@@ -57,20 +64,27 @@ struct FixScale {
   int64_t s1_max;        // Gaussian: see fix_exponent
   int q;                 // fraction bits of u
   int r;                 // right shift to 54 fraction bits (Gaussian, Laplace)
+  int limb;              // bits of the low limb (0: whole 64-bit integers)
   int ok;
 };
 
+// High word of a 64 x 64-bit product, low by at most 2: the product of the low
+// halves is left out, which saves a multiply and its carries (the multiplies
+// are what bounds the products).
 KRR_HD uint64_t fix_mulhi(uint64_t a, uint64_t b) {
-#ifdef __CUDA_ARCH__
-  return __umul64hi(a, b);
-#else
-  return (uint64_t)(((unsigned __int128)a * b) >> 64);
-#endif
+  const uint32_t al = (uint32_t)a, ah = (uint32_t)(a >> 32);
+  const uint32_t bl = (uint32_t)b, bh = (uint32_t)(b >> 32);
+  const uint64_t x = (uint64_t)al * bh, y = (uint64_t)ah * bl;
+  return (uint64_t)ah * bh + (x >> 32) + (y >> 32);
 }
 
+// High word of a 32 x 32-bit product, by the wide multiply (the high-word one
+// runs at half its rate).
 KRR_HD uint32_t fix_mulhi32(uint32_t a, uint32_t b) {
 #ifdef __CUDA_ARCH__
-  return __umulhi(a, b);
+  uint64_t p;
+  asm("mul.wide.u32 %0, %1, %2;" : "=l"(p) : "r"(a), "r"(b));
+  return (uint32_t)(p >> 32);
 #else
   return (uint32_t)(((uint64_t)a * b) >> 32);
 #endif
@@ -172,11 +186,20 @@ KRR_HD int64_t fix_coord(double x, double ctr, double s_hi, double s_lo,
   return (int64_t)pi + (int64_t)rint((ps - pi) + ls);
 }
 
-// u = 2^29 h + l with |l| <= 2^28
-KRR_HD void fix_limbs(int64_t u, int32_t *h, int32_t *l) {
-  const int64_t hh = (u + (1LL << (kFixLimb - 1))) >> kFixLimb;
+// u = 2^limb h + l with |l| <= 2^(limb - 1)
+KRR_HD void fix_limbs(int64_t u, int limb, int32_t *h, int32_t *l) {
+  const int64_t hh = (u + (1LL << (limb - 1))) >> limb;
   *h = (int32_t)hh;
-  *l = (int32_t)(u - hh * (1LL << kFixLimb));
+  *l = (int32_t)(u - hh * (1LL << limb));
+}
+
+// fix_exponent without S3: E from 2^50 S1 + 2^26 (S2 + bias), bias the mean of
+// S3 2^-26.  Near points can fall below zero by what is missing: 0 then.
+KRR_HD uint64_t fix_exponent_ff(int64_t S1, int64_t S2, int r, int64_t bias, int64_t s1_max) {
+  const int64_t a = (S2 + bias + (1LL << (r - 1))) >> r;
+  const uint64_t b = (uint64_t)S1 << (24 - r);
+  if (a < 0 && b < (uint64_t)-a) return 0;
+  return S1 >= s1_max ? ~0ull : b + (uint64_t)a;
 }
 
 // E at 54 fraction bits from the partial sums of squares, rounded to nearest;
@@ -189,13 +212,12 @@ KRR_HD uint64_t fix_exponent(int64_t S1, int64_t S2, uint64_t S3, int r,
   return S1 >= s1_max ? ~0ull : E;
 }
 
-// 2^-E for E at 54 fraction bits.  The top 8 fraction bits select 2^(-j/256)
+// 2^-f at 2^-63, f the fraction of E (54 fraction bits).  The top 8 fraction bits select 2^(-j/256)
 // from tab (units 2^-63); the rest, g < 2^-8, goes through 1 - 2^-g =
 // g (c1 - g (c2 - g (c3 - g (c4 - g c5)))), c_i = ln(2)^i / i! (Taylor; the
 // next term is below 2^-60): the inner coefficients in 32 bits, where their
 // powers of g leave at most 2^-55 of the result to them, the outer two in 64.
-KRR_HD double fix_exp2(uint64_t E, const uint64_t *__restrict__ tab) {
-  const int n = (int)(E >> 54);
+KRR_HD uint64_t fix_exp2_mantissa(uint64_t E, const uint64_t *__restrict__ tab) {
   const int j = (int)(E >> 46) & 255;
   const uint64_t g = E & ((1ull << 46) - 1);               // units 2^-54
   const uint32_t gs = (uint32_t)(g >> 14);                  // units 2^-40
@@ -209,17 +231,22 @@ KRR_HD double fix_exp2(uint64_t E, const uint64_t *__restrict__ tab) {
   const uint64_t t1 = 0x58B90BFBE8E7BCD6ull - (fix_mulhi(G, t2) >> 7);
   const uint64_t p = fix_mulhi(G, t1);                      // 1 - 2^-g at 2^-71
   const uint64_t T = tab[j];
-  const uint64_t m = T - (fix_mulhi(T, p) >> 7);            // 2^-f at 2^-63
-  // m 2^-63 2^-n as a float64: bit 53 of the rounded mantissa carries into
-  // the exponent field
+  return T - (fix_mulhi(T, p) >> 7);                        // 2^-f at 2^-63
+}
+
+// 2^-E as a float64 (0 below 2^-1021): bit 53 of the rounded mantissa carries
+// into the exponent field.
+KRR_HD double fix_exp2(uint64_t E, const uint64_t *__restrict__ tab) {
+  const int n = (int)(E >> 54);
+  const uint64_t m = fix_exp2_mantissa(E, tab);
   const uint64_t bits = ((uint64_t)(1021 - n) << 52) + ((m + 512) >> 10);
   return n > 1020 ? 0.0 : fix_bits_double(bits);
 }
 
 // E of the Laplace kernel at 54 fraction bits from the sum of |d| at
-// 2^-(54 + r), -1 <= r.
+// 2^-(54 + r).
 KRR_HD uint64_t fix_exponent_l1(uint64_t S, int r) {
-  if (r < 0) return (S >> 63) ? ~0ull : S << 1;
+  if (r < 0) return (S >> (64 + r)) ? ~0ull : S << -r;
   return r > 0 ? (S >> r) + ((S >> (r - 1)) & 1) : S;
 }
 
@@ -255,7 +282,12 @@ KRR_HD double fix_matern(int64_t S1, int64_t S2, uint64_t S3, double scale,
   const uint64_t mant = (b & ((1ull << 52) - 1)) | (1ull << 52);
   const uint64_t qf = sh >= 0 ? mant << sh : (mant + (1ull << (-sh - 1))) >> (-sh);
   const uint64_t L = 0xB8AA3B295C17F0BCull;                 // log2 e at 2^-63
-  const uint64_t E = (fix_mulhi(qf, L) << 1) | ((qf * L) >> 63);
+#ifdef __CUDA_ARCH__
+  const uint64_t hi = __umul64hi(qf, L);
+#else
+  const uint64_t hi = (uint64_t)(((unsigned __int128)qf * L) >> 64);
+#endif
+  const uint64_t E = (hi << 1) | ((qf * L) >> 63);
   return fma(q, fma(q, 1.0 / 3.0, 1.0), 1.0) * fix_exp2(E, tab);
 }
 

@@ -217,16 +217,26 @@ __global__ void prepare_ff_kernel(const double *__restrict__ X, int64_t N, int d
 }
 
 krr_status prepare_points_ff(const double *Xd, int64_t N, int d, int kern, double sigma,
-                             cudaStream_t s, PointsFF &P, const double *mean_dev) {
+                             cudaStream_t s, PointsFF &P, const PointsFF *like) {
   P.dp = (d + 3) / 4 * 4;
   P.d = d;
   P.N = N;
   P.kern = kern;
+  if (like) {
+    P.fixed = like->fixed;
+  } else {
+    int ok = 0;
+    KRR_TRY(fix_scale(Xd, N, nullptr, 0, d, kern, sigma, true, s, P.scale));
+    KRR_CUDA_TRY(cudaMemcpyAsync(&ok, &P.scale.p->ok, sizeof(int), cudaMemcpyDeviceToHost, s));
+    KRR_CUDA_TRY(cudaStreamSynchronize(s));
+    P.fixed = ok != 0;
+  }
+  if (P.fixed) return fix_points(Xd, N, d, (like ? *like : P).scale.p, s, P.u);
   KRR_TRY(P.xh.alloc((size_t)N * P.dp, s));
   KRR_TRY(P.xl.alloc((size_t)N * P.dp, s));
   KRR_TRY(P.ch.alloc((size_t)N, s));
   KRR_TRY(P.cl.alloc((size_t)N, s));
-  const double *mean = mean_dev;
+  const double *mean = like ? like->mean.p : nullptr;
   if (!mean) {
     KRR_TRY(points_mean(Xd, N, d, s, P.mean));
     mean = P.mean.p;
@@ -504,8 +514,84 @@ krr_status kmv_f32(const PointsF32 &P, float lambda, const float *V, int64_t ldv
   return KRR_OK;
 }
 
-cudaError_t launch_kmvfix_any(int kern, int DP, int M, dim3 grid, cudaStream_t s,
+cudaError_t launch_kmvfix_any(int kern, bool ff, int DP, int M, dim3 grid, cudaStream_t s,
                               const KmvFixArgs &a);
+cudaError_t launch_kmvfixsym_any(int kern, bool ff, int DP, int M, cudaStream_t s,
+                                 const KmvFixSymArgs &a);
+
+// Y = the row sums of a row's pairs (t, J) and the column sums of the pairs (I,
+// t) above it (+ lambda V): 32 rows a block, whose eight warps take every
+// eighth of the nt tiles each.  32 divides RT, so a block lies in one tile.
+__global__ void __launch_bounds__(32 * KRED_WARPS)
+fixsym_reduce_kernel(const double *__restrict__ rowpart, const double *__restrict__ colpart,
+                     int64_t N, int M, int RT, int nt, double lambda,
+                     const double *__restrict__ V, int64_t ldv, double *__restrict__ Y,
+                     int64_t ldy) {
+  __shared__ double red[KRED_WARPS][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, c = blockIdx.y;
+  const int64_t i0 = (int64_t)blockIdx.x * 32, i = i0 + lane;
+  const int t = (int)(i0 / RT), r = (int)(i0 % RT) + lane;
+  double acc = 0.0;
+#pragma unroll 2
+  for (int k = warp; k < nt; k += KRED_WARPS) {
+    const int64_t p = k < t ? ffsym_start(k, nt) + (t - k) : ffsym_start(t, nt) + (k - t);
+    acc += (k < t ? colpart : rowpart)[(p * M + c) * RT + r];
+  }
+  red[warp][lane] = acc;
+  __syncthreads();
+  if (warp != 0 || i >= N) return;
+#pragma unroll
+  for (int w = 1; w < KRED_WARPS; ++w) acc += red[w][lane];
+  Y[(int64_t)c * ldy + i] = acc + lambda * V[(int64_t)c * ldv + i];
+}
+
+// Tiles of the symmetric fixed-point product: as wide as leaves about 2500
+// pairs (four waves of the resident CTAs) and 32 KB of column sums.
+static void fixsym_shape(int64_t N, int M, int *RT, int *nt) {
+  int rt = KFIX_THREADS;
+  while (rt * 2 * M <= 4096 && rt < 1024 && (N + 2 * rt - 1) / (2 * rt) >= 70) rt *= 2;
+  *RT = rt;
+  *nt = (int)((N + rt - 1) / rt);
+}
+
+// Where the symmetric product is the faster one: from 20 tiles (at N = 2000
+// its 136 pairs leave the SMs half empty: 49 us against 47; at 3000 60 against
+// 80) and up to four right-hand sides, whose column sums it adds to every
+// entry (float64 at d <= 8 up to two: 150 us against 148 with four at N =
+// 4096, the DFMA of both sums bounding it).  Its partial sums stay within 4 GiB.
+bool fixsym_applies(int64_t N, int d, int m, bool ff) {
+  if (m > 4 || (!ff && m > 2 && d <= 8)) return false;
+  const int M = pad_m(m);
+  int RT, nt;
+  fixsym_shape(N, M, &RT, &nt);
+  return nt >= 20 && (double)nt * (nt + 1) * M * RT * 8.0 <= 4.0 * 1024 * 1024 * 1024;
+}
+
+// Symmetric square product of fixed-point points (known to fit).
+static krr_status fixsym_product(const int2 *u, int64_t N, int d, int kern, const FixScale *scale,
+                                 bool ff, double lambda, const double *V, int64_t ldv, int m,
+                                 double *Y, int64_t ldy, cudaStream_t s, DevBuf<double> &part) {
+  static const ExpFFConsts ec = make_exp_consts();
+  const int M = pad_m(m);
+  int RT, nt;
+  fixsym_shape(N, M, &RT, &nt);
+  const size_t half = (size_t)nt * (nt + 1) / 2 * M * RT;
+  if (part.n < 2 * half) KRR_TRY(part.alloc(2 * half, s));
+  const KmvFixSymArgs a{u, N, scale, V, ldv, m, RT, nt, ec, part.p, part.p + half};
+  KmvTimer tm(ff ? 2 : 1);
+  tm.begin(s);
+  const cudaError_t e = launch_kmvfixsym_any(kern, ff, (d + 3) / 4 * 4, M, s, a);
+  tm.end(s);
+  count_launch();
+  if (e != cudaSuccess) {
+    set_error("symmetric product launch failed: %s", cudaGetErrorString(e));
+    return KRR_ECUDA;
+  }
+  fixsym_reduce_kernel<<<dim3(ceil_div(N, 32), m), 32 * KRED_WARPS, 0, s>>>(
+      part.p, part.p + half, N, M, RT, nt, lambda, V, ldv, Y, ldy);
+  KRR_LAUNCH_CHECK();
+  return KRR_OK;
+}
 
 // Float64 product between row points (Xr, ur) and column points (Xc, uc) of
 // one scale; known as in PointsF64.
@@ -516,6 +602,7 @@ static krr_status f64_products(const double *Xr, const int2 *ur, int64_t Nr, con
                                DevBuf<double> &part) {
   const int dp = (d + 3) / 4 * 4;
   const double inv_scale = (kern == KGAUSS) ? 1.0 / (2.0 * sigma * sigma) : 1.0 / sigma;
+  static const ExpFFConsts ec = make_exp_consts();
   for (int c0 = 0; c0 < m; c0 += 16) {
     const int mg = (m - c0 < 16) ? (m - c0) : 16;
     const int M = pad_m(mg);
@@ -534,8 +621,8 @@ static krr_status f64_products(const double *Xr, const int2 *ur, int64_t Nr, con
     tm.begin(s);
     cudaError_t e = cudaSuccess;
     if (known != 0) {
-      const KmvFixArgs a{ur, Nr, uc, scale, Vg, ldv, N, mg, chunk, part.p};
-      e = launch_kmvfix_any(kern, dp, M, dim3((unsigned)fix_tiles, nsplit), s, a);
+      const KmvFixArgs a{ur, Nr, uc, scale, Vg, ldv, N, mg, chunk, ec, part.p};
+      e = launch_kmvfix_any(kern, false, dp, M, dim3((unsigned)fix_tiles, nsplit), s, a);
       count_launch();
     }
     if (known != 1 && e == cudaSuccess) {
@@ -559,6 +646,9 @@ static krr_status f64_products(const double *Xr, const int2 *ur, int64_t Nr, con
 krr_status kmv_f64(const PointsF64 &P, double lambda, const double *V, int64_t ldv, int m,
                    double *Y, int64_t ldy, cudaStream_t s, DevBuf<double> &part) {
   if (P.N == 0 || m == 0) return KRR_OK;
+  if (P.known == 1 && fixsym_applies(P.N, P.d, m, false))
+    return fixsym_product(P.u.p, P.N, P.d, P.kern, P.scale.p, false, lambda, V, ldv, m, Y, ldy, s,
+                          part);
   return f64_products(P.X, P.u.p, P.N, P.X, P.u.p, P.N, P.d, P.kern, P.sigma, P.scale.p, P.known,
                       lambda, true, V, ldv, m, Y, ldy, s, part);
 }
@@ -622,6 +712,38 @@ krr_status kff_cross(const PointsFF &R, const PointsFF &P, double lambda, const 
   const int64_t N = P.N, Nr = R.N;
   if (N == 0 || Nr == 0 || m == 0) return KRR_OK;
   static const ExpFFConsts ec = make_exp_consts();
+  if (R.fixed && P.fixed) {
+    const bool sq = (&R == &P);
+    const FixScale *scale = P.scale.p ? P.scale.p : R.scale.p;
+    if (sq && fixsym_applies(N, P.d, m, true))
+      return fixsym_product(P.u.p, N, P.d, P.kern, scale, true, lambda, V, ldv, m, Y, ldy, s, part);
+    for (int c0 = 0; c0 < m; c0 += 16) {
+      const int mg = std::min(16, m - c0), M = pad_m(mg);
+      const int rows = KFIX_THREADS * kmvfix_rows_per_thread(P.dp);
+      const int64_t tiles = (Nr + rows - 1) / rows;
+      int64_t chunk;
+      int nsplit;
+      split_shape(N, choose_splits(tiles, N, KFIX_TJ, 8, 2), KFIX_TJ, &chunk, &nsplit);
+      const size_t need = (size_t)nsplit * M * Nr;
+      if (part.n < need) KRR_TRY(part.alloc(need, s));
+      const double *Vg = V + (int64_t)c0 * ldv;
+      const KmvFixArgs a{R.u.p, Nr, P.u.p, scale, Vg, ldv, N, mg, chunk, ec, part.p};
+      KmvTimer tm(2);
+      tm.begin(s);
+      const cudaError_t e =
+          launch_kmvfix_any(P.kern, true, P.dp, M, dim3((unsigned)tiles, nsplit), s, a);
+      tm.end(s);
+      count_launch();
+      if (e != cudaSuccess) {
+        set_error("float-float product launch failed: %s", cudaGetErrorString(e));
+        return KRR_ECUDA;
+      }
+      KRR_TRY(kmv_reduce<double>(part.p, nsplit, M, Nr, mg, sq ? lambda : 0.0, sq ? Vg : nullptr,
+                                 ldv, Y + (int64_t)c0 * ldy, ldy, s));
+    }
+    return KRR_OK;
+  }
+  KRR_REQUIRE(!R.fixed && !P.fixed, "float-float product: point sets prepared differently");
   if (vsplit.n < (size_t)2 * N * m) KRR_TRY(vsplit.alloc((size_t)2 * N * m, s));
   float *vh = vsplit.p, *vl = vsplit.p + (size_t)N * m;
   {
@@ -723,9 +845,9 @@ krr_status kcross_f64(const double *Xr, int64_t Nr, const double *Xd, int64_t N,
   if (N == 0 || Nr == 0 || m == 0) return KRR_OK;
   DevBuf<FixScale> scale;
   DevBuf<int2> ur, uc;
-  KRR_TRY(fix_scale(Xr, Nr, Xd, N, d, kern, sigma, s, scale));
-  KRR_TRY(fix_points(Xr, Nr, d, kern, scale.p, s, ur));
-  KRR_TRY(fix_points(Xd, N, d, kern, scale.p, s, uc));
+  KRR_TRY(fix_scale(Xr, Nr, Xd, N, d, kern, sigma, false, s, scale));
+  KRR_TRY(fix_points(Xr, Nr, d, scale.p, s, ur));
+  KRR_TRY(fix_points(Xd, N, d, scale.p, s, uc));
   return f64_products(Xr, ur.p, Nr, Xd, uc.p, N, d, kern, sigma, scale.p, -1, 0.0, false, V, ldv,
                       m, Y, ldy, s, part);
 }

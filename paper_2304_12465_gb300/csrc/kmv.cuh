@@ -136,12 +136,17 @@ struct PointsF64 {
 krr_status prepare_points_f64(const double *Xd, int64_t N, int d, int kern, double sigma,
                               cudaStream_t s, PointsF64 &P, bool wait);
 
-// Common scale of one or two point sets (B may be NULL) and the integer
-// coordinates of one set under it.
+// Whether a square product of fixed-point points takes the symmetric kernel.
+// A single float64 product then waits for scale->ok: 10 us, against at least
+// 20 saved.
+bool fixsym_applies(int64_t N, int d, int m, bool ff);
+
+// Common scale of one or two point sets (B may be NULL) for float64 or
+// float-float products, and the integer coordinates of one set under it.
 krr_status fix_scale(const double *A, int64_t na, const double *B, int64_t nb, int d, int kern,
-                     double sigma, cudaStream_t s, DevBuf<FixScale> &out);
-krr_status fix_points(const double *Xd, int64_t N, int d, int kern, const FixScale *scale,
-                      cudaStream_t s, DevBuf<int2> &u);
+                     double sigma, bool ff, cudaStream_t s, DevBuf<FixScale> &out);
+krr_status fix_points(const double *Xd, int64_t N, int d, const FixScale *scale, cudaStream_t s,
+                      DevBuf<int2> &u);
 
 // G (nc columns, ld ldg) = A(:, cols) from fixed-point coordinates; writes
 // nothing when the range does not allow them.
@@ -157,7 +162,12 @@ krr_status kcross_f64(const double *Xr, int64_t Nr, const double *Xd, int64_t N,
 
 // Points split for the float-float product: centred, scaled x = xh + xl and
 // c = -|x|^2/2 = ch + cl (unused for Laplace).
+// When the range of the points allows it (fixed) the set holds its fixed-point
+// coordinates (kfix.cuh) instead, under a scale of its own or another set's.
 struct PointsFF {
+  bool fixed = false;
+  DevBuf<FixScale> scale;
+  DevBuf<int2> u;         // N x dp
   DevBuf<float> xh, xl;   // N x dp
   DevBuf<float> ch, cl;   // N
   DevBuf<double> mean;    // d
@@ -167,8 +177,10 @@ struct PointsFF {
   int kern = 0;
 };
 
+// like (optional): a prepared set whose scale and centre this one, a subset of
+// its points, shares.  Synchronises s otherwise.
 krr_status prepare_points_ff(const double *Xd, int64_t N, int d, int kern, double sigma,
-                             cudaStream_t s, PointsFF &P, const double *mean_dev = nullptr);
+                             cudaStream_t s, PointsFF &P, const PointsFF *like = nullptr);
 
 // Rectangular float-float product Y (R.N x m) = K(R, P) V; when &R == &P the
 // shift lambda V is added (square product).

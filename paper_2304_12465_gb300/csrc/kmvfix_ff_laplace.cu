@@ -1,0 +1,10 @@
+// Instantiates the fixed-point float-float products for one kernel function.
+#include "kmvfix_kernels.cuh"
+
+namespace krr {
+
+cudaError_t launch_kmvfix_ff_laplace(int DP, int M, dim3 grid, cudaStream_t s, const KmvFixArgs &a) {
+  return launch_kmvfix<FixAccFF, KLAPLACE>(DP, M, grid, s, a);
+}
+
+}  // namespace krr

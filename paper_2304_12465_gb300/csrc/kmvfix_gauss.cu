@@ -4,7 +4,7 @@
 namespace krr {
 
 cudaError_t launch_kmvfix_gauss(int DP, int M, dim3 grid, cudaStream_t s, const KmvFixArgs &a) {
-  return launch_kmvfix<KGAUSS>(DP, M, grid, s, a);
+  return launch_kmvfix<FixAccD, KGAUSS>(DP, M, grid, s, a);
 }
 
 cudaError_t launch_kfix_columns_gauss(int DP, const int2 *ua, int64_t N, const FixScale *scale,

@@ -4,7 +4,7 @@
 namespace krr {
 
 cudaError_t launch_kmvfix_laplace(int DP, int M, dim3 grid, cudaStream_t s, const KmvFixArgs &a) {
-  return launch_kmvfix<KLAPLACE>(DP, M, grid, s, a);
+  return launch_kmvfix<FixAccD, KLAPLACE>(DP, M, grid, s, a);
 }
 
 cudaError_t launch_kfix_columns_laplace(int DP, const int2 *ua, int64_t N, const FixScale *scale,

@@ -4,7 +4,7 @@
 namespace krr {
 
 cudaError_t launch_kmvfix_matern(int DP, int M, dim3 grid, cudaStream_t s, const KmvFixArgs &a) {
-  return launch_kmvfix<KMATERN>(DP, M, grid, s, a);
+  return launch_kmvfix<FixAccD, KMATERN>(DP, M, grid, s, a);
 }
 
 cudaError_t launch_kfix_columns_matern(int DP, const int2 *ua, int64_t N, const FixScale *scale,

@@ -572,7 +572,7 @@ krr_status krill_points_ff(const krill_precond *P, cudaStream_t s, KrillFF &Q) {
   gather_points_kernel<<<ceil_div((int64_t)P->k * P->d, 256), 256, 0, s>>>(P->X, P->d, P->S,
                                                                           P->k, xc.p);
   KRR_LAUNCH_CHECK();
-  KRR_TRY(prepare_points_ff(xc.p, P->k, P->d, P->kern, P->sigma, s, Q.centers, Q.all.mean.p));
+  KRR_TRY(prepare_points_ff(xc.p, P->k, P->d, P->kern, P->sigma, s, Q.centers, &Q.all));
   return KRR_OK;
 }
 

@@ -677,11 +677,13 @@ double serve_footprint(int64_t N, int d, int m, int k) {
   b += 4.0 * n * m * 8 + 5.0 * n * m * 4;
   // product partials, preconditioner partials, reductions
   b += splits * M * n * 4 + nbt * k * m * 8 + 3.0 * k * m * 8 + 2.0 * nbv * m * 8;
-  // float-float residual product: split partials and split right-hand sides
+  // float-float residual product: split partials (or the symmetric product's
+  // sums of every pair of tiles) and split right-hand sides
   const double rows_ff = 128.0 * (dpff <= 16 ? 2 : 1);
   const double tiles_ff = std::ceil(n / rows_ff);
   const double ffsplits = std::min(std::ceil(3648.0 / tiles_ff) + 1.0, std::ceil(n / 32.0));
-  b += ffsplits * M * n * 8 + 2.0 * n * m * 4;
+  const double sym_tiles = std::max(std::min(n / 128.0, 140.0), n / 1024.0) + 2.0;
+  b += std::max(ffsplits, sym_tiles) * M * n * 8 + 2.0 * n * m * 4;
   return b * 1.05 + 16.0 * 1024 * 1024;
 }
 
@@ -952,7 +954,7 @@ static krr_status build_slot(krr_server *S, Slot *sl, cudaStream_t s) {
   const size_t ot = take((size_t)rank * m * 8), ou = take((size_t)rank * m * 8),
                ov = take((size_t)rank * m * 8);
   const size_t od0 = take((size_t)D.nbv * m * 8), od1 = take((size_t)D.nbv * m * 8);
-  KRR_CUDA_TRY(cudaMallocAsync(&sl->arena, off, s));
+  KRR_CUDA_TRY(pool_malloc((void **)&sl->arena, off, s));
   char *base = (char *)sl->arena;
   sl->Y64 = (double *)(base + oY);
   sl->alpha64 = (double *)(base + oA);
@@ -1007,6 +1009,8 @@ static krr_status build_slot(krr_server *S, Slot *sl, cudaStream_t s) {
   rebind(sl->Pff.ch, S->s_free);
   rebind(sl->Pff.cl, S->s_free);
   rebind(sl->Pff.mean, S->s_free);
+  rebind(sl->Pff.scale, S->s_free);
+  rebind(sl->Pff.u, S->s_free);
   return KRR_OK;
 }
 
@@ -1117,6 +1121,8 @@ static void release_device(krr_server *S, Slot *sl) {
   sl->Pff.ch.release();
   sl->Pff.cl.release();
   sl->Pff.mean.release();
+  sl->Pff.scale.release();
+  sl->Pff.u.release();
   sl->ffpart.release();
   sl->ffvsplit.release();
 }

@@ -34,8 +34,8 @@ extern "C" double entry(int kern, int d, int e, const double *x, const double *y
     const int64_t D = a - b;
     S += (uint64_t)(D < 0 ? -D : D);
     int32_t ah, al, bh, bl;
-    fix_limbs(a, &ah, &al);
-    fix_limbs(b, &bh, &bl);
+    fix_limbs(a, kFixLimb, &ah, &al);
+    fix_limbs(b, kFixLimb, &bh, &bl);
     const int64_t dh = (int64_t)ah - bh, dl = (int64_t)al - bl;
     if (dh != (int32_t)dh || dl != (int32_t)dl) return -1.0;
     S1 += dh * dh; S2 += dh * dl; S3 += (uint64_t)(dl * dl);

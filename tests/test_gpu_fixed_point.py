@@ -80,3 +80,48 @@ def test_reduction_of_many_splits(K, N):
     ref = O.kmatvec(X, 0, 1.0, 0.3, V)
     scale = O.kmatvec(X, 0, 1.0, 0.3, np.abs(V))
     assert np.all(np.abs(got - ref) <= (N + 64) * 2.0 ** -53 * scale)
+
+
+# --------------------------------------------- symmetric and float-float products
+# Sizes around the symmetric kernel's limits: 20 tiles of 128 points (2432 and
+# 2433), ragged last tiles, the step to wider tiles, one to four right-hand
+# sides (five take the rectangular kernel), one point past 16 coordinates.
+# Float64: |error| <= (N + 64) 2^-53 sum |a v| as above with the entries' own
+# bound; float-float: 2^-44 sum |a v| for the entries (d 2^(2 e - 56) and 2^-46
+# of their value) plus N 2^-47 sum |a v| for the sums' low parts.
+SYM = [(2432, 8, 1), (2433, 8, 2), (2500, 3, 4), (3001, 17, 3), (2700, 32, 1), (17950, 4, 1),
+       (3000, 8, 5)]
+
+
+@pytest.mark.parametrize("prec", ["fp64", "ff"])
+@pytest.mark.parametrize("kern", [O.GAUSSIAN, O.LAPLACE_L1, O.MATERN52])
+@pytest.mark.parametrize("N,d,m", SYM)
+def test_symmetric_product(K, prec, kern, N, d, m):
+    if N > 4000 and kern != O.GAUSSIAN:
+        pytest.skip("one kernel at the larger size")
+    rng = np.random.default_rng(N + d + m)
+    X, V = rng.standard_normal((N, d)), rng.standard_normal((m, N))
+    X[5] = X[4]
+    X[N - 1] = X[0] + 1e-8
+    sigma = 1.0 + d / 8.0
+    rows = np.unique(np.concatenate([[0, 4, 5, N - 1], rng.integers(0, N, 400)]))
+    got = K.krr_kmatvec(to_dev(X), kern, sigma, 0.25, to_dev(V), prec=prec).cpu().numpy()[:, rows]
+    ref = O.kmatvec(X, kern, sigma, 0.25, V, rows)
+    scale = O.kmatvec(X, kern, sigma, 0.25, np.abs(V), rows)
+    eps = (N + 64) * 2.0 ** -53 if prec == "fp64" else 2.0 ** -44 + N * 2.0 ** -47
+    assert np.all(np.abs(got - ref) <= eps * scale)
+
+
+@pytest.mark.parametrize("kern", [O.GAUSSIAN, O.LAPLACE_L1, O.MATERN52])
+def test_float_float_beyond_the_range(K, kern):
+    """Points too spread for the fixed-point float-float product take the
+    float-float kernels, to the same bound."""
+    rng = np.random.default_rng(1)
+    N = 2600
+    X, V = 300.0 * rng.standard_normal((N, 5)), rng.standard_normal((2, N))
+    X[:50] = X[50:100] + rng.standard_normal((50, 5))
+    got = K.krr_kmatvec(to_dev(X), kern, 1.0, 0.25, to_dev(V), prec="ff").cpu().numpy()
+    ref = O.kmatvec(X, kern, 1.0, 0.25, V)
+    scale = O.kmatvec(X, kern, 1.0, 0.25, np.abs(V))
+    # beyond the float-float coordinates' own 2^-48 |x| = 2^-39: dE <= 2 |d| 2^-39 sqrt(d)
+    assert np.all(np.abs(got - ref) <= 2.0 ** -34 * scale)
