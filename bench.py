@@ -774,7 +774,7 @@ def measure_config(K, workload, steps, warmup, dist=None, rank=0, world=1):
         t_flop = pairs * extra["roofline_model"]["flop_per_pair"] / peak_flop
         t_mufu = pairs * extra["roofline_model"]["mufu_per_pair"] / peak_mufu
         res["roofline"] = {
-            "kernel": "kmvb_kernel (batched 8-setting product)", "bound": "alu",
+            "kernel": "kmvb_kernel (batched product, 8 settings in two launches)", "bound": "alu",
             "achieved": pairs * extra["roofline_model"]["flop_per_pair"] / sec / 1e12,
             "peak": peak_flop / 1e12, "unit": "TFLOP/s",
             "frac": max(t_flop, t_mufu) / sec, "traffic": None,
