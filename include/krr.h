@@ -609,7 +609,8 @@ KRR_API krr_status krr_set_product_path(int path);
 /* column's largest |v| per term (the FMA variants: 2^-24 of each term), so   */
 /* they serve square products (krr_kmatvec, the solvers) only; prediction and */
 /* the restricted products keep 1..7.  Variants 2, 4..7, 10 and 11 serve m <= */
-/* 4 per launch.  A forced variant that does not serve a launch leaves that   */
+/* 4 per launch; 8 and 9 also take 13 to 16 right-hand sides in one launch.   */
+/* A forced variant that does not serve a launch leaves that                  */
 /* launch to the autotuner or the default.  Results differ between variants   */
 /* at the rounding level only.  Process-wide.  KRR_EINVAL outside             */
 /* 0..KRR_PRODUCT_VARIANTS.                                                   */

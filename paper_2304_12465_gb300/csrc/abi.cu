@@ -352,8 +352,7 @@ krr_status krr_autotune_variant(krr_kernel kern, int d, int m, int64_t N, int *v
   KRR_REQUIRE(variant, "variant is NULL");
   KRR_REQUIRE(valid_kernel(kern), "unknown kernel %d", (int)kern);
   KRR_REQUIRE(d >= 1 && d <= 32 && m >= 1 && m <= 16 && N >= 1, "bad shape");
-  const int mg = m > 8 ? 8 : m;
-  const int M = mg <= 2 ? 2 : mg <= 4 ? 4 : 8;
+  const int M = m <= 2 ? 2 : m <= 4 ? 4 : m <= 12 ? 8 : 16;
   int best = 0;
   float t[KRR_PRODUCT_VARIANTS] = {};
   if (!tc5_tuned((int)kern, d, M, N, &best, t)) best = 0;

@@ -199,7 +199,7 @@ __device__ __forceinline__ void mma_commit(uint32_t bar) {
 // ------------------------------------------------------------ TMEM loads
 // 32x32b.x16: thread t of the warp receives lane (lane(taddr) + t), columns
 // col(taddr) .. col(taddr) + 15.
-__device__ __forceinline__ void tmem_ld_32x32b_x16(uint32_t taddr, uint32_t (&r)[16]) {
+__device__ __forceinline__ void tmem_ld_32x32b_x16(uint32_t taddr, uint32_t *r) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,"
       "%14,%15}, [%16];"

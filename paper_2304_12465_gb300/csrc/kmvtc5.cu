@@ -1,6 +1,6 @@
 // Host side of the tcgen05 product (kmvtc5_kernels.cuh): the split operands
 // and their TMA tensor maps, the launch over right-hand-side groups of at
-// most 8, and the reduction of the per-CTA segment partial sums.
+// most 16, and the reduction of the per-CTA segment partial sums.
 #include <cuda_fp16.h>
 #include <cudaTypedefs.h>
 
@@ -329,38 +329,36 @@ t5_reduce_many_kernel(const float *__restrict__ part, int64_t Nr, int m, int M, 
 }
 
 // Right-hand sides of the column points as the kernel's shared tiles hold
-// them: for column tile t (of TN points), pair cp and column jl, {v_2cp,
-// v_2cp, v_2cp+1, v_2cp+1} of point t TN + jl times vscale (zero beyond Nc
-// or m); vscale = 2^-14 for the Gaussian, whose kernel values come scaled by
-// 2^14.
+// them: for column tile t (of TN points), pair cp of right-hand sides and pair
+// jp of columns, {v_2cp(j), v_2cp(j + 1), v_2cp+1(j), v_2cp+1(j + 1)}, j = t TN
+// + 2 jp, times vscale (zero beyond Nc or m); vscale = 2^-14 for the Gaussian,
+// whose kernel values come scaled by 2^14.
 template <typename TV5>
-__global__ void t5_vdup_kernel(const TV5 *__restrict__ V, int64_t ldv, int64_t Nc, int m,
-                               int MP, int C, int TN, float vscale, float4 *__restrict__ vdup) {
-  const int64_t total = (int64_t)C * MP * TN;
+__global__ void t5_vpair_kernel(const TV5 *__restrict__ V, int64_t ldv, int64_t Nc, int m,
+                                int MP, int C, int TN, float vscale, float4 *__restrict__ vpair) {
+  const int TN2 = TN / 2;
+  const int64_t total = (int64_t)C * MP * TN2;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
        e += (int64_t)gridDim.x * blockDim.x) {
-    const int jl = (int)(e % TN);
-    const int cp = (int)((e / TN) % MP);
-    const int64_t t = e / ((int64_t)TN * MP);
-    const int64_t j = t * TN + jl;
-    float va = 0.0f, vb = 0.0f;
-    if (j < Nc) {
-      if (2 * cp < m) va = (float)V[(int64_t)(2 * cp) * ldv + j] * vscale;
-      if (2 * cp + 1 < m) vb = (float)V[(int64_t)(2 * cp + 1) * ldv + j] * vscale;
-    }
-    vdup[e] = make_float4(va, va, vb, vb);
+    const int c = 2 * (int)((e / TN2) % MP);
+    const int64_t j = e / ((int64_t)TN2 * MP) * TN + 2 * (e % TN2);
+    auto val = [&](int cc, int64_t jj) {
+      return cc < m && jj < Nc ? (float)V[(int64_t)cc * ldv + jj] * vscale : 0.0f;
+    };
+    vpair[e] = make_float4(val(c, j), val(c, j + 1), val(c + 1, j), val(c + 1, j + 1));
   }
 }
 
-// Largest |v| of each right-hand side (m <= 8) over this block's grid-stride
+// Largest |v| of each right-hand side (m <= 16) over this block's grid-stride
 // share of the Nc points: bmax[block][c].
 constexpr int T5_VMAX_BLOCKS = 256;
+constexpr int T5_MAX_M = 16;   // right-hand sides of one launch
 template <typename TV5>
 __global__ void t5_vmax_kernel(const TV5 *__restrict__ V, int64_t ldv, int64_t Nc, int m,
                                float *__restrict__ bmax) {
-  __shared__ float red[8][8];
+  __shared__ float red[8][T5_MAX_M];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int c = 0; c < 8; ++c) {
+  for (int c = 0; c < T5_MAX_M; ++c) {
     float mx = 0.0f;
     if (c < m)
       for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < Nc;
@@ -370,10 +368,10 @@ __global__ void t5_vmax_kernel(const TV5 *__restrict__ V, int64_t ldv, int64_t N
     if (lane == 0) red[warp][c] = mx;
   }
   __syncthreads();
-  if (threadIdx.x < 8) {
+  if (threadIdx.x < T5_MAX_M) {
     float mx = 0.0f;
     for (int w = 0; w < (int)(blockDim.x >> 5); ++w) mx = fmaxf(mx, red[w][threadIdx.x]);
-    bmax[blockIdx.x * 8 + threadIdx.x] = mx;
+    bmax[blockIdx.x * T5_MAX_M + threadIdx.x] = mx;
   }
 }
 
@@ -385,7 +383,8 @@ __device__ __forceinline__ uint32_t t5_pack_halves(__half lo, __half hi) {
 // scaled by s_c = 2^vexp[c], the power of two that brings its largest |v|
 // into [2^13, 2^14), and split into fp16 halves v s_c = v_hi + v_lo.  B slot n
 // of fragment f: v_hi of column n (n < M) and v_lo of column n - M (M <= n <
-// 2M) for M <= 4; v_hi (f = 0) or v_lo (f = 1) of column n for M = 8.  For
+// 2M) for M <= 4; for M = 8 and 16, v_hi (f < M / 8) or v_lo of column n + 8
+// (f mod M / 8).  For
 // column tile t, batch bt of 16 columns, fragment f and lane 4 g + q, frag
 // holds {B(2q, g), B(2q + 1, g)}, {B(2q + 8, g), B(2q + 9, g)} over the
 // batch's columns (zero beyond Nc, m or 2M).  Every block derives the scales
@@ -394,10 +393,10 @@ template <typename TV5>
 __global__ void t5_vfrag_kernel(const TV5 *__restrict__ V, int64_t ldv, int64_t Nc, int m,
                                 int M, int C, int TN, const float *__restrict__ bmax, int gmax,
                                 uint2 *__restrict__ frag, int *__restrict__ vexp) {
-  __shared__ float sc[8];
-  if (threadIdx.x < 8) {
+  __shared__ float sc[T5_MAX_M];
+  if (threadIdx.x < T5_MAX_M) {
     float mx = 0.0f;
-    for (int q = 0; q < gmax; ++q) mx = fmaxf(mx, bmax[q * 8 + threadIdx.x]);
+    for (int q = 0; q < gmax; ++q) mx = fmaxf(mx, bmax[q * T5_MAX_M + threadIdx.x]);
     int e = 0;
     if (mx > 0.0f && mx <= 3.4028234663852886e38f) {
       int E = 0;
@@ -408,7 +407,7 @@ __global__ void t5_vfrag_kernel(const TV5 *__restrict__ V, int64_t ldv, int64_t 
     if (blockIdx.x == 0) vexp[threadIdx.x] = e;
   }
   __syncthreads();
-  const int NB = (M == 8) ? 2 : 1;
+  const int NB = t5_nfrag(M);
   const int nbat = TN / 16;
   const int64_t total = (int64_t)C * nbat * NB * 32;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
@@ -418,8 +417,8 @@ __global__ void t5_vfrag_kernel(const TV5 *__restrict__ V, int64_t ldv, int64_t 
     const int bt = (int)((e / (32 * NB)) % nbat);
     const int64_t t = e / ((int64_t)32 * NB * nbat);
     const int g = lane >> 2, q = lane & 3;
-    int c = g;
-    bool lo = (f == 1), live = true;
+    int c = g + 8 * (NB > 1 ? f % (NB / 2) : 0);
+    bool lo = 2 * f >= NB, live = true;
     if (NB == 1) {
       lo = g >= M;
       c = lo ? g - M : g;
@@ -445,10 +444,16 @@ __global__ void t5_vfrag_kernel(const TV5 *__restrict__ V, int64_t ldv, int64_t 
 // Results of different variants differ only in the summation order of the
 // column groups (rounding level).
 static_assert(T5_NVARIANTS == KRR_PRODUCT_VARIANTS, "variant count of the ABI");
-// Untuned default: the FMA sums (3) up to 4 right-hand sides per launch, the
-// tensor-core sums (9) for 5..8, where they measured 2.96 ms against 4.35 ms
-// per product at N = 1e5, d = 16.
-static int t5_default_variant(int M, bool square) { return (M == 8 && square) ? 9 : 3; }
+// Untuned default.  Square products of 5 and more right-hand sides take the
+// tensor-core sums (9): 2.93 ms against 3.59 ms at N = 1e5, d = 16, m = 8.
+// Below, the FMA sums, with 8 warps (3) where they are bound by the FMA pipe
+// (Gaussian, 3 or 4 right-hand sides, d <= 16: 2.15 ms against 2.25 ms with
+// 16) and with 16 (2) otherwise: 1.61 against 1.98 ms for m = 2, 2.43 against
+// 2.60 for d = 30, 4.35 against 5.15 for Matern.
+static int t5_default_variant(const PointsF32 &P, int M, bool square) {
+  if (M >= 8) return square ? 9 : 3;
+  return P.kern == KGAUSS && M == 4 && P.nh5 == 1 ? 3 : 2;
+}
 static std::atomic<int> g_t5_variant{0};
 static std::mutex g_t5_mtx;
 struct T5Tune {
@@ -500,14 +505,14 @@ static T5Geometry t5_geometry(int64_t Nr, int64_t Nc, int TN) {
 // right-hand-side quadruples or B fragments (16-byte aligned), the block
 // maxima of V and the scale exponents (TV variants).
 static size_t t5_npart(const T5Geometry &g, int M) { return (size_t)g.G * g.J * 4 * M * T5_RB; }
-static size_t t5_nvdup(const T5Geometry &g, int M) {
-  return (size_t)g.C * g.TN * 4 * (M / 2);   // quadruples, or (fewer) B fragments
+static size_t t5_nrhs(const T5Geometry &g, int M) {
+  return (size_t)g.C * g.TN * t5_vstage(M) / (4 * 128);   // floats of a column tile's stage
 }
 static size_t t5_scratch_floats(const T5Geometry &g, int M) {
-  return t5_npart(g, M) + t5_nvdup(g, M) + T5_VMAX_BLOCKS * 8 + 8;
+  return t5_npart(g, M) + t5_nrhs(g, M) + (T5_VMAX_BLOCKS + 1) * T5_MAX_M;
 }
 static int *t5_vexp(float *part, const T5Geometry &g, int M) {
-  return reinterpret_cast<int *>(part + t5_npart(g, M) + t5_nvdup(g, M) + T5_VMAX_BLOCKS * 8);
+  return reinterpret_cast<int *>(part + t5_npart(g, M) + t5_nrhs(g, M) + T5_VMAX_BLOCKS * T5_MAX_M);
 }
 
 // Stages V for this geometry and launches the product; returns the launch's
@@ -519,22 +524,22 @@ static cudaError_t t5_launch(const PointsF32 &R, const PointsF32 &P, int M, int 
   float *vbuf = part + t5_npart(g, M);
   cudaError_t e = cudaSuccess;
   if (t5_variant_tv(variant)) {
-    float *bmax = vbuf + t5_nvdup(g, M);
+    float *bmax = vbuf + t5_nrhs(g, M);
     const int gmax = (int)std::min<int64_t>((P.N + 255) / 256, T5_VMAX_BLOCKS);
     t5_vmax_kernel<<<gmax, 256, 0, s>>>(Vg, ldv, P.N, mg, bmax);
     count_launch();
-    const int NB = (M == 8) ? 2 : 1;
+    const int NB = t5_nfrag(M);
     const int64_t total = (int64_t)g.C * (g.TN / 16) * NB * 32;
     const int blocks = (int)std::min<int64_t>((total + 255) / 256, 4096);
     t5_vfrag_kernel<<<blocks, 256, 0, s>>>(Vg, ldv, P.N, mg, M, g.C, g.TN, bmax, gmax,
                                            reinterpret_cast<uint2 *>(vbuf), t5_vexp(part, g, M));
     count_launch();
   } else {
-    const int64_t total = (int64_t)g.C * (M / 2) * g.TN;
+    const int64_t total = (int64_t)g.C * (M / 2) * (g.TN / 2);
     const int blocks = (int)std::min<int64_t>((total + 255) / 256, 4096);
-    t5_vdup_kernel<<<blocks, 256, 0, s>>>(Vg, ldv, P.N, mg, M / 2, g.C, g.TN,
-                                          P.kern == KGAUSS ? 0x1p-14f : 1.0f,
-                                          reinterpret_cast<float4 *>(vbuf));
+    t5_vpair_kernel<<<blocks, 256, 0, s>>>(Vg, ldv, P.N, mg, M / 2, g.C, g.TN,
+                                           P.kern == KGAUSS ? 0x1p-14f : 1.0f,
+                                           reinterpret_cast<float4 *>(vbuf));
     count_launch();
   }
   e = cudaGetLastError();
@@ -545,7 +550,7 @@ static cudaError_t t5_launch(const PointsF32 &R, const PointsF32 &P, int M, int 
   // 512 TMEM columns)
   const int ew = t5_variant_ew(variant);
   const size_t smem = std::max<size_t>(
-      t5_smem_bytes(kb, M, t5_tot_floats(ew, M, variant == 5, t5_variant_tv(variant))),
+      t5_smem_bytes(kb, M, t5_tot_floats(ew, M, t5_variant_tv(variant))),
       116 * 1024);
   const bool tv = t5_variant_tv(variant), gauss = P.kern == KGAUSS;
   KmvTimer tm;
@@ -569,26 +574,26 @@ static int choose_variant(const PointsF32 &R, const PointsF32 &P, bool square, i
                           bool quiet) {
   const int forced = g_t5_variant.load();
   if (forced > 0 && t5_variant_valid(forced, M, square)) return forced;
-  if (quiet) return t5_default_variant(M, square);
+  if (quiet) return t5_default_variant(P, M, square);
   const auto key = std::make_tuple(P.kern, P.nh5, P.csep5, M, R.N, P.N, square);
   {
     std::lock_guard<std::mutex> lk(g_t5_mtx);
     auto it = g_t5_tuned.find(key);
     if (it != g_t5_tuned.end()) return it->second.best;
   }
-  if (!autotune_on()) return t5_default_variant(M, square);
+  if (!autotune_on()) return t5_default_variant(P, M, square);
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone)
-    return t5_default_variant(M, square);   // timing would synchronise a capturing stream
+    return t5_default_variant(P, M, square);   // timing would synchronise a capturing stream
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) {
     if (e0) cudaEventDestroy(e0);
     cudaGetLastError();
-    return t5_default_variant(M, square);
+    return t5_default_variant(P, M, square);
   }
   T5Tune tune;
   float best_ms = 1e30f;
-  tune.best = t5_default_variant(M, square);
+  tune.best = t5_default_variant(P, M, square);
   for (int v = 1; v <= T5_NVARIANTS; ++v) {
     if (!t5_variant_valid(v, M, square)) continue;
     const T5Geometry g = t5_geometry(R.N, P.N, t5_variant_tn(v));
@@ -630,9 +635,17 @@ static krr_status tc5_products(const PointsF32 &R, const PointsF32 &P, double la
               "tcgen05 product: operands missing or of different layouts");
   int *fault = fault_ptr();
   KRR_REQUIRE(fault != nullptr, "tcgen05 product: no fault flag on this device");
-  for (int c0 = 0; c0 < m; c0 += 8) {
-    const int mg = std::min(8, m - c0);
-    const int M = mg <= 2 ? 2 : mg <= 4 ? 4 : 8;
+  // One launch of 16 where two of 8 would both take their sums on the tensor
+  // cores: the kernel values, their split and the distances are formed once.
+  // N = 50021, d = 32, Matern, m = 16: 2.93 -> 1.79 ms (N = 1e5, d = 16,
+  // Gaussian: 5.9 -> 4.2 ms).  From 9 to 12 a launch of 8 and
+  // one of 4 keep the float32 sums of the latter.
+  const int forced = g_t5_variant.load();
+  const bool wide = square && (forced == 0 || forced == 8 || forced == 9);
+  int mg = 0;
+  for (int c0 = 0; c0 < m; c0 += mg) {
+    mg = std::min(wide && m - c0 > 12 ? 16 : 8, m - c0);
+    const int M = mg <= 2 ? 2 : mg <= 4 ? 4 : mg <= 8 ? 8 : 16;
     const TV5 *Vg = V + (int64_t)c0 * ldv;
     const int variant = choose_variant(R, P, square, M, Vg, ldv, mg, part, fault, s, quiet);
     const T5Geometry g = t5_geometry(Nr, Nc, t5_variant_tn(variant));

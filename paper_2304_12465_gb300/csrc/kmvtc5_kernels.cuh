@@ -36,20 +36,31 @@
 // Warp roles (320 threads):
 //   warp 8 (producer): one lane issues the TMA loads of the row operand (both
 //     row tiles, once per segment) and of each column tile's operand into a
-//     ring of t5_stages(kb, M) stages (up to 8), plus a bulk copy of the tile's right-hand sides,
-//     prepared once per product as {v_c, v_c, v_c+1, v_c+1} quadruples
-//     (t5_vdup_kernel), all completing on the stage's barrier.
+//     ring of t5_stages(kb, M) stages (up to 8), plus a bulk copy of the tile's
+//     right-hand sides, prepared once per product (t5_vpair_kernel,
+//     t5_vfrag_kernel), all completing on the stage's barrier.
 //   warp 9 (MMA): allocates all 512 TMEM columns; one lane issues, per column
 //     tile and row tile, the MMAs of D into one of two accumulator buffers
 //     (2 buffers x 2 row tiles x 128 columns), and commits them to the
 //     barriers that release the column stage and hand the buffer to the
 //     epilogue.
-//   warps 0-7 (epilogue): warp w reads TMEM lanes 32 (w % 4) .. + 31 of both
-//     row tiles for columns 64 (w / 4) .. + 63 of the tile with tcgen05.ld
-//     16x256b (a lane holds rows g, g + 8, g + 16, g + 24 of each row tile and
-//     two columns of every 8), forms kappa with ex2 on the MUFU, and
-//     accumulates V with packed FFMA2 on row pairs; each quadruple of V read
-//     from shared memory serves eight rows.
+//   warps 0-7 (epilogue; 12 or 16 in other variants): warps 0-3 take the even
+//     tiles and warps 4-7 the odd ones.  Warp w reads TMEM lanes 32 (w % 4) ..
+//     + 31 with tcgen05.ld 32x32b, 16 columns of both row tiles at a time: a
+//     lane holds one row of each row tile, forms kappa with ex2 on the MUFU and
+//     accumulates V with FFMA2 over pairs of columns of one row, so that V is
+//     read undoubled, as warp-wide broadcasts, and sums need no shuffles.
+//
+// What bounds it (N = 1e5, d = 16, m = 4, 1e10 entries, 2.15 ms): FFMA2, ex2
+// and the issue slots each need 1.0-1.1 ms; the hand-over of a tile costs an
+// epilogue warp about 700 cycles, measured with the work itself taken out, and
+// the eight MMAs 510.  With all eight warps on every tile these were waits of
+// both warps of a scheduler at once; alternate tiles let one warp compute
+// meanwhile.  Against a layout of eight rows a lane (16x256b), V doubled and
+// every warp on every tile: m = 4 2.30 -> 2.15 ms, m = 2 1.75 -> 1.61 (16
+// warps), m = 8 without tensor-core sums 4.35 -> 3.59, Matern m = 4 4.74 ->
+// 4.35 (16 warps).  Taken with alternate tiles too, eight rows a lane
+// and column pairs need a quarter of the V loads but 168 registers: 2.27 ms.
 //
 // Every mbarrier wait is bounded (T5_WAIT_BUDGET cycles); a wait that gives
 // up sets *fault, raises a CTA-wide abort flag so the other roles leave too,
@@ -79,26 +90,34 @@ __host__ __device__ constexpr int t5_nh(int d) { return (d + 15) / 16; }
 __host__ __device__ constexpr int t5_csep(int d) { return (d % 16 == 0 || d % 16 > 10) ? 1 : 0; }
 __host__ __device__ constexpr int t5_kb(int nh, int csep) { return 2 * nh + csep; }
 
-// Floats of shared memory that hold the epilogue's running totals (the second
-// accumulation level) for the FMA variants whose registers would not hold
-// them (16 epilogue warps, or the software-pipelined variant, at M = 4): 8
-// per right-hand side per thread (2 row tiles x 2 row halves x a row pair).
-// 0 (totals in registers) otherwise.  At M = 8 with 8 warps the registers
-// spill about 270 bytes, which measured faster (4.49 ms against 4.64 ms at
-// N = 1e5) than the totals in shared memory and the two stages they cost.
-__host__ __device__ constexpr int t5_tot_floats(int EW, int M, int LAG, int TV) {
-  return (!TV && M == 4 && (EW == 16 || LAG)) ? EW * 32 * 8 * M : 0;
+// B fragments of 8 slots per batch of 16 columns (TV variants).
+__host__ __device__ constexpr int t5_nfrag(int M) { return M >= 8 ? M / 4 : 1; }
+
+// Floats of shared memory that hold the running totals of the TV variants at
+// M = 16 (four fragments' accumulators of four row groups; totals in registers
+// spilled 390 bytes).  0 otherwise: totals in registers.
+__host__ __device__ constexpr int t5_tot_floats(int EW, int M, int TV) {
+  return (TV && M == 16) ? EW * 32 * 16 * t5_nfrag(M) : 0;
+}
+
+// 16-byte words of right-hand sides per pair of columns: M / 2 of {v_c(j),
+// v_c(j + 1), v_c+1(j), v_c+1(j + 1)} (FMA sums), or the B fragments (TV).
+__host__ __device__ constexpr int t5_vwords(int M, int TV) { return TV ? 2 * t5_nfrag(M) : M / 2; }
+
+// Shared-memory bytes of a stage's right-hand sides (enough for either).
+__host__ __device__ constexpr int t5_vstage(int M) {
+  return (t5_vwords(M, 1) > t5_vwords(M, 0) ? t5_vwords(M, 1) : t5_vwords(M, 0)) * T5_TN / 2 * 16;
 }
 
 // Column-tile pipeline stages: as many as fit (at most 8) in about 200 KB of
 // shared memory beside the row operand and the totals, so that TMA latency is
 // hidden.
 __host__ __device__ constexpr int t5_stages(int kb, int M, int tot_floats = 0) {
-  return ((204800 - 1024 - T5_RT * kb * T5_BLK - 4 * tot_floats) /
-          (kb * T5_BLK + (M / 2) * T5_TN * 16)) > 8
+  return ((204800 - 1024 - T5_RT * kb * T5_BLK - 4 * tot_floats) / (kb * T5_BLK + t5_vstage(M))) >
+                 8
              ? 8
              : ((204800 - 1024 - T5_RT * kb * T5_BLK - 4 * tot_floats) /
-                (kb * T5_BLK + (M / 2) * T5_TN * 16));
+                (kb * T5_BLK + t5_vstage(M)));
 }
 
 // Barrier indices in shared memory for ST stages.
@@ -115,12 +134,12 @@ __host__ __device__ constexpr int t5_nbar(int st) { return 7 + 3 * st; }
 // Shared memory of one CTA (bytes, including 1024 bytes of alignment slack).
 __host__ __device__ constexpr int t5_smem_bytes(int kb, int M, int tot_floats = 0) {
   return 1024 + T5_RT * kb * T5_BLK +
-         t5_stages(kb, M, tot_floats) * (kb * T5_BLK + (M / 2) * T5_TN * 16) + 4 * tot_floats +
+         t5_stages(kb, M, tot_floats) * (kb * T5_BLK + t5_vstage(M)) + 4 * tot_floats +
          8 * t5_nbar(t5_stages(kb, M, tot_floats)) + 16;
 }
 
 struct T5Args {
-  const float4 *vdup;   // C x (M/2) x TN right-hand-side quadruples (t5_vdup_kernel)
+  const float4 *v;      // right-hand sides of the column tiles (t5_vpair_kernel, t5_vfrag_kernel)
   int64_t Nc;           // column points
   float *part;          // G x J x (EW / 4) x M x T5_RB partial sums
   int C;            // column tiles
@@ -169,9 +188,8 @@ __device__ __forceinline__ void t5_mma_16816(float (&d)[4], const uint32_t (&a)[
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b.x), "r"(b.y));
 }
 
-// Epilogue variants: EW epilogue warps (8, 12 or 16; EW / 4 column groups of
-// TN / (EW / 4) columns per tile, TN the column tile: 128, or 96 for 12
-// warps), PIPE = 1 keeps the TMEM loads of the
+// Epilogue variants: EW epilogue warps (8, 12 or 16; TN the column tile: 128,
+// or 96 for 12 warps, which share every tile), PIPE = 1 keeps the TMEM loads of the
 // next 16 columns in flight while the current ones are computed, LAG = 1
 // (with PIPE) software-pipelines the epilogue by one batch of 16 columns:
 // the kernel values (ex2 on the MUFU) of batch b are formed while the FFMA2
@@ -184,7 +202,7 @@ __device__ __forceinline__ void t5_mma_16816(float (&d)[4], const uint32_t (&a)[
 // B operand holds the right-hand sides split likewise, v s_c = v_hi + v_lo
 // with a power-of-two scale s_c per right-hand side (t5_vfrag_kernel): B
 // slots 0..M-1 the v_hi, M..2M-1 the v_lo (M <= 4), or one fragment of each
-// (M = 8).  Products of fp16 halves are exact in float32, so the result is
+// for every eight right-hand sides (M = 8, 16).  Products of fp16 halves are exact in float32, so the result is
 // (hi + lo)(v_hi + v_lo) summed in float32 per tile, then added to the
 // segment total (two levels, as the FMA variants).
 template <int KERN, int NH, int CSEP, int M, int EW, int PIPE, int LAG, int TN, int TV = 0>
@@ -196,9 +214,9 @@ kmvtc5_kernel(const __grid_constant__ CUtensorMap rowmap,
   constexpr int T5_TN = TN;
   constexpr int KB = 2 * NH + CSEP;
   constexpr int MP = M / 2;   // right-hand-side pairs
-  constexpr int NB = (M == 8) ? 2 : 1;   // B fragments per batch (TV)
-  constexpr int VQ = TV ? NB : MP;       // 16-byte right-hand-side words per column
-  constexpr int TOTF = t5_tot_floats(EW, M, LAG, TV);   // running totals in shared memory
+  constexpr int NB = t5_nfrag(M);        // B fragments per batch (TV)
+  constexpr int VF = t5_vwords(M, TV) * T5_TN / 2;   // 16-byte right-hand-side words of a tile
+  constexpr int TOTF = t5_tot_floats(EW, M, TV);     // running totals in shared memory
   constexpr int T5_ST = t5_stages(KB, M, TOTF);
   constexpr int T5_BAR_A_FULL = t5_bar_a_full();
   constexpr int T5_BAR_A_EMPTY = t5_bar_a_empty();
@@ -210,7 +228,12 @@ kmvtc5_kernel(const __grid_constant__ CUtensorMap rowmap,
   constexpr int T5_BAR_FIN = t5_bar_fin(T5_ST);
   constexpr int T5_NBAR = t5_nbar(T5_ST);
   constexpr int T5_EPI_WARPS = EW;
-  constexpr int T5_CG = EW / 4;                 // column groups of the epilogue
+  // The two halves of 8 or 16 epilogue warps take alternate tiles (one D buffer
+  // each), so that one half computes while the other hands over.
+  // Not for the Matern tensor-core sums, whose warps issue without a pause (N =
+  // 50021, d = 32, m = 8: 1.49 ms together, 1.56 in turn).
+  constexpr int TG = EW % 8 == 0 && !(TV && KERN == KMATERN) ? 2 : 1;
+  constexpr int T5_CG = EW / 4 / TG;            // column groups of a tile
   constexpr int T5_WCOLS = T5_TN / T5_CG;       // columns per epilogue warp per tile
   constexpr int T5_PRODUCER_WARP = EW;
   constexpr int T5_MMA_WARP = EW + 1;
@@ -221,9 +244,9 @@ kmvtc5_kernel(const __grid_constant__ CUtensorMap rowmap,
   const uint32_t sA = base;                                   // [rt][kb][128 x 32 B]
   const uint32_t sB = sA + T5_RT * KB * T5_BLK;               // [stage][kb][128 x 32 B]
   const uint32_t vOff = sB + T5_ST * KB * T5_BLK - base;
-  float4 *sV = reinterpret_cast<float4 *>(gbase + vOff);       // [stage][MP][128]
-  const uint32_t totOff = vOff + T5_ST * MP * 128 * 16;
-  float4 *sTot = reinterpret_cast<float4 *>(gbase + totOff);   // [warp][2M][32 lanes]
+  float4 *sV = reinterpret_cast<float4 *>(gbase + vOff);       // [stage][VF]
+  const uint32_t totOff = vOff + T5_ST * t5_vstage(M);
+  float4 *sTot = reinterpret_cast<float4 *>(gbase + totOff);   // [warp][4 NB][32 lanes]
   const uint32_t sBar = base + totOff + 4 * TOTF;
   uint32_t *tslot = reinterpret_cast<uint32_t *>(gbase + (sBar - base) + 8 * T5_NBAR);
   volatile int *abort_flag = reinterpret_cast<volatile int *>(tslot + 1);
@@ -243,11 +266,11 @@ kmvtc5_kernel(const __grid_constant__ CUtensorMap rowmap,
     for (int s = 0; s < T5_ST; ++s) {
       bw::mbar_init(bar(T5_BAR_B_FULL + s), 1);
       bw::mbar_init(bar(T5_BAR_B_EMPTY + s), 1);
-      bw::mbar_init(bar(T5_BAR_V_EMPTY + s), T5_EPI_WARPS);   // one arrival per warp
+      bw::mbar_init(bar(T5_BAR_V_EMPTY + s), T5_EPI_WARPS / TG);   // one arrival per warp
     }
     for (int i = 0; i < 2; ++i) {
       bw::mbar_init(bar(T5_BAR_D_FULL + i), 1);
-      bw::mbar_init(bar(T5_BAR_D_EMPTY + i), T5_EPI_WARPS);
+      bw::mbar_init(bar(T5_BAR_D_EMPTY + i), T5_EPI_WARPS / TG);
     }
     bw::mbar_init(bar(T5_BAR_FIN), 1);
     *abort_flag = 0;
@@ -277,7 +300,7 @@ kmvtc5_kernel(const __grid_constant__ CUtensorMap rowmap,
   if (warp == T5_PRODUCER_WARP) {
     // ------------------------------------------------------------ producer
     if (lane == 0) {
-      constexpr uint32_t VBYTES = VQ * T5_TN * 16;
+      constexpr uint32_t VBYTES = VF * 16;
       int64_t kt = 0, issued_b = 0;
       int issued_a = 0;
       int64_t rb = rb_first;
@@ -297,7 +320,7 @@ kmvtc5_kernel(const __grid_constant__ CUtensorMap rowmap,
         if (!wait(T5_BAR_B_EMPTY + s, ph ^ 1u) || !wait(T5_BAR_V_EMPTY + s, ph ^ 1u)) break;
         bw::mbar_arrive_expect_tx(bar(T5_BAR_B_FULL + s), KB * T5_BLK + VBYTES);
         bw::tma_load_3d(sB + s * KB * T5_BLK, &colmap, bar(T5_BAR_B_FULL + s), 0, ct * T5_TN, 0);
-        bw::bulk_load(base + vOff + (uint32_t)s * VBYTES, a.vdup + (size_t)ct * VQ * T5_TN,
+        bw::bulk_load(base + vOff + (uint32_t)s * VBYTES, a.v + (size_t)ct * VF,
                       VBYTES, bar(T5_BAR_B_FULL + s));
         ++issued_b;
       }
@@ -361,97 +384,88 @@ kmvtc5_kernel(const __grid_constant__ CUtensorMap rowmap,
   } else {
     // ------------------------------------------------------------ epilogue
     const int qd = warp & 3;        // TMEM lane quarter
-    const int cg = warp >> 2;       // column group
-    const int g = lane >> 2, tq = lane & 3;
-    // sums over the current tile's columns (acc) and over the segment's
-    // finished tiles (tot): two-level float32 accumulation, so a long segment
-    // (up to about 1e5 columns per row) adds one tile sum at a time to its
-    // running total instead of one entry at a time
-    float2 acc[T5_RT][2][M];        // [row tile][rows g,g+8 | g+16,g+24][rhs]
-    // running totals: registers, or (TOTF > 0) this thread's 2M float4 in
-    // shared memory, float4 q holding acc entries 2q and 2q + 1 (flattened)
-    float2 tot[TOTF ? 1 : T5_RT][2][M];
-    float4 *mytot = sTot + warp * (2 * M) * 32 + lane;
-#pragma unroll
-    for (int rt = 0; rt < T5_RT; ++rt)
-#pragma unroll
-      for (int hf = 0; hf < 2; ++hf)
-#pragma unroll
-        for (int c = 0; c < M; ++c) acc[rt][hf][c] = f2(0.0f, 0.0f);
-    if constexpr (TOTF > 0) {
-#pragma unroll
-      for (int q = 0; q < 2 * M; ++q) mytot[q * 32] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-    } else {
-#pragma unroll
-      for (int rt = 0; rt < T5_RT; ++rt)
-#pragma unroll
-        for (int hf = 0; hf < 2; ++hf)
-#pragma unroll
-          for (int c = 0; c < M; ++c) tot[rt][hf][c] = f2(0.0f, 0.0f);
-    }
-    auto fold_tile = [&]() {
-      if constexpr (TOTF > 0) {
-        float2 *af = &acc[0][0][0];
-#pragma unroll
-        for (int q = 0; q < 2 * M; ++q) {
-          const float4 t = mytot[q * 32];
-          const float2 lo = __fadd2_rn(f2(t.x, t.y), af[2 * q]);
-          const float2 hi = __fadd2_rn(f2(t.z, t.w), af[2 * q + 1]);
-          mytot[q * 32] = make_float4(lo.x, lo.y, hi.x, hi.y);
-          af[2 * q] = af[2 * q + 1] = f2(0.0f, 0.0f);
-        }
-      } else {
-#pragma unroll
-        for (int rt = 0; rt < T5_RT; ++rt)
-#pragma unroll
-          for (int hf = 0; hf < 2; ++hf)
-#pragma unroll
-            for (int c = 0; c < M; ++c) {
-              tot[rt][hf][c] = __fadd2_rn(tot[rt][hf][c], acc[rt][hf][c]);
-              acc[rt][hf][c] = f2(0.0f, 0.0f);
-            }
-      }
-    };
-    // running total of (rt, hf, c), cleared as it is read (segment end)
-    auto take_tot = [&](int rt, int hf, int c) -> float2 {
-      if constexpr (TOTF > 0) {
-        const int i = (rt * 2 + hf) * M + c;
-        float4 *t = mytot + (i >> 1) * 32;
-        const float4 v = *t;
-        if (i & 1) {
-          t->z = 0.0f;
-          t->w = 0.0f;
-          return f2(v.z, v.w);
-        }
-        t->x = 0.0f;
-        t->y = 0.0f;
-        return f2(v.x, v.y);
-      } else {
-        const float2 v = tot[rt][hf][c];
-        tot[rt][hf][c] = f2(0.0f, 0.0f);
-        return v;
-      }
-    };
+    const int slot = warp >> 2;     // slot of the partial sums
+    const int cg = slot % T5_CG;    // column group
+    const int tg = slot / T5_CG;    // tiles of this parity (TG = 2)
     constexpr int NBT = T5_WCOLS / 16;   // batches of 16 columns per tile
     if constexpr (TV) {
+      const int g = lane >> 2, tq = lane & 3;
       constexpr int NG = T5_RT * 2;      // m16 row groups of a warp: (row tile, half)
-      float yacc[NG][NB][4], ytot[NG][NB][4];
+      float yacc[NG][NB][4], ytot[TOTF ? 1 : NG][TOTF ? 1 : NB][4];
+      float4 *mytot = sTot + warp * (NG * NB) * 32 + lane;   // TOTF: group gr, fragment f at gr NB + f
 #pragma unroll
       for (int gr = 0; gr < NG; ++gr)
 #pragma unroll
         for (int f = 0; f < NB; ++f)
 #pragma unroll
-          for (int i = 0; i < 4; ++i) yacc[gr][f][i] = ytot[gr][f][i] = 0.0f;
+          for (int i = 0; i < 4; ++i) {
+            yacc[gr][f][i] = 0.0f;
+            if constexpr (!TOTF) ytot[gr][f][i] = 0.0f;
+          }
+      if constexpr (TOTF > 0) {
+#pragma unroll
+        for (int q = 0; q < NG * NB; ++q) mytot[q * 32] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      }
       int64_t kt = 0, rb = rb_first;
       int ct = ct_first;
+      // segment end: accumulator (g, 2t + e) / (g + 8, 2t + e) holds B slot 2t + e;
+      // add each v_hi slot's v_lo partner and write this warp's partial sums
+      // (scaled by 2^14 s_c; t5_reduce_kernel undoes it)
+      auto flush = [&](int64_t rbq) {
+        const int j = (int)(rbq - rb_first);
+        float *out = a.part + (((int64_t)b * a.J + j) * (EW / 4) + slot) * (int64_t)M * T5_RB;
+#pragma unroll
+        for (int gr = 0; gr < NG; ++gr) {
+          float yt[NB][4];   // the totals, cleared as they are read
+#pragma unroll
+          for (int f = 0; f < NB; ++f) {
+            if constexpr (TOTF > 0) {
+              float4 &t = mytot[(gr * NB + f) * 32];
+              yt[f][0] = t.x, yt[f][1] = t.y, yt[f][2] = t.z, yt[f][3] = t.w;
+              t = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            } else {
+#pragma unroll
+              for (int i = 0; i < 4; ++i) {
+                yt[f][i] = ytot[gr][f][i];
+                ytot[gr][f][i] = 0.0f;
+              }
+            }
+          }
+          // columns 8 h .. 8 h + 7 of the right-hand sides
+#pragma unroll
+          for (int h = 0; h < (NB + 1) / 2; ++h) {
+            float y[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              if constexpr (NB >= 2)
+                y[i] = yt[h][i] + yt[h + NB / 2][i];
+              else
+                y[i] = yt[0][i] + __shfl_xor_sync(0xffffffffu, yt[0][i], M / 2);
+            }
+            const int c0 = 8 * h + 2 * tq;
+            if (c0 < M) {
+              const int row = (gr >> 1) * T5_TM + 32 * qd + 16 * (gr & 1) + g;
+              out[c0 * T5_RB + row] = y[0];
+              out[(c0 + 1) * T5_RB + row] = y[1];
+              out[c0 * T5_RB + row + 8] = y[2];
+              out[(c0 + 1) * T5_RB + row + 8] = y[3];
+            }
+          }
+        }
+      };
       for (int64_t p = p_begin; p < p_end; ++p, ++kt, (++ct == a.C ? (ct = 0, ++rb) : 0)) {
+        const bool segend = p + 1 == p_end || ct + 1 == a.C;
+        if (TG == 2 && (int)(kt & 1) != tg) {
+          if (segend) flush(rb);
+          continue;
+        }
         const int s = (int)(kt % T5_ST);
         const int buf = (int)(kt & 1);
         const bool ok = __all_sync(0xffffffffu, wait(T5_BAR_D_FULL + buf, (uint32_t)((kt >> 1) & 1)) &&
                                                     wait(T5_BAR_B_FULL + s, (uint32_t)((kt / T5_ST) & 1)));
         if (!ok) break;
         bw::tc_fence_after();
-        const uint2 *vf = reinterpret_cast<const uint2 *>(sV + (size_t)s * VQ * T5_TN);
+        const uint2 *vf = reinterpret_cast<const uint2 *>(sV + (size_t)s * VF);
         const uint32_t tcol = tmem + (uint32_t)(buf * T5_RT * T5_TN + cg * T5_WCOLS);
         uint32_t r[PIPE ? 2 : 1][32];   // [batch parity][row group][8]
         auto load_batch = [&](int bt, uint32_t *rr) {
@@ -506,283 +520,185 @@ kmvtc5_kernel(const __grid_constant__ CUtensorMap rowmap,
             bw::tmem_wait_ld32(r[(bt + 1) & 1]);
             if (bt + 2 == NBT) release_buffer();
           }
-        }
+          if ((bt & 3) == 3 || bt + 1 == NBT) {   // sums of 64 columns
 #pragma unroll
-        for (int gr = 0; gr < NG; ++gr)
+            for (int gr = 0; gr < NG; ++gr)
 #pragma unroll
-          for (int f = 0; f < NB; ++f)
+              for (int f = 0; f < NB; ++f) {
+                if constexpr (TOTF > 0) {
+                  float4 &t = mytot[(gr * NB + f) * 32];
+                  const float4 v = t;
+                  t = make_float4(v.x + yacc[gr][f][0], v.y + yacc[gr][f][1], v.z + yacc[gr][f][2],
+                                  v.w + yacc[gr][f][3]);
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              ytot[gr][f][i] += yacc[gr][f][i];
-              yacc[gr][f][i] = 0.0f;
-            }
-        __syncwarp();
-        if (lane == 0) bw::mbar_arrive(bar(T5_BAR_V_EMPTY + s));
-        if (p + 1 == p_end || ct + 1 == a.C) {
-          // end of a segment: accumulator (g, 2t + e) / (g + 8, 2t + e) holds
-          // B slot 2t + e; add each v_hi slot's v_lo partner and write this
-          // warp's partial sums (scaled by 2^14 s_c; t5_reduce_kernel undoes it)
-          const int j = (int)(rb - rb_first);
-          float *out = a.part + (((int64_t)b * a.J + j) * T5_CG + cg) * (int64_t)M * T5_RB;
+                  for (int i = 0; i < 4; ++i) yacc[gr][f][i] = 0.0f;
+                } else {
 #pragma unroll
-          for (int gr = 0; gr < NG; ++gr) {
-            float y[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              if constexpr (NB == 2)
-                y[i] = ytot[gr][0][i] + ytot[gr][1][i];
-              else
-                y[i] = ytot[gr][0][i] + __shfl_xor_sync(0xffffffffu, ytot[gr][0][i], M / 2);
-#pragma unroll
-              for (int f = 0; f < NB; ++f) ytot[gr][f][i] = 0.0f;
-            }
-            const int c0 = 2 * tq;
-            if (c0 < M) {
-              const int row = (gr >> 1) * T5_TM + 32 * qd + 16 * (gr & 1) + g;
-              out[c0 * T5_RB + row] = y[0];
-              out[(c0 + 1) * T5_RB + row] = y[1];
-              out[c0 * T5_RB + row + 8] = y[2];
-              out[(c0 + 1) * T5_RB + row + 8] = y[3];
-            }
+                  for (int i = 0; i < 4; ++i) {
+                    ytot[gr][f][i] += yacc[gr][f][i];
+                    yacc[gr][f][i] = 0.0f;
+                  }
+                }
+              }
           }
         }
+        __syncwarp();
+        if (lane == 0) bw::mbar_arrive(bar(T5_BAR_V_EMPTY + s));
+        if (segend) flush(rb);
       }
-    } else if constexpr (LAG) {
-      // segment end: the four lanes of a row group hold sums over different
-      // columns; add them and write this warp's partial sums
-      auto flush = [&](int64_t rbq) {
-        const int j = (int)(rbq - rb_first);
-        float *out = a.part + (((int64_t)b * a.J + j) * T5_CG + cg) * (int64_t)M * T5_RB;
+    } else {
+      // a lane's rows of the two row tiles: packed sums over the even and odd
+      // columns of the current tile (acc), and over the segment's finished
+      // tiles (tot): two-level float32 accumulation, so a long segment (up to
+      // about 1e5 columns per row) adds one tile sum at a time to its running
+      // total instead of one entry at a time
+      float2 acc[T5_RT][M];
+      float tot[T5_RT][M];
+#pragma unroll
+      for (int rt = 0; rt < T5_RT; ++rt)
+#pragma unroll
+        for (int c = 0; c < M; ++c) {
+          acc[rt][c] = f2(0.0f, 0.0f);
+          tot[rt][c] = 0.0f;
+        }
+      auto fold_tile = [&]() {
 #pragma unroll
         for (int rt = 0; rt < T5_RT; ++rt)
 #pragma unroll
-          for (int hf = 0; hf < 2; ++hf)
-#pragma unroll
-            for (int c = 0; c < M; ++c) {
-              float2 v = take_tot(rt, hf, c);
-              v.x += __shfl_xor_sync(0xffffffffu, v.x, 1);
-              v.y += __shfl_xor_sync(0xffffffffu, v.y, 1);
-              v.x += __shfl_xor_sync(0xffffffffu, v.x, 2);
-              v.y += __shfl_xor_sync(0xffffffffu, v.y, 2);
-              if ((c & 3) == tq) {
-                const int row = rt * T5_TM + 32 * qd + 16 * hf + g;
-                out[c * T5_RB + row] = v.x;
-                out[c * T5_RB + row + 8] = v.y;
-              }
-            }
+          for (int c = 0; c < M; ++c) {
+            tot[rt][c] += acc[rt][c].x + acc[rt][c].y;
+            acc[rt][c] = f2(0.0f, 0.0f);
+          }
       };
-      // kernel values of one batch: [ch][e][rt][hf] -> rows (g, g + 8) pair
+      // segment end: this warp's partial sums
+      auto flush = [&](int64_t rbq) {
+        const int j = (int)(rbq - rb_first);
+        float *out = a.part + (((int64_t)b * a.J + j) * (EW / 4) + slot) * (int64_t)M * T5_RB +
+                     32 * qd + lane;
+#pragma unroll
+        for (int rt = 0; rt < T5_RT; ++rt)
+#pragma unroll
+          for (int c = 0; c < M; ++c) {
+            out[c * T5_RB + rt * T5_TM] = tot[rt][c];
+            tot[rt][c] = 0.0f;
+          }
+      };
+      // kernel values of one batch: [row tile][column pair]
       auto kappa_batch = [&](const uint32_t *cur, float2 *kq) {
 #pragma unroll
-        for (int ch = 0; ch < 2; ++ch)
-#pragma unroll
-          for (int e = 0; e < 2; ++e)
-#pragma unroll
-            for (int rt = 0; rt < T5_RT; ++rt)
-#pragma unroll
-              for (int hf = 0; hf < 2; ++hf) {
-                const uint32_t *q = &cur[(rt * 2 + hf) * 8 + ch * 4];
-                kq[((ch * 2 + e) * 2 + rt) * 2 + hf] =
-                    f2(t5_kappa<KERN>(q[e]), t5_kappa<KERN>(q[2 + e]));
-              }
+        for (int i = 0; i < T5_RT * 8; ++i)
+          kq[i] = f2(t5_kappa<KERN>(cur[2 * i]), t5_kappa<KERN>(cur[2 * i + 1]));
       };
-      auto ffma_batch = [&](const float2 *kq, const float4 *vq, int col0) {
+      auto ffma_batch = [&](const float2 *kq, const float4 *vq) {
 #pragma unroll
-        for (int ch = 0; ch < 2; ++ch)
+        for (int jp = 0; jp < 8; ++jp)
 #pragma unroll
-          for (int e = 0; e < 2; ++e) {
-            const int jl = col0 + ch * 8 + 2 * tq + e;
+          for (int cp = 0; cp < MP; ++cp) {
+            const float4 v = vq[cp * (T5_TN / 2) + jp];
 #pragma unroll
-            for (int cp = 0; cp < MP; ++cp) {
-              const float4 v = vq[cp * T5_TN + jl];
-#pragma unroll
-              for (int rt = 0; rt < T5_RT; ++rt)
-#pragma unroll
-                for (int hf = 0; hf < 2; ++hf) {
-                  const float2 k2 = kq[((ch * 2 + e) * 2 + rt) * 2 + hf];
-                  acc[rt][hf][2 * cp] = __ffma2_rn(k2, f2(v.x, v.y), acc[rt][hf][2 * cp]);
-                  acc[rt][hf][2 * cp + 1] = __ffma2_rn(k2, f2(v.z, v.w), acc[rt][hf][2 * cp + 1]);
-                }
+            for (int rt = 0; rt < T5_RT; ++rt) {
+              acc[rt][2 * cp] = __ffma2_rn(kq[rt * 8 + jp], f2(v.x, v.y), acc[rt][2 * cp]);
+              acc[rt][2 * cp + 1] = __ffma2_rn(kq[rt * 8 + jp], f2(v.z, v.w), acc[rt][2 * cp + 1]);
             }
           }
       };
-      // the batch whose accumulation is pending
-      float2 kp[16];
+      // LAG: the batch whose accumulation is pending
+      float2 kp[T5_RT * 8];
       const float4 *vp = sV;
-      int colp = 0, sp = 0;
-      bool havep = false, p_last = false, p_segend = false;
+      int sp = 0;
+      bool havep = false, p_fold = false, p_last = false, p_segend = false;
       int64_t p_rb = 0;
-      auto retire_pending = [&]() {
-        ffma_batch(kp, vp, colp);
-        if (p_last) {
-          fold_tile();
+      auto retire = [&](const float2 *kq, const float4 *vq, int sq, bool fold, bool last,
+                        bool segend, int64_t rbq) {
+        ffma_batch(kq, vq);
+        if (fold) fold_tile();   // every 64 columns: sums of 32 entries
+        if (last) {
           __syncwarp();
-          if (lane == 0) bw::mbar_arrive(bar(T5_BAR_V_EMPTY + sp));
-          if (p_segend) flush(p_rb);
+          if (lane == 0) bw::mbar_arrive(bar(T5_BAR_V_EMPTY + sq));
+          if (segend) flush(rbq);
         }
       };
       int64_t kt = 0, rb = rb_first;
       int ct = ct_first;
       for (int64_t p = p_begin; p < p_end; ++p, ++kt, (++ct == a.C ? (ct = 0, ++rb) : 0)) {
+        const bool segend = (p + 1 == p_end) || (ct + 1 == a.C);
+        if (TG == 2 && (int)(kt & 1) != tg) {
+          if (segend) {
+            if (LAG && havep) retire(kp, vp, sp, p_fold, p_last, p_segend, p_rb);
+            havep = false;
+            flush(rb);
+          }
+          continue;
+        }
         const int s = (int)(kt % T5_ST);
         const int buf = (int)(kt & 1);
+        // D of this tile, and (for the visibility of the bulk-copied V) the
+        // stage's arrival
         const bool ok =
             __all_sync(0xffffffffu, wait(T5_BAR_D_FULL + buf, (uint32_t)((kt >> 1) & 1)) &&
                                         wait(T5_BAR_B_FULL + s, (uint32_t)((kt / T5_ST) & 1)));
         if (!ok) break;
         bw::tc_fence_after();
-        const float4 *vt = sV + (size_t)s * MP * T5_TN;
-        const uint32_t tcol = tmem + (uint32_t)(buf * T5_RT * T5_TN + cg * T5_WCOLS);
-        const bool segend = (p + 1 == p_end) || (ct + 1 == a.C);
-        uint32_t r[2][32];
+        const float4 *vt = sV + (size_t)s * VF + cg * (T5_WCOLS / 2);
+        const uint32_t tcol = tmem + ((uint32_t)(32 * qd) << 16) +
+                              (uint32_t)(buf * T5_RT * T5_TN + cg * T5_WCOLS);
+        // with PIPE, the TMEM loads of batch bt + 1 are in flight while batch bt
+        // is computed
+        uint32_t r[PIPE ? 2 : 1][32];   // [batch parity][row tile][column]
         auto load_batch = [&](int bt, uint32_t *rr) {
 #pragma unroll
           for (int rt = 0; rt < T5_RT; ++rt)
-#pragma unroll
-            for (int hf = 0; hf < 2; ++hf)
-              bw::tmem_ld_16x256b_x2(tcol + ((uint32_t)(32 * qd + 16 * hf) << 16) +
-                                         (uint32_t)(rt * T5_TN + bt * 16),
-                                     &rr[(rt * 2 + hf) * 8]);
+            bw::tmem_ld_32x32b_x16(tcol + (uint32_t)(rt * T5_TN + bt * 16), rr + rt * 16);
         };
         auto release_buffer = [&]() {
+          // this warp's TMEM loads of the buffer have landed: hand it back
           bw::tc_fence_before();
           __syncwarp();
           if (lane == 0) bw::mbar_arrive(bar(T5_BAR_D_EMPTY + buf));
         };
-        load_batch(0, r[0]);
-        bw::tmem_wait_ld32(r[0]);
-        if (NBT == 1) release_buffer();
+        if (PIPE) {
+          load_batch(0, r[0]);
+          bw::tmem_wait_ld32(r[0]);
+          if (NBT == 1) release_buffer();
+        }
 #pragma unroll
         for (int bt = 0; bt < NBT; ++bt) {
-          if (bt + 1 < NBT) load_batch(bt + 1, r[(bt + 1) & 1]);
-          float2 kc[16];
-          kappa_batch(r[bt & 1], kc);
-          if (havep) retire_pending();
-          if (bt + 1 < NBT) {
+          uint32_t *cur = r[PIPE ? (bt & 1) : 0];
+          if (PIPE) {
+            if (bt + 1 < NBT) load_batch(bt + 1, r[(bt + 1) & 1]);
+          } else {
+            load_batch(bt, cur);
+            bw::tmem_wait_ld32(cur);
+            if (bt + 1 == NBT) release_buffer();
+          }
+          float2 kc[T5_RT * 8];
+          kappa_batch(cur, kc);
+          const bool last = bt + 1 == NBT, fold = last || (bt & 3) == 3;
+          if constexpr (LAG) {
+            if (havep) retire(kp, vp, sp, p_fold, p_last, p_segend, p_rb);
+          } else {
+            retire(kc, vt + bt * 8, s, fold, last, segend, rb);
+          }
+          if (PIPE && bt + 1 < NBT) {
             bw::tmem_wait_ld32(r[(bt + 1) & 1]);
             if (bt + 2 == NBT) release_buffer();
           }
+          if constexpr (LAG) {
 #pragma unroll
-          for (int i = 0; i < 16; ++i) kp[i] = kc[i];
-          vp = vt;
-          colp = cg * T5_WCOLS + bt * 16;
-          sp = s;
-          havep = true;
-          p_last = (bt + 1 == NBT);
-          p_segend = p_last && segend;
-          p_rb = rb;
-        }
-      }
-      if (havep) retire_pending();
-    } else {
-    int64_t kt = 0, rb = rb_first;
-    int ct = ct_first;
-    for (int64_t p = p_begin; p < p_end; ++p, ++kt, (++ct == a.C ? (ct = 0, ++rb) : 0)) {
-      const int s = (int)(kt % T5_ST);
-      const int buf = (int)(kt & 1);
-      // D of this tile, and (for the visibility of the bulk-copied V) the
-      // stage's arrival
-      const bool ok = __all_sync(0xffffffffu, wait(T5_BAR_D_FULL + buf, (uint32_t)((kt >> 1) & 1)) &&
-                                                  wait(T5_BAR_B_FULL + s, (uint32_t)((kt / T5_ST) & 1)));
-      if (!ok) break;
-      bw::tc_fence_after();
-      const float4 *vt = sV + (size_t)s * MP * T5_TN;
-      const uint32_t tcol = tmem + (uint32_t)(buf * T5_RT * T5_TN + cg * T5_WCOLS);
-      // with PIPE, the TMEM loads of batch bt + 1 are in flight while batch bt
-      // is computed
-      uint32_t r[PIPE ? 2 : 1][32];   // [batch parity][rt][hf][8]
-      auto load_batch = [&](int bt, uint32_t *rr) {
-#pragma unroll
-        for (int rt = 0; rt < T5_RT; ++rt)
-#pragma unroll
-          for (int hf = 0; hf < 2; ++hf)
-            bw::tmem_ld_16x256b_x2(tcol + ((uint32_t)(32 * qd + 16 * hf) << 16) +
-                                       (uint32_t)(rt * T5_TN + bt * 16),
-                                   &rr[(rt * 2 + hf) * 8]);
-      };
-      auto release_buffer = [&]() {
-        // every TMEM load of this buffer has landed: hand it back
-        bw::tc_fence_before();
-        __syncwarp();
-        if (lane == 0) bw::mbar_arrive(bar(T5_BAR_D_EMPTY + buf));
-      };
-      if (PIPE) {
-        load_batch(0, r[0]);
-        bw::tmem_wait_ld32(r[0]);
-        if (NBT == 1) release_buffer();
-      }
-#pragma unroll
-      for (int bt = 0; bt < NBT; ++bt) {
-        uint32_t *cur = r[PIPE ? (bt & 1) : 0];
-        if (PIPE) {
-          if (bt + 1 < NBT) load_batch(bt + 1, r[(bt + 1) & 1]);
-        } else {
-          load_batch(bt, cur);
-          bw::tmem_wait_ld32(cur);
-          if (bt + 1 == NBT) release_buffer();
-        }
-        const int col0 = cg * T5_WCOLS + bt * 16;
-#pragma unroll
-        for (int ch = 0; ch < 2; ++ch) {
-#pragma unroll
-          for (int e = 0; e < 2; ++e) {
-            const int jl = col0 + ch * 8 + 2 * tq + e;
-            float2 kk[T5_RT][2];
-#pragma unroll
-            for (int rt = 0; rt < T5_RT; ++rt)
-#pragma unroll
-              for (int hf = 0; hf < 2; ++hf) {
-                const uint32_t *q = &cur[(rt * 2 + hf) * 8 + ch * 4];
-                kk[rt][hf] = f2(t5_kappa<KERN>(q[e]), t5_kappa<KERN>(q[2 + e]));
-              }
-#pragma unroll
-            for (int cp = 0; cp < MP; ++cp) {
-              const float4 v = vt[cp * T5_TN + jl];
-#pragma unroll
-              for (int rt = 0; rt < T5_RT; ++rt)
-#pragma unroll
-                for (int hf = 0; hf < 2; ++hf) {
-                  acc[rt][hf][2 * cp] = __ffma2_rn(kk[rt][hf], f2(v.x, v.y), acc[rt][hf][2 * cp]);
-                  acc[rt][hf][2 * cp + 1] =
-                      __ffma2_rn(kk[rt][hf], f2(v.z, v.w), acc[rt][hf][2 * cp + 1]);
-                }
-            }
+            for (int i = 0; i < T5_RT * 8; ++i) kp[i] = kc[i];
+            vp = vt + bt * 8;
+            sp = s;
+            havep = true;
+            p_fold = fold;
+            p_last = last;
+            p_segend = last && segend;
+            p_rb = rb;
           }
         }
-        if (PIPE && bt + 1 < NBT) {
-          bw::tmem_wait_ld32(r[(bt + 1) & 1]);
-          if (bt + 2 == NBT) release_buffer();
-        }
       }
-      fold_tile();
-      __syncwarp();
-      if (lane == 0) bw::mbar_arrive(bar(T5_BAR_V_EMPTY + s));
-      if (p + 1 == p_end || ct + 1 == a.C) {
-        // end of a segment: the four lanes of a row group hold sums over
-        // different columns; add them and write this warp's partial sums
-        const int j = (int)(rb - rb_first);
-        float *out = a.part + (((int64_t)b * a.J + j) * T5_CG + cg) * (int64_t)M * T5_RB;
-#pragma unroll
-        for (int rt = 0; rt < T5_RT; ++rt)
-#pragma unroll
-          for (int hf = 0; hf < 2; ++hf)
-#pragma unroll
-            for (int c = 0; c < M; ++c) {
-              float2 v = take_tot(rt, hf, c);
-              v.x += __shfl_xor_sync(0xffffffffu, v.x, 1);
-              v.y += __shfl_xor_sync(0xffffffffu, v.y, 1);
-              v.x += __shfl_xor_sync(0xffffffffu, v.x, 2);
-              v.y += __shfl_xor_sync(0xffffffffu, v.y, 2);
-              if ((c & 3) == tq) {
-                const int row = rt * T5_TM + 32 * qd + 16 * hf + g;
-                out[c * T5_RB + row] = v.x;
-                out[c * T5_RB + row + 8] = v.y;
-              }
-            }
-      }
+      if (LAG && havep) retire(kp, vp, sp, p_fold, p_last, p_segend, p_rb);
     }
-    }
-}
+  }
 
   bw::tc_fence_before();
   __syncthreads();
@@ -816,7 +732,8 @@ namespace krr {
 // on 96-column tiles with pipelined loads, 7 = the same without; 8..11 take
 // the sums over V on the tensor cores (TV): 8 = 8 warps with pipelined loads,
 // 9 = 8 warps without, 10 = 16 warps without, 11 = 16 warps with.  The 12-
-// and 16-warp and software-pipelined variants serve M <= 4 only.
+// and 16-warp and software-pipelined variants serve M <= 4 only; M = 16 has
+// the TV variants 8 and 9.
 constexpr int T5_NVARIANTS = 11;
 __host__ __device__ constexpr bool t5_variant_tv(int v) { return v >= 8; }
 __host__ __device__ constexpr int t5_variant_ew(int v) {
@@ -828,7 +745,8 @@ __host__ __device__ constexpr int t5_variant_tn(int v) { return (v == 6 || v == 
 // restricted KRR) may have rows whose kernel values all lie below 2^-20,
 // where their fp16 halves (even scaled by 2^14) keep too few bits.
 inline bool t5_variant_valid(int v, int M, bool square) {
-  return v >= 1 && v <= T5_NVARIANTS && (v == 1 || v == 3 || v == 8 || v == 9 || M <= 4) &&
+  return v >= 1 && v <= T5_NVARIANTS &&
+         (v == 8 || v == 9 || ((v == 1 || v == 3) && M <= 8) || M <= 4) &&
          (square || !t5_variant_tv(v));
 }
 
@@ -907,6 +825,9 @@ cudaError_t launch_kmvtc5(int nh, int csep, int M, int variant, int G, size_t sm
   KRR_T5_CASE(1, 1, 2) KRR_T5_CASE(1, 1, 4) KRR_T5_CASE(1, 1, 8)
   KRR_T5_CASE(2, 0, 2) KRR_T5_CASE(2, 0, 4) KRR_T5_CASE(2, 0, 8)
   KRR_T5_CASE(2, 1, 2) KRR_T5_CASE(2, 1, 4) KRR_T5_CASE(2, 1, 8)
+  if constexpr (TVSET) {
+    KRR_T5_CASE(1, 0, 16) KRR_T5_CASE(1, 1, 16) KRR_T5_CASE(2, 0, 16) KRR_T5_CASE(2, 1, 16)
+  }
 #undef KRR_T5_CASE
   return cudaErrorInvalidValue;
 }
