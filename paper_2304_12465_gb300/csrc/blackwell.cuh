@@ -82,6 +82,12 @@ __device__ __forceinline__ bool mbar_wait_abortable(uint32_t bar, uint32_t parit
   }
 }
 
+// Makes this thread's shared-memory writes visible to the async proxy (MMA
+// operands written by threads).
+__device__ __forceinline__ void fence_async_shared() {
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+}
+
 // --------------------------------------------------------------- TMA loads
 // 2-D tiled tensor load into shared memory, completing on `bar` (tx bytes).
 // c0 is the innermost coordinate (elements), c1 the row.
@@ -207,6 +213,14 @@ __device__ __forceinline__ void tmem_ld_32x32b_x16(uint32_t taddr, uint32_t *r) 
         "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
         "=r"(r[14]), "=r"(r[15])
       : "r"(taddr));
+}
+
+// 32x32b.x8: as x16 with eight columns.
+__device__ __forceinline__ void tmem_ld_32x32b_x8(uint32_t taddr, uint32_t *r) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]),
+                 "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr));
 }
 
 // 16x256b.x1: 16 lanes x 8 columns; thread t receives (lane0 + t/4, columns

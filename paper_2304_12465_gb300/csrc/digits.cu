@@ -1,234 +1,373 @@
-// C -= A B^T by digits on the fp16 tensor cores (digits.cuh): the Schur update
-// of Alg. 3 and the off-diagonal part of its triangular solve.
+// C -= A B^T by digits on the fifth-generation tensor cores (digits.cuh): the
+// Schur update of Alg. 3 and the off-diagonal part of its triangular solve.
 #include <algorithm>
 
+#include "blackwell.cuh"
 #include "dense.cuh"
 #include "digits.cuh"
+#include "kmv.cuh"
 
 namespace krr {
 
-constexpr int DG_THREADS = 256;
-constexpr int DG_ROWS = 64;        // rows of C per CTA: four 16-row tiles
-constexpr int DG_STAGES = 4;       // ring of B digits: two pairs of steps
-constexpr int DG_KSTEPS = DIG_CHUNK / 16;
+constexpr int DG_ROWS = 128;       // rows of C per CTA (TMEM lanes)
+constexpr int DG_WORKERS = 8;      // warps that convert A and read the sums out
+constexpr int DG_THREADS = (DG_WORKERS + 2) * 32;
+constexpr int DG_ADIG = DG_ROWS * 32;           // bytes of one digit of 128 x 16 of A
+constexpr int DG_LOWSTEPS = DIG_LOW / 16;       // steps of 16 terms between read-outs
+constexpr int DG_HIGHCHUNKS = DIG_HIGH / DIG_LOW;
+constexpr long long DG_WAIT_BUDGET = 1LL << 32;   // about 2 s
 
-__device__ __forceinline__ void dg_mma(float (&c)[4], const uint4 &a, const uint2 &b) {
-  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, "
-      "{%8,%9}, {%0,%1,%2,%3};"
-      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-      : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b.x), "r"(b.y));
+// Columns of one group: 64, or what is left rounded up to 16.
+__host__ __device__ constexpr int dg_group_cols(int nc, int g) {
+  return nc - 64 * g >= 64 ? 64 : (nc - 64 * g + 15) / 16 * 16;
+}
+// Instances for up to NC columns: stages of the ring, TMEM columns.
+__host__ __device__ constexpr int dg_stages(int NC) { return NC == 32 ? 2 : 4; }
+__host__ __device__ constexpr int dg_stage_bytes(int NC) { return DIG_N * (DG_ADIG + NC * 32); }
+// Steps of A in flight to shared memory, 16 KB each (a thread's own entries).
+__host__ __device__ constexpr int dg_ahead(int NC) { return NC == 32 ? 2 : 3; }
+constexpr int DG_AHEAD_BYTES = DG_WORKERS * 32 * 8 * 8;
+constexpr size_t dg_smem(int NC) {
+  return 1024 + (size_t)dg_stages(NC) * dg_stage_bytes(NC) +
+         (size_t)dg_ahead(NC) * DG_AHEAD_BYTES + 8 * (3 * dg_stages(NC) + 3) + 16;
 }
 
 // Digits of B (nc rows of K entries: row c at B + rows[c] (rows NULL: c), step
-// ldb between entries) as MMA B fragments, zero padded to K16 steps of 16 and
-// NT tiles of 8 rows: frag[((step NT + tile) 7 + digit) 32 + lane].
+// ldb between entries) as the kernel's shared tiles hold them: for column group
+// g and step of 16 terms, the seven digits one after the other, each a
+// K-major operand of dg_group_cols rows of 32 bytes in the 32-byte swizzle
+// (zero padded).  A thread makes half a row.
 __global__ void dig_rows_kernel(const double *__restrict__ B, int64_t ldb,
-                                const int64_t *__restrict__ rows, int nc, int K, int K16, int NT, uint2 *__restrict__ frag) {
-  const int64_t total = (int64_t)K16 * NT * 32;
+                                const int64_t *__restrict__ rows, int nc, int K, int K16,
+                                uint4 *__restrict__ img) {
+  const int ncp = (nc + 15) / 16 * 16;
+  const int64_t total = (int64_t)K16 * ncp * 2;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
        e += (int64_t)gridDim.x * blockDim.x) {
-    const int lane = (int)(e & 31), tile = (int)((e >> 5) % NT);
-    const int step = (int)((e >> 5) / NT);
-    const int c = tile * 8 + (lane >> 2), k = step * 16 + 2 * (lane & 3);
-    double x[4] = {0.0, 0.0, 0.0, 0.0};
-    if (c < nc) {
-      const int64_t r = rows ? rows[c] : c;
+    const int c = (int)(e % ncp), half = (int)((e / ncp) & 1);
+    const int step = (int)(e / ncp / 2);
+    const int k = step * 16 + half * 8;
+    double x[8];
+    const int64_t r = c < nc ? (rows ? rows[c] : c) : 0;
 #pragma unroll
-      for (int t = 0; t < 4; ++t) {
-        const int kk = k + (t & 1) + 8 * (t >> 1);
-        if (kk < K) x[t] = B[r + (int64_t)kk * ldb];
-      }
-    }
-    uint32_t d0[DIG_N], d1[DIG_N];
-    dig_pair(x[0], x[1], d0);
-    dig_pair(x[2], x[3], d1);
-    uint2 *dst = frag + ((int64_t)(step * NT + tile) * DIG_N) * 32 + lane;
+    for (int t = 0; t < 8; ++t)
+      x[t] = (c < nc && k + t < K) ? B[r + (int64_t)(k + t) * ldb] : 0.0;
+    uint32_t d[4][DIG_N];
 #pragma unroll
-    for (int s = 0; s < DIG_N; ++s) dst[s * 32] = make_uint2(d0[s], d1[s]);
-  }
-}
-
-// C (N x nc, ldc) -= A (N x K, lda) B^T, B as fragments; cmap (optional) gives
-// the column of C for each row of B.  A CTA takes 64 rows
-// and all columns; warp (r, h) the 16 rows of tile r and NTW column tiles of
-// half h.  Per step of 16 terms each warp converts its half of its row tile's
-// entries (read column by column, 64-byte segments), the two halves meet in
-// shared memory as MMA A fragments, and B fragments arrive through a ring of
-// asynchronous copies.  Tensor bound: 28 MMAs a tile and step against about
-// 30 other instructions.  The accumulators (28 floats a tile) set NTW <= 7
-// and one CTA a SM.  Measured at N = 1e5, 100 columns: 1.04 ms for K = 500 and
-// 1.75 ms for K = 900, against 3.35 and 5.87 ms for a float-float product on
-// the float32 pipe (3.3 clocks an MMA where the pipe's best is 2.1: eight
-// warps a SM do not fill it, and converting inside the MMA sequence spilled
-// and took 2.48 ms).
-template <int NTW>
-__global__ void __launch_bounds__(DG_THREADS, 1)
-dig_gemm_kernel(const double *__restrict__ A, int64_t lda, int64_t N, int K,
-                const uint2 *__restrict__ frag, int nc, double *__restrict__ C, int64_t ldc,
-                const int *__restrict__ cmap) {
-  constexpr int NT = 2 * NTW;
-  constexpr int BSTEP = NT * DIG_N * 32;                 // uint2 of one step
-  extern __shared__ __align__(16) unsigned char dg_smem[];
-  uint2 *sB = reinterpret_cast<uint2 *>(dg_smem);        // [DG_STAGES][BSTEP]
-  uint4 *sA = reinterpret_cast<uint4 *>(sB + DG_STAGES * BSTEP);   // [2][4][DIG_N][32]
-  int64_t *tot = reinterpret_cast<int64_t *>(sA + 2 * 4 * DIG_N * 32);   // [NTW 4][256]
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int rt = warp >> 1, half = warp & 1;
-  const int g = lane >> 2, q = lane & 3;
-  const int64_t r0 = (int64_t)blockIdx.x * DG_ROWS + rt * 16 + g;
-  const bool ok0 = r0 < N, ok1 = r0 + 8 < N;
-  const int steps = (K + 15) / 16;
-
-  auto load_a = [&](int step, double (&x)[4]) {
-    const int k = step * 16 + half * 8 + 2 * q;
-    const double *p = A + r0 + (int64_t)k * lda;
-    x[0] = (ok0 && k < K) ? p[0] : 0.0;
-    x[1] = (ok0 && k + 1 < K) ? p[lda] : 0.0;
-    x[2] = (ok1 && k < K) ? p[8] : 0.0;
-    x[3] = (ok1 && k + 1 < K) ? p[lda + 8] : 0.0;
-  };
-  auto copy_b = [&](int step) {
-    if (step < steps) {
-      const char *src = reinterpret_cast<const char *>(frag + (int64_t)step * BSTEP);
-      const uint32_t dst =
-          (uint32_t)__cvta_generic_to_shared(sB + (step % DG_STAGES) * BSTEP);
-      for (int i = tid; i < BSTEP / 2; i += DG_THREADS)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + i * 16),
-                     "l"(src + i * 16));
-    }
-  };
-
-  float acc[NTW][DIG_N][4];
-#pragma unroll
-  for (int j = 0; j < NTW; ++j)
+    for (int t = 0; t < 4; ++t) dig_pair(x[2 * t], x[2 * t + 1], d[t]);
+    const int g = c / 64, n = c % 64, ncol = dg_group_cols(nc, g);
+    uint4 *dst = img + ((int64_t)g * K16 * 64 + (int64_t)step * ncol) * DIG_N * 2;
 #pragma unroll
     for (int s = 0; s < DIG_N; ++s)
-#pragma unroll
-      for (int e = 0; e < 4; ++e) acc[j][s][e] = 0.0f;
-#pragma unroll
-  for (int j = 0; j < NTW * 4; ++j) tot[j * DG_THREADS + tid] = 0;
+      dst[(s * ncol + n) * 2 + (half ^ ((n >> 2) & 1))] =
+          make_uint4(d[0][s], d[1][s], d[2][s], d[3][s]);
+  }
+}
 
-  double x[4];
-  auto store_a = [&](int step) {
-    uint2 *dst = reinterpret_cast<uint2 *>(sA + ((step & 1) * 4 + rt) * DIG_N * 32 + lane) + half;
-    uint32_t d0[DIG_N], d1[DIG_N];
-    dig_pair(x[0], x[1], d0);
-    dig_pair(x[2], x[3], d1);
-#pragma unroll
-    for (int s = 0; s < DIG_N; ++s) dst[s * 64] = make_uint2(d0[s], d1[s]);
-  };
-  load_a(0, x);
-  copy_b(0);
-  copy_b(1);
-  for (int step = 0; step < steps; ++step) {
-    store_a(step);
-    if ((step & 1) == 0) {
-      // a pair of steps of B has arrived, and every warp is done with the
-      // pair before it, whose place the next pair takes
-      asm volatile("cp.async.wait_all;" ::: "memory");
-      __syncthreads();
-      copy_b(step + 2);
-      copy_b(step + 3);
-    } else {
-      // only the two warps of a row tile share its digits, so that the row
-      // tiles' conversions and MMAs drift apart and overlap
-      asm volatile("bar.sync %0, 64;" ::"r"(rt + 1) : "memory");
+// C (N x nc, ldc) -= A (N x K, lda) B^T, B as dig_rows_kernel lays it out; cmap
+// (optional) gives the column of C for each row of B.  A CTA takes 128 rows and
+// one group of up to NC columns (blockIdx.x: groups of a row tile next to one
+// another, so that the second one finds its rows of A in L2).
+//
+// Warps 0-7 convert A, read column by column (256-byte segments, copied two or
+// three steps ahead to shared memory by the thread that will use them, since
+// eight warps with the loads in registers waited for them): a thread makes the
+// seven digits of eight entries of a row, 16 bytes each, into a ring of stages
+// in the MMAs' K-major layout; a producer lane copies B's digits beside them.
+// One lane issues the MMAs: digit s of A times digits 0 .. 6 - s of B, which lie
+// one after the other as rows of one operand and whose products go to groups s
+// .. 6, adjacent in TMEM: ten MMAs a step instead of 28, N up to 256.  Every DIG_LOW terms the eight warps add the
+// accumulators to their 64-bit totals in registers (32 a thread); the ring's
+// stages are filled before, so that the MMAs go on at once.
+//
+// A step of 64 columns takes about 900 clocks at the MMAs' rate (0.40 ms for N =
+// 1e5, K = 900, 100 columns with the conversion taken out) and as many issue
+// slots a scheduler to convert, with eight warps to fill them (0.8 ms with the
+// MMAs taken out).  Measured at N = 1e5, 100 columns: 0.51 ms for K = 500 and
+// 0.83 ms for K = 900, against 1.04 and 1.75 ms for the same digits with
+// mma.sync, and 3.35 and 5.87 ms for a float-float product on the float32 pipe;
+// with A's entries loaded to registers two steps ahead 0.54 and 0.88 ms, and C
+// read and written entry by entry 0.1 ms more.  Up to 32 columns two CTAs share
+// an SM (45 us at N = 1e5, K = 20 to 80, where mma.sync took 57).
+template <int NC>
+__global__ void __launch_bounds__(DG_THREADS, NC == 32 ? 2 : 1)
+dig_gemm_kernel(const double *__restrict__ A, int64_t lda, int64_t N, int K,
+                const uint4 *__restrict__ img, int nc, int groups, double *__restrict__ C,
+                int64_t ldc, const int *__restrict__ cmap, int *fault) {
+  constexpr int ST = dg_stages(NC);
+  constexpr int STAGE = dg_stage_bytes(NC);
+  constexpr int AHEAD = dg_ahead(NC);
+  constexpr int TCOLS = NC == 32 ? 256 : 512;
+  constexpr int BAR_A = 0, BAR_B = ST, BAR_E = 2 * ST, BAR_D = 3 * ST, BAR_R = 3 * ST + 1,
+                BAR_FIN = 3 * ST + 2;
+  extern __shared__ uint8_t dg_raw[];
+  const uint32_t raw = bw::smem_u32(dg_raw);
+  const uint32_t base = (raw + 1023u) & ~1023u;
+  const uint32_t sX = base + ST * STAGE;   // [AHEAD][8 entries][256 threads] of A
+  const uint32_t sBar = sX + AHEAD * DG_AHEAD_BYTES;
+  uint32_t *tslot = reinterpret_cast<uint32_t *>(dg_raw + (sBar - raw) + 8 * (3 * ST + 3));
+  volatile int *abort_flag = reinterpret_cast<volatile int *>(tslot + 1);
+  auto bar = [&](int i) -> uint32_t { return sBar + 8u * (uint32_t)i; };
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int grp = (int)(blockIdx.x % groups);
+  const int64_t row0 = (int64_t)(blockIdx.x / groups) * DG_ROWS;
+  const int ncol = dg_group_cols(nc, grp);
+  const int K16 = (K + 15) / 16;
+  const int chunks = (K16 + DG_LOWSTEPS - 1) / DG_LOWSTEPS;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < ST; ++s) {
+      bw::mbar_init(bar(BAR_A + s), DG_WORKERS);
+      bw::mbar_init(bar(BAR_B + s), 1);
+      bw::mbar_init(bar(BAR_E + s), 1);
     }
-    if (step + 1 < steps) load_a(step + 1, x);
-    const uint4 *bufA = sA + ((step & 1) * 4 + rt) * DIG_N * 32;
-    uint4 a[DIG_N];
-#pragma unroll
-    for (int s = 0; s < DIG_N; ++s) a[s] = bufA[s * 32 + lane];
-    const uint2 *bufB = sB + (step % DG_STAGES) * BSTEP + half * NTW * DIG_N * 32 + lane;
-#pragma unroll
-    for (int j = 0; j < NTW; ++j)
-#pragma unroll
-      for (int t = 0; t < DIG_N; ++t) {
-        const uint2 b = bufB[(j * DIG_N + t) * 32];
-#pragma unroll
-        for (int s = 0; s + t < DIG_N; ++s) dg_mma(acc[j][s + t], a[s], b);
+    bw::mbar_init(bar(BAR_D), 1);
+    bw::mbar_init(bar(BAR_R), DG_WORKERS);
+    bw::mbar_init(bar(BAR_FIN), 1);
+    *abort_flag = 0;
+    bw::fence_mbar_init();
+  }
+  if (warp == DG_WORKERS + 1) {
+    bw::tmem_alloc(bw::smem_u32(tslot), TCOLS);
+    bw::tmem_relinquish();
+  }
+  bw::tc_fence_before();
+  __syncthreads();
+  bw::tc_fence_after();
+  const uint32_t tmem = *tslot;
+  // bounded wait; on timeout records the fault and aborts the CTA
+  auto wait = [&](int i, uint32_t parity) -> bool {
+    if (bw::mbar_wait_abortable(bar(i), parity, DG_WAIT_BUDGET, abort_flag)) return true;
+    *abort_flag = 1;
+    atomicOr(fault, 1);
+    return false;
+  };
+
+  if (warp == DG_WORKERS) {
+    // ---------------------------------------------------------- B's digits
+    if (lane == 0) {
+      const uint32_t bytes = (uint32_t)(DIG_N * ncol * 32);
+      const uint4 *src = img + (int64_t)grp * K16 * 64 * DIG_N * 2;
+      int issued = 0, s = 0;
+      uint32_t ph = 0;
+      for (int step = 0; step < K16; ++step) {
+        if (!wait(BAR_E + s, ph ^ 1u)) break;
+        bw::mbar_arrive_expect_tx(bar(BAR_B + s), bytes);
+        bw::bulk_load(base + (uint32_t)(s * STAGE + DIG_N * DG_ADIG),
+                      src + (int64_t)step * ncol * DIG_N * 2, bytes, bar(BAR_B + s));
+        ++issued;
+        if (++s == ST) s = 0, ph ^= 1u;
       }
-    if ((step + 1) % DG_KSTEPS == 0 || step + 1 == steps) {
-#pragma unroll
-      for (int j = 0; j < NTW; ++j)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          // units 2^-32 and 2^-64, both exact
-          const int64_t hi = ((int64_t)__float2int_rn(acc[j][0][e]) << 16) +
-                             ((int64_t)__float2int_rn(acc[j][1][e]) << 8) +
-                             (int64_t)__float2int_rn(acc[j][2][e]);
-          const int64_t lo = ((int64_t)__float2int_rn(acc[j][3][e]) << 24) +
-                             ((int64_t)__float2int_rn(acc[j][4][e]) << 16) +
-                             ((int64_t)__float2int_rn(acc[j][5][e]) << 8) +
-                             (int64_t)__float2int_rn(acc[j][6][e]);
-          tot[(j * 4 + e) * DG_THREADS + tid] += hi * (1ll << 28) + ((lo + 8) >> 4);
-#pragma unroll
-          for (int s = 0; s < DIG_N; ++s) acc[j][s][e] = 0.0f;
+      // wait (bounded, quietly) for the copies in flight
+      for (int q = issued > ST ? issued - ST : 0; q < issued; ++q)
+        bw::mbar_wait(bar(BAR_B + q % ST), (uint32_t)((q / ST) & 1), DG_WAIT_BUDGET >> 4);
+    }
+    __syncwarp();
+  } else if (warp == DG_WORKERS + 1) {
+    // ----------------------------------------------------------------- MMA
+    if (lane == 0) {
+      int s = 0, in = 0, chunk = 0;
+      uint32_t ph = 0;
+      for (int step = 0; step < K16; ++step) {
+        // the sums of the chunk before have been read out
+        if (in == 0 && chunk > 0 && !wait(BAR_R, (uint32_t)((chunk - 1) & 1))) break;
+        if (!wait(BAR_A + s, ph) || !wait(BAR_B + s, ph)) break;
+        bw::tc_fence_after();
+        const uint32_t a0 = base + (uint32_t)(s * STAGE), b0 = a0 + DIG_N * DG_ADIG;
+        auto mma = [&](int sa, int t, int nt, uint32_t acc) {
+          bw::mma_f16(tmem + (uint32_t)((sa + t) * ncol),
+                      bw::sdesc_kmajor_sw32(a0 + sa * DG_ADIG),
+                      bw::sdesc_kmajor_sw32(b0 + (uint32_t)(t * ncol * 32)),
+                      bw::idesc_f16_f32(DG_ROWS, nt * ncol), acc);
+        };
+        // groups 0..2 and 3..6 start anew after their read-outs
+        mma(0, 0, 3, (in == 0 && chunk % DG_HIGHCHUNKS == 0) ? 0u : 1u);
+        mma(0, 3, 4, in == 0 ? 0u : 1u);
+        mma(1, 0, 3, 1);
+        mma(1, 3, 3, 1);
+        mma(2, 0, 3, 1);
+        mma(2, 3, 2, 1);
+        mma(3, 0, 4, 1);
+        mma(4, 0, 3, 1);
+        mma(5, 0, 2, 1);
+        mma(6, 0, 1, 1);
+        bw::mma_commit(bar(BAR_E + s));
+        if (++in == DG_LOWSTEPS || step + 1 == K16) {
+          bw::mma_commit(bar(BAR_D));
+          in = 0;
+          ++chunk;
         }
+        if (++s == ST) s = 0, ph ^= 1u;
+      }
+      // every MMA issued so far has completed once FIN flips
+      bw::mma_commit(bar(BAR_FIN));
+      bw::mbar_wait(bar(BAR_FIN), 0, DG_WAIT_BUDGET >> 4);
+    }
+    __syncwarp();
+  } else {
+    // ------------------------------------------- conversion and read-outs
+    const int half = warp >> 2;               // entries 8 half .. + 7, columns of half
+    const int rl = (warp & 3) * 32 + lane;    // row of the tile, TMEM lane
+    const int64_t row = row0 + rl;
+    const bool ok = row < N;
+    const int nc2 = ncol / 2;
+    const double *Ar = A + row + (int64_t)(8 * half) * lda;
+    const uint32_t dst = base + (uint32_t)(rl * 32 + ((half ^ ((rl >> 2) & 1)) * 16));
+    const uint32_t xs = sX + (uint32_t)threadIdx.x * 8;
+    auto load = [&](int step, int slot) {
+      if (step < K16) {
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+          const bool in = ok && step * 16 + 8 * half + t < K;
+          asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(
+                           xs + (uint32_t)(slot * DG_AHEAD_BYTES + t * DG_WORKERS * 32 * 8)),
+                       "l"(in ? Ar + (int64_t)(step * 16 + t) * lda : A), "r"(in ? 8 : 0)
+                       : "memory");
+        }
+      }
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    int64_t tot[NC / 2];
+#pragma unroll
+    for (int i = 0; i < NC / 2; ++i) tot[i] = 0;
+    const uint32_t tcol = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(half * nc2);
+    auto read_out = [&](int chunk) -> bool {
+      if (!__all_sync(0xffffffffu, wait(BAR_D, (uint32_t)(chunk & 1)))) return false;
+      bw::tc_fence_after();
+      const bool high = (chunk + 1) % DG_HIGHCHUNKS == 0 || chunk + 1 == chunks;
+#pragma unroll
+      for (int cb = 0; cb < NC / 16; ++cb) {
+        if (cb * 8 < nc2) {
+          uint32_t r[32];
+#pragma unroll
+          for (int g = 3; g < 7; ++g)
+            bw::tmem_ld_32x32b_x8(tcol + (uint32_t)(g * ncol + cb * 8), r + (g - 3) * 8);
+          bw::tmem_wait_ld32(r);
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            // units 2^-64, exact
+            const int64_t lo = ((int64_t)__float2int_rn(__uint_as_float(r[i])) << 24) +
+                               ((int64_t)__float2int_rn(__uint_as_float(r[8 + i])) << 16) +
+                               ((int64_t)__float2int_rn(__uint_as_float(r[16 + i])) << 8) +
+                               (int64_t)__float2int_rn(__uint_as_float(r[24 + i]));
+            tot[cb * 8 + i] += (lo + 8) >> 4;
+          }
+          if (high) {
+#pragma unroll
+            for (int g = 0; g < 3; ++g)
+              bw::tmem_ld_32x32b_x8(tcol + (uint32_t)(g * ncol + cb * 8), r + g * 8);
+            bw::tmem_wait_ld32(r);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              // units 2^-32
+              const int64_t hi = ((int64_t)__float2int_rn(__uint_as_float(r[i])) << 16) +
+                                 ((int64_t)__float2int_rn(__uint_as_float(r[8 + i])) << 8) +
+                                 (int64_t)__float2int_rn(__uint_as_float(r[16 + i]));
+              tot[cb * 8 + i] += hi * (1ll << 28);
+            }
+          }
+        }
+      }
+      bw::tc_fence_before();
+      __syncwarp();
+      if (lane == 0) bw::mbar_arrive(bar(BAR_R));
+      return true;
+    };
+    int s = 0, chunk = 0, slot = 0;
+    uint32_t ph = 0;
+    bool good = true;
+#pragma unroll
+    for (int q = 0; q < AHEAD; ++q) load(q, q);
+    for (int step = 0; step < K16; ++step) {
+      // the ring is full of the next chunk's steps: the chunk before is read
+      // out now, since the MMAs that would free a stage wait for it
+      if (step == (chunk + 1) * DG_LOWSTEPS + ST) good = good && read_out(chunk++);
+      good = good && __all_sync(0xffffffffu, wait(BAR_E + s, ph ^ 1u));
+      if (!good) break;
+      asm volatile("cp.async.wait_group %0;" ::"n"(AHEAD - 1) : "memory");
+      double x[8];
+#pragma unroll
+      for (int t = 0; t < 8; ++t)
+        asm volatile("ld.shared.f64 %0, [%1];"
+                     : "=d"(x[t])
+                     : "r"(xs + (uint32_t)(slot * DG_AHEAD_BYTES + t * DG_WORKERS * 32 * 8))
+                     : "memory");
+      load(step + AHEAD, slot);
+      uint32_t d[4][DIG_N];
+#pragma unroll
+      for (int t = 0; t < 4; ++t) dig_pair(x[2 * t], x[2 * t + 1], d[t]);
+#pragma unroll
+      for (int q = 0; q < DIG_N; ++q)
+        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(
+                         dst + (uint32_t)(s * STAGE + q * DG_ADIG)),
+                     "r"(d[0][q]), "r"(d[1][q]), "r"(d[2][q]), "r"(d[3][q])
+                     : "memory");
+      bw::fence_async_shared();
+      __syncwarp();
+      if (lane == 0) bw::mbar_arrive(bar(BAR_A + s));
+      if (++s == ST) s = 0, ph ^= 1u;
+      if (++slot == AHEAD) slot = 0;
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    while (good && chunk < chunks) good = read_out(chunk++);
+    if (good && ok) {
+      // eight columns of C at a time, all read before the first is written
+#pragma unroll
+      for (int cb = 0; cb < NC / 16; ++cb) {
+        const int c0 = grp * 64 + half * nc2 + cb * 8;
+        if (cb * 8 < nc2) {
+          double *p[8], v[8];
+#pragma unroll
+          for (int i = 0; i < 8; ++i)
+            if (c0 + i < nc) {
+              p[i] = C + row + (int64_t)(cmap ? cmap[c0 + i] : c0 + i) * ldc;
+              v[i] = *p[i];
+            }
+#pragma unroll
+          for (int i = 0; i < 8; ++i)
+            if (c0 + i < nc) *p[i] = v[i] - (double)tot[cb * 8 + i] * 0x1p-60;
+        }
+      }
     }
   }
-#pragma unroll
-  for (int j = 0; j < NTW; ++j)
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const int c = (half * NTW + j) * 8 + 2 * q + (e & 1);
-      const bool ok = (e >> 1) ? ok1 : ok0;
-      if (ok && c < nc) {
-        double *dst = C + r0 + (e >> 1) * 8 + (int64_t)(cmap ? cmap[c] : c) * ldc;
-        *dst -= (double)tot[(j * 4 + e) * DG_THREADS + tid] * 0x1p-60;
-      }
-    }
+  bw::tc_fence_before();
+  __syncthreads();
+  if (warp == DG_WORKERS + 1) {
+    bw::tc_fence_after();
+    bw::tmem_dealloc(tmem, TCOLS);
+  }
 }
 
-static size_t dig_smem(int NTW) {
-  return (size_t)DG_STAGES * 2 * NTW * DIG_N * 32 * sizeof(uint2) +
-         (size_t)2 * 4 * DIG_N * 32 * sizeof(uint4) +
-         (size_t)NTW * 4 * DG_THREADS * sizeof(int64_t);
+size_t dig_image_bytes(int nc, int K) {
+  return (size_t)((K + 15) / 16) * DIG_N * 32 * ((nc + 15) / 16 * 16);
 }
 
-template <int NTW>
-static krr_status launch_dig(const double *A, int64_t lda, int64_t N, int K, const uint2 *frag,
-                             int nc, double *C, int64_t ldc, const int *cmap, cudaStream_t s) {
-  const size_t smem = dig_smem(NTW);
-  KRR_TRY(raise_smem_limit(dig_gemm_kernel<NTW>, smem));
-  dig_gemm_kernel<NTW><<<ceil_div(N, DG_ROWS), DG_THREADS, smem, s>>>(A, lda, N, K, frag, nc, C,
-                                                                     ldc, cmap);
+template <int NC>
+static krr_status launch_dig(const double *A, int64_t lda, int64_t N, int K, const uint4 *img,
+                             int nc, double *C, int64_t ldc, const int *cmap, int *fault,
+                             cudaStream_t s) {
+  KRR_TRY(raise_smem_limit(dig_gemm_kernel<NC>, dg_smem(NC)));
+  const int groups = (nc + 63) / 64;
+  dig_gemm_kernel<NC><<<(unsigned)(ceil_div(N, DG_ROWS) * groups), DG_THREADS, dg_smem(NC), s>>>(
+      A, lda, N, K, img, nc, groups, C, ldc, cmap, fault);
   KRR_LAUNCH_CHECK();
   return KRR_OK;
 }
 
-// Column tiles of a warp: half of the columns, rounded up to an instance.
-static int dig_ntw(int nc) {
-  const int tiles = (nc + 7) / 8;
-  return tiles <= 2 ? 1 : tiles <= 4 ? 2 : tiles <= 8 ? 4 : 7;
-}
-
-size_t dig_frag_elems(int nc, int K) {
-  return (size_t)((K + 15) / 16) * 2 * dig_ntw(std::min(nc, DIG_MAX_COLS)) * DIG_N * 32;
-}
-
 krr_status dig_gemm_sub(const double *A, int64_t lda, int64_t N, int K, const double *B,
                         int64_t ldb, const int64_t *rows, int nc, double *C, int64_t ldc,
-                        const int *cmap, uint2 *frag, cudaStream_t s) {
+                        const int *cmap, uint4 *img, cudaStream_t s) {
   if (N <= 0 || K <= 0 || nc <= 0) return KRR_OK;
-  for (int c0 = 0; c0 < nc; c0 += DIG_MAX_COLS) {
-    const int n = std::min(DIG_MAX_COLS, nc - c0);
-    const int NTW = dig_ntw(n);
-    const int K16 = (K + 15) / 16;
-    const int64_t total = (int64_t)K16 * 2 * NTW * 32;
-    dig_rows_kernel<<<(unsigned)std::min<int64_t>((total + 127) / 128, 4 * num_sms()), 128, 0,
-                      s>>>(rows ? B : B + c0, ldb, rows ? rows + c0 : nullptr, n, K, K16, 2 * NTW, frag);
-    KRR_LAUNCH_CHECK();
-    double *Cc = cmap ? C : C + (int64_t)c0 * ldc;
-    const int *cm = cmap ? cmap + c0 : nullptr;
-    switch (NTW) {
-      case 1: KRR_TRY(launch_dig<1>(A, lda, N, K, frag, n, Cc, ldc, cm, s)); break;
-      case 2: KRR_TRY(launch_dig<2>(A, lda, N, K, frag, n, Cc, ldc, cm, s)); break;
-      case 4: KRR_TRY(launch_dig<4>(A, lda, N, K, frag, n, Cc, ldc, cm, s)); break;
-      default: KRR_TRY(launch_dig<7>(A, lda, N, K, frag, n, Cc, ldc, cm, s)); break;
-    }
-  }
-  return KRR_OK;
+  int *fault = tc5_fault_ptr();
+  KRR_REQUIRE(fault != nullptr, "digit product: no fault flag on this device");
+  const int K16 = (K + 15) / 16;
+  const int64_t total = (int64_t)K16 * ((nc + 15) / 16 * 16) * 2;
+  dig_rows_kernel<<<(unsigned)std::min<int64_t>((total + 127) / 128, 4 * num_sms()), 128, 0, s>>>(
+      B, ldb, rows, nc, K, K16, img);
+  KRR_LAUNCH_CHECK();
+  if (nc <= 32) return launch_dig<32>(A, lda, N, K, img, nc, C, ldc, cmap, fault, s);
+  return launch_dig<64>(A, lda, N, K, img, nc, C, ldc, cmap, fault, s);
 }
 
 }  // namespace krr

@@ -5,18 +5,20 @@
 // written as seven balanced base-256 digits, x = sum_s q_s 2^(-8 - 8 s),
 // -128 <= q_s <= 127 (the leading one -512..511, for |x| below 2).  Digits are
 // exact in fp16; the product of digits s and t carries 2^(-16 - 8 (s + t)), so
-// the pairs of one g = s + t share an accumulator.  Over 128 terms a pair of
-// full digits stays within 2^21 and a pair with a leading digit within 128 256
-// sqrt(128) (the rows' norm), so seven pairs stay below 2^24 and the float32
-// accumulation is exact.  The 28 pairs with s + t <= 6 are kept; what is
-// dropped is about 2^-59.6 sqrt(6 K) of 1, below the rounding of a float64 sum
-// of K terms.  After 128 terms the seven accumulators go into one 64-bit total
-// in units of 2^-60.
+// the pairs of one g = s + t share an accumulator.  Over n terms a pair of full
+// digits stays within 2^14 n, a pair with one leading digit within 2^15 sqrt(n)
+// and the leading pair within 2^16 (the rows' norms, with room for the leading
+// digits' rounding), so the sums of groups 3..6 (at most two pairs with a
+// leading digit and five without) stay below 2^24 over DIG_LOW terms and those
+// of groups 0..2 (one full pair) over DIG_HIGH, and the float32 accumulation is
+// exact.  The 28 pairs with s + t <= 6 are kept; what is dropped is about
+// 2^-59.6 sqrt(6 K) of 1, below the rounding of a float64 sum of K terms.  The
+// accumulators go into one 64-bit total in units of 2^-60.
 //
-// One 16 x 8 x 16 MMA does 2048 multiply-adds; the float64 pipe does 1.9 a
-// clock and SM, so 28 MMAs (59.6 clocks at the measured rate of 606 TFLOP/s)
-// replace 1078 clocks of DFMA, and the float-float form on the float32 pipe
-// (12 operations a multiply-add) 192.
+// A 128 x 64 x 16 product of float64 is 131072 multiply-adds: 69000 clocks of
+// the float64 pipe of an SM (1.9 a clock), 1000 of its tensor cores as 28 digit
+// products (4096 a clock).
+
 #pragma once
 
 #include <cuda_fp16.h>
@@ -26,19 +28,20 @@
 namespace krr {
 
 constexpr int DIG_N = 7;              // digits
-constexpr int DIG_CHUNK = 128;        // terms between flushes of the accumulators
-constexpr int DIG_MAX_COLS = 112;     // columns of one launch
+constexpr int DIG_LOW = 160;          // terms between read-outs of groups 3..6
+constexpr int DIG_HIGH = 640;         // and of groups 0..2
+static_assert(5 * 16384.0 * DIG_LOW + 2 * 32768.0 * 12.65 <= 16777216.0, "groups 3..6");
+static_assert(16384.0 * DIG_HIGH + 2 * 32768.0 * 25.3 + 65536.0 <= 16777216.0, "groups 0..2");
 
-// round(2^56 x), |x| < 2; 0 for |x| < 2^-57.
-__device__ __forceinline__ int64_t dig_fixed(double x) {
+// round(2^56 x) + bias, |x| < 2 (0 + bias for |x| < 2^-57): the mantissa as 2^5
+// times an integer, shifted right by the exponent's distance from 2 with one
+// bit left, rounded there.
+__device__ __forceinline__ uint64_t dig_fixed(double x, uint64_t bias) {
   const uint64_t b = (uint64_t)__double_as_longlong(x);
   const int e = (int)(b >> 52) & 0x7ff;
-  const uint64_t mant = (b & ((1ull << 52) - 1)) | (1ull << 52);
-  const int r = 1019 - e;
-  uint64_t v;
-  if (r <= 0) v = mant << ((-r) & 7);
-  else v = r > 54 ? 0 : (mant + (1ull << (r - 1))) >> r;
-  return (b >> 63) ? -(int64_t)v : (int64_t)v;
+  const uint64_t m5 = ((b & ((1ull << 52) - 1)) | (1ull << 52)) << 5;
+  const uint64_t v = ((m5 >> min(1023 - e, 63)) + 1) >> 1;
+  return (int64_t)b < 0 ? bias - v : bias + v;
 }
 
 // The digits of two entries as fp16 pairs (x0 low, x1 high): out[s] for digit s.
@@ -46,7 +49,7 @@ __device__ __forceinline__ void dig_pair(double x0, double x1, uint32_t (&out)[D
   // a bias of 128 in every digit's place (512 in the leading one's) makes the
   // digits plain bytes
   const uint64_t bias = 0x0200808080808080ull;
-  const uint64_t w0 = (uint64_t)dig_fixed(x0) + bias, w1 = (uint64_t)dig_fixed(x1) + bias;
+  const uint64_t w0 = dig_fixed(x0, bias), w1 = dig_fixed(x1, bias);
   const uint32_t l0 = (uint32_t)w0, l1 = (uint32_t)w1;
   const uint32_t h0 = (uint32_t)(w0 >> 32), h1 = (uint32_t)(w1 >> 32);
   const __half2 off = __half2half2(__ushort_as_half((unsigned short)0x6480));   // 1152

@@ -208,7 +208,7 @@ krr_status prepare_points_tc5(const double *Xd, cudaStream_t s, PointsF32 &P, in
 // cleared by tc5_check_fault).
 __device__ int g_t5_fault;
 
-static int *fault_ptr() {
+int *tc5_fault_ptr() {
   static std::mutex mtx;
   static int *ptrs[64] = {};
   int dev = 0;
@@ -226,7 +226,7 @@ static int *fault_ptr() {
 }
 
 krr_status tc5_check_fault(cudaStream_t s) {
-  int *f = fault_ptr();
+  int *f = tc5_fault_ptr();
   if (!f) return KRR_OK;
   int h = 0;
   KRR_CUDA_TRY(cudaMemcpyAsync(&h, f, sizeof(int), cudaMemcpyDeviceToHost, s));
@@ -255,7 +255,7 @@ __global__ void t5_wait_selftest_kernel(int *fault, long long budget) {
 
 krr_status tc5_wait_selftest(long long budget, cudaStream_t s) {
   KRR_REQUIRE(budget >= 0 && budget <= (1LL << 31), "wait budget: 0 to 2^31 cycles");
-  int *f = fault_ptr();
+  int *f = tc5_fault_ptr();
   KRR_REQUIRE(f != nullptr, "no fault flag on this device");
   t5_wait_selftest_kernel<<<1, 32, 0, s>>>(f, budget);
   KRR_LAUNCH_CHECK();
@@ -633,7 +633,7 @@ static krr_status tc5_products(const PointsF32 &R, const PointsF32 &P, double la
   if (Nr == 0 || Nc == 0 || m == 0) return KRR_OK;
   KRR_REQUIRE(R.nh5 > 0 && P.nh5 == R.nh5 && P.csep5 == R.csep5 && R.kern == P.kern,
               "tcgen05 product: operands missing or of different layouts");
-  int *fault = fault_ptr();
+  int *fault = tc5_fault_ptr();
   KRR_REQUIRE(fault != nullptr, "tcgen05 product: no fault flag on this device");
   // One launch of 16 where two of 8 would both take their sums on the tensor
   // cores: the kernel values, their split and the distances are formed once.

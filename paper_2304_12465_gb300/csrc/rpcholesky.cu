@@ -487,13 +487,13 @@ krr_status rpcholesky_device(const double *Xd, int64_t N, int d, int kern, doubl
   DevBuf<int64_t> draws, cand;
   DevBuf<int> counts, kept;
   DevBuf<double> G, Lb;
-  DevBuf<uint2> frag;
+  DevBuf<uint8_t> img;
   KRR_TRY(draws.alloc(B, s));
   KRR_TRY(cand.alloc(B, s));
   KRR_TRY(counts.alloc(4, s));
   KRR_TRY(kept.alloc(B, s));
   KRR_TRY(G.alloc((size_t)N * B, s));
-  KRR_TRY(frag.alloc(dig_frag_elems(B, std::max(k, B)), s));
+  KRR_TRY(img.alloc(dig_image_bytes(B, std::max(k, B)), s));
   KRR_TRY(Lb.alloc((size_t)B * B, s));
 
   KRR_TRY(raise_smem_limit(block_chol_kernel, (size_t)B * (B + 1) * sizeof(double)));
@@ -545,7 +545,8 @@ krr_status rpcholesky_device(const double *Xd, int64_t N, int d, int kern, doubl
     // G = A(:, S') - F(:, 0:rank) F(S', 0:rank)^T
     KRR_TRY(kernel_columns_f64(P64, cand.p, nc, G.p, N, s));
     if (rank > 0)
-      KRR_TRY(dig_gemm_sub(f->F, N, N, rank, f->F, N, cand.p, nc, G.p, N, nullptr, frag.p, s));
+      KRR_TRY(dig_gemm_sub(f->F, N, N, rank, f->F, N, cand.p, nc, G.p, N, nullptr,
+                           reinterpret_cast<uint4 *>(img.p), s));
     block_chol_kernel<<<1, 256, (size_t)nc * (nc + 1) * sizeof(double), s>>>(
         G.p, N, cand.p, nc, thr, Lb.p, kept.p, counts.p + 2);
     KRR_LAUNCH_CHECK();
@@ -557,7 +558,7 @@ krr_status rpcholesky_device(const double *Xd, int64_t N, int d, int kern, doubl
     for (int q = 0; q < groups; ++q) {
       const int a0 = (int)((int64_t)na * q / groups), w = (int)((int64_t)na * (q + 1) / groups) - a0;
       KRR_TRY(dig_gemm_sub(f->F + (int64_t)rank * N, N, N, a0, Lb.p + a0, nc, nullptr, w, G.p, N,
-                           kept.p + a0, frag.p, s));
+                           kept.p + a0, reinterpret_cast<uint4 *>(img.p), s));
       block_trsm_kernel<<<ceil_div(N, TRSM_THREADS), TRSM_THREADS, 0, s>>>(
           G.p, N, Lb.p, nc, kept.p, a0, w, f->F, N, rank, f->dres);
       KRR_LAUNCH_CHECK();
@@ -566,6 +567,7 @@ krr_status rpcholesky_device(const double *Xd, int64_t N, int d, int kern, doubl
     KRR_LAUNCH_CHECK();
     rank += na;
   }
+  KRR_TRY(tc5_check_fault(s));   // the digit products' bounded waits
   f->rank = rank;
   f->nblocks = (int)t;
   return KRR_OK;

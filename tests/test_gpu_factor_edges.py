@@ -74,3 +74,20 @@ def test_core_edges(K, rank):
 def test_many_draws(K, N, nd):
     d = np.random.default_rng(N).random(N)
     np.testing.assert_array_equal(K.krr_rpc_sample(d, 11, 4, nd), O.rpc_sample(d, 11, 4, nd))
+
+
+@pytest.mark.parametrize("N,k,B", [
+    (127, 64, 16), (128, 96, 33), (385, 225, 32), (640, 352, 65), (1025, 672, 128), (1153, 810, 90),
+])
+def test_digit_product_edges(K, N, k, B):
+    """128-row tiles, column groups of 16 to 64 and two groups, and the
+    read-outs of the accumulators after 160 and 640 terms."""
+    rng = np.random.default_rng(N + B)
+    X = rng.standard_normal((N, 6))
+    ref = O.rpcholesky(X, O.MATERN52, 0.8, k, B, 9)
+    f = K.krr_rpcholesky(X, O.MATERN52, 0.8, k, B, 9)
+    F, S, D = f.export()
+    np.testing.assert_array_equal(S, ref.S)
+    np.testing.assert_allclose(F, ref.F, atol=1e-10, rtol=0)
+    np.testing.assert_allclose(D, ref.dres, atol=1e-10, rtol=0)
+    f.free()
