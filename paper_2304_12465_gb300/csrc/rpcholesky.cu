@@ -296,11 +296,13 @@ __device__ __forceinline__ double div_by(double x, double d, double r) {
 // candidate whose current Schur value is <= thr is dropped and does not
 // update the rest.  Outputs the factor of the kept candidates Lb (ld nc,
 // column-major, lower, in their order), their positions, and their count.
-// Panels of eight columns are factored by one warp in registers (a lane keeps
-// every 32nd row; rows meet by shuffles, without barriers), the rest is
-// updated by all warps between two barriers: 100 candidates took 262 us with
-// three barriers a column, now about 75 us, of which the 1.7e5 DFMA at 1.9 a
-// clock on one SM are 43.
+// Panels of eight columns are factored in registers by up to four warps, one
+// for each float64 pipe of the SM: a lane keeps one row below the panel's
+// diagonal block, and every warp the block itself, so that they need no
+// barriers; the rest is updated by all warps between two barriers.  100
+// candidates took 262 us with three barriers a column, 231 us with the panel in
+// one warp, whose 272 float64 instructions a panel take 67 clocks each, now
+// 187.
 constexpr int CHOL_PW = 8;
 __global__ void __launch_bounds__(256)
 block_chol_kernel(const double *__restrict__ G, int64_t ldg, const int64_t *__restrict__ cand,
@@ -320,43 +322,42 @@ block_chol_kernel(const double *__restrict__ G, int64_t ldg, const int64_t *__re
   __syncthreads();
   for (int c0 = 0; c0 < nc; c0 += CHOL_PW) {
     const int pw = min(CHOL_PW, nc - c0);
-    if (warp == 0) {
-      // row c0 + lane + 32 r, columns c0 .. c0 + pw
-      double P[4][CHOL_PW];
+    double top[CHOL_PW];   // warp 0: the diagonal block, stored once every warp has read it
+    const int a = c0 + CHOL_PW + 32 * warp + lane;   // this lane's row below the diagonal block
+    if (warp == 0 || (warp < 4 && c0 + CHOL_PW + 32 * warp < nc)) {
+      // rows c0 .. c0 + 7 in lanes 0..7 of every warp (T), rows below (P);
+      // columns c0 .. c0 + pw
+      double T[CHOL_PW], P[CHOL_PW];
 #pragma unroll
-      for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int q = 0; q < CHOL_PW; ++q) {
-          const int a = c0 + lane + 32 * r;
-          P[r][q] = (a < nc && q < pw) ? sT[a * ld + c0 + q] : 0.0;
-        }
+      for (int q = 0; q < CHOL_PW; ++q) {
+        T[q] = (lane < pw && q < pw) ? sT[(c0 + lane) * ld + c0 + q] : 0.0;
+        P[q] = (a < nc && q < pw) ? sT[a * ld + c0 + q] : 0.0;
+      }
       unsigned mask = 0;
 #pragma unroll
       for (int q = 0; q < CHOL_PW; ++q) {
-        const double p = __shfl_sync(0xffffffffu, P[0][q], q);
+        const double p = __shfl_sync(0xffffffffu, T[q], q);
         if (q < pw && p > thr) {
           mask |= 1u << q;
           double d, rd;
           sqrt_and_inverse(p, &d, &rd);
-#pragma unroll
-          for (int r = 0; r < 4; ++r) P[r][q] = div_by(P[r][q], d, rd);
-          if (lane == q) P[0][q] = d;
+          T[q] = div_by(T[q], d, rd);
+          P[q] = div_by(P[q], d, rd);
+          if (lane == q) T[q] = d;
 #pragma unroll
           for (int u = q + 1; u < CHOL_PW; ++u) {
-            const double l = __shfl_sync(0xffffffffu, P[0][q], u);
-#pragma unroll
-            for (int r = 0; r < 4; ++r) P[r][u] = fma(-P[r][q], l, P[r][u]);
+            const double l = __shfl_sync(0xffffffffu, T[q], u);
+            T[u] = fma(-T[q], l, T[u]);
+            P[u] = fma(-P[q], l, P[u]);
           }
         }
       }
 #pragma unroll
-      for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int q = 0; q < CHOL_PW; ++q) {
-          const int a = c0 + lane + 32 * r;
-          if (a < nc && q < pw) sT[a * ld + c0 + q] = P[r][q];
-        }
-      if (lane == 0) {
+      for (int q = 0; q < CHOL_PW; ++q) {
+        if (a < nc && q < pw) sT[a * ld + c0 + q] = P[q];
+        top[q] = T[q];
+      }
+      if (tid == 0) {
         s_mask = mask;
         int na = s_na;
         for (int q = 0; q < pw; ++q)
@@ -365,6 +366,11 @@ block_chol_kernel(const double *__restrict__ G, int64_t ldg, const int64_t *__re
       }
     }
     __syncthreads();
+    if (warp == 0 && lane < pw) {
+#pragma unroll
+      for (int q = 0; q < CHOL_PW; ++q)
+        if (q < pw) sT[(c0 + lane) * ld + c0 + q] = top[q];
+    }
     const unsigned mask = s_mask;
     const int t0 = c0 + pw;
     // 16 x 16 threads over the lower triangle that is left
