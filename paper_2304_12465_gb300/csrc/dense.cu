@@ -7,58 +7,62 @@
 
 namespace krr {
 
-constexpr int GB_M = 64, GB_N = 64, GB_K = 16, G_THREADS = 256;
-
 // ------------------------------------------------------------ Gram (F^T F)
-// Lower-triangular output tiles only.  float input: each K tile of GB_K
-// products is summed in float32, then added to a float-float accumulator
-// (Knuth's TwoSum, the rounding errors gathered in a float32 correction that
-// is folded back every 8 tiles) -- float64 adds, at a small fraction of the
-// float32 rate on this GPU, bounded the kernel; double input: float64
-// throughout.
-template <typename T>
+// Lower-triangular output tiles only; the terms go in chunks of GB_K through
+// shared memory, the next chunk's on their way to registers meanwhile.
+constexpr int GB_K = 16, G_THREADS = 256;
+constexpr int GD_T = 64;               // float64: 64 x 64 tiles
+constexpr int GF_M = 128, GF_N = 64;   // float32: 128 x 64 tiles,
+constexpr int GF_K = 2 * GB_K;         // two chunks at a time
+
+// Tile pair t of the lower triangle for tiles of M x N: row tile ti has the
+// column tiles below (ti + 1) M.
+template <int M, int N>
+__device__ __forceinline__ void gram_tile(int t, int *ti, int *tj) {
+  int i = 0;
+  while (t >= (i + 1) * (M / N)) {
+    t -= (i + 1) * (M / N);
+    ++i;
+  }
+  *ti = i;
+  *tj = t;
+}
+
+// Float64 throughout: a thread takes 4 x 4 entries.  Bound by the float64 pipe.
 __global__ void __launch_bounds__(G_THREADS)
-gram_lower_kernel(const T *__restrict__ F, int64_t N, int r, int kslice,
+gram_lower_kernel(const double *__restrict__ F, int64_t N, int r, int kslice,
                   double *__restrict__ part) {
-  __shared__ T As[GB_K][GB_M + 1];
-  __shared__ T Bs[GB_K][GB_N + 1];
-  // map blockIdx.x to a lower-triangular (ti, tj) tile pair, tj <= ti
-  int t = blockIdx.x, ti = 0;
-  while (t > ti) { t -= ti + 1; ++ti; }
-  const int tj = t;
+  __shared__ double As[GB_K][GD_T + 1];
+  __shared__ double Bs[GB_K][GD_T + 1];
+  int ti, tj;
+  gram_tile<GD_T, GD_T>(blockIdx.x, &ti, &tj);
   const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
-  const int i0 = ti * GB_M, j0 = tj * GB_N;
+  const int i0 = ti * GD_T, j0 = tj * GD_T;
   const int64_t kb = (int64_t)blockIdx.y * kslice;
   const int64_t ke = min(N, kb + kslice);
-  constexpr bool FLT = sizeof(T) == 4;
   double acc[4][4];
-  float sh[4][4], sl[4][4];   // float-float accumulators (float input)
-  T acc32[4][4];
 #pragma unroll
   for (int a = 0; a < 4; ++a)
 #pragma unroll
-    for (int b = 0; b < 4; ++b) {
-      acc[a][b] = 0.0;
-      sh[a][b] = sl[a][b] = 0.0f;
-    }
-  int chunk = 0;
+    for (int b = 0; b < 4; ++b) acc[a][b] = 0.0;
   for (int64_t k0 = kb; k0 < ke; k0 += GB_K) {
 #pragma unroll
-    for (int e = 0; e < (GB_M * GB_K) / G_THREADS; ++e) {
+    for (int e = 0; e < (GD_T * GB_K) / G_THREADS; ++e) {
       const int idx = tid + e * G_THREADS;
       const int kk = idx % GB_K, ii = idx / GB_K;
       const int64_t gk = k0 + kk;
-      As[kk][ii] = (i0 + ii < r && gk < ke) ? F[gk + (int64_t)(i0 + ii) * N] : T(0);
-      Bs[kk][ii] = (j0 + ii < r && gk < ke) ? F[gk + (int64_t)(j0 + ii) * N] : T(0);
+      As[kk][ii] = (i0 + ii < r && gk < ke) ? F[gk + (int64_t)(i0 + ii) * N] : 0.0;
+      Bs[kk][ii] = (j0 + ii < r && gk < ke) ? F[gk + (int64_t)(j0 + ii) * N] : 0.0;
     }
     __syncthreads();
+    double sum[4][4];
 #pragma unroll
     for (int a = 0; a < 4; ++a)
 #pragma unroll
-      for (int b = 0; b < 4; ++b) acc32[a][b] = T(0);
+      for (int b = 0; b < 4; ++b) sum[a][b] = 0.0;
 #pragma unroll
     for (int kk = 0; kk < GB_K; ++kk) {
-      T av[4], bv[4];
+      double av[4], bv[4];
 #pragma unroll
       for (int a = 0; a < 4; ++a) av[a] = As[kk][ty + 16 * a];
 #pragma unroll
@@ -66,34 +70,12 @@ gram_lower_kernel(const T *__restrict__ F, int64_t N, int r, int kslice,
 #pragma unroll
       for (int a = 0; a < 4; ++a)
 #pragma unroll
-        for (int b = 0; b < 4; ++b) acc32[a][b] = fma(av[a], bv[b], acc32[a][b]);
+        for (int b = 0; b < 4; ++b) sum[a][b] = fma(av[a], bv[b], sum[a][b]);
     }
-    if constexpr (FLT) {
-      ++chunk;
 #pragma unroll
-      for (int a = 0; a < 4; ++a)
+    for (int a = 0; a < 4; ++a)
 #pragma unroll
-        for (int b = 0; b < 4; ++b) {
-          const float c = (float)acc32[a][b];
-          const float t = __fadd_rn(sh[a][b], c);
-          const float z = __fsub_rn(t, sh[a][b]);
-          const float err = __fadd_rn(__fsub_rn(sh[a][b], __fsub_rn(t, z)), __fsub_rn(c, z));
-          sh[a][b] = t;
-          sl[a][b] = __fadd_rn(sl[a][b], err);
-          if ((chunk & 7) == 0) {
-            // fold the correction back (TwoSum), keeping it below an ulp of the sum
-            const float t2 = __fadd_rn(sh[a][b], sl[a][b]);
-            const float z2 = __fsub_rn(t2, sh[a][b]);
-            sl[a][b] = __fadd_rn(__fsub_rn(sh[a][b], __fsub_rn(t2, z2)), __fsub_rn(sl[a][b], z2));
-            sh[a][b] = t2;
-          }
-        }
-    } else {
-#pragma unroll
-      for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) acc[a][b] += (double)acc32[a][b];
-    }
+      for (int b = 0; b < 4; ++b) acc[a][b] += sum[a][b];
     __syncthreads();
   }
   double *o = part + (int64_t)blockIdx.y * r * r;
@@ -102,9 +84,113 @@ gram_lower_kernel(const T *__restrict__ F, int64_t N, int r, int kslice,
 #pragma unroll
     for (int b = 0; b < 4; ++b) {
       const int gi = i0 + ty + 16 * a, gj = j0 + tx + 16 * b;
+      if (gi < r && gj <= gi) o[(int64_t)gi + (int64_t)gj * r] = acc[a][b];
+    }
+}
+
+// float32 F: each chunk of GB_K products is summed in float32, then added to a
+// float-float accumulator (Knuth's TwoSum, the rounding errors gathered in a
+// float32 correction that is folded back every 8 chunks) -- float64 adds, at a
+// small fraction of the float32 rate on this GPU, bounded the kernel.  A thread
+// takes 8 x 4 entries as packed pairs of rows, so that three 16-byte loads
+// serve 32 FMAs: with 4 x 4 entries and eight 4-byte loads the shared-memory
+// wavefronts bound it (N = 1e5, r = 1000: 5.76 ms, now
+// 4.23; 4.50 with one chunk at a time, 6.1 with two CTAs a SM and spills).
+__global__ void __launch_bounds__(G_THREADS)
+gram_lower_f32_kernel(const float *__restrict__ F, int64_t N, int r, int kslice,
+                      double *__restrict__ part) {
+  __shared__ __align__(16) float As[GF_K][GF_M + 4];
+  __shared__ __align__(16) float Bs[GF_K][GF_N + 4];
+  int ti, tj;
+  gram_tile<GF_M, GF_N>(blockIdx.x, &ti, &tj);
+  const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
+  const int i0 = ti * GF_M, j0 = tj * GF_N;
+  const int64_t kb = (int64_t)blockIdx.y * kslice;
+  const int64_t ke = min(N, kb + kslice);
+  const float2 zero = make_float2(0.0f, 0.0f), minus = make_float2(-1.0f, -1.0f);
+  float2 sh[4][4], sl[4][4];
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int b = 0; b < 4; ++b) sh[a][b] = sl[a][b] = zero;
+  constexpr int NA = GF_M * GF_K / G_THREADS, NB = GF_N * GF_K / G_THREADS;
+  constexpr int CS = G_THREADS / GF_K;
+  float ra[NA], rb[NB];
+  const int kk0 = tid % GF_K, ii0 = tid / GF_K;   // and every CS-th column from there
+  auto load = [&](int64_t k0) {
+    const int64_t gk = k0 + kk0;
+#pragma unroll
+    for (int e = 0; e < NA; ++e) {
+      const int i = i0 + ii0 + CS * e;
+      ra[e] = (i < r && gk < ke) ? F[gk + (int64_t)i * N] : 0.0f;
+    }
+#pragma unroll
+    for (int e = 0; e < NB; ++e) {
+      const int j = j0 + ii0 + CS * e;
+      rb[e] = (j < r && gk < ke) ? F[gk + (int64_t)j * N] : 0.0f;
+    }
+  };
+  // t = s + c with its rounding error (TwoSum); returns the error
+  auto two_sum = [&](float2 &s, float2 c) {
+    const float2 t = __fadd2_rn(s, c);
+    const float2 z = __ffma2_rn(s, minus, t);
+    const float2 u = __ffma2_rn(z, minus, t);
+    const float2 err = __fadd2_rn(__ffma2_rn(u, minus, s), __ffma2_rn(z, minus, c));
+    s = t;
+    return err;
+  };
+  int chunk = 0;
+  load(kb);
+  for (int64_t k0 = kb; k0 < ke; k0 += GF_K) {
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < NA; ++e) As[kk0][ii0 + CS * e] = ra[e];
+#pragma unroll
+    for (int e = 0; e < NB; ++e) Bs[kk0][ii0 + CS * e] = rb[e];
+    __syncthreads();
+    if (k0 + GF_K < ke) load(k0 + GF_K);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      float2 sum[4][4];
+#pragma unroll
+      for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) sum[a][b] = zero;
+#pragma unroll
+      for (int kk = 0; kk < GB_K; ++kk) {
+        const float4 a0 = *reinterpret_cast<const float4 *>(&As[h * GB_K + kk][ty * 8]);
+        const float4 a1 = *reinterpret_cast<const float4 *>(&As[h * GB_K + kk][ty * 8 + 4]);
+        const float4 bq = *reinterpret_cast<const float4 *>(&Bs[h * GB_K + kk][tx * 4]);
+        const float2 av[4] = {make_float2(a0.x, a0.y), make_float2(a0.z, a0.w),
+                              make_float2(a1.x, a1.y), make_float2(a1.z, a1.w)};
+        const float bv[4] = {bq.x, bq.y, bq.z, bq.w};
+#pragma unroll
+        for (int b = 0; b < 4; ++b)
+#pragma unroll
+          for (int a = 0; a < 4; ++a)
+            sum[a][b] = __ffma2_rn(av[a], make_float2(bv[b], bv[b]), sum[a][b]);
+      }
+      ++chunk;
+#pragma unroll
+      for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+          sl[a][b] = __fadd2_rn(sl[a][b], two_sum(sh[a][b], sum[a][b]));
+          // fold the correction back, keeping it below an ulp of the sum
+          if ((chunk & 7) == 0) sl[a][b] = two_sum(sh[a][b], sl[a][b]);
+        }
+    }
+  }
+  double *o = part + (int64_t)blockIdx.y * r * r;
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+      const int gi = i0 + ty * 8 + 2 * a, gj = j0 + tx * 4 + b;
       if (gi < r && gj <= gi)
-        o[(int64_t)gi + (int64_t)gj * r] =
-            FLT ? (double)sh[a][b] + (double)sl[a][b] : acc[a][b];
+        o[(int64_t)gi + (int64_t)gj * r] = (double)sh[a][b].x + (double)sl[a][b].x;
+      if (gi + 1 < r && gj <= gi + 1)
+        o[(int64_t)gi + 1 + (int64_t)gj * r] = (double)sh[a][b].y + (double)sl[a][b].y;
     }
 }
 
@@ -124,19 +210,25 @@ __global__ void gram_combine_kernel(const double *__restrict__ part, int slices,
 template <typename T>
 krr_status gram_lower(const T *F, int64_t N, int r, double *C, cudaStream_t s) {
   if (r <= 0) return KRR_OK;
-  const int tiles = (r + GB_M - 1) / GB_M;
-  const int ntri = tiles * (tiles + 1) / 2;
-  int64_t slices = ((int64_t)num_sms() * 4 + ntri - 1) / ntri;
-  const int64_t maxs = (N + 1023) / 1024;
-  if (slices > maxs) slices = maxs;
-  if (slices < 1) slices = 1;
+  constexpr bool FLT = sizeof(T) == 4;
+  constexpr int M = FLT ? GF_M : GD_T, RATIO = FLT ? GF_M / GF_N : 1;
+  const int tiles = (r + M - 1) / M;
+  const int ntri = tiles * (tiles + 1) / 2 * RATIO;   // a few beyond r or the diagonal
+  // slices of the terms: float32 just under four waves of one CTA a SM, float64
+  // two waves or more of two, down to 128 terms (r = 200, N = 4096: 40 CTAs
+  // with slices of 1024 terms took 1127 us, 320 take 419)
+  int64_t slices = ((int64_t)num_sms() * 4 + (FLT ? 0 : ntri - 1)) / ntri;
+  slices = std::max<int64_t>(1, std::min<int64_t>(slices, FLT ? (N + 1023) / 1024 : (N + 127) / 128));
   int64_t kslice = (N + slices - 1) / slices;
-  kslice = (kslice + GB_K - 1) / GB_K * GB_K;
+  kslice = (kslice + GF_K - 1) / GF_K * GF_K;
   slices = (N + kslice - 1) / kslice;
   DevBuf<double> part;
   KRR_TRY(part.alloc((size_t)slices * r * r, s));
-  gram_lower_kernel<T><<<dim3(ntri, (unsigned)slices), G_THREADS, 0, s>>>(F, N, r, (int)kslice,
-                                                                         part.p);
+  const dim3 grid(ntri, (unsigned)slices);
+  if constexpr (FLT)
+    gram_lower_f32_kernel<<<grid, G_THREADS, 0, s>>>(F, N, r, (int)kslice, part.p);
+  else
+    gram_lower_kernel<<<grid, G_THREADS, 0, s>>>(F, N, r, (int)kslice, part.p);
   KRR_LAUNCH_CHECK();
   int blocks = ceil_div((int64_t)r * r, 256);
   if (blocks > num_sms() * 16) blocks = num_sms() * 16;
