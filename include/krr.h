@@ -67,10 +67,10 @@ typedef enum {
                             outer iterative refinement, float64 CG scalars and
                             k x k core                                         */
     KRR_PREC_FLOAT_FLOAT = 2  /* krr_kmatvec and krr_pcg_solve: float64-accurate
-                            product (about 2^-46 per entry) evaluated in
-                            float-float arithmetic on the float32 pipes; the
-                            product the mixed path uses for its refinement
-                            residuals                                         */
+                            product (about 2^-46 per entry) on the integer and
+                            float32 pipes (fixed-point kernel values, sums in
+                            float-float); the product the mixed path uses for
+                            its refinement residuals                          */
 } krr_precision;
 
 /* Pivot rule of the partial Cholesky factorization: RPCholesky (Alg. 3)    */
@@ -115,13 +115,16 @@ typedef struct {
 /* ------------------------------------------------------------------------ */
 /* Fused matrix-free product (Alg. 1 "Product"):                             */
 /*   Y = (A + lambda I) V,  A_ij = kappa(x_i, x_j), never stored.            */
-/* precision KRR_PREC_FP64 evaluates in float64 with direct differences;     */
+/* precision KRR_PREC_FP64 evaluates entries to float64 accuracy, in fixed   */
+/* point where the points' range allows it (differences of coordinates       */
+/* rounded once to 57 bits of the range, exact squared distances) and in     */
+/* float64 with direct differences elsewhere, and sums in float64;           */
 /* KRR_PREC_MIXED evaluates kernel tiles in float32 (distances from row      */
 /* norms of centred points) and accumulates in float32 -- for the Gaussian   */
 /* and Matern kernels by default with the inner products on the tensor cores */
 /* (see krr_set_product_path), prepared once per call (synchronises stream);  */
-/* KRR_PREC_FLOAT_FLOAT evaluates entries and sums in float-float arithmetic */
-/* (error-free transformations on the float32 pipes, ~2^-46 per entry).     */
+/* KRR_PREC_FLOAT_FLOAT evaluates entries in fixed point likewise (float-    */
+/* float elsewhere) and sums in float-float arithmetic (~2^-46 per entry).   */
 /* V, Y: N x m column-major float64.  Y may not alias V.                     */
 /* ------------------------------------------------------------------------ */
 KRR_API krr_status krr_kmatvec(const double *X, int64_t N, int d, krr_kernel kern,
@@ -184,7 +187,9 @@ KRR_API krr_status krr_rpc_sample(const double *dres, int64_t N, double dfloor,
 /* is <= N * 2^-52 * max_i A_ii, appends G R^{-1} to F and subtracts its      */
 /* squared row norms from the residual diagonal; every candidate of a block   */
 /* gets residual 0.  Stops early (rank < k) if every weight becomes zero.     */
-/* All arithmetic is float64.  *F_out receives a new handle (free with        */
+/* Results are float64 throughout: the entries as for KRR_PREC_FP64, the      */
+/* products with F from 57-bit fixed-point digits whose sums are exact, at    */
+/* most as far off as float64 sums.  *F_out receives a new handle (free with  */
 /* krr_factor_free).                                                          */
 /* ------------------------------------------------------------------------ */
 KRR_API krr_status krr_rpcholesky(const double *X, int64_t N, int d, krr_kernel kern,

@@ -40,7 +40,8 @@ __device__ __forceinline__ uint64_t dig_fixed(double x, uint64_t bias) {
   const uint64_t b = (uint64_t)__double_as_longlong(x);
   const int e = (int)(b >> 52) & 0x7ff;
   const uint64_t m5 = ((b & ((1ull << 52) - 1)) | (1ull << 52)) << 5;
-  const uint64_t v = ((m5 >> min(1023 - e, 63)) + 1) >> 1;
+  // (beyond 2, infinities and NaN: 0, without an undefined shift)
+  const uint64_t v = ((m5 >> min((unsigned)(1023 - e), 63u)) + 1) >> 1;
   return (int64_t)b < 0 ? bias - v : bias + v;
 }
 

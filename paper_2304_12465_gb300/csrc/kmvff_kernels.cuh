@@ -1,4 +1,6 @@
-// Float64-accurate fused product on the float32 pipes ("double-float").
+// Float64-accurate fused product on the float32 pipes ("double-float"), for
+// point sets outside the range of the fixed-point products (kmvfix_kernels.cuh),
+// which take a fraction of its instructions elsewhere.
 //
 // The mixed-precision refinement needs its residual y - (A + lambda I)x with
 // kernel entries accurate far beyond float32, but this part's float64 pipe
