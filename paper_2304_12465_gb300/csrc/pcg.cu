@@ -28,12 +28,16 @@ constexpr int RED_BLOCKS = 512;
 // loaded before any arithmetic so that many loads are in flight.  M is m
 // rounded up to 1, 2, 4, 8 or 16 (specialised: a runtime column count costs
 // the unrolled loops several times their work).
-constexpr int TT_COLS = 64;
+// A block takes TT_COLS columns of F, or TT_COLS_FEW where that leaves the grid
+// below two blocks a SM: a block's passes over its columns then are a chain of
+// latencies (N = 4096, rank 200: 64 blocks of four passes 14.4 us, 208 of one
+// 5.2).  The partial sums do not depend on it.
+constexpr int TT_COLS = 64, TT_COLS_FEW = 16;
 
 template <typename T, int M>
 __global__ void __launch_bounds__(256)
 tall_t_kernel(const T *__restrict__ F, int64_t N, int rank, const T *__restrict__ R, int m,
-              double *__restrict__ part) {
+              int cols, double *__restrict__ part) {
   constexpr int PER_LANE = TT_ROWS / 32;
   __shared__ T sR[M][TT_ROWS];
   const int64_t n0 = (int64_t)blockIdx.x * TT_ROWS;
@@ -45,9 +49,9 @@ tall_t_kernel(const T *__restrict__ F, int64_t N, int rank, const T *__restrict_
   __syncthreads();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int nw = blockDim.x >> 5;
-  const int l1 = min(rank, (int)(blockIdx.y + 1) * TT_COLS);
+  const int l1 = min(rank, (int)(blockIdx.y + 1) * cols);
   // two columns per pass: each R value read from shared memory serves both
-  for (int l = (int)blockIdx.y * TT_COLS + warp; l < l1; l += 2 * nw) {
+  for (int l = (int)blockIdx.y * cols + warp; l < l1; l += 2 * nw) {
     const bool two = l + nw < l1;
     const T *col = F + (int64_t)l * N + n0;
     const T *col2 = col + (int64_t)nw * N;
@@ -159,18 +163,26 @@ static void launch_tri_gemv(const double *Mt, int rank, const double *x, int m, 
   }
 }
 
+// Blocks of 64 threads: about ten per SM at N = 1e5, so the last wave of
+// blocks leaves few SMs idle (256-thread blocks left 2.6 per SM).
+constexpr int TN_THREADS = 64;
+constexpr int TN_GROUPS = 4;   // threads a row where N leaves less than two blocks a SM
+
 // Z[c][n] = (R[c][n] - sum_l F[n + l N] v[c][l]) / lambda
 // One thread per row (blocks of TN_THREADS); the column loop loads LU
 // values of F before using them so that enough loads are in flight to stream
 // F at HBM speed.  M as above.
-template <typename T, int M>
+// GRP > 1: as many threads a row, each with every GRP-th group of LU columns,
+// whose sums are added in order.
+template <typename T, int M, int GRP = 1>
 __global__ void __launch_bounds__(256)
 tall_n_kernel(const T *__restrict__ F, int64_t N, int rank, const double *__restrict__ v,
               int m, const T *__restrict__ R, double inv_lambda, T *__restrict__ Z) {
   constexpr int LCH = 256;
   constexpr int LU = 32;
   __shared__ T sv[LCH][M];
-  const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int rows = blockDim.x / GRP, grp = threadIdx.x / rows, nl0 = threadIdx.x % rows;
+  const int64_t n = (int64_t)blockIdx.x * rows + nl0;
   const bool ok = n < N;
   T acc[M];
 #pragma unroll
@@ -183,7 +195,7 @@ tall_n_kernel(const T *__restrict__ F, int64_t N, int rank, const double *__rest
       sv[l][c] = (l < nl && c < m) ? (T)v[(int64_t)c * rank + l0 + l] : T(0);
     }
     __syncthreads();
-    for (int lb = 0; lb < nl; lb += LU) {
+    for (int lb = grp * LU; lb < nl; lb += GRP * LU) {
       T f[LU];
 #pragma unroll
       for (int u = 0; u < LU; ++u)
@@ -194,6 +206,19 @@ tall_n_kernel(const T *__restrict__ F, int64_t N, int rank, const double *__rest
         for (int c = 0; c < M; ++c) acc[c] = fma(f[u], sv[lb + u][c], acc[c]);
       }
     }
+  }
+  if constexpr (GRP > 1) {
+    __shared__ T red[GRP - 1][TN_THREADS][M];
+    if (grp > 0) {
+#pragma unroll
+      for (int c = 0; c < M; ++c) red[grp - 1][nl0][c] = acc[c];
+    }
+    __syncthreads();
+    if (grp > 0) return;
+#pragma unroll
+    for (int q = 0; q < GRP - 1; ++q)
+#pragma unroll
+      for (int c = 0; c < M; ++c) acc[c] += red[q][nl0][c];
   }
   if (ok) {
 #pragma unroll
@@ -209,27 +234,37 @@ static int tall_pad_m(int m) { return m <= 1 ? 1 : m <= 2 ? 2 : m <= 4 ? 4 : m <
 template <typename T>
 static krr_status launch_tall_t(const T *F, int64_t N, int rank, const T *R, int m,
                                 double *part, cudaStream_t s) {
-  const dim3 grid(ceil_div(N, TT_ROWS), ceil_div(rank, TT_COLS));
+  const int nb = ceil_div(N, TT_ROWS);
+  const int cols = (int64_t)nb * ceil_div(rank, TT_COLS) < 2 * num_sms() ? TT_COLS_FEW : TT_COLS;
+  const dim3 grid(nb, ceil_div(rank, cols));
   switch (tall_pad_m(m)) {
-    case 1: tall_t_kernel<T, 1><<<grid, 256, 0, s>>>(F, N, rank, R, m, part); break;
-    case 2: tall_t_kernel<T, 2><<<grid, 256, 0, s>>>(F, N, rank, R, m, part); break;
-    case 4: tall_t_kernel<T, 4><<<grid, 256, 0, s>>>(F, N, rank, R, m, part); break;
-    case 8: tall_t_kernel<T, 8><<<grid, 256, 0, s>>>(F, N, rank, R, m, part); break;
-    default: tall_t_kernel<T, 16><<<grid, 256, 0, s>>>(F, N, rank, R, m, part); break;
+    case 1: tall_t_kernel<T, 1><<<grid, 256, 0, s>>>(F, N, rank, R, m, cols, part); break;
+    case 2: tall_t_kernel<T, 2><<<grid, 256, 0, s>>>(F, N, rank, R, m, cols, part); break;
+    case 4: tall_t_kernel<T, 4><<<grid, 256, 0, s>>>(F, N, rank, R, m, cols, part); break;
+    case 8: tall_t_kernel<T, 8><<<grid, 256, 0, s>>>(F, N, rank, R, m, cols, part); break;
+    default: tall_t_kernel<T, 16><<<grid, 256, 0, s>>>(F, N, rank, R, m, cols, part); break;
   }
   KRR_LAUNCH_CHECK();
   return KRR_OK;
 }
-
-// Blocks of 64 threads: about ten per SM at N = 1e5, so the last wave of
-// blocks leaves few SMs idle (256-thread blocks left 2.6 per SM).
-constexpr int TN_THREADS = 64;
 
 template <typename T>
 static krr_status launch_tall_n(const T *F, int64_t N, int rank, const double *v, int m,
                                 const T *R, double inv_lambda, T *Z, cudaStream_t s) {
   const unsigned grid = ceil_div(N, TN_THREADS);
   constexpr int B = TN_THREADS;
+  // few rows: the columns of a row are a chain of latencies, split over four
+  // threads (N = 4096, rank 200, m = 1: 12.4 us with one, 6.1)
+  if (m <= 4 && rank > 0 && grid < 2u * (unsigned)num_sms()) {
+    constexpr int GB = TN_THREADS * TN_GROUPS;
+    switch (tall_pad_m(m)) {
+      case 1: tall_n_kernel<T, 1, TN_GROUPS><<<grid, GB, 0, s>>>(F, N, rank, v, m, R, inv_lambda, Z); break;
+      case 2: tall_n_kernel<T, 2, TN_GROUPS><<<grid, GB, 0, s>>>(F, N, rank, v, m, R, inv_lambda, Z); break;
+      default: tall_n_kernel<T, 4, TN_GROUPS><<<grid, GB, 0, s>>>(F, N, rank, v, m, R, inv_lambda, Z); break;
+    }
+    KRR_LAUNCH_CHECK();
+    return KRR_OK;
+  }
   switch (tall_pad_m(m)) {
     case 1: tall_n_kernel<T, 1><<<grid, B, 0, s>>>(F, N, rank, v, m, R, inv_lambda, Z); break;
     case 2: tall_n_kernel<T, 2><<<grid, B, 0, s>>>(F, N, rank, v, m, R, inv_lambda, Z); break;
