@@ -169,6 +169,7 @@ class ClockSampler:
 # tcgen05 kernel.  Any other shape or tile has no capture and reports None; a
 # change to the kernel invalidates the entry until it is captured again.
 KMV32_TRAFFIC = {("fma", 0, 100_000, 16, 4, 50): 8_748_117 + 16_672_768,
+                 ("tensor", 0, 100_000, 16, 4, 1): 20_839_936 + 0,
                  ("tensor", 0, 100_000, 16, 4, 3): 20_839_680 + 0}
 
 # Register-operand mma.sync (m16n8k16, f16 inputs, f32 accumulator) measured by
