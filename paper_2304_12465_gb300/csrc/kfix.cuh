@@ -250,10 +250,15 @@ KRR_HD uint64_t fix_exponent_l1(uint64_t S, int r) {
   return r > 0 ? (S >> r) + ((S >> (r - 1)) & 1) : S;
 }
 
+constexpr double kFixMaternEnd = 708.39;   // 1022 ln 2 = 708.396
+
 // (1 + q + q^2/3) exp(-q) from the partial sums of squares; scale = 2^(30-2Q).
 // The square root starts from the float32 reciprocal square root (2^-22) and
 // takes one Goldschmidt step and a final residual correction in float64; q
-// log2 e is a 64 x 64-bit fixed-point product.
+// log2 e is a 64 x 64-bit fixed-point product.  E has ten integer bits, so it
+// would wrap at q = 1024 ln 2 = 709.8, which opposite corners of the accepted
+// range pass from d = 31 on (q up to 128 sqrt(d)): from E = 1022 on kappa, below
+// 1e-302 there, is 0, as in the Gaussian and Laplace forms.
 KRR_HD double fix_matern(int64_t S1, int64_t S2, uint64_t S3, double scale,
                                              const uint64_t *__restrict__ tab) {
   const int64_t A = S2 + (int64_t)(S3 >> 30);
@@ -269,7 +274,7 @@ KRR_HD double fix_matern(int64_t S1, int64_t S2, uint64_t S3, double scale,
   g = fma(g, e, g);
   h = fma(h, e, h);
   const double q = fma(fma(-g, g, r2), h, g);
-  if (q > 720.0) return 0.0;
+  if (q >= kFixMaternEnd) return 0.0;
   uint64_t b;
 #ifdef __CUDA_ARCH__
   b = (uint64_t)__double_as_longlong(q);
