@@ -567,6 +567,14 @@ bool fixsym_applies(int64_t N, int d, int m, bool ff) {
   return nt >= 20 && (double)nt * (nt + 1) * M * RT * 8.0 <= 4.0 * 1024 * 1024 * 1024;
 }
 
+double fixsym_scratch_bytes(int64_t N, int d, int m, bool ff) {
+  if (!fixsym_applies(N, d, m, ff)) return 0.0;
+  const int M = pad_m(m);
+  int RT, nt;
+  fixsym_shape(N, M, &RT, &nt);
+  return (double)nt * (nt + 1) * M * RT * 8.0;
+}
+
 // Symmetric square product of fixed-point points (known to fit).
 static krr_status fixsym_product(const int2 *u, int64_t N, int d, int kern, const FixScale *scale,
                                  bool ff, double lambda, const double *V, int64_t ldv, int m,

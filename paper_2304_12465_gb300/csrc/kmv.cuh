@@ -142,6 +142,8 @@ krr_status prepare_points_f64(const double *Xd, int64_t N, int d, int kern, doub
 // A single float64 product then waits for scale->ok: 10 us, against at least
 // 20 saved.
 bool fixsym_applies(int64_t N, int d, int m, bool ff);
+// Device bytes of that product's partial sums, 0 where it does not apply.
+double fixsym_scratch_bytes(int64_t N, int d, int m, bool ff);
 
 // Common scale of one or two point sets (B may be NULL) for float64 or
 // float-float products, and the integer coordinates of one set under it.

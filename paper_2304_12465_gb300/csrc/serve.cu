@@ -677,13 +677,13 @@ double serve_footprint(int64_t N, int d, int m, int k) {
   b += 4.0 * n * m * 8 + 5.0 * n * m * 4;
   // product partials, preconditioner partials, reductions
   b += splits * M * n * 4 + nbt * k * m * 8 + 3.0 * k * m * 8 + 2.0 * nbv * m * 8;
-  // float-float residual product: split partials (or the symmetric product's
-  // sums of every pair of tiles) and split right-hand sides
+  // float-float residual product: split partials (or, for the shapes that take
+  // it, the symmetric product's sums of every pair of tiles) and split
+  // right-hand sides
   const double rows_ff = 128.0 * (dpff <= 16 ? 2 : 1);
   const double tiles_ff = std::ceil(n / rows_ff);
   const double ffsplits = std::min(std::ceil(3648.0 / tiles_ff) + 1.0, std::ceil(n / 32.0));
-  const double sym_tiles = std::max(std::min(n / 128.0, 140.0), n / 1024.0) + 2.0;
-  b += std::max(ffsplits, sym_tiles) * M * n * 8 + 2.0 * n * m * 4;
+  b += std::max(ffsplits * M * n * 8, fixsym_scratch_bytes(N, d, m, true)) + 2.0 * n * m * 4;
   return b * 1.05 + 16.0 * 1024 * 1024;
 }
 

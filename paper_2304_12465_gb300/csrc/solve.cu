@@ -497,7 +497,7 @@ static double escalation_worst(const Escalation &e) {
 krr_status escalate_refine(Escalation &e, cudaStream_t s) {
   const int64_t N = e.N, nm = N * e.m;
   const int m = e.m;
-  DevBuf<double> b64, d64, F64, X64, part64;
+  DevBuf<double> b64, d64, F64, X64;
   KRR_TRY(b64.alloc((size_t)nm, s));
   KRR_TRY(d64.alloc((size_t)nm, s));
   // the float32 factor in float64 (exactly representable), consistent with
@@ -527,8 +527,8 @@ krr_status escalate_refine(Escalation &e, cudaStream_t s) {
   const double *Xdev = nullptr;
   PointsF64 P64;
   auto residual = [&]() -> krr_status {
-    if (res64)
-      KRR_TRY(kmv_f64(P64, e.lambda, e.alpha, N, m, e.mx, N, s, part64));
+    if (res64)   // in the float-float product's scratch: the two shapes' sizes agree
+      KRR_TRY(kmv_f64(P64, e.lambda, e.alpha, N, m, e.mx, N, s, *e.ffpart));
     else
       KRR_TRY(kmv_ff(*e.Pff, e.lambda, e.alpha, N, m, e.mx, N, s, *e.ffpart, *e.ffvsplit));
     e.entries += kmv_entries(N);
