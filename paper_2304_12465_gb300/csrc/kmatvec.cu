@@ -9,6 +9,7 @@
 #include "kmv_dispatch.cuh"
 #include "kmvfix_kernels.cuh"
 #include "kmvtc_kernels.cuh"
+#include "route.cuh"
 
 namespace krr {
 
@@ -479,10 +480,12 @@ krr_status kmv_f32(const PointsF32 &P, float lambda, const float *V, int64_t ldv
                    float *Y, int64_t ldy, cudaStream_t s, DevBuf<float> &part) {
   const int64_t N = P.N;
   if (N == 0 || m == 0) return KRR_OK;
-  if (P.nh5 > 0 && g_product_path.load() == 0)
-    return kmv_tc5(P, P, lambda, true, V, ldv, m, Y, ldy, s, part);
-  if (P.kc16 > 0 && path_of(P.kern, P.dp) == 1)
-    return kmv_tc(P, lambda, V, ldv, m, Y, ldy, s, part);
+  switch (product_route(product_path(), P.nh5 > 0, P.kc16 > 0, P.xt.p != nullptr)) {
+    case kRouteTcgen05: return kmv_tc5(P, P, lambda, true, V, ldv, m, Y, ldy, s, part);
+    case kRouteMmaSync: return kmv_tc(P, lambda, V, ldv, m, Y, ldy, s, part);
+    case kRouteFma: break;
+    default: KRR_REQUIRE(false, "float32 product: points without operands");
+  }
   for (int c0 = 0; c0 < m; c0 += 16) {
     const int mg = (m - c0 < 16) ? (m - c0) : 16;
     const int M = pad_m(mg);
