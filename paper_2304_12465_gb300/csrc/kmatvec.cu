@@ -177,8 +177,8 @@ krr_status prepare_points_f32(const double *Xd, int64_t N, int d, int kern, doub
 }
 
 krr_status prepare_points_product(const double *Xd, int64_t N, int d, int kern, double sigma,
-                                  cudaStream_t s, PointsF32 &P) {
-  if (product_path() == 0 && kern != KLAPLACE) {
+                                  cudaStream_t s, PointsF32 &P, bool try_tc5) {
+  if (try_tc5 && product_path() == 0 && kern != KLAPLACE) {
     P.dp = (d + 3) / 4 * 4;
     P.d = d;
     P.N = N;

@@ -56,9 +56,10 @@ krr_status prepare_points_tc(const double *Xd, cudaStream_t s, PointsF32 &P,
 
 // Points of a square float32 product (kmv_f32) by the process's path: the
 // tcgen05 operands alone when they apply, else the float32 points and, where
-// it applies, the mma.sync layout.  Synchronises s.
+// it applies, the mma.sync layout.  try_tc5 = false: the caller knows that they
+// do not.  Synchronises s.
 krr_status prepare_points_product(const double *Xd, int64_t N, int d, int kern, double sigma,
-                                  cudaStream_t s, PointsF32 &P);
+                                  cudaStream_t s, PointsF32 &P, bool try_tc5 = true);
 
 // Builds only the tcgen05 operands of P (P.nh5 > 0); *bad = 1 (and nh5 = 0)
 // when a point is outside the split's range.  P's kern, sigma, N and d are
@@ -77,8 +78,9 @@ krr_status kmv_tc5(const PointsF32 &R, const PointsF32 &P, float lambda, bool sq
 
 // One whole tcgen05 product from and to float64 arrays: Y = K(Xr, X) V, or (A
 // + lambda I) V when Xr is NULL.  Every launch is issued before the host
-// learns whether the points fit the split: *done = false when the path does
-// not apply or they did not fit (Y is then to be computed another way).
+// learns whether the points fit the split; the product itself returns at once
+// when they do not.  *done = false when the path does not apply or they did not
+// fit (Y is then to be computed another way).
 // Synchronises s.
 krr_status kmv_tc5_call(const double *Xr, int64_t Nr, const double *Xd, int64_t N, int d,
                         int kern, double sigma, double lambda, const double *V, int m, double *Y,

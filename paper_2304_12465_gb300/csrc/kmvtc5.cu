@@ -264,7 +264,8 @@ krr_status tc5_wait_selftest(long long budget, cudaStream_t s) {
 
 // ------------------------------------------------------------ reduction
 // TV5: the type of V and Y.  flags (optional): {a point outside the split's
-// range, a bounded wait gave up}, for one read-back after the product.
+// range (nothing was summed then), a bounded wait gave up}, for one read-back
+// after the product.
 template <typename TV5>
 __global__ void t5_reduce_kernel(const float *__restrict__ part, int64_t Nr, int m, int M, int C,
                                  int64_t T, int G, int J, int CG, const int *__restrict__ vexp,
@@ -273,7 +274,7 @@ __global__ void t5_reduce_kernel(const float *__restrict__ part, int64_t Nr, int
                                  int *__restrict__ flags) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (flags && i == 0) flags[1] = *fault;
-  if (i >= Nr) return;
+  if (i >= Nr || (flags && flags[0])) return;
   const int64_t rb = i / T5_RB;
   const int r = (int)(i % T5_RB);
   const int b_lo = t5_cta_of(rb * C, T, G);
@@ -308,6 +309,7 @@ t5_reduce_many_kernel(const float *__restrict__ part, int64_t Nr, int m, int M, 
   const int64_t i0 = (int64_t)blockIdx.x * 32, i = i0 + lane;
   const int c = blockIdx.y;
   if (flags && i0 == 0 && c == 0 && threadIdx.x == 0) flags[1] = *fault;
+  if (flags && flags[0]) return;
   const int64_t rb = i0 / T5_RB;
   const int r = (int)(i0 % T5_RB) + lane;
   const int b_lo = t5_cta_of(rb * C, T, G);
@@ -516,11 +518,13 @@ static int *t5_vexp(float *part, const T5Geometry &g, int M) {
 }
 
 // Stages V for this geometry and launches the product; returns the launch's
-// error.  part must hold t5_scratch_floats(g, M) floats.
+// error.  part must hold t5_scratch_floats(g, M) floats.  skip: see T5Args (NULL
+// while tuning, whose times would be those of an empty kernel).
 template <typename TV5>
 static cudaError_t t5_launch(const PointsF32 &R, const PointsF32 &P, int M, int variant,
                              const T5Geometry &g, const TV5 *Vg, int64_t ldv, int mg,
-                             float *part, int *fault, cudaStream_t s, bool timed) {
+                             float *part, int *fault, const int *skip, cudaStream_t s,
+                             bool timed) {
   float *vbuf = part + t5_npart(g, M);
   cudaError_t e = cudaSuccess;
   if (t5_variant_tv(variant)) {
@@ -544,7 +548,7 @@ static cudaError_t t5_launch(const PointsF32 &R, const PointsF32 &P, int M, int 
   }
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  const T5Args args{reinterpret_cast<const float4 *>(vbuf), P.N, part, g.C, g.T, g.J, fault};
+  const T5Args args{reinterpret_cast<const float4 *>(vbuf), P.N, part, g.C, g.T, g.J, fault, skip};
   const int nh = P.nh5, csep = P.csep5, kb = t5_kb(nh, csep);
   // at least half of an SM's shared memory: one CTA per SM (each takes all
   // 512 TMEM columns)
@@ -602,9 +606,9 @@ static int choose_variant(const PointsF32 &R, const PointsF32 &P, bool square, i
     float ms = 0.0f;
     bool ok = true;
     for (int rep = 0; rep < 2 && ok; ++rep) {   // the second launch is timed
-      ok = t5_launch(R, P, M, v, g, Vg, ldv, mg, part.p, fault, s, false) == cudaSuccess &&
+      ok = t5_launch(R, P, M, v, g, Vg, ldv, mg, part.p, fault, nullptr, s, false) == cudaSuccess &&
            cudaEventRecord(e0, s) == cudaSuccess &&
-           t5_launch(R, P, M, v, g, Vg, ldv, mg, part.p, fault, s, false) == cudaSuccess &&
+           t5_launch(R, P, M, v, g, Vg, ldv, mg, part.p, fault, nullptr, s, false) == cudaSuccess &&
            cudaEventRecord(e1, s) == cudaSuccess && cudaEventSynchronize(e1) == cudaSuccess &&
            cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess;
     }
@@ -651,7 +655,7 @@ static krr_status tc5_products(const PointsF32 &R, const PointsF32 &P, double la
     const T5Geometry g = t5_geometry(Nr, Nc, t5_variant_tn(variant));
     const size_t need = t5_scratch_floats(g, M);
     if (part.n < need) KRR_TRY(part.alloc(need, s));
-    cudaError_t e = t5_launch(R, P, M, variant, g, Vg, ldv, mg, part.p, fault, s, !quiet);
+    cudaError_t e = t5_launch(R, P, M, variant, g, Vg, ldv, mg, part.p, fault, flags, s, !quiet);
     if (e != cudaSuccess) {
       set_error("tcgen05 product launch failed: %s", cudaGetErrorString(e));
       return KRR_ECUDA;

@@ -146,6 +146,9 @@ struct T5Args {
   int64_t T;        // row blocks x column tiles
   int J;            // segments per CTA (maximum)
   int *fault;       // set to 1 when a bounded wait gives up
+  // optional: not zero when the points turned out not to fit the split (known
+  // on the device before the host knows): every CTA then has no pairs
+  const int *skip;
 };
 
 // Kernel values of the MMA accumulator D.
@@ -254,7 +257,8 @@ kmvtc5_kernel(const __grid_constant__ CUtensorMap rowmap,
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int G = gridDim.x, b = blockIdx.x;
-  const int64_t p_begin = (int64_t)b * a.T / G, p_end = (int64_t)(b + 1) * a.T / G;
+  const int64_t p_begin = (int64_t)b * a.T / G;
+  const int64_t p_end = (a.skip && *a.skip) ? p_begin : (int64_t)(b + 1) * a.T / G;
   const int64_t rb_first = p_begin / a.C;
   const int ct_first = (int)(p_begin - rb_first * a.C);
   // (row block, column tile) of pair p are kept incrementally along the range
@@ -377,8 +381,10 @@ kmvtc5_kernel(const __grid_constant__ CUtensorMap rowmap,
         if (p + 1 == p_end || ct + 1 == a.C) bw::mma_commit(bar(T5_BAR_A_EMPTY));
       }
       // every MMA issued so far has completed once FIN flips
-      bw::mma_commit(bar(T5_BAR_FIN));
-      bw::mbar_wait(bar(T5_BAR_FIN), 0, T5_WAIT_BUDGET >> 4);
+      if (p_begin < p_end) {
+        bw::mma_commit(bar(T5_BAR_FIN));
+        bw::mbar_wait(bar(T5_BAR_FIN), 0, T5_WAIT_BUDGET >> 4);
+      }
     }
     __syncwarp();
   } else {
