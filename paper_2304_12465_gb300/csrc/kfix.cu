@@ -91,6 +91,7 @@ __global__ void fix_scale_kernel(const double *__restrict__ part, int blocks, in
   out->s_lo = s_lo;
   out->s1_max = 0;
   out->r2_scale = 0.0;
+  out->bias = out->s1_near = 0;
   if (kern == KLAPLACE) {
     out->limb = 0;
     out->q = 58 - e;
@@ -104,6 +105,13 @@ __global__ void fix_scale_kernel(const double *__restrict__ part, int blocks, in
   out->r2_scale = ldexp(1.0, 30 - 2 * out->q);
   // (without a shift every sum of squares stays below E = 512)
   out->s1_max = left == 0 ? INT64_MAX : (int64_t)((1022ull << 54) >> left);
+  if (ff) {
+    // the mean of a squared difference of low limbs uniform over 2^25 values is
+    // 2^50 / 6 a coordinate (padded coordinates have none); 2^50 S1 is worth
+    // 2^(2 e - 56) S1
+    out->bias = (int64_t)d * (1 << 24) / 6;
+    out->s1_near = 1LL << (56 - 2 * e - kFixNearExp);
+  }
 }
 
 __global__ void fix_convert_kernel(const double *__restrict__ X, int64_t N, int d, int dp,

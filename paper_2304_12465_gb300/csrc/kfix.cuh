@@ -50,8 +50,12 @@ constexpr int kFixMinExp = 1;    // a smaller range gains nothing: E is kept at 
 constexpr int kFixLimb = 29;
 // The float-float products keep |u| < 2^53 with low limbs of 25 bits and leave
 // out S3 but for its mean over low limbs: what is missing stays below d 2^(2 e
-// - 56) of E at the accepted ranges, and two multiply-adds a coordinate remain.
+// - 56) of E (a fifth of 2^(2 e - 56) sqrt(d) in the mean square), and two
+// multiply-adds a coordinate remain.  Pairs nearer than 2^-8 in E or q^2 take
+// the whole sum (s1_near): there kappa is 1 but for a small difference, and
+// equal points give exactly 1, as direct differences do.
 constexpr int kFixFFLimb = 25;
+constexpr int kFixNearExp = 8;
 constexpr int kFixTab = 256;
 
 // What the conversion and the products of one point set (or two: rows and
@@ -62,6 +66,8 @@ struct FixScale {
   double s_hi, s_lo;     // scale factor as an unevaluated sum
   double r2_scale;       // Matern: 2^(30 - 2 q)
   int64_t s1_max;        // Gaussian: see fix_exponent
+  int64_t bias, s1_near; // float-float products: mean of S3 2^-26; limit of S1
+                         // below which S3 is formed
   int q;                 // fraction bits of u
   int r;                 // right shift to 54 fraction bits (Gaussian, Laplace)
   int limb;              // bits of the low limb (0: whole 64-bit integers)
@@ -193,10 +199,10 @@ KRR_HD void fix_limbs(int64_t u, int limb, int32_t *h, int32_t *l) {
   *l = (int32_t)(u - hh * (1LL << limb));
 }
 
-// fix_exponent without S3: E from 2^50 S1 + 2^26 (S2 + bias), bias the mean of
-// S3 2^-26.  Near points can fall below zero by what is missing: 0 then.
-KRR_HD uint64_t fix_exponent_ff(int64_t S1, int64_t S2, int r, int64_t bias, int64_t s1_max) {
-  const int64_t a = (S2 + bias + (1LL << (r - 1))) >> r;
+// The float-float products' E from 2^50 S1 + 2^26 A, A = S2 + S3 2^-26 or its
+// mean.  A sum that falls below zero by the rounding of A is 0.
+KRR_HD uint64_t fix_exponent_ff(int64_t S1, int64_t A, int r, int64_t s1_max) {
+  const int64_t a = (A + (1LL << (r - 1))) >> r;
   const uint64_t b = (uint64_t)S1 << (24 - r);
   if (a < 0 && b < (uint64_t)-a) return 0;
   return S1 >= s1_max ? ~0ull : b + (uint64_t)a;

@@ -51,27 +51,26 @@ struct FixAccFF {
   static __device__ __forceinline__ double value(T a) { return (double)a.h + (double)a.l; }
 };
 
-// 2^-E as hi + lo floats: the leading 48 bits of the mantissa.
+// 2^-E as hi + lo floats: 24 bits rounded to nearest and the signed rest (32
+// bits, rounded to 24 by the conversion), 49 bits of the mantissa or more.
 __device__ __forceinline__ FF fix_exp2_ff(uint64_t E, const uint64_t *__restrict__ tab) {
   const int n = (int)(E >> 54);
-  const uint64_t m = fix_exp2_mantissa(E, tab);
-  // m in [2^62, 2^63]: 24 bits from bit 39 up (bit 63 carries into the
-  // exponent field), 24 from bit 15 up
-  const float h = __uint_as_float(0x4B000000u + ((uint32_t)(m >> 39) - 0x800000u));
-  const float l = __fsub_rn(__uint_as_float(0x4B000000u | ((uint32_t)(m >> 15) & 0xffffffu & 0x7fffffu)),
-                            8388608.0f) +
-                  ((m >> 38) & 1 ? 8388608.0f : 0.0f);
-  if (n < 100) {
+  // m in [2^62, 2^63]: hi from bit 39 up (bit 63 carries into the exponent
+  // field), lo the 32 bits below less half of hi's unit, in units of 2^-56
+  const uint64_t t = fix_exp2_mantissa(E, tab) + (1ull << 38);
+  const float h = __uint_as_float(0x4B000000u + ((uint32_t)(t >> 39) - 0x800000u));
+  const float l = (float)(int32_t)((uint32_t)(t >> 7) ^ 0x80000000u);
+  if (n < 64) {
     const float s = __uint_as_float((uint32_t)(127 - 24 - n) << 23);   // 2^(-24 - n)
-    return {h * s, l * (s * 0x1p-24f)};
+    return {h * s, l * (s * 0x1p-32f)};
   }
   if (n > 150) return {0.0f, 0.0f};
   const float s = __uint_as_float((uint32_t)(127 + 40 - n) << 23);     // 2^(40 - n)
-  return {(h * 0x1p-64f) * s, 0.0f};
+  return {(h * 0x1p-64f) * s, n < 100 ? (l * 0x1p-96f) * s : 0.0f};
 }
 
-// The squared distance 2^(26 - 2 q) (2^24 S1 + A) as a float-float value (the
-// leading 48 bits).
+// The squared distance 2^(26 - 2 q) (2^24 S1 + A) as a float-float value (its
+// leading 48 bits or more).
 __device__ __forceinline__ FF fix_r2_ff(int64_t S1, int64_t A, int q) {
   uint64_t lo = (uint64_t)S1 << 24;
   int64_t hi = S1 >> 40;
@@ -92,10 +91,10 @@ __device__ __forceinline__ FF fix_r2_ff(int64_t S1, int64_t A, int q) {
   }
   // value = top 2^(ex - 64) 2^(26 - 2 q), top in [2^63, 2^64)
   const float h = __uint_as_float(0x4B000000u + ((uint32_t)(top >> 40) - 0x800000u));
-  const float l = (float)((uint32_t)(top >> 16) & 0xffffffu);
+  const float l = (float)(uint32_t)(top >> 8);
   const int e2 = ex - 24 + 26 - 2 * q;                                  // exponent of h's unit
   const float s = __uint_as_float((uint32_t)max(127 + e2, 1) << 23);
-  return {h * s, (l * s) * 0x1p-24f};
+  return {h * s, (l * s) * 0x1p-32f};
 }
 
 // kappa of one pair from the row's coordinates (registers) and the column's
@@ -138,16 +137,24 @@ __device__ __forceinline__ typename A::T fix_kappa(const int2 (&u)[DP],
       }
     }
     if constexpr (A::kFF) {
-      // mean of a squared difference of low limbs uniform over 2^25 values:
-      // 2^50 / 6, a coordinate, in units of 2^26
-      constexpr int64_t bias = (int64_t)DP * (1 << 24) / 6;
+      int64_t low = S2 + fs.bias;
+      if (S1 < fs.s1_near) {   // near points are few in most sets
+#pragma unroll
+        for (int k = 0; k < DP; k += 2) {
+          const int4 b = v[k / 2];
+          const int l0 = u[k].y - b.y, l1 = u[k + 1].y - b.w;
+          S3 += (uint64_t)((int64_t)l0 * l0);
+          S3 += (uint64_t)((int64_t)l1 * l1);
+        }
+        low = S2 + (int64_t)(S3 >> 26);
+      }
       if constexpr (KERN == KMATERN) {
-        const FF q = sqrt_ff(fix_r2_ff(S1, S2 + bias, fs.q));
+        const FF q = sqrt_ff(fix_r2_ff(S1, low, fs.q));
         const FF e = exp_ff({-q.h, -q.l}, cst, cst + 4);
         const FF third = {0.3333333433f, -9.9341077e-09f};
         return ff_mul(ff_add({1.0f, 0.0f}, ff_add(q, ff_mul(ff_mul(q, q), third))), e);
       } else {
-        return fix_exp2_ff(fix_exponent_ff(S1, S2, fs.r, bias, fs.s1_max), tab);
+        return fix_exp2_ff(fix_exponent_ff(S1, low, fs.r, fs.s1_max), tab);
       }
     } else if constexpr (KERN == KMATERN) {
       return fix_matern(S1, S2, S3, fs.r2_scale, tab);
@@ -165,6 +172,8 @@ __device__ __forceinline__ FixScale fix_load_scale(const FixScale *__restrict__ 
   fs.q = scale->q;
   fs.s1_max = scale->s1_max;
   fs.r2_scale = scale->r2_scale;
+  fs.bias = scale->bias;
+  fs.s1_near = scale->s1_near;
   return fs;
 }
 template <typename A, int KERN>
