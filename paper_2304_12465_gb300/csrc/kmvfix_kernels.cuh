@@ -64,9 +64,10 @@ __device__ __forceinline__ FF fix_exp2_ff(uint64_t E, const uint64_t *__restrict
     const float s = __uint_as_float((uint32_t)(127 - 24 - n) << 23);   // 2^(-24 - n)
     return {h * s, l * (s * 0x1p-32f)};
   }
+  // down to the smallest float, both parts (subnormal ones rounded once)
   if (n > 150) return {0.0f, 0.0f};
   const float s = __uint_as_float((uint32_t)(127 + 40 - n) << 23);     // 2^(40 - n)
-  return {(h * 0x1p-64f) * s, n < 100 ? (l * 0x1p-96f) * s : 0.0f};
+  return {(h * 0x1p-64f) * s, (l * 0x1p-96f) * s};
 }
 
 // The squared distance 2^(26 - 2 q) (2^24 S1 + A) as a float-float value (its

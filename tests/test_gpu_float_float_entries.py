@@ -83,3 +83,23 @@ def test_entries(d, kern, e, N, cols):
                 err.append(float(decimal.Decimal(got[c, 8 * g + c]) - want) * 2.0 ** 53)
         dev = 0.137 * np.sqrt(d) * 2.0 ** (2 * e - 3)
         assert np.sqrt(np.mean(np.square(err))) <= 9 + 2 * np.sqrt(d) * 2.0 ** (e - 1) / 2 + 1.5 * dev
+
+
+@pytest.mark.parametrize("kern", [O.GAUSSIAN, O.LAPLACE_L1])
+def test_small_entries(kern):
+    """Down to 2^-148 both floats count: the mantissa's 2^-49, E = 2 sqrt(E) 2^3
+    (Gaussian, e = 3) or 4 (Laplace, e <= 7) units of 2^-53 times ln 2, and the
+    two roundings to subnormal floats, 2^-150 each."""
+    K = require_gpu()
+    decimal.getcontext().prec = 50
+    E = np.linspace(90, 148, 117)
+    x = {O.GAUSSIAN: np.sqrt(2 * np.log(2) * E), O.LAPLACE_L1: np.log(2) * E}[kern]
+    X = np.concatenate([[0.0], x])[:, None]
+    V = np.zeros((1, len(X)))
+    V[0, 0] = 1.0
+    got = K.krr_kmatvec(to_dev(X), kern, 1.0, 0.0, to_dev(V), prec="ff").cpu().numpy()[0]
+    for i in range(1, len(X)):
+        _, want = exact(kern, X[i], X[0], 1.0)
+        rel = (17 + (16 * np.sqrt(E[i - 1]) if kern == O.GAUSSIAN else 4)) * 2.0 ** -53
+        lim = decimal.Decimal(rel) * want + decimal.Decimal(2) ** -149
+        assert abs(decimal.Decimal(got[i]) - want) <= lim, (E[i - 1], got[i])
