@@ -553,26 +553,39 @@ kmvtc5_kernel(const __grid_constant__ CUtensorMap rowmap,
         if (segend) flush(rb);
       }
     } else {
-      // a lane's rows of the two row tiles: packed sums over the even and odd
-      // columns of the current tile (acc), and over the segment's finished
-      // tiles (tot): two-level float32 accumulation, so a long segment (up to
-      // about 1e5 columns per row) adds one tile sum at a time to its running
-      // total instead of one entry at a time
+      // a lane's rows of the two row tiles: packed sums over 32 even and 32 odd
+      // columns (acc) and over the segment's finished tiles (tot): two-level
+      // float32 accumulation, so a long segment (up to about 1e5 columns per
+      // row) adds one sum at a time to its running total instead of one entry at
+      // a time.  With up to two right-hand sides, where ex2 leaves the FMA pipe
+      // idle (1.75 ms either way at N = 1e5, d = 16; with four 2.30 -> 2.35), the
+      // chains are half as long and the tile's sums make a level of their own
+      // (mid): a small product's error is its chains'.
+      constexpr bool FINE = M == 2 && EW == 16;
       float2 acc[T5_RT][M];
-      float tot[T5_RT][M];
+      float mid[T5_RT][FINE ? M : 1], tot[T5_RT][M];
 #pragma unroll
       for (int rt = 0; rt < T5_RT; ++rt)
 #pragma unroll
         for (int c = 0; c < M; ++c) {
           acc[rt][c] = f2(0.0f, 0.0f);
+          if constexpr (FINE) mid[rt][c] = 0.0f;
           tot[rt][c] = 0.0f;
         }
-      auto fold_tile = [&]() {
+      auto fold = [&](bool last) {
 #pragma unroll
         for (int rt = 0; rt < T5_RT; ++rt)
 #pragma unroll
           for (int c = 0; c < M; ++c) {
-            tot[rt][c] += acc[rt][c].x + acc[rt][c].y;
+            if constexpr (FINE) {
+              mid[rt][c] += acc[rt][c].x + acc[rt][c].y;
+              if (last) {
+                tot[rt][c] += mid[rt][c];
+                mid[rt][c] = 0.0f;
+              }
+            } else {
+              tot[rt][c] += acc[rt][c].x + acc[rt][c].y;
+            }
             acc[rt][c] = f2(0.0f, 0.0f);
           }
       };
@@ -612,12 +625,12 @@ kmvtc5_kernel(const __grid_constant__ CUtensorMap rowmap,
       float2 kp[T5_RT * 8];
       const float4 *vp = sV;
       int sp = 0;
-      bool havep = false, p_fold = false, p_last = false, p_segend = false;
+      bool havep = false, p_full = false, p_last = false, p_segend = false;
       int64_t p_rb = 0;
-      auto retire = [&](const float2 *kq, const float4 *vq, int sq, bool fold, bool last,
+      auto retire = [&](const float2 *kq, const float4 *vq, int sq, bool full, bool last,
                         bool segend, int64_t rbq) {
         ffma_batch(kq, vq);
-        if (fold) fold_tile();   // every 64 columns: sums of 32 entries
+        if (full) fold(last);   // every 32 or 64 columns
         if (last) {
           __syncwarp();
           if (lane == 0) bw::mbar_arrive(bar(T5_BAR_V_EMPTY + sq));
@@ -630,7 +643,7 @@ kmvtc5_kernel(const __grid_constant__ CUtensorMap rowmap,
         const bool segend = (p + 1 == p_end) || (ct + 1 == a.C);
         if (TG == 2 && (int)(kt & 1) != tg) {
           if (segend) {
-            if (LAG && havep) retire(kp, vp, sp, p_fold, p_last, p_segend, p_rb);
+            if (LAG && havep) retire(kp, vp, sp, p_full, p_last, p_segend, p_rb);
             havep = false;
             flush(rb);
           }
@@ -679,11 +692,11 @@ kmvtc5_kernel(const __grid_constant__ CUtensorMap rowmap,
           }
           float2 kc[T5_RT * 8];
           kappa_batch(cur, kc);
-          const bool last = bt + 1 == NBT, fold = last || (bt & 3) == 3;
+          const bool last = bt + 1 == NBT, full = last || (FINE ? bt & 1 : (bt & 3) == 3);
           if constexpr (LAG) {
-            if (havep) retire(kp, vp, sp, p_fold, p_last, p_segend, p_rb);
+            if (havep) retire(kp, vp, sp, p_full, p_last, p_segend, p_rb);
           } else {
-            retire(kc, vt + bt * 8, s, fold, last, segend, rb);
+            retire(kc, vt + bt * 8, s, full, last, segend, rb);
           }
           if (PIPE && bt + 1 < NBT) {
             bw::tmem_wait_ld32(r[(bt + 1) & 1]);
@@ -695,14 +708,14 @@ kmvtc5_kernel(const __grid_constant__ CUtensorMap rowmap,
             vp = vt + bt * 8;
             sp = s;
             havep = true;
-            p_fold = fold;
+            p_full = full;
             p_last = last;
             p_segend = last && segend;
             p_rb = rb;
           }
         }
       }
-      if (LAG && havep) retire(kp, vp, sp, p_fold, p_last, p_segend, p_rb);
+      if (LAG && havep) retire(kp, vp, sp, p_full, p_last, p_segend, p_rb);
     }
   }
 
