@@ -94,8 +94,8 @@ __global__ void fix_scale_kernel(const double *__restrict__ part, int blocks, in
   out->bias = out->s1_near = 0;
   if (kern == KLAPLACE) {
     out->limb = 0;
-    out->q = 58 - e;
-    out->r = 4 - e;
+    out->q = kFixL1Bits - e;
+    out->r = kFixL1Bits - 54 - e;
     return;
   }
   out->limb = ff ? kFixFFLimb : kFixLimb;

@@ -11,17 +11,18 @@
 // the kernel into a plain sum, and rounded once to integers:
 //   Gaussian  u = round(2^Q (x - ctr) sqrt(log2 e / 2) / sigma):  E = sum d^2 2^(-2Q)
 //   Matern    u = round(2^Q (x - ctr) sqrt(5) / sigma):           q^2 = sum d^2 2^(-2Q)
-//   Laplace   u = round(2^53 (x - ctr) log2 e / sigma):           E = sum |d| 2^(-53)
+//   Laplace   u = round(2^Q (x - ctr) log2 e / sigma):            E = sum |d| 2^(-Q)
 // with d = u_i - u_j and kappa = 2^-E (Matern: the polynomial times exp(-q)).
 // Gaussian and Matern coordinates have |u| < 2^57 and are kept as limbs
 // u = 2^29 h + l, |l| <= 2^28, so that the three partial sums of squares
 //   S1 = sum dh^2, S2 = sum dh dl, S3 = sum dl^2,  sum d^2 = 2^58 S1 + 2^30 S2 + S3
 // of up to 32 coordinates are exact in 64 bits: five instructions (two
 // subtractions, three multiply-adds) a coordinate.  Laplace coordinates have
-// |u| < 2^58 as plain 64-bit integers.
+// |u| < 2^60 as plain 64-bit integers; their differences are summed over groups
+// of eight, whose two lowest bits are summed apart.
 //
 // Error: the coordinates are rounded once, to 2^-58 of the range's power of
-// two (2^-54 absolute for Laplace); everything after that is exact up to one
+// two (2^-61 for Laplace); everything after that is exact up to one
 // rounding of E at 2^-55 and the mantissa of 2^-E, good to 2^-60, rounded to
 // 53 bits.  Float64 arithmetic rounds every difference, square and sum and E
 // itself at 2^-53 of E.  Point sets whose scaled half-range exceeds
@@ -48,6 +49,13 @@ constexpr int kFixMaxExpGauss = 4, kFixMaxExpMatern = 6, kFixMaxExpLaplace = 5;
 constexpr int kFixFFMaxExpGauss = 4, kFixFFMaxExpMatern = 5, kFixFFMaxExpLaplace = 9;
 constexpr int kFixMinExp = 1;    // a smaller range gains nothing: E is kept at 2^-54
 constexpr int kFixLimb = 29;
+// Fraction bits of Laplace coordinates plus the range's exponent: |u| < 2^60, and
+// eight differences below 2^61 stay within 64 bits.  From the second group on a
+// sum keeps its two lowest bits apart (kFixL1Low): four shifted ones stay within
+// 64 bits too.  With 58 bits and one plain sum, near pairs in 32 dimensions were
+// off by up to 3.8 units of 2^-53 at the widest range, where the float64 formula
+// is off by half a unit.
+constexpr int kFixL1Bits = 60, kFixL1Group = 8, kFixL1Low = 2;
 // The float-float products keep |u| < 2^53 with low limbs of 25 bits and leave
 // out S3 but for its mean over low limbs: what is missing stays below d 2^(2 e
 // - 56) of E (a fifth of 2^(2 e - 56) sqrt(d) in the mean square), and two
@@ -254,6 +262,17 @@ KRR_HD double fix_exp2(uint64_t E, const uint64_t *__restrict__ tab) {
 KRR_HD uint64_t fix_exponent_l1(uint64_t S, int r) {
   if (r < 0) return (S >> (64 + r)) ? ~0ull : S << -r;
   return r > 0 ? (S >> r) + ((S >> (r - 1)) & 1) : S;
+}
+
+// The same from the sums of the groups without their lowest bits (S, at
+// 2^-(54 + r)) and of those bits (L, at 2^-(54 + kFixL1Low + r)).
+KRR_HD uint64_t fix_exponent_l1_groups(uint64_t S, uint32_t L, int r) {
+  S += L >> kFixL1Low;
+  L &= (1u << kFixL1Low) - 1;
+  if (r > 0) return fix_exponent_l1(S, r);
+  if (r == 0) return S + (L >> 1);
+  if (S >> (64 + r)) return ~0ull;
+  return (S << -r) + (r == -1 ? (uint64_t)(L >> 1) : (uint64_t)L << (-r - kFixL1Low));
 }
 
 constexpr double kFixMaternEnd = 708.39;   // 1022 ln 2 = 708.396
