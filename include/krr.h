@@ -188,8 +188,10 @@ KRR_API krr_status krr_rpc_sample(const double *dres, int64_t N, double dfloor,
 /* squared row norms from the residual diagonal; every candidate of a block   */
 /* gets residual 0.  Stops early (rank < k) if every weight becomes zero.     */
 /* Results are float64 throughout: the entries as for KRR_PREC_FP64, the      */
-/* products with F from 57-bit fixed-point digits whose sums are exact, at    */
-/* most as far off as float64 sums.  *F_out receives a new handle (free with  */
+/* products with F from 57-bit digits of rows scaled by their norms, whose    */
+/* sums are exact: off by about 2^-57 of the two rows' norms.  KRR_ETIMEOUT   */
+/* if a bounded device-side wait of those products gave up (likewise for the  */
+/* solves that build a factor).  *F_out receives a new handle (free with      */
 /* krr_factor_free).                                                          */
 /* ------------------------------------------------------------------------ */
 KRR_API krr_status krr_rpcholesky(const double *X, int64_t N, int d, krr_kernel kern,

@@ -7,16 +7,18 @@
 
 namespace krr {
 
-// C (N x nc, ldc) -= A (N x K, lda) B^T for float64 matrices with entries in
-// [-1, 1] whose products' sums stay below 4 in magnitude, on the tensor cores
-// by digits (digits.cuh): row c of B starts at B + rows[c] (rows NULL: B + c)
-// with a step of ldb between its K entries and updates column cmap[c] of C
-// (cmap NULL: c).  img: dig_image_bytes(nc, K) bytes of scratch.  A bounded wait
+// C (N x nc, ldc) -= A (N x K, lda) B^T in float64, on the tensor cores by digits
+// (digits.cuh): row c of B starts at B + rows[c] (rows NULL: B + c) with a step of
+// ldb between its K entries and updates column cmap[c] of C (cmap NULL: c).  an2,
+// bn2: the squared norms of the rows of A and of B (bn2 indexed like the rows), to
+// rounding; they scale the rows, and an entry is off by about 2^-57 of the two
+// norms' product.  img: dig_image_bytes(nc, K) bytes of scratch.  A bounded wait
 // that gives up sets the flag that tc5_check_fault reads.
 size_t dig_image_bytes(int nc, int K);
-krr_status dig_gemm_sub(const double *A, int64_t lda, int64_t N, int K, const double *B,
-                        int64_t ldb, const int64_t *rows, int nc, double *C, int64_t ldc,
-                        const int *cmap, uint4 *img, cudaStream_t s);
+krr_status dig_gemm_sub(const double *A, int64_t lda, int64_t N, int K, const double *an2,
+                        const double *B, int64_t ldb, const int64_t *rows, const double *bn2,
+                        int nc, double *C, int64_t ldc, const int *cmap, uint4 *img,
+                        cudaStream_t s);
 
 // Lower triangle of C (r x r, column-major) = F^T F for F N x r column-major.
 // float F: float32 products summed in float32 over 16-term chunks, the chunk

@@ -36,10 +36,12 @@ constexpr size_t dg_smem(int NC) {
 // ldb between entries) as the kernel's shared tiles hold them: for column group
 // g and step of 16 terms, the seven digits one after the other, each a
 // K-major operand of dg_group_cols rows of 32 bytes in the 32-byte swizzle
-// (zero padded).  A thread makes half a row.
+// (zero padded).  A thread makes half a row.  n2: squared norms of the rows,
+// indexed like them; their scales go to shift.
 __global__ void dig_rows_kernel(const double *__restrict__ B, int64_t ldb,
-                                const int64_t *__restrict__ rows, int nc, int K, int K16,
-                                uint4 *__restrict__ img) {
+                                const int64_t *__restrict__ rows,
+                                const double *__restrict__ n2, int nc, int K, int K16,
+                                uint4 *__restrict__ img, int *__restrict__ shift) {
   const int ncp = (nc + 15) / 16 * 16;
   const int64_t total = (int64_t)K16 * ncp * 2;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
@@ -49,12 +51,14 @@ __global__ void dig_rows_kernel(const double *__restrict__ B, int64_t ldb,
     const int k = step * 16 + half * 8;
     double x[8];
     const int64_t r = c < nc ? (rows ? rows[c] : c) : 0;
+    const int sh = c < nc ? dig_shift(n2[r]) : 0;
+    if (step == 0 && half == 0) shift[c] = sh;
 #pragma unroll
     for (int t = 0; t < 8; ++t)
       x[t] = (c < nc && k + t < K) ? B[r + (int64_t)(k + t) * ldb] : 0.0;
     uint32_t d[4][DIG_N];
 #pragma unroll
-    for (int t = 0; t < 4; ++t) dig_pair(x[2 * t], x[2 * t + 1], d[t]);
+    for (int t = 0; t < 4; ++t) dig_pair(x[2 * t], x[2 * t + 1], sh, d[t]);
     const int g = c / 64, n = c % 64, ncol = dg_group_cols(nc, g);
     uint4 *dst = img + ((int64_t)g * K16 * 64 + (int64_t)step * ncol) * DIG_N * 2;
 #pragma unroll
@@ -64,8 +68,9 @@ __global__ void dig_rows_kernel(const double *__restrict__ B, int64_t ldb,
   }
 }
 
-// C (N x nc, ldc) -= A (N x K, lda) B^T, B as dig_rows_kernel lays it out; cmap
-// (optional) gives the column of C for each row of B.  A CTA takes 128 rows and
+// C (N x nc, ldc) -= A (N x K, lda) B^T, B and its scales as dig_rows_kernel lays
+// them out, an2 the squared norms of A's rows; cmap (optional) gives the column of
+// C for each row of B.  A CTA takes 128 rows and
 // one group of up to NC columns (blockIdx.x: groups of a row tile next to one
 // another, so that the second one finds its rows of A in L2).
 //
@@ -92,7 +97,8 @@ __global__ void dig_rows_kernel(const double *__restrict__ B, int64_t ldb,
 template <int NC>
 __global__ void __launch_bounds__(DG_THREADS, NC == 32 ? 2 : 1)
 dig_gemm_kernel(const double *__restrict__ A, int64_t lda, int64_t N, int K,
-                const uint4 *__restrict__ img, int nc, int groups, double *__restrict__ C,
+                const double *__restrict__ an2, const uint4 *__restrict__ img,
+                const int *__restrict__ bshift, int nc, int groups, double *__restrict__ C,
                 int64_t ldc, const int *__restrict__ cmap, int *fault) {
   constexpr int ST = dg_stages(NC);
   constexpr int STAGE = dg_stage_bytes(NC);
@@ -211,6 +217,7 @@ dig_gemm_kernel(const double *__restrict__ A, int64_t lda, int64_t N, int K,
     const int rl = (warp & 3) * 32 + lane;    // row of the tile, TMEM lane
     const int64_t row = row0 + rl;
     const bool ok = row < N;
+    const int sa = ok ? dig_shift(an2[row]) : 0;
     const int nc2 = ncol / 2;
     const double *Ar = A + row + (int64_t)(8 * half) * lda;
     const uint32_t dst = base + (uint32_t)(rl * 32 + ((half ^ ((rl >> 2) & 1)) * 16));
@@ -296,7 +303,7 @@ dig_gemm_kernel(const double *__restrict__ A, int64_t lda, int64_t N, int K,
       load(step + AHEAD, slot);
       uint32_t d[4][DIG_N];
 #pragma unroll
-      for (int t = 0; t < 4; ++t) dig_pair(x[2 * t], x[2 * t + 1], d[t]);
+      for (int t = 0; t < 4; ++t) dig_pair(x[2 * t], x[2 * t + 1], sa, d[t]);
 #pragma unroll
       for (int q = 0; q < DIG_N; ++q)
         asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(
@@ -318,15 +325,19 @@ dig_gemm_kernel(const double *__restrict__ A, int64_t lda, int64_t N, int K,
         const int c0 = grp * 64 + half * nc2 + cb * 8;
         if (cb * 8 < nc2) {
           double *p[8], v[8];
+          int sb[8];
 #pragma unroll
           for (int i = 0; i < 8; ++i)
             if (c0 + i < nc) {
               p[i] = C + row + (int64_t)(cmap ? cmap[c0 + i] : c0 + i) * ldc;
               v[i] = *p[i];
+              sb[i] = bshift[c0 + i];
             }
 #pragma unroll
           for (int i = 0; i < 8; ++i)
-            if (c0 + i < nc) *p[i] = v[i] - (double)tot[cb * 8 + i] * 0x1p-60;
+            if (c0 + i < nc)   // the total's unit is 2^(-60 - the two rows' scales)
+              *p[i] = v[i] - (double)tot[cb * 8 + i] *
+                                 __hiloint2double((1023 - 60 - sa - sb[i]) << 20, 0);
         }
       }
     }
@@ -339,35 +350,39 @@ dig_gemm_kernel(const double *__restrict__ A, int64_t lda, int64_t N, int K,
   }
 }
 
+// B's digits, then its scales.
 size_t dig_image_bytes(int nc, int K) {
-  return (size_t)((K + 15) / 16) * DIG_N * 32 * ((nc + 15) / 16 * 16);
+  return (size_t)((K + 15) / 16 * DIG_N * 32 + 4) * ((nc + 15) / 16 * 16);
 }
 
 template <int NC>
-static krr_status launch_dig(const double *A, int64_t lda, int64_t N, int K, const uint4 *img,
-                             int nc, double *C, int64_t ldc, const int *cmap, int *fault,
-                             cudaStream_t s) {
+static krr_status launch_dig(const double *A, int64_t lda, int64_t N, int K, const double *an2,
+                             const uint4 *img, const int *bshift, int nc, double *C, int64_t ldc,
+                             const int *cmap, int *fault, cudaStream_t s) {
   KRR_TRY(raise_smem_limit(dig_gemm_kernel<NC>, dg_smem(NC)));
   const int groups = (nc + 63) / 64;
   dig_gemm_kernel<NC><<<(unsigned)(ceil_div(N, DG_ROWS) * groups), DG_THREADS, dg_smem(NC), s>>>(
-      A, lda, N, K, img, nc, groups, C, ldc, cmap, fault);
+      A, lda, N, K, an2, img, bshift, nc, groups, C, ldc, cmap, fault);
   KRR_LAUNCH_CHECK();
   return KRR_OK;
 }
 
-krr_status dig_gemm_sub(const double *A, int64_t lda, int64_t N, int K, const double *B,
-                        int64_t ldb, const int64_t *rows, int nc, double *C, int64_t ldc,
-                        const int *cmap, uint4 *img, cudaStream_t s) {
+krr_status dig_gemm_sub(const double *A, int64_t lda, int64_t N, int K, const double *an2,
+                        const double *B, int64_t ldb, const int64_t *rows, const double *bn2,
+                        int nc, double *C, int64_t ldc, const int *cmap, uint4 *img,
+                        cudaStream_t s) {
   if (N <= 0 || K <= 0 || nc <= 0) return KRR_OK;
   int *fault = tc5_fault_ptr();
   KRR_REQUIRE(fault != nullptr, "digit product: no fault flag on this device");
-  const int K16 = (K + 15) / 16;
-  const int64_t total = (int64_t)K16 * ((nc + 15) / 16 * 16) * 2;
+  const int K16 = (K + 15) / 16, ncp = (nc + 15) / 16 * 16;
+  int *bshift = reinterpret_cast<int *>(img + (size_t)K16 * DIG_N * 2 * ncp);
+  const int64_t total = (int64_t)K16 * ncp * 2;
   dig_rows_kernel<<<(unsigned)std::min<int64_t>((total + 127) / 128, 4 * num_sms()), 128, 0, s>>>(
-      B, ldb, rows, nc, K, K16, img);
+      B, ldb, rows, bn2, nc, K, K16, img, bshift);
   KRR_LAUNCH_CHECK();
-  if (nc <= 32) return launch_dig<32>(A, lda, N, K, img, nc, C, ldc, cmap, fault, s);
-  return launch_dig<64>(A, lda, N, K, img, nc, C, ldc, cmap, fault, s);
+  if (nc <= 32)
+    return launch_dig<32>(A, lda, N, K, an2, img, bshift, nc, C, ldc, cmap, fault, s);
+  return launch_dig<64>(A, lda, N, K, an2, img, bshift, nc, C, ldc, cmap, fault, s);
 }
 
 }  // namespace krr

@@ -302,12 +302,18 @@ __device__ __forceinline__ double div_by(double x, double d, double r) {
 // barriers; the rest is updated by all warps between two barriers.  100
 // candidates took 262 us with three barriers a column, 231 us with the panel in
 // one warp, whose 272 float64 instructions a panel take 67 clocks each, now
-// 187.
+// 187.  n2[a]: squared norm of row a of Lb over the columns before its group of
+// the triangular solve (trsm_group_start).
+constexpr int TRSM_W = 20;   // columns of a group at most, see block_trsm_kernel
+__host__ __device__ inline int trsm_groups(int na) { return (na + TRSM_W - 1) / TRSM_W; }
+__host__ __device__ inline int trsm_group_start(int na, int q) {
+  return (int)((int64_t)na * q / trsm_groups(na));
+}
 constexpr int CHOL_PW = 8;
 __global__ void __launch_bounds__(256)
 block_chol_kernel(const double *__restrict__ G, int64_t ldg, const int64_t *__restrict__ cand,
                   int nc, double thr, double *__restrict__ Lb, int *__restrict__ kept,
-                  int *__restrict__ nkept) {
+                  int *__restrict__ nkept, double *__restrict__ n2) {
   extern __shared__ double sT[];  // nc x (nc + 1), row-major
   __shared__ int s_list[RPC_MAX_BLOCK];
   __shared__ unsigned s_mask;     // kept columns of the panel
@@ -393,22 +399,34 @@ block_chol_kernel(const double *__restrict__ G, int64_t ldg, const int64_t *__re
     const int c = e / na, a = e - c * na;
     Lb[a + (int64_t)c * nc] = (a >= c) ? sT[s_list[a] * ld + s_list[c]] : 0.0;
   }
-  for (int e = tid; e < na; e += blockDim.x) kept[e] = s_list[e];
+  for (int e = tid; e < na; e += blockDim.x) {
+    kept[e] = s_list[e];
+    int q = 0;
+    while (trsm_group_start(na, q + 1) <= e) ++q;
+    const int a0 = trsm_group_start(na, q);
+    double v = 0.0;
+    for (int c = 0; c < a0; ++c) {
+      const double x = sT[s_list[e] * ld + s_list[c]];
+      v = fma(x, x, v);
+    }
+    n2[e] = v;
+  }
   if (tid == 0) *nkept = na;
 }
 
 // Columns a0 .. a0 + w of the new part of F: row n solves x L^T = G(n, kept)
 // over them by forward substitution (G already holds the part of the columns
-// before a0) and writes x to F(n, rank + a0 ..); dres(n) -= |x|^2.  The row
-// stays in registers, so a group is at most TRSM_W columns: the float64 work
-// of a row is w^2 / 2 + 4 w of the na^2 / 2 + 10 na that substitution over all
-// na columns (with divisions) took.
-constexpr int TRSM_W = 20;
+// before a0) and writes x to F(n, rank + a0 ..); dres(n) -= |x|^2.  rn2 and bn2
+// collect |x|^2 over all columns and over this block's, the scales of the products
+// by digits.  The row stays in registers, so a group is at most TRSM_W columns:
+// the float64 work of a row is w^2 / 2 + 4 w of the na^2 / 2 + 10 na that
+// substitution over all na columns (with divisions) took.
 constexpr int TRSM_THREADS = 64;
 __global__ void __launch_bounds__(TRSM_THREADS)
 block_trsm_kernel(const double *__restrict__ G, int64_t ldg, const double *__restrict__ Lb,
                   int nc, const int *__restrict__ kept, int a0, int w, double *__restrict__ F,
-                  int64_t N, int rank, double *__restrict__ dres) {
+                  int64_t N, int rank, double *__restrict__ dres, double *__restrict__ rn2,
+                  double *__restrict__ bn2) {
   __shared__ double sL[TRSM_W][TRSM_W + 1];
   __shared__ double sR[TRSM_W];
   for (int e = threadIdx.x; e < w * w; e += TRSM_THREADS) {
@@ -437,6 +455,8 @@ block_trsm_kernel(const double *__restrict__ G, int64_t ldg, const double *__res
     }
   }
   dres[n] -= s2;
+  rn2[n] += s2;
+  bn2[n] = a0 == 0 ? s2 : bn2[n] + s2;
 }
 
 __global__ void block_finish_kernel(const int64_t *__restrict__ cand, int nc,
@@ -492,7 +512,7 @@ krr_status rpcholesky_device(const double *Xd, int64_t N, int d, int kern, doubl
 
   DevBuf<int64_t> draws, cand;
   DevBuf<int> counts, kept;
-  DevBuf<double> G, Lb;
+  DevBuf<double> G, Lb, rn2, bn2, ln2;   // (squared row norms of F, its new block and Lb)
   DevBuf<uint8_t> img;
   KRR_TRY(draws.alloc(B, s));
   KRR_TRY(cand.alloc(B, s));
@@ -501,6 +521,10 @@ krr_status rpcholesky_device(const double *Xd, int64_t N, int d, int kern, doubl
   KRR_TRY(G.alloc((size_t)N * B, s));
   KRR_TRY(img.alloc(dig_image_bytes(B, std::max(k, B)), s));
   KRR_TRY(Lb.alloc((size_t)B * B, s));
+  KRR_TRY(rn2.alloc((size_t)N, s));
+  KRR_TRY(bn2.alloc((size_t)N, s));
+  KRR_TRY(ln2.alloc((size_t)B, s));
+  KRR_CUDA_TRY(cudaMemsetAsync(rn2.p, 0, sizeof(double) * (size_t)N, s));
 
   KRR_TRY(raise_smem_limit(block_chol_kernel, (size_t)B * (B + 1) * sizeof(double)));
 
@@ -551,22 +575,22 @@ krr_status rpcholesky_device(const double *Xd, int64_t N, int d, int kern, doubl
     // G = A(:, S') - F(:, 0:rank) F(S', 0:rank)^T
     KRR_TRY(kernel_columns_f64(P64, cand.p, nc, G.p, N, s));
     if (rank > 0)
-      KRR_TRY(dig_gemm_sub(f->F, N, N, rank, f->F, N, cand.p, nc, G.p, N, nullptr,
+      KRR_TRY(dig_gemm_sub(f->F, N, N, rank, rn2.p, f->F, N, cand.p, rn2.p, nc, G.p, N, nullptr,
                            reinterpret_cast<uint4 *>(img.p), s));
     block_chol_kernel<<<1, 256, (size_t)nc * (nc + 1) * sizeof(double), s>>>(
-        G.p, N, cand.p, nc, thr, Lb.p, kept.p, counts.p + 2);
+        G.p, N, cand.p, nc, thr, Lb.p, kept.p, counts.p + 2, ln2.p);
     KRR_LAUNCH_CHECK();
     int na = 0;
     KRR_CUDA_TRY(cudaMemcpyAsync(&na, counts.p + 2, sizeof(int), cudaMemcpyDeviceToHost, s));
     KRR_CUDA_TRY(cudaStreamSynchronize(s));
     // equal groups of at most TRSM_W columns
-    const int groups = (na + TRSM_W - 1) / TRSM_W;
-    for (int q = 0; q < groups; ++q) {
-      const int a0 = (int)((int64_t)na * q / groups), w = (int)((int64_t)na * (q + 1) / groups) - a0;
-      KRR_TRY(dig_gemm_sub(f->F + (int64_t)rank * N, N, N, a0, Lb.p + a0, nc, nullptr, w, G.p, N,
-                           kept.p + a0, reinterpret_cast<uint4 *>(img.p), s));
+    for (int q = 0; q < trsm_groups(na); ++q) {
+      const int a0 = trsm_group_start(na, q), w = trsm_group_start(na, q + 1) - a0;
+      KRR_TRY(dig_gemm_sub(f->F + (int64_t)rank * N, N, N, a0, bn2.p, Lb.p + a0, nc, nullptr,
+                           ln2.p + a0, w, G.p, N, kept.p + a0, reinterpret_cast<uint4 *>(img.p),
+                           s));
       block_trsm_kernel<<<ceil_div(N, TRSM_THREADS), TRSM_THREADS, 0, s>>>(
-          G.p, N, Lb.p, nc, kept.p, a0, w, f->F, N, rank, f->dres);
+          G.p, N, Lb.p, nc, kept.p, a0, w, f->F, N, rank, f->dres, rn2.p, bn2.p);
       KRR_LAUNCH_CHECK();
     }
     block_finish_kernel<<<1, 128, 0, s>>>(cand.p, nc, kept.p, counts.p + 2, f->S, rank, f->dres);
