@@ -12,6 +12,7 @@
 #include "kmv.cuh"
 #include "krill.cuh"
 #include "pcg.cuh"
+#include "retry.cuh"
 #include "rpc.cuh"
 #include "solve.cuh"
 
@@ -53,43 +54,58 @@ static thread_local cudaStream_t g_alloc_stream = nullptr;
 void set_alloc_stream(cudaStream_t s) { g_alloc_stream = s; }
 cudaStream_t alloc_stream() { return g_alloc_stream; }
 
-cudaError_t pool_malloc(void **p, size_t bytes, cudaStream_t s) {
+// The library's pool of the current device, made by the first allocation from it
+// (create); NULL: none.
+static cudaMemPool_t device_pool(bool create) {
   constexpr int kMaxDevices = 64;
   static std::mutex mtx;
   static cudaMemPool_t pools[kMaxDevices] = {};
   static bool tried[kMaxDevices] = {};
   int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  cudaMemPool_t pool = nullptr;
-  if (dev >= 0 && dev < kMaxDevices) {
-    std::lock_guard<std::mutex> lk(mtx);
-    if (!tried[dev]) {
-      tried[dev] = true;
-      cudaMemPoolProps props = {};
-      props.allocType = cudaMemAllocationTypePinned;
-      props.location.type = cudaMemLocationTypeDevice;
-      props.location.id = dev;
-      unsigned long long keep = kPoolKeepBytes;
-      cudaMemPool_t np = nullptr;
-      if (cudaMemPoolCreate(&np, &props) == cudaSuccess) {
-        if (cudaMemPoolSetAttribute(np, cudaMemPoolAttrReleaseThreshold, &keep) == cudaSuccess)
-          pools[dev] = np;
-        else
-          cudaMemPoolDestroy(np);
-      }
-      cudaGetLastError();
-    }
-    pool = pools[dev];
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) {
+    cudaGetLastError();
+    return nullptr;
   }
-  if (pool) {
-    e = cudaMallocFromPoolAsync(p, bytes, pool, s);
+  std::lock_guard<std::mutex> lk(mtx);
+  if (create && !tried[dev]) {
+    tried[dev] = true;
+    cudaMemPoolProps props = {};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    unsigned long long keep = kPoolKeepBytes;
+    cudaMemPool_t np = nullptr;
+    if (cudaMemPoolCreate(&np, &props) == cudaSuccess) {
+      if (cudaMemPoolSetAttribute(np, cudaMemPoolAttrReleaseThreshold, &keep) == cudaSuccess)
+        pools[dev] = np;
+      else
+        cudaMemPoolDestroy(np);
+    }
+    cudaGetLastError();
+  }
+  return pools[dev];
+}
+
+static bool pool_trim() {
+  cudaGetLastError();
+  const cudaMemPool_t pool = device_pool(false);
+  if (!pool) return false;
+  cudaMemPoolTrimTo(pool, 0);
+  cudaGetLastError();
+  return true;
+}
+
+cudaError_t pool_malloc(void **p, size_t bytes, cudaStream_t s) {
+  if (const cudaMemPool_t pool = device_pool(true)) {
+    const cudaError_t e = cudaMallocFromPoolAsync(p, bytes, pool, s);
     if (e == cudaSuccess) return e;
-    cudaGetLastError();
-    cudaMemPoolTrimTo(pool, 0);
-    cudaGetLastError();
+    pool_trim();
   }
   return cudaMallocAsync(p, bytes, s);
+}
+
+cudaError_t plain_malloc(void **p, size_t bytes) {
+  return alloc_or_trim(cudaSuccess, [&] { return cudaMalloc(p, bytes); }, [] { return pool_trim(); });
 }
 
 bool is_device_ptr(const void *p) {

@@ -92,10 +92,12 @@ krr_status raise_smem_limit(F *func, size_t bytes) {
 // synchronisation, so a call that allocates a dozen buffers and waits for its
 // result paid 120-160 us for mapping them again (measured; 15 us from this
 // pool).  The pool keeps at most kPoolKeepBytes of unused memory beyond a
-// synchronisation and gives the rest back; when an allocation fails it gives
-// back everything unused and tries the default pool.
+// synchronisation and gives the rest back; when an allocation of the library
+// fails, from the pool or from plain device memory, it gives back everything
+// unused, and the allocation is tried again (from the default pool or plainly).
 constexpr unsigned long long kPoolKeepBytes = 256ull << 20;
 cudaError_t pool_malloc(void **p, size_t bytes, cudaStream_t s);
+cudaError_t plain_malloc(void **p, size_t bytes);
 
 // Stream-ordered scratch owned by one call (freed with cudaFreeAsync).
 template <typename T>
@@ -137,7 +139,7 @@ krr_status dev_alloc(T **p, size_t count) {
   if (count == 0) return KRR_OK;
   cudaStream_t s = alloc_stream();
   if (s) KRR_CUDA_TRY(pool_malloc((void **)p, count * sizeof(T), s));
-  else KRR_CUDA_TRY(cudaMalloc((void **)p, count * sizeof(T)));
+  else KRR_CUDA_TRY(plain_malloc((void **)p, count * sizeof(T)));
   return KRR_OK;
 }
 

@@ -1584,7 +1584,7 @@ static krr_status server_init(krr_server *S) {
     KRR_CUDA_TRY(cudaEventCreateWithFlags(&L.ev_done, cudaEventDisableTiming));
     KRR_CUDA_TRY(cudaEventCreate(&L.ev_t0));
     KRR_CUDA_TRY(cudaEventCreate(&L.ev_t1));
-    KRR_CUDA_TRY(cudaMalloc(&L.table_dev, sizeof(ServeTable)));
+    KRR_CUDA_TRY(plain_malloc((void **)&L.table_dev, sizeof(ServeTable)));
     KRR_CUDA_TRY(cudaMemset(L.table_dev, 0, sizeof(ServeTable)));
     KRR_CUDA_TRY(cudaMallocHost(&L.table_host, sizeof(ServeTable)));
     std::memset(L.table_host, 0, sizeof(ServeTable));
@@ -1603,9 +1603,9 @@ static krr_status server_init(krr_server *S) {
     KRR_CUDA_TRY(cudaStreamCreateWithPriority(&S->s_slot[i], cudaStreamNonBlocking, hi));
     KRR_CUDA_TRY(cudaEventCreateWithFlags(&S->ev_slot[i], cudaEventDisableTiming));
   }
-  KRR_CUDA_TRY(cudaMalloc(&S->init_dev, sizeof(ServeTable) * SERVE_MAX_SLOTS));
-  KRR_CUDA_TRY(cudaMalloc(&S->scalars_dev, sizeof(ServeScalars) * SERVE_MAX_SLOTS));
-  KRR_CUDA_TRY(cudaMalloc(&S->status_dev, sizeof(ServeStatus) * SERVE_MAX_SLOTS));
+  KRR_CUDA_TRY(plain_malloc((void **)&S->init_dev, sizeof(ServeTable) * SERVE_MAX_SLOTS));
+  KRR_CUDA_TRY(plain_malloc((void **)&S->scalars_dev, sizeof(ServeScalars) * SERVE_MAX_SLOTS));
+  KRR_CUDA_TRY(plain_malloc((void **)&S->status_dev, sizeof(ServeStatus) * SERVE_MAX_SLOTS));
   KRR_CUDA_TRY(cudaMemset(S->scalars_dev, 0, sizeof(ServeScalars) * SERVE_MAX_SLOTS));
   KRR_CUDA_TRY(cudaMemset(S->status_dev, 0, sizeof(ServeStatus) * SERVE_MAX_SLOTS));
   KRR_CUDA_TRY(cudaMallocHost(&S->init_host, sizeof(ServeTable) * SERVE_MAX_SLOTS));
