@@ -112,9 +112,9 @@ struct DevBuf {
   krr_status alloc(size_t count, cudaStream_t stream) {
     release();
     s = stream;
-    n = count;
     if (count == 0) return KRR_OK;
     KRR_CUDA_TRY(pool_malloc((void **)&p, count * sizeof(T), stream));
+    n = count;   // 0 after a failure: callers compare n with what they need
     return KRR_OK;
   }
   void release() {
