@@ -10,6 +10,7 @@
 #include <vector>
 
 #include "krr.h"
+#include "rsqrt.cuh"
 
 namespace krr {
 
@@ -237,18 +238,12 @@ __device__ inline T warp_sum(T v) {
 // d = sqrt(p) and r = 1 / d for p > 0.  A float64 instruction of one warp holds
 // its sub-core's float64 pipe for 67 clocks whatever its active lanes, so on
 // the serial path of a factorisation the instruction count is the time: the
-// library's square root and division took about 23 of them.  Here the float32
-// reciprocal square root (2^-22) takes one third-order step (2^-63) and d one
-// residual correction: 9.  Outside float32's range the library functions.
+// library's square root and division took about 23 of them, the steps from the
+// float32 reciprocal square root (2 units of its last place, 2^-22) take 9.
+// Outside float32's range the library functions.
 __device__ __forceinline__ void sqrt_and_inverse(double p, double *d, double *r) {
   if (p > 1e-30 && p < 1e30) {
-    const double y = (double)rsqrtf((float)p);
-    const double t = p * y;
-    const double e = fma(-t, y, 1.0);
-    const double y1 = fma(y * e, fma(e, 0.375, 0.5), y);
-    const double q = p * y1;
-    *d = fma(fma(-q, q, p), 0.5 * y1, q);
-    *r = y1;
+    sqrt_from_estimate(p, (double)rsqrtf((float)p), d, r);
   } else {
     *d = sqrt(p);
     *r = 1.0 / *d;
