@@ -263,6 +263,10 @@ krr_status tc5_wait_selftest(long long budget, cudaStream_t s) {
 }
 
 // ------------------------------------------------------------ reduction
+// Y[c][i] = sum of the partial sums of row i over the CTAs covering its row
+// block (CTA order) and column groups, + lambda V[c][i] when V is given.  With
+// vexp (TV variants) the partial sums of right-hand side c carry the factor
+// 2^(14 + vexp[c]), which is divided out in float64.
 // TV5: the type of V and Y.  flags (optional): {a point outside the split's
 // range (nothing was summed then), a bounded wait gave up}, for one read-back
 // after the product.

@@ -732,19 +732,6 @@ __host__ __device__ inline int t5_cta_of(int64_t p, int64_t T, int G) {
   return (int)(((p + 1) * (int64_t)G + T - 1) / T) - 1;
 }
 
-// Y[c][i] = sum of the partial sums of row i over the CTAs covering its row
-// block (CTA order) and column groups, + lambda V[c][i] when V is given.
-// With vexp (TV variants) the partial sums of right-hand side c carry the
-// factor 2^(14 + vexp[c]), which is divided out in float64.
-__global__ void t5_reduce_kernel(const float *__restrict__ part, int64_t Nr, int m, int M, int C,
-                                 int64_t T, int G, int J, int CG, const int *__restrict__ vexp,
-                                 float lambda, const float *__restrict__ V, int64_t ldv,
-                                 float *__restrict__ Y, int64_t ldy);
-
-}  // namespace krr
-
-namespace krr {
-
 // Epilogue variants of the tcgen05 product: 1 = 8 warps with pipelined TMEM
 // loads, 2 = 16 warps, 3 = 8 warps without the pipelining, 4 = 16 warps with
 // it, 5 = 8 warps, pipelined and software-pipelined by one batch, 6 = 12 warps
