@@ -58,7 +58,7 @@ __global__ void dig_rows_kernel(const double *__restrict__ B, int64_t ldb,
       x[t] = (c < nc && k + t < K) ? B[r + (int64_t)(k + t) * ldb] : 0.0;
     uint32_t d[4][DIG_N];
 #pragma unroll
-    for (int t = 0; t < 4; ++t) dig_pair(x[2 * t], x[2 * t + 1], sh, d[t]);
+    for (int t = 0; t < 4; ++t) dig_pair(x[2 * t], x[2 * t + 1], 1023 - sh, d[t]);
     const int g = c / 64, n = c % 64, ncol = dg_group_cols(nc, g);
     uint4 *dst = img + ((int64_t)g * K16 * 64 + (int64_t)step * ncol) * DIG_N * 2;
 #pragma unroll
@@ -217,7 +217,7 @@ dig_gemm_kernel(const double *__restrict__ A, int64_t lda, int64_t N, int K,
     const int rl = (warp & 3) * 32 + lane;    // row of the tile, TMEM lane
     const int64_t row = row0 + rl;
     const bool ok = row < N;
-    const int sa = ok ? dig_shift(an2[row]) : 0;
+    const int top = 1023 - (ok ? dig_shift(an2[row]) : 0);
     const int nc2 = ncol / 2;
     const double *Ar = A + row + (int64_t)(8 * half) * lda;
     const uint32_t dst = base + (uint32_t)(rl * 32 + ((half ^ ((rl >> 2) & 1)) * 16));
@@ -303,7 +303,7 @@ dig_gemm_kernel(const double *__restrict__ A, int64_t lda, int64_t N, int K,
       load(step + AHEAD, slot);
       uint32_t d[4][DIG_N];
 #pragma unroll
-      for (int t = 0; t < 4; ++t) dig_pair(x[2 * t], x[2 * t + 1], sa, d[t]);
+      for (int t = 0; t < 4; ++t) dig_pair(x[2 * t], x[2 * t + 1], top, d[t]);
 #pragma unroll
       for (int q = 0; q < DIG_N; ++q)
         asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(
@@ -337,7 +337,7 @@ dig_gemm_kernel(const double *__restrict__ A, int64_t lda, int64_t N, int K,
           for (int i = 0; i < 8; ++i)
             if (c0 + i < nc)   // the total's unit is 2^(-60 - the two rows' scales)
               *p[i] = v[i] - (double)tot[cb * 8 + i] *
-                                 __hiloint2double((1023 - 60 - sa - sb[i]) << 20, 0);
+                                 __hiloint2double((top - 60 - sb[i]) << 20, 0);
         }
       }
     }

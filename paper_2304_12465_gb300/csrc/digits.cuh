@@ -47,25 +47,25 @@ __device__ __forceinline__ int dig_shift(double n2) {
   return min((1022 - e) >> 1, DIG_MAX_SHIFT);
 }
 
-// round(2^(56 + s) x) + bias, |2^s x| < 2 (0 + bias for |2^s x| < 2^-57): the
-// mantissa as 2^5 times an integer, shifted right by the exponent's distance from
-// 2 with one bit left, rounded there.
-__device__ __forceinline__ uint64_t dig_fixed(double x, int s, uint64_t bias) {
+// round(2^(56 + s) x) + bias, top = 1023 - s, |2^s x| < 2 (0 + bias for |2^s x| <
+// 2^-57): the mantissa as 2^5 times an integer, shifted right by the exponent's
+// distance from 2 with one bit left, rounded there.
+__device__ __forceinline__ uint64_t dig_fixed(double x, int top, uint64_t bias) {
   const uint64_t b = (uint64_t)__double_as_longlong(x);
   const int e = (int)(b >> 52) & 0x7ff;
   const uint64_t m5 = ((b & ((1ull << 52) - 1)) | (1ull << 52)) << 5;
   // (beyond 2, infinities and NaN: 0, without an undefined shift)
-  const uint64_t v = ((m5 >> min((unsigned)(1023 - e - s), 63u)) + 1) >> 1;
+  const uint64_t v = ((m5 >> min((unsigned)(top - e), 63u)) + 1) >> 1;
   return (int64_t)b < 0 ? bias - v : bias + v;
 }
 
 // The digits of two entries of rows scaled by 2^s as fp16 pairs (x0 low, x1
-// high): out[q] for digit q.
-__device__ __forceinline__ void dig_pair(double x0, double x1, int s, uint32_t (&out)[DIG_N]) {
+// high): out[q] for digit q.  top = 1023 - s.
+__device__ __forceinline__ void dig_pair(double x0, double x1, int top, uint32_t (&out)[DIG_N]) {
   // a bias of 128 in every digit's place (512 in the leading one's) makes the
   // digits plain bytes
   const uint64_t bias = 0x0200808080808080ull;
-  const uint64_t w0 = dig_fixed(x0, s, bias), w1 = dig_fixed(x1, s, bias);
+  const uint64_t w0 = dig_fixed(x0, top, bias), w1 = dig_fixed(x1, top, bias);
   const uint32_t l0 = (uint32_t)w0, l1 = (uint32_t)w1;
   const uint32_t h0 = (uint32_t)(w0 >> 32), h1 = (uint32_t)(w1 >> 32);
   const __half2 off = __half2half2(__ushort_as_half((unsigned short)0x6480));   // 1152

@@ -94,8 +94,8 @@ __global__ void fix_scale_kernel(const double *__restrict__ part, int blocks, in
   out->bias = out->s1_near = 0;
   if (kern == KLAPLACE) {
     out->limb = 0;
-    out->q = kFixL1Bits - e;
-    out->r = kFixL1Bits - 54 - e;
+    out->q = (ff ? kFixFFL1Bits : kFixL1Bits) - e;
+    out->r = out->q - 54;
     return;
   }
   out->limb = ff ? kFixFFLimb : kFixLimb;

@@ -54,8 +54,10 @@ constexpr int kFixLimb = 29;
 // sum keeps its two lowest bits apart (kFixL1Low): four shifted ones stay within
 // 64 bits too.  With 58 bits and one plain sum, near pairs in 32 dimensions were
 // off by up to 3.8 units of 2^-53 at the widest range, where the float64 formula
-// is off by half a unit.
+// is off by half a unit.  The float-float values, 8 units apart, keep 58 bits and
+// one sum.
 constexpr int kFixL1Bits = 60, kFixL1Group = 8, kFixL1Low = 2;
+constexpr int kFixFFL1Bits = 58;
 // The float-float products keep |u| < 2^53 with low limbs of 25 bits and leave
 // out S3 but for its mean over low limbs: what is missing stays below d 2^(2 e
 // - 56) of E (a fifth of 2^(2 e - 56) sqrt(d) in the mean square), and two

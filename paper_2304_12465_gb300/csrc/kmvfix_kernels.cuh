@@ -107,6 +107,8 @@ __device__ __forceinline__ typename A::T fix_kappa(const int2 (&u)[DP],
                                                    const uint64_t *__restrict__ tab,
                                                    const float *__restrict__ cst) {
   if constexpr (KERN == KLAPLACE) {
+    // the float64 sums of more than one group of coordinates keep their lowest bits
+    constexpr bool GROUPS = DP > kFixL1Group && !A::kFF;
     uint64_t S = 0, G = 0;   // sums of the groups before without their low bits
     uint32_t L = 0;          // (those apart), and of the present one
 #pragma unroll
@@ -117,15 +119,15 @@ __device__ __forceinline__ typename A::T fix_kappa(const int2 (&u)[DP],
       const int64_t d1 = (int64_t)(((uint64_t)(uint32_t)u[k + 1].y << 32) | (uint32_t)u[k + 1].x) -
                          (int64_t)(((uint64_t)(uint32_t)b.w << 32) | (uint32_t)b.z);
       G += (uint64_t)llabs(d0) + (uint64_t)llabs(d1);
-      if constexpr (DP > kFixL1Group)
+      if constexpr (GROUPS)
         if ((k + 2) % kFixL1Group == 0 || k + 2 == DP) {
           S += G >> kFixL1Low;
           L += (uint32_t)G & ((1u << kFixL1Low) - 1);
           G = 0;
         }
     }
-    const uint64_t E = DP > kFixL1Group ? fix_exponent_l1_groups(S, L, fs.r - kFixL1Low)
-                                        : fix_exponent_l1(G, fs.r);
+    const uint64_t E = GROUPS ? fix_exponent_l1_groups(S, L, fs.r - kFixL1Low)
+                              : fix_exponent_l1(G, fs.r);
     if constexpr (A::kFF) return fix_exp2_ff(E, tab);
     else return fix_exp2(E, tab);
   } else {

@@ -307,7 +307,7 @@ __device__ __forceinline__ double div_by(double x, double d, double r) {
 constexpr int TRSM_W = 20;   // columns of a group at most, see block_trsm_kernel
 __host__ __device__ inline int trsm_groups(int na) { return (na + TRSM_W - 1) / TRSM_W; }
 __host__ __device__ inline int trsm_group_start(int na, int q) {
-  return (int)((int64_t)na * q / trsm_groups(na));
+  return na * q / trsm_groups(na);   // na <= 128
 }
 constexpr int CHOL_PW = 8;
 __global__ void __launch_bounds__(256)
@@ -399,17 +399,23 @@ block_chol_kernel(const double *__restrict__ G, int64_t ldg, const int64_t *__re
     const int c = e / na, a = e - c * na;
     Lb[a + (int64_t)c * nc] = (a >= c) ? sT[s_list[a] * ld + s_list[c]] : 0.0;
   }
-  for (int e = tid; e < na; e += blockDim.x) {
-    kept[e] = s_list[e];
-    int q = 0;
-    while (trsm_group_start(na, q + 1) <= e) ++q;
-    const int a0 = trsm_group_start(na, q);
+  for (int e = tid; e < na; e += blockDim.x) kept[e] = s_list[e];
+  {
+    // two threads a row (256 threads, at most 128 rows)
+    const int e = tid >> 1;
     double v = 0.0;
-    for (int c = 0; c < a0; ++c) {
-      const double x = sT[s_list[e] * ld + s_list[c]];
-      v = fma(x, x, v);
+    if (e < na) {
+      int a0 = 0;
+      for (int q = 1; trsm_group_start(na, q) <= e; ++q) a0 = trsm_group_start(na, q);
+      const double *row = sT + s_list[e] * ld;
+#pragma unroll 8
+      for (int c = tid & 1; c < a0; c += 2) {
+        const double x = row[s_list[c]];
+        v = fma(x, x, v);
+      }
     }
-    n2[e] = v;
+    v += __shfl_xor_sync(0xffffffffu, v, 1);
+    if (e < na && (tid & 1) == 0) n2[e] = v;
   }
   if (tid == 0) *nkept = na;
 }
