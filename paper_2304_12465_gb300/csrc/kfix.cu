@@ -91,7 +91,8 @@ __global__ void fix_scale_kernel(const double *__restrict__ part, int blocks, in
   out->s_lo = s_lo;
   out->s1_max = 0;
   out->r2_scale = 0.0;
-  out->bias = out->s1_near = 0;
+  out->bias = 0;
+  out->s1_near = 0;
   if (kern == KLAPLACE) {
     out->limb = 0;
     out->q = (ff ? kFixFFL1Bits : kFixL1Bits) - e;
@@ -110,7 +111,7 @@ __global__ void fix_scale_kernel(const double *__restrict__ part, int blocks, in
     // 2^50 / 6 a coordinate (padded coordinates have none); 2^50 S1 is worth
     // 2^(2 e - 56) S1
     out->bias = (int64_t)d * (1 << 24) / 6;
-    out->s1_near = 1LL << (56 - 2 * e - kFixNearExp);
+    out->s1_near = 1u << (56 - 2 * e - kFixNearExp - 32);
   }
 }
 

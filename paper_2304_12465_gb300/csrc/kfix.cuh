@@ -76,8 +76,8 @@ struct FixScale {
   double s_hi, s_lo;     // scale factor as an unevaluated sum
   double r2_scale;       // Matern: 2^(30 - 2 q)
   int64_t s1_max;        // Gaussian: see fix_exponent
-  int64_t bias, s1_near; // float-float products: mean of S3 2^-26; limit of S1
-                         // below which S3 is formed
+  int64_t bias;          // float-float products: mean of S3 2^-26
+  uint32_t s1_near;      // and the limit of S1 2^-32 below which S3 is formed
   int q;                 // fraction bits of u
   int r;                 // right shift to 54 fraction bits (Gaussian, Laplace)
   int limb;              // bits of the low limb (0: whole 64-bit integers)
