@@ -115,16 +115,19 @@ typedef struct {
 /* ------------------------------------------------------------------------ */
 /* Fused matrix-free product (Alg. 1 "Product"):                             */
 /*   Y = (A + lambda I) V,  A_ij = kappa(x_i, x_j), never stored.            */
-/* precision KRR_PREC_FP64 evaluates entries to float64 accuracy, in fixed   */
-/* point where the points' range allows it (differences of coordinates       */
-/* rounded once to 57 bits of the range, exact squared distances) and in     */
-/* float64 with direct differences elsewhere, and sums in float64;           */
-/* KRR_PREC_MIXED evaluates kernel tiles in float32 (distances from row      */
-/* norms of centred points) and accumulates in float32 -- for the Gaussian   */
-/* and Matern kernels by default with the inner products on the tensor cores */
+/* precision KRR_PREC_FP64 evaluates entries to float64 accuracy and sums in  */
+/* float64.  Entries are formed in fixed point (coordinates rounded once to 57*/
+/* bits of the range, exact squared distances; values below 2^-1021, Matern   */
+/* ones below 1e-302, are 0) where half the range of every coordinate is at   */
+/* most 18 sigma (Gaussian), 22 (Laplace) or 28 (Matern), else in float64 with*/
+/* direct differences: one point beyond sends the whole set to those kernels. */
+/* KRR_PREC_MIXED evaluates kernel tiles in float32 (distances from row       */
+/* norms of centred points) and accumulates in float32 -- for the Gaussian    */
+/* and Matern kernels by default with the inner products on the tensor cores  */
 /* (see krr_set_product_path), prepared once per call (synchronises stream);  */
-/* KRR_PREC_FLOAT_FLOAT evaluates entries in fixed point likewise (float-    */
-/* float elsewhere) and sums in float-float arithmetic (~2^-46 per entry).   */
+/* KRR_PREC_FLOAT_FLOAT evaluates entries in fixed point likewise (half-ranges*/
+/* of 18, 354 and 14 sigma; float-float elsewhere) and sums in float-float    */
+/* arithmetic (about 2^-46 per entry; equal points give exactly 1).           */
 /* V, Y: N x m column-major float64.  Y may not alias V.                     */
 /* ------------------------------------------------------------------------ */
 KRR_API krr_status krr_kmatvec(const double *X, int64_t N, int d, krr_kernel kern,
@@ -153,8 +156,9 @@ KRR_API krr_status krr_kmatvec_batched(const double *X, int64_t N, int d, int S,
 /* Prediction at test points (Sec. 2.1: f(x) = sum_i alpha_i K(x_i, x)):      */
 /*   out (Nt x m) = K(Xtest, Xtrain) alpha,  alpha N x m.                     */
 /* Xtrain N x d and Xtest Nt x d row-major.  KRR_PREC_FP64 evaluates entries  */
-/* in float64; KRR_PREC_MIXED in float32 tiles with float32 accumulation     */
-/* (both point sets centred on the training mean).                           */
+/* to float64 accuracy as for krr_kmatvec (one range for both point sets);    */
+/* KRR_PREC_MIXED in float32 tiles with float32 accumulation (both point sets */
+/* centred on the training mean).                                             */
 /* ------------------------------------------------------------------------ */
 KRR_API krr_status krr_predict(const double *Xtrain, int64_t N, int d, krr_kernel kern,
                                double sigma, const double *alpha, int m,
@@ -600,8 +604,9 @@ KRR_API krr_status krr_set_product_path(int path);
 /* Epilogue variant of the tcgen05 product (KRR_PRODUCT_TENSOR): 0 (default)  */
 /* = chosen per shape by the autotuner while krr_set_autotune is on (every    */
 /* valid variant timed once on the caller's stream at the first product of    */
-/* the shape), else variant 3 (9 for 5..8 right-hand sides per launch of a    */
-/* square product).  Variants 1..7 sum over the right-hand sides with FFMA2   */
+/* the shape), else 9 for square products of 5 or more right-hand sides per   */
+/* launch, 3 for rectangular ones of 5 to 8 and for Gaussian products of 3 or */
+/* 4 with d <= 16, and 2 otherwise.  Variants 1..7 sum over the right-hand sides with FFMA2   */
 /* on the FMA pipe: 1 = 8 epilogue warps with the next columns' Tensor Memory */
 /* loads in flight while the current ones are computed; 2 = 16 epilogue       */
 /* warps; 3 = 8 warps without that overlap; 4 = 16 warps with it; 5 = 8       */
