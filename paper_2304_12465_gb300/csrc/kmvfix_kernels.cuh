@@ -202,10 +202,20 @@ __device__ __forceinline__ void fix_load_tables(const ExpFFConsts &ec, uint64_t 
   }
 }
 
+// CTAs a SM that a rectangular product of one or two right-hand sides keeps room
+// for (1: the compiler's choice).  The branch of the float-float near pairs takes 8
+// to 36 registers more than the rest and would cost one or two of them: 4e5 points,
+// one right-hand side, 2000 columns, d = 20: 8.30 ms, 7.96 with the limit (7.75
+// without near pairs); 1000 columns, d = 16: 3.73 and 3.47.
+__host__ __device__ constexpr int kmvfix_min_ctas(bool ff, int DP, int M) {
+  if (!ff || M > 2 || DP <= 4) return 1;
+  return DP <= 8 ? 7 : DP <= 16 ? 4 : DP <= 20 ? 7 : DP <= 24 ? 6 : 5;
+}
+
 // part[split][c][row] = sum over the split's columns of kappa v; ur (Nr x DP),
 // uc (N x DP): coordinates of rows and columns.
 template <typename A, int KERN, int DP, int M>
-__global__ void __launch_bounds__(KFIX_THREADS)
+__global__ void __launch_bounds__(KFIX_THREADS, kmvfix_min_ctas(A::kFF, DP, M))
 kmvfix_kernel(const int2 *__restrict__ ur, int64_t Nr, const int2 *__restrict__ uc,
               const FixScale *__restrict__ scale, const double *__restrict__ V, int64_t ldv,
               int64_t N, int m, int64_t chunk, const ExpFFConsts ec, double *__restrict__ part) {
